@@ -381,7 +381,9 @@ tbsci_status tbsci_davidson(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *
  * 0..l_b-1. Determinant (w, u) has the compressed index off[w] + (position of
  * u in I_w); vectors on a pruned space are DEVICE arrays [nvec][off[l_a]].
  * H on the space is the principal submatrix of H on its determinants. Arrays
- * are copied. Errors: EINVAL (null pointers, a malformed CSR, an index out of
+ * are copied. Where at most 16 distinct sets I_w occur (irreps, excitation
+ * levels) the links between those sets are listed here, once, on the device
+ * (within an eighth of what is left of a budget). Errors: EINVAL (null pointers, a malformed CSR, an index out of
  * range or not ascending), ENOMEM, ECUDA. */
 typedef struct tbsci_pruned tbsci_pruned;
 tbsci_status tbsci_pruned_create(tbsci_ctx *ctx, const tbsci_tables *a, const tbsci_tables *b, const int64_t *off,

@@ -275,6 +275,21 @@ struct tbsci_pruned {
     tbsci::DevBuf<int32_t> d_rows;  // alpha rows ordered by work (descending)
     std::vector<int64_t> h_off;
     size_t charged = 0;
+    // Classes of alpha rows with equal I_w (none when ncls == 0): the links of every
+    // class's columns into every class's columns, as positions in the compressed rows,
+    // in sliced-ELL slices of 32 consecutive members (see pruned.cu).
+    int ncls = 0, cmax = 0;              // classes, members of the largest
+    tbsci::DevBuf<int32_t> d_cls;        // class of each alpha row
+    tbsci::DevBuf<int64_t> d_cbeg;       // [ncls] where a row of the class starts in d_cols
+    tbsci::DevBuf<int32_t> d_ccnt;       // [ncls] members
+    tbsci::DevBuf<int32_t> d_pos;        // [ncls][lb] member index of a column, or -1
+    tbsci::DevBuf<int> d_ov;             // [ncls][ncls] bit 0: a column in common, bit 1: a single link
+    tbsci::DevBuf<int64_t> d_sbase, d_dbase;  // first slice of (class, target class) / of a class
+    tbsci::DevBuf<int64_t> d_s_off, d_d_off;
+    tbsci::DevBuf<int32_t> d_s_w, d_d_w;
+    tbsci::DevBuf<uint32_t> d_s_ci;      // member index << 13 | 2 pair + (sign < 0)
+    tbsci::DevBuf<int32_t> d_s_li;       // the link's place in the space's single links (-1: padding)
+    tbsci::DevBuf<int2> d_d_ent;         // doubles: member index, place in the double links (-1: padding)
 };
 
 struct tbsci_ham {

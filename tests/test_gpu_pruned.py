@@ -184,3 +184,42 @@ def test_pruned_edge_cases_and_errors(tb, ctx):
             sp.prune(off, cols)
         assert err.value.status == tb.TBSCI_EINVAL
     sp.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("sizes,kernel", [
+    ((33,), "k_sigma_classes"),                        # one class, one member past a slice of 32
+    ((0, 1, 257), "k_sigma_classes"),                  # empty rows, single members, past one sweep of 256 threads
+    ((1100, 64, 7), "k_sigma_classes"),                # 512-thread rows beside short ones
+    (tuple(range(20, 36)), "k_sigma_classes"),         # as many classes as are taken
+    (tuple(range(20, 37)), "k_sigma_pruned"),          # one more: the general kernel
+])
+def test_pruned_row_classes(tb, ctx, sizes, kernel, dtype):
+    """Alpha rows drawn from a few sets I_w (random beta indices, unrelated sets):
+    the kernel for rows in classes, and the general one for more sets, against the
+    oracle with three vectors."""
+    import torch
+    n, na, nb = 13, 6, 6
+    rng = np.random.default_rng(len(sizes) * 100 + sizes[-1])
+    h, eri, _ = synth_hamiltonian(n, seed=601)
+    asel, bsel = selected_strings(n, na, 60, 602), selected_strings(n, nb, 1200, 603)
+    sp = tb.Space(ctx, n, na, nb, h, eri, 0.3, alpha=asel, beta=bsel)
+    osp = oracle.make_space(n, na, nb, asel, bsel)
+    sets = [np.sort(rng.choice(sp.lb, k, replace=False)).astype(np.int32) for k in sizes]
+    rows = [sets[k % len(sets)] for k in rng.permutation(sp.la)]
+    off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64)
+    pr = sp.prune(off, np.concatenate(rows))
+    ops = oracle.PrunedSpace(osp, off, np.concatenate(rows))
+    tdt = torch.float64 if dtype == "f64" else torch.float32
+    C = torch.from_numpy(rng.standard_normal((3, pr.ndet))).to(tdt).cuda()
+    tb.tbsci_trace_enable(ctx.handle, True)
+    s = pr.sigma(C)
+    tb.tbsci_trace_enable(ctx.handle, False)
+    assert {k for k, _ in tb.tbsci_trace_read(ctx.handle)[0]} == {kernel}
+    ref, bound = oracle.sigma_pruned(ops, h, eri, 0.3, C.double().cpu().numpy(), with_bound=True)
+    if dtype == "f64":
+        assert_sigma_close(s.cpu().numpy(), ref, bound)
+    else:
+        assert_sigma_close(s.double().cpu().numpy(), ref, bound, rel=64 * 2.0 ** -24, norm_rel=1e-5)
+    pr.close()
+    sp.close()
