@@ -12,8 +12,8 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libtbsci.so")
 SOURCES = ["api.cu", "strings_tables.cu", "plan.cu", "sigma.cu", "davidson.cu", "server.cu", "sigma_tc.cu",
-           "pruned.cu", "sigma_split.cu", "select.cu", "sigma_dense.cu"]
-HEADERS = [os.path.join(CSRC, "internal.cuh"), os.path.join(ROOT, "include", "tbsci.h")]
+           "pruned.cu", "sigma_split.cu", "select.cu", "sigma_dense.cu", "sigma_exact.cu"]
+HEADERS = [os.path.join(CSRC, "internal.cuh"), os.path.join(CSRC, "tensor.cuh"), os.path.join(ROOT, "include", "tbsci.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "-I" + os.path.join(ROOT, "include")]

@@ -7,6 +7,7 @@
 
 #include <array>
 #include <atomic>
+#include <functional>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -217,6 +218,9 @@ struct DenseSameSpin {
     DevBuf<unsigned char> scratch;  // padded split vector and product
 };
 
+struct ExactData;  // sigma_exact.cu
+struct AbPlanes;   // sigma_tc.cu
+
 struct Plan {
     uint64_t ida = 0, idb = 0;
     int norb = 0, npair = 0;
@@ -244,6 +248,12 @@ struct Plan {
     int npoff = 0;
     DevBuf<int32_t> d_lbp, d_offpair;
     DevBuf<int> d_tc_err;
+    // their links by tile of 64 source columns (see sigma_tc.cu); tl_kpmax = 0: none
+    DevBuf<uint4> d_tl_pos;
+    DevBuf<int2> d_tl_piece;
+    DevBuf<int> d_tl_rounds;
+    int tl_nslot = 0, tl_npiece = 0, tl_kpmax = 0;
+    std::shared_ptr<AbPlanes> ab[2];  // one BF16 plane per operand, three
     // autotuned launch shape per sigma type (index = tbsci_dtype F64 / F32): threads per CTA, vectors per CTA
     int tune_threads[2] = {0, 0}, tune_nv[2] = {0, 0}, tune_stage[2] = {0, 0};
     // autotuned SIMT pass of the tensor-core sigma types (shared-memory mode, threads; 0 = default)
@@ -258,6 +268,7 @@ struct Plan {
     DevBuf<int32_t> d_bss_col;
     DevBuf<float> d_bss_valf;
     DenseSameSpin dense;
+    std::shared_ptr<ExactData> exact;  // tables of the exact tensor-core path, made on first use
     tbsci_sigma_counts counts{};
     size_t charged = 0;  // device bytes counted against the context's budget
 };
@@ -373,10 +384,20 @@ tbsci_status rest_products_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P,
 tbsci_status rest_dense_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const float *c, float *s, int nvec,
                                bool bf16, cudaStream_t st);
 void dense_context_release(tbsci_ctx *ctx);
-// sigma_tc.cu: the diagonal, alpha singles and all alpha-beta classes on the
-// tensor cores (3xTF32 or BF16 products, FP32 accumulation), added into s.
-tbsci_status sigma_tc_add(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan, const float *c, float *s, int nvec,
-                          bool bf16, cudaStream_t st);
+// sigma_exact.cu: FP64 / FP32 sigma summed exactly on the tensor cores (norb <= 16);
+// *ran = false where it does not apply. simt(v, skip) launches the SIMT sigma of
+// vector v, which returns at once where *skip (device memory) is set.
+tbsci_status exact_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const double *c, double *s, int nvec,
+                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, const int *)> &simt);
+tbsci_status exact_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const float *c, float *s, int nvec,
+                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, const int *)> &simt);
+tbsci_status udiag_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, const float *c, float *s, bool add,
+                          bool singles, cudaStream_t st);
+// sigma_tc.cu: the alpha-beta classes on the tensor cores with np = 1 or 3 BF16 planes
+// per operand, FP32 accumulation, added into s
+tbsci_status tile_links_build(tbsci_ctx *ctx, Plan *P, cudaStream_t st);
+tbsci_status sigma_tc_prepare(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int np, cudaStream_t st, bool *ready);
+tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, const int *info, cudaStream_t st);
 tbsci_status diagonal_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan, double *diag,
                              cudaStream_t st);
 

@@ -232,6 +232,7 @@ size_t plan_device_bytes(const Plan &P) {
          P.d_s2_valf.bytes() + P.d_d2_valf.bytes() + P.d_d2_col.bytes();
     b += P.d_U1.bytes() + P.d_U2.bytes() + P.d_Eb2.bytes() + P.d_U1f.bytes() + P.d_U2f.bytes() + P.d_Eb2f.bytes();
     b += P.d_rowsa.bytes() + P.d_pairs.bytes() + P.d_lbp.bytes() + P.d_offpair.bytes() + P.d_tc_err.bytes();
+    b += P.d_tl_pos.bytes() + P.d_tl_piece.bytes() + P.d_tl_rounds.bytes();
     return b;
 }
 
@@ -395,6 +396,7 @@ tbsci_status plan_get(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *a, con
             TB_CUDA(ctx, cudaMemcpy(plan->d_offpair.p, op.data(), op.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
             TB_CUDA(ctx, plan->d_tc_err.alloc(1));
             TB_CUDA(ctx, cudaMemsetAsync(plan->d_tc_err.p, 0, sizeof(int), st));
+            TB_TRY(tile_links_build(ctx, plan.get(), st));
         }
     }
     // work counts: non-zeros of H by class (Sec. II.C, Table I)

@@ -61,6 +61,7 @@ struct SigArgs {
     const T *s2_val, *d2_val;
     const int32_t *d2_col;
     const T *U1, *U2, *Eb2;
+    const int *skip;  // device flag: nothing to do where it is set (NULL: none)
 };
 
 // One alpha row Ia of sigma (the whole body of a CTA). REST: only the classes
@@ -304,6 +305,7 @@ __device__ __forceinline__ void sigma_row(const SigArgs<T> &A, const int64_t Ia,
 template <typename T, int NV, bool STAGE, bool ACCS, int kThreads, bool REST = false>
 __global__ void __launch_bounds__(kThreads) k_sigma(SigArgs<T> A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (A.skip && *A.skip) return;
     sigma_row<T, NV, STAGE, ACCS, kThreads, REST>(A, A.rowsa[blockIdx.x], smem_raw);
 }
 
@@ -509,8 +511,9 @@ tbsci_status launch_nv(tbsci_ctx *ctx, SigArgs<T> A, cudaStream_t st, int thread
 template <typename T>
 tbsci_status launch_typed(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, const T *c, T *s, int nvec,
                           cudaStream_t st, int nv_max = 0, int threads = 0, int stage = -1,
-                          const int32_t *rows = nullptr, int64_t nrows = 0) {
+                          const int32_t *rows = nullptr, int64_t nrows = 0, const int *skip = nullptr) {
     SigArgs<T> A = make_args<T>(ham, P);
+    A.skip = skip;
     if (A.la == 0 || A.lb == 0) return TBSCI_OK;
     const int ti = sizeof(T) == 8 ? 0 : 1;
     if (nv_max == 0 && P->tune_nv[ti] > 0) {
@@ -848,7 +851,7 @@ tbsci_status sigma_autotune(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *plan, co
     const int64_t la = plan->A.l, lb = plan->B.l;
     if (la == 0 || lb == 0 || nvec <= 0) return TBSCI_OK;
     if (dt == TBSCI_F32_TC_TF32 || dt == TBSCI_F32_TC_BF16) {
-        if (plan->npoff > 128 || !plan->d_lbp.p) dt = TBSCI_F32;  // these run on the SIMT path
+        if (plan->tl_kpmax == 0) dt = TBSCI_F32;  // these run on the SIMT path
         else return autotune_rest(ctx, ham, plan, static_cast<const float *>(c), static_cast<float *>(s), nvec, dt,
                                   st, best_ms);
     }
@@ -976,8 +979,14 @@ tbsci_status sigma_autotune(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *plan, co
         plan->tune_nv[ti] = bn;
         plan->tune_stage[ti] = bs;
         // the chosen shape on the whole space: leaves sigma computed, and its time
+        for (int rep = 0; rep < 2 && ret == TBSCI_OK; ++rep) {
+            ret = cu(cudaEventRecord(e0, st));
+            if (ret == TBSCI_OK) ret = sigma_launch(ctx, ham, plan, c, s, nvec, dt, st);
+            if (ret == TBSCI_OK) ret = cu(cudaEventRecord(e1, st));
+            if (ret == TBSCI_OK) ret = cu(cudaEventSynchronize(e1));
+        }
         float ms = 0.f;
-        ret = trial(0, 0, -1, nullptr, 0, 1, &ms);
+        if (ret == TBSCI_OK) ret = cu(cudaEventElapsedTime(&ms, e0, e1));
         if (ret == TBSCI_OK && best_ms) *best_ms = ms;
     }
     cudaEventDestroy(e0);
@@ -1096,19 +1105,43 @@ tbsci_status sigma_launch_rest(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan 
     return TBSCI_OK;
 }
 
+namespace {
+
+// FP64 / FP32: the exact tensor-core path where it applies, else the SIMT kernels
+template <typename T>
+tbsci_status launch_full(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan, const T *c, T *s, int nvec,
+                         cudaStream_t st) {
+    const size_t n = (size_t)plan->A.l * plan->B.l;
+    bool ran = false;
+    TB_TRY(exact_launch(ctx, ham, const_cast<Plan *>(plan), c, s, nvec, st, &ran, [&](int v, const int *skip) {
+        return launch_typed<T>(ctx, ham, plan, c + v * n, s + v * n, 1, st, 0, 0, -1, nullptr, 0, skip);
+    }));
+    return ran ? TBSCI_OK : launch_typed<T>(ctx, ham, plan, c, s, nvec, st);
+}
+
+}  // namespace
+
 tbsci_status sigma_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan, const void *c, void *s, int nvec,
                           tbsci_dtype dt, cudaStream_t st) {
     if (dt == TBSCI_F64)
-        return launch_typed<double>(ctx, ham, plan, static_cast<const double *>(c), static_cast<double *>(s), nvec, st);
+        return launch_full<double>(ctx, ham, plan, static_cast<const double *>(c), static_cast<double *>(s), nvec, st);
     if (dt == TBSCI_F32)
-        return launch_typed<float>(ctx, ham, plan, static_cast<const float *>(c), static_cast<float *>(s), nvec, st);
+        return launch_full<float>(ctx, ham, plan, static_cast<const float *>(c), static_cast<float *>(s), nvec, st);
     if (dt == TBSCI_F32_TC_TF32 || dt == TBSCI_F32_TC_BF16) {
         const float *cf = static_cast<const float *>(c);
         float *sf = static_cast<float *>(s);
-        if (plan->npoff > 128 || !plan->d_lbp.p)  // no tensor-core tile for this norb: FP32 on the SIMT path
+        const int np = dt == TBSCI_F32_TC_BF16 ? 1 : 3;
+        bool ready = false;
+        TB_TRY(sigma_tc_prepare(ctx, ham, const_cast<Plan *>(plan), np, st, &ready));
+        if (!ready)  // no tensor-core tile for this norb, or no room for its planes: FP32 on the SIMT path
             return launch_typed<float>(ctx, ham, plan, cf, sf, nvec, st);
-        TB_TRY(sigma_launch_rest(ctx, ham, plan, cf, sf, nvec, st, -1, 0, nullptr, 0, dt == TBSCI_F32_TC_BF16));
-        return sigma_tc_add(ctx, ham, plan, cf, sf, nvec, dt == TBSCI_F32_TC_BF16, st);
+        TB_TRY(sigma_launch_rest(ctx, ham, plan, cf, sf, nvec, st, -1, 0, nullptr, 0, np == 1));
+        const size_t n = (size_t)plan->A.l * plan->B.l;
+        for (int v = 0; v < nvec; ++v) {
+            TB_TRY(udiag_launch(ctx, ham, plan, cf + v * n, sf + v * n, true, true, st));
+            TB_TRY(sigma_tc_ab(ctx, const_cast<Plan *>(plan), np, cf + v * n, sf + v * n, nullptr, st));
+        }
+        return TBSCI_OK;
     }
     return fail(ctx, TBSCI_EINVAL, "unknown dtype");
 }

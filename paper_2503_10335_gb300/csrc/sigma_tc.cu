@@ -1,4 +1,4 @@
-// The alpha-beta classes of sigma on the 5th-generation tensor cores.
+// The alpha-beta classes of sigma on the 5th-generation tensor cores, in FP32.
 //
 // For one alpha row Ia (one CTA), with K alpha terms k = (Ja_k, pq_k, s_k):
 // k = 0 is Ja = Ia ("W" row: sum_{p in Ia} (pp|rs)), k >= 1 the alpha singles.
@@ -7,380 +7,602 @@
 //                                            F[k][Jb] = c(Ja_k, Jb)
 // over the off-diagonal orbital pairs rs (one 128-row MMA tile for norb <= 16),
 // then sigma(Ia, Ib) += sign * G[rs][Jb] for every beta single link
-// Ib = E_rs Jb (the gather D of the classic formulation, done as a scatter from
-// the accumulator rows). The beta-diagonal pairs (r = s in Ib), the alpha-single
-// string-Hamiltonian values and the whole diagonal are added by the threads that
-// stage F, as  (h_a(Ia,Ja_k) + s_k U[pq_k][Jb]) c(Ja_k, Jb)  and
-// Hd(Ia, Jb) c(Ia, Jb). Together: classes [1,1], [1,0], [0,1] (alpha-beta
-// part) and [0,0] of Sec. II.C; the rest (same-spin beta singles/doubles,
-// alpha doubles) comes from the SIMT kernel run first.
+// Ib = E_rs Jb (the gather D of the classic formulation, done from the accumulators).
+// The beta-diagonal pairs (r = s in Ib), the alpha-single string-Hamiltonian values
+// and the diagonal are added by k_udiag (sigma_exact.cu). Together: classes [1,1],
+// [1,0], [0,1] (alpha-beta part) and [0,0] of Sec. II.C; the same-spin classes come
+// from the passes of sigma.cu, sigma_split.cu or sigma_dense.cu run first.
 //
-// Operands are staged in shared memory in the K-major no-swizzle core-matrix
-// layout: element (row r, k) at (r/8)*SBO + (k/E)*128 + (r%8)*16 + (k%E)*es,
-// E = 16 / es elements per 16-byte core row; tcgen05.mma (cta_group::1,
-// M = 128, N = 64) accumulates FP32 in TMEM; tcgen05.ld brings rows back.
-// Precision: 3xTF32 (A = Ah + Al, F = Fh + Fl, G = Ah Fh + Ah Fl + Al Fh) for
-// FP32-level accuracy, or one BF16 product (fast, ~3 significant digits).
-// Every mbarrier wait is bounded; on timeout the CTA records an error, skips
-// the rest of its row and still frees its TMEM.
+// Precision: three BF16 planes per operand (x = x0 + x1 + x2 holds all 24 bits of an
+// FP32 value) and the six products x_i y_j with i + j <= 2, FP32 accumulation, for the
+// split-TF32 type and the FP32 type (at least the accuracy of three TF32 products, at
+// the same tensor-core time); or one BF16 product (~3 significant digits).
+//
+// What bounds it: not the products (512 to 960 tensor-core cycles per 64 columns) but
+// the way of G into the sigma row. So it keeps the products' operands out of the
+// warps' hands (A lies in TMEM for the whole row; c arrives as BF16 planes cut once
+// per vector, a 128-byte segment per coupled row) and gives the accumulators a plan of
+// the links made once per space: every link of a 64-column tile has a slot, the slots
+// of a target column are consecutive, and a thread sums up to four of them. No atomics:
+// results are run-to-run identical.
+// Norb 16, full space (165.6M determinants), one vector: 35.7 ms with three planes, 30.4
+// ms with one; 85 and 53 ms with operands staged element by element and sums by
+// shared-memory atomics.
+// Every mbarrier wait is bounded; on timeout the CTA records an error, writes a NaN,
+// skips the rest of its row and still frees its TMEM.
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.cuh"
+#include "tensor.cuh"
 
 namespace tbsci {
 
 namespace {
 
-// CTA size: the first half of the warps drains the accumulator, the second
-// stages F. Split TF32 writes two planes per staged element and gains from 32
-// warps; BF16 staging is lighter and runs best with 16.
-template <bool BF16>
-__host__ __device__ constexpr int tc_threads() { return BF16 ? 512 : 1024; }
-constexpr int kTileN = 64;    // beta columns per MMA tile
-constexpr int kTileM = 128;   // off-diagonal pair rows (norb <= 16: <= 120 used)
-constexpr int kKStep = 16;    // K padding granule (a BF16 MMA step; two TF32 steps)
+// ------------------------------------------------------------------ link plan
 
-struct TcArgs {
-    int64_t la, lb;
-    const float *C;
+constexpr int kLinkThreads = 256;
+
+// One CTA per tile of 64 columns Jb. counts -> places of the target columns' lists ->
+// ranks of the links. Lists of n slots are summed by ceil(n / 4) consecutive lanes,
+// aligned to a power of two so that a list stays in one warp, longest lists first.
+// Within a list: positive links by column and pair, then negative ones.
+__global__ void __launch_bounds__(kLinkThreads) k_tile_links(const int32_t *__restrict__ lbp, int64_t lb, int npoff, int npiece,
+                                                             int nslot, uint16_t *pos, int2 *piece, int *rounds) {
+    extern __shared__ uint32_t scnt[];  // [lb] positive links | negative links << 16, then the next slots
+    __shared__ int sOff[6][kLinkThreads];
+    __shared__ int sTot[6];
+    const int t = blockIdx.x, tid = threadIdx.x;
+    const int64_t j0 = (int64_t)t * kAbTile;
+    const int ncol = (int)min((int64_t)kAbTile, lb - j0);
+    const int32_t *L = lbp + j0 * npoff;
+    for (int64_t i = tid; i < lb; i += kLinkThreads) scnt[i] = 0;
+    __syncthreads();
+    for (int x = tid; x < ncol * npoff; x += kLinkThreads) {
+        const int32_t e = L[x];
+        if (e >= 0) atomicAdd(&scnt[e >> 1], (e & 1) ? 0x10000u : 1u);
+    }
+    __syncthreads();
+    const int64_t per = (lb + kLinkThreads - 1) / kLinkThreads, a = min(lb, tid * per), b = min(lb, a + per);
+    int own[6] = {0, 0, 0, 0, 0, 0};  // lists by size class (1, 2, 4, 8, 16 lanes), slots
+    for (int64_t i = a; i < b; ++i) {
+        const int n = (int)(scnt[i] & 0xFFFF) + (int)(scnt[i] >> 16);
+        if (!n) continue;
+        const int np = (n + kPiece - 1) / kPiece;
+        ++own[np <= 1 ? 0 : np <= 2 ? 1 : np <= 4 ? 2 : np <= 8 ? 3 : 4];
+        own[5] += n;
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) sOff[k][tid] = own[k];
+    __syncthreads();
+    if (tid < 6) {  // exclusive sums in thread order
+        int run = 0;
+        for (int k = 0; k < kLinkThreads; ++k) {
+            const int x = sOff[tid][k];
+            sOff[tid][k] = run;
+            run += x;
+        }
+        sTot[tid] = run;
+    }
+    __syncthreads();
+    int base[5], lanes = 0;
+#pragma unroll
+    for (int k = 4; k >= 0; --k) {
+        base[k] = lanes;
+        lanes += sTot[k] << k;
+    }
+    int2 *P = piece + (int64_t)t * npiece;
+    int at[5], slot = sOff[5][tid];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) at[k] = base[k] + (sOff[k][tid] << k);
+    for (int64_t i = a; i < b; ++i) {
+        const int plus = (int)(scnt[i] & 0xFFFF), n = plus + (int)(scnt[i] >> 16);
+        if (!n) continue;
+        const int np = (n + kPiece - 1) / kPiece, cl = np <= 1 ? 0 : np <= 2 ? 1 : np <= 4 ? 2 : np <= 8 ? 3 : 4;
+        int p = 0;
+#pragma unroll
+        for (int k = 0; k < 5; ++k)
+            if (k == cl) {
+                p = at[k];
+                at[k] += 1 << k;
+            }
+        for (int k = 0; k < (1 << cl); ++k) {
+            int2 v = make_int2(-1, 0);
+            if (k < np) {
+                const int s = k * kPiece, cnt = min(kPiece, n - s), pc = min(cnt, max(0, plus - s));
+                v = make_int2(k ? -1 : (int)i, (int)((uint32_t)(slot + s) | ((uint32_t)pc << 16) | ((uint32_t)(cnt - pc) << 20) |
+                                                     ((uint32_t)(np - 1 - k) << 24)));
+            }
+            P[p + k] = v;
+        }
+        scnt[i] = (uint32_t)slot | ((uint32_t)(slot + plus) << 16);
+        slot += n;
+    }
+    for (int k = lanes + tid; k < npiece; k += kLinkThreads) P[k] = make_int2(-1, 0);
+    if (tid == 0) rounds[t] = (lanes + kAbDrain - 1) / kAbDrain;
+    __syncthreads();
+    for (int c = 0; c < kAbTile; ++c) {  // a target occurs at most once per column
+        for (int rs = tid; rs < 128; rs += kLinkThreads) {
+            uint16_t s = (uint16_t)(nslot - 1);
+            const int32_t e = c < ncol && rs < npoff ? L[c * npoff + rs] : -1;
+            if (e >= 0) {
+                const uint32_t x = scnt[e >> 1];
+                s = (uint16_t)((e & 1) ? x >> 16 : x & 0xFFFF);
+                scnt[e >> 1] = x + ((e & 1) ? 0x10000u : 1u);
+            }
+            pos[((((size_t)t * 4 + (c >> 4)) * 2 + ((c >> 3) & 1)) * 128 + rs) * 8 + (c & 7)] = s;
+        }
+        __syncthreads();
+    }
+}
+
+// ------------------------------------------------------------------ planes
+
+// x = sum of NP BF16 values, each the rounded rest of the ones before
+template <int NP>
+__device__ __forceinline__ void bf16_planes(float x, uint32_t (&h)[NP]) {
+#pragma unroll
+    for (int s = 0; s < NP; ++s) {
+        const __nv_bfloat16 b = __float2bfloat16_rn(x);
+        h[s] = __bfloat16_as_ushort(b);
+        if (s + 1 < NP) {
+            const float r = x - __bfloat162float(b);
+            x = isfinite(r) ? r : 0.f;  // infinities and NaN lie in the first plane
+        }
+    }
+}
+
+// planes [NP][la][lbp] of a vector, columns lb .. lbp - 1 zero; 8 columns per thread
+template <int NP>
+__global__ void __launch_bounds__(256) k_planes(const float *__restrict__ c, int64_t la, int64_t lb, int64_t lbp,
+                                                const int *__restrict__ info, __nv_bfloat16 *out) {
+    if (info && !info[0]) return;
+    const int64_t per = lbp / 8, n = la * per, plane = la * lbp;
+    for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+        const int64_t r = i / per, j = (i - r * per) * 8;
+        uint32_t h[8][NP];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) bf16_planes<NP>(j + u < lb ? __ldg(c + r * lb + j + u) : 0.f, h[u]);
+#pragma unroll
+        for (int s = 0; s < NP; ++s)
+            *reinterpret_cast<uint4 *>(out + s * plane + r * lbp + j) =
+                make_uint4(h[0][s] | (h[1][s] << 16), h[2][s] | (h[3][s] << 16), h[4][s] | (h[5][s] << 16), h[6][s] | (h[7][s] << 16));
+    }
+}
+
+// planes of the integral columns, [pair][128 off-diagonal pairs] x 4 BF16, or of W_Ia, [la][128] x 4
+template <int NP>
+__global__ void k_ab_planes(const float *__restrict__ V, int npair, int npoff, const int32_t *__restrict__ offpair,
+                            const uint64_t *__restrict__ str, int64_t rows, uint2 *out) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= rows * 128) return;
+    const int64_t row = i >> 7;
+    const int rs = (int)(i & 127);
+    float x = 0.f;
+    if (rs < npoff) {
+        const int col = offpair[rs];
+        if (str) {
+            for (uint64_t s = str[row]; s; s &= s - 1) {
+                const int p = __ffsll((long long)s) - 1;
+                x += V[(size_t)(p * (p + 1) / 2 + p) * npair + col];
+            }
+        } else {
+            x = V[(size_t)row * npair + col];
+        }
+    }
+    uint32_t h[NP];
+    bf16_planes<NP>(x, h);
+    out[i] = make_uint2(h[0] | (NP > 1 ? h[NP > 1 ? 1 : 0] << 16 : 0u), NP > 2 ? h[NP > 2 ? 2 : 0] : 0u);
+}
+
+// ------------------------------------------------------------------ the kernel
+
+struct FpArgs {
+    int64_t la, lb, lbp;
+    const __nv_bfloat16 *Cs;
     float *S;
-    int npair, npoff, na, kmax;
-    const uint64_t *stra;
+    const int *info;       // run only where info[0] is set (NULL: always)
+    const uint2 *Vd, *Wd;  // [pair][128], [la][128] x 4 BF16
     const int64_t *a_soff;
     const int2 *a_sci;
-    const float *a_sval;
-    const float *Vf;   // [npair][npair]
-    const float *Uf;   // [npair][lb]
-    const float *Ea, *Eb;
-    float ecore;
-    const int32_t *lbp;      // [lb][npoff]
-    const int32_t *offpair;  // [npoff]
+    const uint4 *pos;      // [tile][4][2][128] x 8: slot of (pair, column); nslot - 1: no link
+    const int2 *piece;     // [tile][npiece]: {target column (-1: not the first piece of its list), first slot |
+                           // positive links << 16 | negative links << 20 | further pieces << 24}
+    const int *rounds;     // [tile] pieces / kAbDrain, rounded up
+    int npiece, nslot;
+    int stage_bytes;       // shared memory for the gathered c rows
     const int32_t *rowsa;
     int *err;
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-    d |= (uint64_t)1 << 46;  // descriptor version of this architecture; no swizzle, base offset 0
-    return d;
-}
-
-__device__ __forceinline__ float tf32_round(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
-}
-
-// byte offset of element (r, k) in a K-major no-swizzle tile with Kp columns
-template <int ES>
-__device__ __forceinline__ uint32_t core_off(int r, int k, int Kp) {
-    constexpr int E = 16 / ES;
-    return (uint32_t)((r >> 3) * (Kp / E) * 128 + (k / E) * 128 + (r & 7) * 16 + (k % E) * ES);
-}
-
-template <bool BF16>
-__device__ __forceinline__ void put(unsigned char *hi, unsigned char *lo, uint32_t off_hi, uint32_t off_lo, float v) {
-    if (BF16) {
-        *reinterpret_cast<__nv_bfloat16 *>(hi + off_hi) = __float2bfloat16_rn(v);
-    } else {
-        const float h = tf32_round(v);
-        *reinterpret_cast<float *>(hi + off_hi) = h;
-        *reinterpret_cast<float *>(lo + off_lo) = tf32_round(v - h);
-    }
-}
-
-template <bool BF16>
-__global__ void __launch_bounds__(tc_threads<BF16>()) k_sigma_ab_tc(TcArgs A) {
-    constexpr int kTcThreads = tc_threads<BF16>();
-    constexpr int kEpiThreads = kTcThreads / 2;
-    constexpr int kEpiParts = kEpiThreads / 128;  // warps per TMEM lane quarter
-    static_assert(kTileN % (16 * kEpiParts) == 0, "each draining warp reads whole 16-column TMEM chunks");
-    constexpr int ES = BF16 ? 2 : 4;  // element bytes
-    extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint64_t mbar[2];
+template <int NP>
+__global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab_tc(const FpArgs A) {
+    if (A.info && !A.info[0]) return;
+    extern __shared__ unsigned char smem_dyn[];
+    __shared__ uint64_t bar[16];
     __shared__ uint32_t tmem_base;
-    __shared__ int sJa[256], sPq[256], sOccP[64];
-    __shared__ float sSa[256], sHa[256];
-    __shared__ int sAbort, sAbortTile;
-
+    __shared__ int sAbort;
+    __shared__ int sJa[kAbMaxK], sPq[kAbMaxK];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t lb = A.lb;
-    const int64_t Ia = A.rowsa[blockIdx.x];
-    const int64_t t0 = A.a_soff[Ia];
-    const int K = 1 + (int)(A.a_soff[Ia + 1] - t0);
-    const int Kp = (K + kKStep - 1) / kKStep * kKStep;
-    const uint32_t a_bytes = (uint32_t)kTileM * Kp * ES, b_bytes = (uint32_t)kTileN * Kp * ES;
-    unsigned char *sAh = smem;
-    unsigned char *sAl = sAh + (BF16 ? 0 : a_bytes);
-    unsigned char *sBh = sAh + (BF16 ? 1 : 2) * a_bytes;  // two F buffers of (BF16 ? 1 : 2) planes each
-    float *sAcc = reinterpret_cast<float *>(sBh + 2 * (BF16 ? 1 : 2) * b_bytes);
-
-    // alpha terms of this row
+    const int64_t lb = A.lb, lbp = A.lbp, Ia = A.rowsa[blockIdx.x], t0 = A.a_soff[Ia];
+    const int K = 1 + (int)(A.a_soff[Ia + 1] - t0), Kp = (K + 15) / 16 * 16;
+    const uint32_t stage_sz = (uint32_t)NP * Kp * kAbTile * 2;
+    const int nst = min(4, A.stage_bytes / (int)stage_sz);
+    constexpr int ndb = 4;                                      // accumulators: NP Kp / 2 <= 120 columns of A, then 4 x 64
+    const int dcol0 = (NP * Kp / 2 + 31) / 32 * 32;
+    unsigned char *sm = smem_dyn + ((1024 - (su32(smem_dyn) & 1023)) & 1023);
+    const uint32_t sB = su32(sm);
+    float *sAcc = reinterpret_cast<float *>(sm + A.stage_bytes);  // [lb]
+    float *sSlot = sAcc + lb;                                     // [2][nslot]
+    const uint32_t bfull = su32(&bar[0]), bempty = su32(&bar[4]), dfull = su32(&bar[8]), dempty = su32(&bar[12]);
+    const int ntiles = (int)((lb + kAbTile - 1) / kAbTile);
+    volatile int *ab = &sAbort;
     if (tid == 0) {
-        int k = 0;
-        for (uint64_t s = A.stra[Ia]; s; s &= s - 1) {
-            const int p = __ffsll((long long)s) - 1;
-            sOccP[k++] = p * (p + 1) / 2 + p;
-        }
         sAbort = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[0])));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[1])));
+        for (int s = 0; s < 4; ++s) {
+            mb_init(bfull + 8 * s, 32);
+            mb_init(bempty + 8 * s, 1);
+            mb_init(dfull + 8 * s, 1);
+            mb_init(dempty + 8 * s, 16);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int k = tid; k < K; k += kTcThreads) {
-        if (k == 0) {
-            sJa[0] = (int)Ia;
-            sPq[0] = -1;
-            sSa[0] = 1.f;
-            sHa[0] = 0.f;
-        } else {
+    for (int k = tid; k < Kp; k += kAbThreads) {
+        int ja = (int)Ia, pq = -1;  // padding terms: any row, zero coefficients
+        if (k >= 1 && k < K) {
             const int2 e = A.a_sci[t0 + k - 1];
-            sJa[k] = e.x;
-            sPq[k] = e.y >> 1;
-            sSa[k] = (e.y & 1) ? -1.f : 1.f;
-            sHa[k] = A.a_sval[t0 + k - 1];
+            ja = e.x;
+            pq = e.y;
         }
+        sJa[k] = ja;
+        sPq[k] = pq;
     }
-    for (int64_t j = tid; j < lb; j += kTcThreads) sAcc[j] = 0.f;
-    __syncthreads();
-    // A[rs][k]: rows = off-diagonal pairs, padded to 128 rows and Kp columns
-    for (int x = tid; x < kTileM * Kp; x += kTcThreads) {
-        const int r = x / Kp, k = x - r * Kp;
-        float v = 0.f;
-        if (r < A.npoff && k < K) {
-            const int rs = A.offpair[r];
-            if (k == 0) {
-                for (int i = 0; i < A.na; ++i) v += A.Vf[(size_t)sOccP[i] * A.npair + rs];
-            } else {
-                v = sSa[k] * A.Vf[(size_t)sPq[k] * A.npair + rs];
-            }
-        }
-        put<BF16>(sAh, sAl, core_off<ES>(r, k, Kp), core_off<ES>(r, k, Kp), v);
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(2 * kTileN));
+    for (int64_t j = tid; j < lb; j += kAbThreads) sAcc[j] = 0.f;
+    if (warp == 19) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(su32(&tmem_base)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    tc_before();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    const uint32_t tmem = tmem_base;
-    // instruction descriptor: D F32, A/B BF16 (kind::f16) or TF32 (kind::tf32), K-major, M = 128, N = 64
-    const uint32_t idesc = (1u << 4) | ((BF16 ? 1u : 2u) << 7) | ((BF16 ? 1u : 2u) << 10) |
-                           ((uint32_t)(kTileN >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
-    const uint32_t sbo = (uint32_t)(Kp * ES / 16) * 128;
-    const int ntiles = (int)((lb + kTileN - 1) / kTileN);
-
-    // F tile t into buffer `buf` by `nth` threads starting at thread `t0`; adds the
-    // diagonal, beta-diagonal and alpha-single terms of those columns into sAcc
-    auto stage = [&](int t, int buf, int tid0, int nth) {
-        const int me = tid - tid0;
-        const int jb = me & (kTileN - 1), kstride = nth / kTileN;
-        const int64_t Jb = (int64_t)t * kTileN + jb;
-        const bool col_ok = Jb < lb;
-        unsigned char *bh = sBh + (size_t)buf * (BF16 ? 1 : 2) * b_bytes;
-        unsigned char *bl = bh + (BF16 ? 0 : b_bytes);
-        float part = 0.f;
-        // batches of 8 alpha terms: all loads of a batch are issued before any use
-        for (int kb = me / kTileN; kb < Kp; kb += 8 * kstride) {
-            float c[8], u[8];
+    tc_after();
+    constexpr uint32_t tmem = 0;  // all 512 columns are this CTA's: they start at 0
+    if (tid == 0 && tmem_base != 0) sAbort = 1;
+    if (warp < 16) {
+        // A's planes: lane = pair row, two terms per 32-bit column, plane s at column s Kp / 2
+        const int quarter = warp & 3, rs = quarter * 32 + lane;
+        for (int kb = warp >> 2; kb < Kp / 8; kb += 4) {
+            uint32_t v[8][2];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const int k = kb + q * kstride;
-                const bool ok = k < K && col_ok;
-                c[q] = ok ? __ldg(A.C + (size_t)sJa[k] * lb + Jb) : 0.f;
-                u[q] = (ok && k > 0) ? __ldg(A.Uf + (size_t)sPq[k] * lb + Jb) : 0.f;
+                const int k = kb * 8 + q, pq = sPq[k];
+                uint2 x = make_uint2(0, 0);
+                if (k == 0) x = __ldg(A.Wd + Ia * 128 + rs);
+                else if (pq >= 0) x = __ldg(A.Vd + (size_t)(pq >> 1) * 128 + rs);
+                const uint32_t neg = k > 0 && pq >= 0 && (pq & 1) ? 0x80008000u : 0u;
+                v[q][0] = x.x ^ neg;
+                v[q][1] = x.y ^ neg;
             }
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int k = kb + q * kstride;
-                if (k >= Kp) break;
-                if (k < K && col_ok) {
-                    float coef;
-                    if (k == 0) {
-                        coef = A.ecore + A.Ea[Ia] + __ldg(A.Eb + Jb);
-                        for (int i = 0; i < A.na; ++i) coef += __ldg(A.Uf + (size_t)sOccP[i] * lb + Jb);
-                    } else {
-                        coef = sHa[k] + sSa[k] * u[q];
-                    }
-                    part = fmaf(coef, c[q], part);
-                }
-                put<BF16>(bh, bl, core_off<ES>(jb, k, Kp), core_off<ES>(jb, k, Kp), c[q]);
+            for (int s = 0; s < NP; ++s) {
+                uint32_t o[4];
+#pragma unroll
+                for (int z = 0; z < 4; ++z)
+                    o[z] = __byte_perm(v[2 * z][s >> 1], v[2 * z + 1][s >> 1], (s & 1) ? 0x7632 : 0x5410);
+                asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                                 tmem + ((uint32_t)(quarter * 32) << 16) + s * (Kp / 2) + kb * 4),
+                             "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3])
+                             : "memory");
             }
         }
-        if (col_ok && part != 0.f) atomicAdd(&sAcc[Jb], part);
-        asm volatile("fence.proxy.async.shared::cta;");
-    };
-    auto issue = [&](int t) {
-        const int buf = t & 1;
-        const uint32_t d = tmem + (uint32_t)(buf * kTileN);
-        const uint32_t aH = smem_u32(sAh), aL = smem_u32(sAl);
-        const uint32_t bH = smem_u32(sBh + (size_t)buf * (BF16 ? 1 : 2) * b_bytes), bL = bH + (BF16 ? 0 : b_bytes);
-        const int ksteps = BF16 ? Kp / 16 : Kp / 8;  // each step = two core columns = 32 bytes of K
-        for (int ks = 0; ks < ksteps; ++ks) {
-            const uint32_t o = (uint32_t)ks * 256;
-            const uint32_t acc0 = ks > 0 ? 1u : 0u;
-            const uint64_t dAh = smem_desc(aH + o, 128, sbo), dBh = smem_desc(bH + o, 128, sbo);
-            if (BF16) {
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-                    "l"(dAh), "l"(dBh), "r"(idesc), "r"(acc0));
-            } else {
-                const uint64_t dAl = smem_desc(aL + o, 128, sbo), dBl = smem_desc(bL + o, 128, sbo);
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-                    "l"(dAh), "l"(dBh), "r"(idesc), "r"(acc0));
-                asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, 1;" ::"r"(d), "l"(dAh), "l"(dBl),
-                             "r"(idesc));
-                asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, 1;" ::"r"(d), "l"(dAl), "l"(dBh),
-                             "r"(idesc));
-            }
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_u32(&mbar[buf])));
-    };
-    auto wait_tile = [&](int t) -> uint32_t {
-        uint32_t done = 0;
-        for (int it = 0; it < (1 << 22) && !done; ++it) {
-            asm volatile(
-                "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                : "=r"(done)
-                : "r"(smem_u32(&mbar[t & 1])), "r"((uint32_t)((t >> 1) & 1)));
-        }
-        return done;
-    };
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    tc_before();
+    __syncthreads();
+    tc_after();
 
-    // Pipeline: while the tensor cores run tile t, the staging warps fill the other
-    // F buffer with tile t+1 and the draining warps read tile t from its TMEM
-    // buffer as soon as its MMAs complete; one barrier per tile.
-    if (ntiles > 0) {
-        stage(0, 0, 0, kTcThreads);
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        if (tid == 0) issue(0);
-    }
-    for (int t = 0; t < ntiles; ++t) {
-        if (tid >= kEpiThreads) {
-            if (t + 1 < ntiles) stage(t + 1, (t + 1) & 1, kEpiThreads, kTcThreads - kEpiThreads);
-        } else {
-            uint32_t done = __all_sync(0xffffffffu, wait_tile(t));  // warp-uniform: tcgen05.ld is collective
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            if (!done) {
-                if (lane == 0) {
-                    sAbort = 1;
-                    sAbortTile = t;
+    if (warp == 19) {
+        const uint32_t dbase = uni((uint32_t)dcol0);
+        int st = 0;
+        uint32_t sph = 0;
+        bool ok = true;
+        // unrolled for the row's number of 16-term steps, so that every descriptor is a
+        // uniform base plus an immediate
+        auto tiles = [&](auto ks_tag) {
+            constexpr int KS = decltype(ks_tag)::value;
+            for (int t = 0; t < ntiles && ok; ++t) {
+                const int db = t & (ndb - 1);
+                ok = __all_sync(0xffffffffu, mb_wait(bfull + 8 * st, sph, ab));
+                if (ok && t >= ndb) ok = __all_sync(0xffffffffu, mb_wait(dempty + 8 * db, (t / ndb - 1) & 1, ab));
+                if (!ok) break;
+                tc_after();
+                const uint64_t b0 = op_desc(uni(sB + st * stage_sz), 16, 1024, 2);
+                const uint32_t d = uni(dbase + db * kAbTile);
+                if (elect_one()) {
+                    constexpr uint32_t idesc = inst_desc(kAbTile, true);
+                    // smallest products first
+#pragma unroll
+                    for (int o = NP - 1; o >= 0; --o)
+#pragma unroll
+                        for (int i = 0; i <= o; ++i)
+#pragma unroll
+                            for (int ks = 0; ks < KS; ++ks)
+                                asm volatile(
+                                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                                    " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d),
+                                    "r"(tmem + i * (KS * 8) + ks * 8), "l"(b0 + ((o - i) * KS + ks) * (kAbTile * 2)), "r"(idesc),
+                                    "r"(o == NP - 1 && i == 0 && ks == 0 ? 0u : 1u)
+                                    : "memory");
+                    mma_commit(dfull + 8 * db);
+                    mma_commit(bempty + 8 * st);
                 }
-            } else {
-                // a warp reads the TMEM lanes of its quarter (warp % 4); the warps of
-                // one quarter split the tile's columns
-                const int quarter = warp & 3, part = warp >> 2;
-                const int rs = quarter * 32 + lane;
-                const int64_t Jb0 = (int64_t)t * kTileN;
-                const uint32_t dcol = (uint32_t)((t & 1) * kTileN);
-                constexpr int kCols = kTileN / kEpiParts;
-#pragma unroll
-                for (int c0 = part * kCols; c0 < (part + 1) * kCols; c0 += 16) {
-                    uint32_t r[16];
-                    const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + dcol + (uint32_t)c0;
-                    asm volatile(
-                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                        "[%16];"
-                        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-                          "=r"(r[14]), "=r"(r[15])
-                        : "r"(taddr));
-                    asm volatile("tcgen05.wait::ld.sync.aligned;");
-                    if (rs < A.npoff) {
-                        int32_t e[16];
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int64_t col = Jb0 + c0 + j;
-                            e[j] = col < lb ? __ldg(A.lbp + col * A.npoff + rs) : -1;
-                        }
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (e[j] >= 0) {
-                                const float g = __uint_as_float(r[j]);
-                                atomicAdd(&sAcc[e[j] >> 1], (e[j] & 1) ? -g : g);
-                            }
-                    }
+                __syncwarp();
+                if (++st == nst) {
+                    st = 0;
+                    sph ^= 1;
                 }
             }
-            asm volatile("tcgen05.fence::before_thread_sync;");
+        };
+        switch (Kp / 16) {
+            case 1: tiles(std::integral_constant<int, 1>{}); break;
+            case 2: tiles(std::integral_constant<int, 2>{}); break;
+            case 3: tiles(std::integral_constant<int, 3>{}); break;
+            case 4: tiles(std::integral_constant<int, 4>{}); break;
+            default: tiles(std::integral_constant<int, 5>{}); break;
         }
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        if (sAbort) break;
-        if (tid == 0 && t + 1 < ntiles) issue(t + 1);
-    }
-    if (sAbort) {
-        // only the timed-out tile's MMAs can still be in flight: give them a second
-        // bounded chance to finish before TMEM is freed
-        if (tid == 0) {
-            wait_tile(sAbortTile);
-            atomicExch(A.err, 1);
+        // no MMA (and no arrival of its commit) may outlive the CTA
+        if (ok && ntiles > 0) mb_wait(bempty + 8 * ((ntiles - 1) % nst), ((ntiles - 1) / nst) & 1, ab);
+        if (!ok)
+            for (int it = 0; it < 4096; ++it) __nanosleep(100);
+        __syncwarp();
+    } else if (warp >= 16) {
+        // a warp gathers a whole tile; three tiles are on their way (not more than there are
+        // stages: a wait must not run a phase ahead of its barrier)
+        const int ng = min(3, nst), g = warp - 16;
+        for (int t = g; t < ntiles && g < ng; t += ng) {
+            const int st = t % nst;
+            if (t >= nst && !mb_wait(bempty + 8 * st, (t / nst - 1) & 1, ab)) break;
+            gather_tile<NP>(A.Cs, (size_t)A.la * lbp, lbp, sJa, Kp, t, sB + st * stage_sz);
+            mb_arrive(bfull + 8 * st);
         }
     } else {
-        for (int64_t j = tid; j < lb; j += kTcThreads) A.S[Ia * lb + j] += sAcc[j];
+        const int quarter = warp & 3, part = warp >> 2, rs = quarter * 32 + lane;
+        // slots, pieces and rounds of a tile are read a tile ahead
+        const uint4 *pp = A.pos + (size_t)part * 2 * 128 + rs;
+        const int2 *pc = A.piece + tid;
+        uint4 p0 = __ldg(pp), p1 = __ldg(pp + 128);
+        int nr = __ldg(A.rounds);
+        int2 sg = __ldg(pc), sg1 = nr > 1 ? __ldg(pc + kAbDrain) : make_int2(-1, 0);
+        for (int t = 0; t < ntiles; ++t) {
+            const int db = t & (ndb - 1);
+            float *slots = sSlot + (t & 1) * A.nslot;
+            const bool ok = __all_sync(0xffffffffu, mb_wait(dfull + 8 * db, (t / ndb) & 1, ab));
+            tc_after();
+            uint32_t q[16];
+            if (ok) {
+                tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + dcol0 + db * kAbTile + part * 16, q);
+                pin16(q);
+            } else {
+#pragma unroll
+                for (int x = 0; x < 16; ++x) q[x] = 0;
+            }
+            tc_before();
+            __syncwarp();
+            if (lane == 0) mb_arrive(dempty + 8 * db);
+            const uint32_t pw[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+#pragma unroll
+            for (int x = 0; x < 16; ++x)
+                slots[(pw[x >> 1] >> (16 * (x & 1))) & 0xFFFFu] = __uint_as_float(q[x]);  // no link: the last slot
+            const int rounds = nr;
+            const int2 *cur = pc;
+            int2 c0 = sg, c1 = sg1;
+            if (t + 1 < ntiles) {
+                pp += 4 * 2 * 128;
+                pc += A.npiece;
+                p0 = __ldg(pp);
+                p1 = __ldg(pp + 128);
+                nr = __ldg(A.rounds + t + 1);
+                sg = __ldg(pc);
+                sg1 = A.npiece > kAbDrain ? __ldg(pc + kAbDrain) : make_int2(-1, 0);
+            }
+            // one barrier per tile: a warp that passes it has summed the tile before last,
+            // whose slots this tile's successor writes
+            asm volatile("bar.sync 1, 512;" ::: "memory");
+            for (int i = 0; i < rounds; ++i) {
+                const uint32_t y = (uint32_t)c0.y;
+                const int ib = c0.x, first = y & 0xFFFF, np = (y >> 16) & 0xF, n = np + ((y >> 20) & 0xF);
+                const int more = y >> 24;  // further pieces, in the lanes above
+                c0 = c1;
+                if (i + 2 < rounds) c1 = __ldg(cur + (i + 2) * kAbDrain);
+                float z[kPiece];
+#pragma unroll
+                for (int k = 0; k < kPiece; ++k) z[k] = slots[first + k];
+                float v = 0.f;
+#pragma unroll
+                for (int k = 0; k < kPiece; ++k)
+                    if (k < n) v += k < np ? z[k] : -z[k];
+                const int steps = __reduce_max_sync(0xffffffffu, (unsigned)more);
+                for (int d = 1; d <= steps; d <<= 1) {
+                    const float w = __shfl_down_sync(0xffffffffu, v, d);
+                    if (d <= more) v += w;
+                }
+                if (ib >= 0) sAcc[ib] += v;
+            }
+        }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    tc_before();
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kTileN));
+    float *S = A.S + Ia * lb;
+    for (int64_t j = tid; j < lb; j += kAbThreads) S[j] += sAcc[j];
+    if (sAbort && tid == 0) {
+        atomicExch(A.err, 1);
+        S[0] = NAN;  // fail loudly
+    }
+    if (warp == 19) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base));
+}
+
+inline int64_t pad64(int64_t l) { return (l + 63) / 64 * 64; }
+
+// stages of the fullest row that fit beside the sigma row and the slots (at most four), as bytes; 0: none
+int fp_stage_bytes(const tbsci_ctx *ctx, const Plan *P, int np) {
+    const int64_t one = (int64_t)np * P->tl_kpmax * kAbTile * 2;
+    const int64_t fixed = 1024 + 4 * (P->B.l + 2 * (int64_t)P->tl_nslot);
+    const int64_t room = ((int64_t)ctx->smem_optin - 2048 - fixed) / 1024 * 1024;
+    return room < one ? 0 : (int)std::min<int64_t>(room, 4 * one);
 }
 
 }  // namespace
 
-tbsci_status sigma_tc_add(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, const float *c, float *s, int nvec,
-                          bool bf16, cudaStream_t st) {
+// Link plan of a space (norb <= 16), made when the space is prepared; left out
+// (tl_kpmax = 0) where the alpha-beta kernels do not apply.
+tbsci_status tile_links_build(tbsci_ctx *ctx, Plan *P, cudaStream_t st) {
     const int64_t la = P->A.l, lb = P->B.l;
-    if (la == 0 || lb == 0) return TBSCI_OK;
-    TB_CHECK(ctx, P->npoff <= kTileM && P->d_lbp.p, TBSCI_EINVAL, "tensor-core sigma needs norb <= 16");
+    P->tl_kpmax = 0;
+    if (P->npoff < 1 || P->npoff > 120 || !P->d_lbp.p || la < 1 || lb < 1) return TBSCI_OK;
     int kmax = 1;
-    for (int64_t i = 0; i < la; ++i) kmax = std::max<int64_t>(kmax, 1 + P->A.h_soff[i + 1] - P->A.h_soff[i]);
-    TB_CHECK(ctx, kmax <= 256, TBSCI_EINVAL, "tensor-core sigma: more than 255 alpha singles per string");
-    const int kp = (kmax + kKStep - 1) / kKStep * kKStep;
-    const size_t es = bf16 ? 2 : 4, planes = bf16 ? 1 : 2;
-    const size_t smem = planes * ((size_t)kTileM * kp * es + 2 * (size_t)kTileN * kp * es) + (size_t)lb * sizeof(float);
-    TB_CHECK(ctx, smem <= ctx->smem_optin, TBSCI_EINVAL, "tensor-core sigma: row too long for shared memory");
-    TcArgs A{};
+    for (int64_t i = 0; i < la; ++i) kmax = std::max<int>(kmax, 1 + (int)(P->A.h_soff[i + 1] - P->A.h_soff[i]));
+    const size_t smem = (size_t)lb * 4;
+    if (kmax > 65 || smem + 16384 > ctx->smem_optin) return TBSCI_OK;
+    const int nt = (int)((lb + kAbTile - 1) / kAbTile);
+    int links = 0;
+    for (int t = 0; t < nt; ++t)
+        links = std::max<int>(links, (int)(P->B.h_soff[std::min<int64_t>(lb, (t + 1) * (int64_t)kAbTile)] - P->B.h_soff[(int64_t)t * kAbTile]));
+    P->tl_nslot = (links + kPiece + 2) / 2 * 2;  // a piece is read whole; the last slot takes pairs without a link
+    P->tl_npiece = std::max(1, (links + kAbDrain - 1) / kAbDrain) * kAbDrain;
+    TB_CUDA(ctx, P->d_tl_pos.alloc((size_t)nt * 4 * 2 * 128));
+    TB_CUDA(ctx, P->d_tl_piece.alloc((size_t)nt * P->tl_npiece));
+    TB_CUDA(ctx, P->d_tl_rounds.alloc(nt));
+    TB_CUDA(ctx, cudaFuncSetAttribute(k_tile_links, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_tile_links<<<(unsigned)nt, kLinkThreads, smem, st>>>(P->d_lbp.p, lb, P->npoff, P->tl_npiece, P->tl_nslot,
+                                                          reinterpret_cast<uint16_t *>(P->d_tl_pos.p), P->d_tl_piece.p,
+                                                          P->d_tl_rounds.p);
+    TB_CUDA(ctx, cudaGetLastError());
+    P->tl_kpmax = (kmax + 15) / 16 * 16;
+    return TBSCI_OK;
+}
+
+// What the kernel keeps for one space and number of planes, made by the first sigma that
+// needs it. Calls on several streams share the planes of c: each waits for the event
+// that the one before it recorded, and `mu` keeps the launches of one call together.
+struct AbPlanes {
+    std::mutex mu;
+    cudaEvent_t busy = nullptr;
+    bool tried = false, ready = false;
+    DevBuf<uint2> V, W;
+    DevBuf<__nv_bfloat16> c;
+    ~AbPlanes() {
+        if (busy) cudaEventDestroy(busy);
+    }
+};
+
+namespace {
+
+template <int NP>
+tbsci_status build_planes(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, AbPlanes *X, cudaStream_t st) {
+    X->tried = true;
+    const int64_t la = P->A.l, lb = P->B.l;
+    const size_t nv = (size_t)P->npair * 128, nw = (size_t)la * 128, nc = (size_t)NP * la * pad64(lb);
+    const size_t bytes = (nv + nw) * sizeof(uint2) + nc * 2;
+    if (charge(ctx, bytes, "planes of the alpha-beta products") != TBSCI_OK) return TBSCI_OK;
+    cudaError_t e = X->V.alloc(nv);
+    if (e == cudaSuccess) e = X->W.alloc(nw);
+    if (e == cudaSuccess) e = X->c.alloc(nc);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&X->busy, cudaEventDisableTiming);
+    if (e == cudaSuccess) {
+        k_ab_planes<NP><<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(ham->d_Vf.p, P->npair, P->npoff, P->d_offpair.p, nullptr,
+                                                                     P->npair, X->V.p);
+        k_ab_planes<NP><<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(ham->d_Vf.p, P->npair, P->npoff, P->d_offpair.p, P->A.d_str,
+                                                                     la, X->W.p);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) {
+        X->V.release();
+        X->W.release();
+        X->c.release();
+        uncharge(ctx, bytes);
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? TBSCI_OK : fail(ctx, TBSCI_ECUDA, std::string("alpha-beta planes: ") + cudaGetErrorString(e));
+    }
+    P->charged += bytes;
+    X->ready = true;
+    return TBSCI_OK;
+}
+
+template <int NP>
+tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float *s, const int *info, cudaStream_t st) {
+    const int64_t la = P->A.l, lb = P->B.l;
+    FpArgs A{};
     A.la = la;
     A.lb = lb;
-    A.npair = P->npair;
-    A.npoff = P->npoff;
-    A.na = P->A.nelec;
-    A.kmax = kmax;
-    A.stra = P->A.d_str;
+    A.lbp = pad64(lb);
+    A.Cs = X->c.p;
+    A.S = s;
+    A.info = info;
+    A.Vd = X->V.p;
+    A.Wd = X->W.p;
     A.a_soff = P->A.d_soff;
     A.a_sci = P->A.d_sci.p;
-    A.a_sval = P->A.d_svalf.p;
-    A.Vf = ham->d_Vf.p;
-    A.Uf = P->d_Uf.p;
-    A.Ea = P->A.d_Ef.p;
-    A.Eb = P->B.d_Ef.p;
-    A.ecore = (float)ham->ecore;
-    A.lbp = P->d_lbp.p;
-    A.offpair = P->d_offpair.p;
+    A.pos = P->d_tl_pos.p;
+    A.piece = P->d_tl_piece.p;
+    A.rounds = P->d_tl_rounds.p;
+    A.npiece = P->tl_npiece;
+    A.nslot = P->tl_nslot;
+    A.stage_bytes = fp_stage_bytes(ctx, P, NP);
     A.rowsa = P->d_rowsa.p;
     A.err = P->d_tc_err.p;
-    auto kern = bf16 ? k_sigma_ab_tc<true> : k_sigma_ab_tc<false>;
+    const size_t smem = 1024 + (size_t)A.stage_bytes + 4 * ((size_t)lb + 2 * (size_t)A.nslot);
+    auto kern = k_sigma_ab_tc<NP>;
     TB_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    for (int v = 0; v < nvec; ++v) {
-        A.C = c + (size_t)v * la * lb;
-        A.S = s + (size_t)v * la * lb;
-        TraceScope tr(ctx, "k_sigma_ab_tc", st);
-        kern<<<(unsigned)la, bf16 ? tc_threads<true>() : tc_threads<false>(), smem, st>>>(A);
+    TB_CUDA(ctx, cudaStreamWaitEvent(st, X->busy, 0));
+    {
+        TraceScope tr(ctx, "k_planes", st);
+        k_planes<NP><<<ctx->num_sms * 8, 256, 0, st>>>(c, la, lb, A.lbp, info, X->c.p);
         TB_CUDA(ctx, cudaGetLastError());
     }
+    {
+        TraceScope tr(ctx, "k_sigma_ab_tc", st);
+        kern<<<(unsigned)la, kAbThreads, smem, st>>>(A);
+        TB_CUDA(ctx, cudaGetLastError());
+    }
+    TB_CUDA(ctx, cudaEventRecord(X->busy, st));
     return TBSCI_OK;
+}
+
+}  // namespace
+
+// Makes the kernel's tables for `np` planes (1 or 3); *ready = false where the space, the
+// budget or a stream being captured (the tables are made outside of graphs, and a
+// graph's replays would share the planes of c with other streams) leaves it to the
+// SIMT kernels.
+tbsci_status sigma_tc_prepare(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int np, cudaStream_t st, bool *ready) {
+    *ready = false;
+    if (P->tl_kpmax == 0 || fp_stage_bytes(ctx, P, np) == 0) return TBSCI_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return TBSCI_OK;
+    }
+    std::shared_ptr<AbPlanes> &X = P->ab[np == 1 ? 0 : 1];
+    {
+        static std::mutex make;
+        std::lock_guard<std::mutex> g(make);
+        if (!X) X = std::make_shared<AbPlanes>();
+    }
+    std::lock_guard<std::mutex> g(X->mu);
+    if (!X->tried) TB_TRY(np == 1 ? build_planes<1>(ctx, ham, P, X.get(), st) : build_planes<3>(ctx, ham, P, X.get(), st));
+    *ready = X->ready;
+    return TBSCI_OK;
+}
+
+// Adds the alpha-beta products of one vector into s (after a prepare that said ready);
+// info: a device flag, nothing is done where it is 0 (NULL: always).
+tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, const int *info, cudaStream_t st) {
+    AbPlanes *X = P->ab[np == 1 ? 0 : 1].get();
+    std::lock_guard<std::mutex> g(X->mu);
+    return np == 1 ? ab_add<1>(ctx, P, X, c, s, info, st) : ab_add<3>(ctx, P, X, c, s, info, st);
 }
 
 }  // namespace tbsci

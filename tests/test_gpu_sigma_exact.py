@@ -1,0 +1,152 @@
+"""FP64 / FP32 sigma on the tensor cores (digits summed exactly in integers; three
+BF16 planes for the FP32 alpha-beta products) at the sizes where its tiles end, with
+the vectors that it leaves to the SIMT kernels, on two streams and under capture.
+Sampled rows against the oracle: FP64 to 1e-12 and FP32 to 64 * 2^-24 of
+(|H||c|)_I, the tolerances of the SIMT kernels that this path replaces."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import assert_sigma_close
+from tbsci_inputs import selected_strings, synth_hamiltonian
+
+pytestmark = pytest.mark.gpu
+F32 = dict(rel=64 * 2.0 ** -24, norm_rel=1e-5)
+
+
+@pytest.fixture(scope="module")
+def tb():
+    import paper_2503_10335_gb300 as tb
+    return tb
+
+
+@pytest.fixture(scope="module")
+def ctx(tb):
+    c = tb.Context(0)
+    yield c
+    c.close()
+
+
+def _space(tb, ctx, n, na, nb, la, lb, seed, scale=0.3, ecore=0.25):
+    h, eri, _ = synth_hamiltonian(n, seed=seed, scale=scale)
+    asel = None if la is None else selected_strings(n, na, la, seed + 1)
+    bsel = None if lb is None else selected_strings(n, nb, lb, seed + 2)
+    sp = tb.Space(ctx, n, na, nb, h, eri, ecore, alpha=asel, beta=bsel)
+    return sp, oracle.make_space(n, na, nb, asel, bsel), h, eri
+
+
+def _check(s, osp, h, eri, C, rows, **kw):
+    ref, bound = oracle.sigma(osp, h, eri, 0.25, C.reshape(C.shape[0], -1), rows=rows, with_bound=True)
+    assert_sigma_close(s.reshape(C.shape[0], -1)[:, rows], ref, bound, **kw)
+
+
+def _rows(ndet, seed, k=400):
+    r = np.random.default_rng(seed)
+    return np.unique(np.concatenate([r.choice(ndet, k, replace=False), np.arange(40), np.arange(ndet - 40, ndet)]))
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("n,na,nb,la,lb,nvec", [
+    (13, 6, 6, 1030, 1025, 2),    # one row past a 128-row tile's multiple of 6, one column past 64
+    (16, 8, 8, 1100, 1087, 1),    # rows with all 64 alpha singles (65 terms), a column short of 17 tiles
+    (16, 12, 5, 1024, 1024, 1),   # twelve alpha electrons: W beyond eight integrals; whole tiles
+    (12, 6, 6, None, None, 1),    # 924 x 924: below the size from which this path is taken
+    (13, 6, 5, None, None, 1),    # a full space: every list at its longest
+])
+def test_exact_sigma_parity(tb, ctx, n, na, nb, la, lb, nvec, dtype):
+    import torch
+    sp, osp, h, eri = _space(tb, ctx, n, na, nb, la, lb, seed=700 + n + na)
+    tdt = torch.float64 if dtype == "f64" else torch.float32
+    rng = np.random.default_rng(n)
+    # string weights over two decades, as in a correlated vector
+    C = rng.standard_normal((nvec, sp.la, sp.lb)) * (10.0 ** -rng.uniform(0, 2, sp.la))[None, :, None]
+    Ct = torch.from_numpy(C).to(tdt).cuda()
+    tb.tbsci_trace_enable(ctx.handle, True)
+    s = sp.sigma(Ct)
+    torch.cuda.synchronize()
+    tb.tbsci_trace_enable(ctx.handle, False)
+    names = {k for k, _ in tb.tbsci_trace_read(ctx.handle)[0]}
+    assert ("k_same_spin_ex" in names) == (sp.ndet >= 1 << 20), names
+    assert torch.equal(s, sp.sigma(Ct))  # integer sums: the same in every run
+    _check(s.double().cpu().numpy(), osp, h, eri, Ct.double().cpu().numpy(), _rows(sp.ndet, n), **({} if dtype == "f64" else F32))
+    sp.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_vectors_left_to_the_simt_kernels(tb, ctx, dtype):
+    """Per vector of one call: ordinary, a single determinant (its largest entry a
+    thousand times its root mean square), zero, extreme magnitudes, infinity, NaN. Each
+    agrees with the oracle (or is non-finite exactly where the SIMT kernels are, on a
+    captured stream), whatever the others are."""
+    import torch
+    sp, osp, h, eri = _space(tb, ctx, 13, 6, 6, 1040, 1030, seed=731)
+    tdt = torch.float64 if dtype == "f64" else torch.float32
+    rng = np.random.default_rng(3)
+    C = rng.standard_normal((6, sp.la, sp.lb))
+    C[1] = 0.0
+    C[1, 5, 7] = 1.0
+    C[2] = 0.0
+    C[3] *= 1e-25 if dtype == "f32" else 1e-180
+    C[4, 17, 3] = np.inf
+    C[5, 400, 1000] = np.nan
+    Ct = torch.from_numpy(C).to(tdt).cuda()
+    s = sp.sigma(Ct)
+    got = s.double().cpu().numpy().reshape(6, -1)
+    Cr = Ct.double().cpu().numpy()
+    rows = np.unique(np.concatenate([_rows(sp.ndet, 5), [5 * sp.lb + 7]]))
+    for v in range(4):
+        _check(got[v][None], osp, h, eri, Cr[v][None], rows, **({} if dtype == "f64" else F32))
+    assert torch.equal(s[0:1], sp.sigma(Ct[0:1].contiguous()))
+    out = torch.empty_like(Ct)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):  # a captured call takes the SIMT kernels
+        sp.sigma(Ct, out)
+    g.replay()
+    torch.cuda.synchronize()
+    simt = out.double().cpu().numpy().reshape(6, -1)
+    assert np.array_equal(np.isnan(got), np.isnan(simt)) and np.array_equal(np.isinf(got), np.isinf(simt))
+    _, bound = oracle.sigma(osp, h, eri, 0.25, Cr[0].reshape(1, -1), rows=rows, with_bound=True)
+    assert_sigma_close(got[:1, rows], simt[:1, rows], bound, **({} if dtype == "f64" else F32))
+    sp.close()
+
+
+def test_two_streams_share_a_space(tb, ctx):
+    """Calls on two streams share the digit planes: each result is what it is alone."""
+    import torch
+    sp, _, _, _ = _space(tb, ctx, 13, 6, 6, 1030, 1025, seed=741)
+    C = torch.randn((6, sp.la, sp.lb), dtype=torch.float64, device="cuda")
+    want = [sp.sigma(C[v:v + 1].contiguous()) for v in range(6)]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    parts = [C[v:v + 1].contiguous() for v in range(6)]
+    outs = [torch.empty_like(p) for p in parts]
+    torch.cuda.synchronize()
+    for v in range(6):
+        sp.sigma(parts[v], outs[v], stream=streams[v % 2])
+    torch.cuda.synchronize()
+    for v in range(6):
+        assert torch.equal(outs[v], want[v])
+    sp.close()
+
+
+def test_without_room_for_the_tables(tb):
+    """A budget that holds the prepared space but not the digit tables: the SIMT
+    kernels serve the call, nothing more is counted, and the result stands."""
+    import torch
+    ctx = tb.Context(0)
+    sp, osp, h, eri = _space(tb, ctx, 13, 6, 6, 1030, 1025, seed=751)
+    need = tb.tbsci_hbm_used(ctx.handle)
+    C = np.random.default_rng(4).standard_normal((1, sp.la, sp.lb))
+    full = sp.sigma(torch.from_numpy(C).cuda())
+    assert tb.tbsci_hbm_used(ctx.handle) > need
+    sp.close()
+    ctx.close()
+    ctx = tb.Context(0, hbm_budget=need + (1 << 20))
+    sp, _, _, _ = _space(tb, ctx, 13, 6, 6, 1030, 1025, seed=751)
+    s = sp.sigma(torch.from_numpy(C).cuda())
+    assert tb.tbsci_hbm_used(ctx.handle) == need
+    rows = _rows(sp.ndet, 6)
+    _check(s.cpu().numpy(), osp, h, eri, C, rows)
+    _check(full.cpu().numpy(), osp, h, eri, C, rows)
+    sp.close()
+    ctx.close()
