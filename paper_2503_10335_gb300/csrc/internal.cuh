@@ -385,19 +385,20 @@ tbsci_status rest_dense_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, co
                                bool bf16, cudaStream_t st);
 void dense_context_release(tbsci_ctx *ctx);
 // sigma_exact.cu: FP64 / FP32 sigma summed exactly on the tensor cores (norb <= 16);
-// *ran = false where it does not apply. simt(v, skip) launches the SIMT sigma of
-// vector v, which returns at once where *skip (device memory) is set.
+// *ran = false where it does not apply. simt(v, nv, skip) launches the SIMT sigma of
+// vectors v .. v + nv - 1, each of which returns at once where skip[2 i] (device memory) is set.
 tbsci_status exact_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const double *c, double *s, int nvec,
-                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, const int *)> &simt);
+                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *)> &simt);
 tbsci_status exact_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const float *c, float *s, int nvec,
-                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, const int *)> &simt);
-tbsci_status udiag_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, const float *c, float *s, bool add,
+                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *)> &simt);
+tbsci_status udiag_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, const float *c, float *s, int nv, bool add,
                           bool singles, cudaStream_t st);
 // sigma_tc.cu: the alpha-beta classes on the tensor cores with np = 1 or 3 BF16 planes
 // per operand, FP32 accumulation, added into s
 tbsci_status tile_links_build(tbsci_ctx *ctx, Plan *P, cudaStream_t st);
 tbsci_status sigma_tc_prepare(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int np, cudaStream_t st, bool *ready);
-tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, const int *info, cudaStream_t st);
+tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, int nv, const int *info, cudaStream_t st);
+int sigma_tc_batch(const Plan *P);
 tbsci_status diagonal_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan, double *diag,
                              cudaStream_t st);
 

@@ -61,7 +61,6 @@ struct SigArgs {
     const T *s2_val, *d2_val;
     const int32_t *d2_col;
     const T *U1, *U2, *Eb2;
-    const int *skip;  // device flag: nothing to do where it is set (NULL: none)
 };
 
 // One alpha row Ia of sigma (the whole body of a CTA). REST: only the classes
@@ -305,8 +304,18 @@ __device__ __forceinline__ void sigma_row(const SigArgs<T> &A, const int64_t Ia,
 template <typename T, int NV, bool STAGE, bool ACCS, int kThreads, bool REST = false>
 __global__ void __launch_bounds__(kThreads) k_sigma(SigArgs<T> A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (A.skip && *A.skip) return;
     sigma_row<T, NV, STAGE, ACCS, kThreads, REST>(A, A.rowsa[blockIdx.x], smem_raw);
+}
+
+// The vectors (one per blockIdx.y) that the exact tensor-core path leaves: skip[2 v] = 0.
+// Its own kernel, so that k_sigma's arguments stay constants.
+template <typename T, bool STAGE, bool ACCS>
+__global__ void __launch_bounds__(256) k_sigma_left(SigArgs<T> A, const int *__restrict__ skip) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (skip[2 * blockIdx.y]) return;
+    A.C += blockIdx.y * A.vstride;
+    A.S += blockIdx.y * A.vstride;
+    sigma_row<T, 1, STAGE, ACCS, 256>(A, A.rowsa[blockIdx.x], smem_raw);
 }
 
 // SIMT pass of the tensor-core sigma types over row pairs: A.rowsa holds even
@@ -511,9 +520,8 @@ tbsci_status launch_nv(tbsci_ctx *ctx, SigArgs<T> A, cudaStream_t st, int thread
 template <typename T>
 tbsci_status launch_typed(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, const T *c, T *s, int nvec,
                           cudaStream_t st, int nv_max = 0, int threads = 0, int stage = -1,
-                          const int32_t *rows = nullptr, int64_t nrows = 0, const int *skip = nullptr) {
+                          const int32_t *rows = nullptr, int64_t nrows = 0) {
     SigArgs<T> A = make_args<T>(ham, P);
-    A.skip = skip;
     if (A.la == 0 || A.lb == 0) return TBSCI_OK;
     const int ti = sizeof(T) == 8 ? 0 : 1;
     if (nv_max == 0 && P->tune_nv[ti] > 0) {
@@ -1107,14 +1115,32 @@ tbsci_status sigma_launch_rest(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan 
 
 namespace {
 
+template <typename T, bool STAGE, bool ACCS>
+tbsci_status launch_left(tbsci_ctx *ctx, const SigArgs<T> &A, int nv, const int *skip, cudaStream_t st) {
+    const size_t sm = smem_bytes<T>(A.npair, A.lb, 1, STAGE, ACCS);
+    auto k = k_sigma_left<T, STAGE, ACCS>;
+    TB_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    TraceScope tr(ctx, "k_sigma_left", st);
+    k<<<dim3((unsigned)A.la, (unsigned)nv), 256, sm, st>>>(A, skip);
+    TB_CUDA(ctx, cudaGetLastError());
+    return TBSCI_OK;
+}
+
 // FP64 / FP32: the exact tensor-core path where it applies, else the SIMT kernels
 template <typename T>
 tbsci_status launch_full(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan, const T *c, T *s, int nvec,
                          cudaStream_t st) {
     const size_t n = (size_t)plan->A.l * plan->B.l;
     bool ran = false;
-    TB_TRY(exact_launch(ctx, ham, const_cast<Plan *>(plan), c, s, nvec, st, &ran, [&](int v, const int *skip) {
-        return launch_typed<T>(ctx, ham, plan, c + v * n, s + v * n, 1, st, 0, 0, -1, nullptr, 0, skip);
+    TB_TRY(exact_launch(ctx, ham, const_cast<Plan *>(plan), c, s, nvec, st, &ran, [&](int v, int nv, const int *skip) {
+        SigArgs<T> A = make_args<T>(ham, plan);
+        A.C = c + v * n;
+        A.S = s + v * n;
+        switch (stage_variant<T>(ctx, A.npair, A.lb, 1, 0)) {
+            case 0: return launch_left<T, true, true>(ctx, A, nv, skip, st);
+            case 1: return launch_left<T, false, true>(ctx, A, nv, skip, st);
+            default: return launch_left<T, false, false>(ctx, A, nv, skip, st);
+        }
     }));
     return ran ? TBSCI_OK : launch_typed<T>(ctx, ham, plan, c, s, nvec, st);
 }
@@ -1137,9 +1163,11 @@ tbsci_status sigma_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan
             return launch_typed<float>(ctx, ham, plan, cf, sf, nvec, st);
         TB_TRY(sigma_launch_rest(ctx, ham, plan, cf, sf, nvec, st, -1, 0, nullptr, 0, np == 1));
         const size_t n = (size_t)plan->A.l * plan->B.l;
-        for (int v = 0; v < nvec; ++v) {
-            TB_TRY(udiag_launch(ctx, ham, plan, cf + v * n, sf + v * n, true, true, st));
-            TB_TRY(sigma_tc_ab(ctx, const_cast<Plan *>(plan), np, cf + v * n, sf + v * n, nullptr, st));
+        const int batch = sigma_tc_batch(plan);
+        for (int v = 0; v < nvec; v += batch) {
+            const int nv = std::min(batch, nvec - v);
+            TB_TRY(udiag_launch(ctx, ham, plan, cf + v * n, sf + v * n, nv, true, true, st));
+            TB_TRY(sigma_tc_ab(ctx, const_cast<Plan *>(plan), np, cf + v * n, sf + v * n, nv, nullptr, st));
         }
         return TBSCI_OK;
     }

@@ -8,7 +8,9 @@
 // drained as integers and combined in 64-bit words. Only the digits that are cut off
 // (below 2^-64 of the vector's scale, 2^-56 of the Hamiltonian's) and the products of
 // weight below 256^-9 are lost: less than the rounding of the FP64 sums that they
-// replace (measured below). FP32 sigma takes 4 + 4 digits and weights to 256^-5.
+// replace (norb 16, 3,000 x 3,000 strings: 6.1e-16 of the norm from 64-bit values, the
+// SIMT kernel 1.5e-15). FP32 sigma takes 4 + 4 digits and weights to 256^-5 for the
+// same-spin classes (1.3e-7 in all, the SIMT kernel 6.2e-7).
 // Integer sums are associative: results do not depend on the order of the work.
 //
 // Parts of a sigma (Sec. II.B, Eq. 7; the classes [a,b] of Sec. II.C):
@@ -16,9 +18,11 @@
 //                   with the beta string unchanged (SIMT, one multiply-add per term)
 //   k_same_spin_ex  the same-spin classes as one dense product per 128 x NT tile,
 //                   sigma += c Hb^T + Ha c over the off-diagonal string Hamiltonians
-//   k_sigma_ab_ex   the alpha-beta classes: per alpha row G = A F over the row's
-//                   alpha terms (A: integrals (rs|pq), F: the coupled c rows), then G
-//                   summed into the columns its beta links point to
+//   k_sigma_ab_ex   the alpha-beta classes (FP64; FP32 takes sigma_tc.cu's kernel):
+//                   per alpha row G = A F over the row's alpha terms (A: integrals
+//                   (rs|pq), F: the coupled c rows), then G summed into the columns
+//                   its beta links point to
+// Small spaces take several vectors per launch.
 // A vector is scaled by one power of two. Digits are relative to that scale, so a
 // vector whose largest entry is far above its root mean square would lose digits of
 // the others: k_scale_final refuses such vectors (and NaN, infinities, extreme
@@ -122,9 +126,14 @@ __host__ __device__ inline int scale_exponent(double top) {
 constexpr int kScaleThreads = 256;
 constexpr int kScaleBlocks = 304;
 
-// per-block largest magnitude and sum of squares of one vector
+// Per vector (blockIdx.y) its largest magnitude and sum of squares, in a fixed order;
+// the last block to finish writes info[2 v]: 1 when the digits serve the vector,
+// info[2 v + 1]: its scale exponent. done[v] wraps back to 0.
 template <typename T>
-__global__ void __launch_bounds__(kScaleThreads) k_scale_partial(const T *__restrict__ c, int64_t n, double *part) {
+__global__ void __launch_bounds__(kScaleThreads) k_scale(const T *__restrict__ c0, int64_t n, double ratio, double *part0,
+                                                         unsigned *done, const int *__restrict__ tab, int *info) {
+    const T *__restrict__ c = c0 + blockIdx.y * n;
+    double *part = part0 + (size_t)blockIdx.y * 2 * kScaleBlocks;
     double top = 0.0, sum = 0.0;
     bool bad = false;
     const int64_t step = (int64_t)gridDim.x * kScaleThreads;
@@ -145,55 +154,59 @@ __global__ void __launch_bounds__(kScaleThreads) k_scale_partial(const T *__rest
     }
     if (bad) top = INFINITY;
     __shared__ double st[kScaleThreads], ss[kScaleThreads];
-    st[threadIdx.x] = top;
-    ss[threadIdx.x] = sum;
-    __syncthreads();
-    for (int o = kScaleThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            st[threadIdx.x] = fmax(st[threadIdx.x], st[threadIdx.x + o]);
-            ss[threadIdx.x] += ss[threadIdx.x + o];
-        }
+    __shared__ bool last;
+    auto fold = [&] {
+        st[threadIdx.x] = top;
+        ss[threadIdx.x] = sum;
         __syncthreads();
-    }
+        for (int o = kScaleThreads / 2; o > 0; o >>= 1) {
+            if (threadIdx.x < o) {
+                st[threadIdx.x] = fmax(st[threadIdx.x], st[threadIdx.x + o]);
+                ss[threadIdx.x] += ss[threadIdx.x + o];
+            }
+            __syncthreads();
+        }
+    };
+    fold();
     if (threadIdx.x == 0) {
         part[2 * blockIdx.x] = st[0];
         part[2 * blockIdx.x + 1] = ss[0];
+        __threadfence();
+        last = atomicInc(done + blockIdx.y, gridDim.x - 1) == gridDim.x - 1;
     }
-}
-
-// info[0]: 1 when the digits serve this vector, info[1]: its scale exponent
-__global__ void __launch_bounds__(512) k_scale_final(const double *__restrict__ part, int nblocks, int64_t n, double ratio,
-                                                     int *info) {
-    __shared__ double st[512], ss[512];
-    st[threadIdx.x] = threadIdx.x < nblocks ? part[2 * threadIdx.x] : 0.0;
-    ss[threadIdx.x] = threadIdx.x < nblocks ? part[2 * threadIdx.x + 1] : 0.0;
     __syncthreads();
-    for (int o = 256; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            st[threadIdx.x] = fmax(st[threadIdx.x], st[threadIdx.x + o]);
-            ss[threadIdx.x] += ss[threadIdx.x + o];
-        }
-        __syncthreads();
+    if (!last) return;
+    __threadfence();
+    top = sum = 0.0;
+    for (int b = threadIdx.x; b < gridDim.x; b += kScaleThreads) {
+        top = fmax(top, __ldcg(part + 2 * b));
+        sum += __ldcg(part + 2 * b + 1);
     }
+    fold();
     if (threadIdx.x != 0) return;
-    const double top = st[0];
+    top = st[0];
     int ok = 0, e = 0;
-    if (top == 0.0) {
+    if (!tab[2]) {
+        ok = 0;
+    } else if (top == 0.0) {
         ok = 1;
     } else if (top < 1e15 && top > 1e-15) {
         e = scale_exponent(top);
         ok = ldexp(1.0, e) <= ratio * sqrt(ss[0] / (double)n) ? 1 : 0;
     }
-    info[0] = ok;
-    info[1] = e;
+    info[2 * blockIdx.y] = ok;
+    info[2 * blockIdx.y + 1] = e;
 }
 
-// the digit planes [NSC][la][lbp] of a vector, columns lb .. lbp - 1 zero; 8 columns per thread
+// the digit planes [NSC][la][lbp] of each vector, columns lb .. lbp - 1 zero; 8 columns per thread
 template <int P>
 __global__ void __launch_bounds__(256) k_slice(const typename Prec<P>::T *__restrict__ c, int64_t la, int64_t lb,
                                                int64_t lbp, const int *__restrict__ info, __nv_bfloat16 *out) {
+    info += 2 * blockIdx.y;
     if (!info[0]) return;
     constexpr int N = Prec<P>::NSC;
+    c += blockIdx.y * la * lb;
+    out += blockIdx.y * N * la * lbp;
     const int shift = 8 * N - info[1];
     const int64_t per = lbp / 8, n = la * per, plane = la * lbp;
     for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
@@ -226,31 +239,45 @@ __global__ void k_absmax(const double *__restrict__ v, int64_t n, unsigned long 
     if ((threadIdx.x & 31) == 0 && m) atomicMax(top, m);
 }
 
+// tab[0], tab[1]: scale exponents of the integrals and of the string Hamiltonians from
+// their largest magnitudes (W_Ia / 8 shares the integrals' scale: up to nelec / 8 of
+// them); tab[2]: 0 where a magnitude is far from 1 (or not finite): such a Hamiltonian
+// stays on the SIMT kernels
+__global__ void k_table_scales(const unsigned long long *__restrict__ top, double w, int *tab) {
+    const double v = w * __longlong_as_double((long long)top[0]), h = __longlong_as_double((long long)top[1]);
+    tab[2] = (v == 0.0 || (v > 1e-15 && v < 1e15)) && (h == 0.0 || (h > 1e-15 && h < 1e15)) ? 1 : 0;
+    tab[0] = tab[2] && v > 0.0 ? scale_exponent(v) : 0;
+    tab[1] = tab[2] && h > 0.0 ? scale_exponent(h) : 0;
+}
+
+// the links of one CSR row per warp into dense digit planes [NSA][l][ld] (zeroed before),
+// and their number per 32-column chunk
 template <int P>
-__device__ __forceinline__ void put_digits(double x, int e, __nv_bfloat16 *out, int64_t plane) {
+__global__ void __launch_bounds__(256) k_dense_digits(int64_t l, int64_t ld, int nch, const int64_t *__restrict__ soff,
+                                                      const int2 *__restrict__ sci, const double *__restrict__ sval,
+                                                      const int64_t *__restrict__ doff, const int32_t *__restrict__ dcol,
+                                                      const double *__restrict__ dval, const int *__restrict__ tab,
+                                                      __nv_bfloat16 *out, uint8_t *cnt) {
+    extern __shared__ unsigned scnt[];  // [8][nch]
+    if (!tab[2]) return;
     constexpr int N = Prec<P>::NSA;
-    const int64_t f = to_fixed(x, 8 * N - e);
-    for (int s = 0; s < N; ++s) out[s * plane] = __ushort_as_bfloat16((unsigned short)digit_bf16<N>(f, s));
-}
-
-// the links of one CSR row per warp into dense digit planes [NSA][l][ld] (zeroed before)
-template <int P>
-__global__ void k_dense_digits(int64_t l, int64_t ld, const int64_t *__restrict__ off, const int2 *__restrict__ sci,
-                               const int32_t *__restrict__ dcol, const double *__restrict__ val, int e,
-                               __nv_bfloat16 *out) {
-    const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t r = blockIdx.x * 8ll + warp, plane = l * ld;
     if (r >= l) return;
-    for (int64_t t = off[r] + (threadIdx.x & 31); t < off[r + 1]; t += 32)
-        put_digits<P>(val[t], e, out + r * ld + (sci ? sci[t].x : dcol[t]), l * ld);
-}
-
-// links of each row per 32-column chunk
-__global__ void k_chunk_counts(int64_t l, int nch, const int64_t *__restrict__ soff, const int2 *__restrict__ sci,
-                               const int64_t *__restrict__ doff, const int32_t *__restrict__ dcol, uint8_t *cnt) {
-    const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (r >= l) return;
-    for (int64_t t = soff[r]; t < soff[r + 1]; ++t) ++cnt[r * nch + (sci[t].x >> 5)];
-    for (int64_t t = doff[r]; t < doff[r + 1]; ++t) ++cnt[r * nch + (dcol[t] >> 5)];
+    unsigned *c = scnt + warp * nch;
+    for (int k = lane; k < nch; k += 32) c[k] = 0;
+    __syncwarp();
+    const int shift = 8 * N - tab[1];
+    auto put = [&](int col, double x) {
+        const int64_t f = to_fixed(x, shift);
+#pragma unroll
+        for (int s = 0; s < N; ++s) out[s * plane + r * ld + col] = __ushort_as_bfloat16((unsigned short)digit_bf16<N>(f, s));
+        atomicAdd(c + (col >> 5), 1u);
+    };
+    for (int64_t t = soff[r] + lane; t < soff[r + 1]; t += 32) put(sci[t].x, sval[t]);
+    for (int64_t t = doff[r] + lane; t < doff[r + 1]; t += 32) put(dcol[t], dval[t]);
+    __syncwarp();
+    for (int k = lane; k < nch; k += 32) cnt[r * nch + k] = (uint8_t)c[k];
 }
 
 // The accumulators stay exact while a row has met at most kWindow links: 7 products
@@ -280,7 +307,7 @@ __global__ void k_windows(int64_t l, int nch, int rows, const uint8_t *__restric
 
 // digits of the integral columns: [pair][128 off-diagonal pairs], and of W_Ia / 8 (times 8): [la][128]
 __global__ void k_ab_digits(const double *__restrict__ V, int npair, int npoff, const int32_t *__restrict__ offpair,
-                            const uint64_t *__restrict__ str, int64_t rows, int e, uint4 *out) {
+                            const uint64_t *__restrict__ str, int64_t rows, const int *__restrict__ tab, uint4 *out) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= rows * 128) return;
     const int64_t row = i >> 7;
@@ -299,7 +326,7 @@ __global__ void k_ab_digits(const double *__restrict__ V, int npair, int npoff, 
             x = V[(size_t)row * npair + col];
         }
     }
-    const int64_t f = to_fixed(x, 8 * N - e);
+    const int64_t f = tab[2] ? to_fixed(x, 8 * N - tab[0]) : 0;
     union {
         uint16_t h[8];
         uint4 v;
@@ -326,29 +353,36 @@ struct UdArgs {
     const int2 *a_sci;
     const T *a_sval, *Ea, *Eb, *U;
     T ecore;
-    int na, add, singles;  // add: accumulate; singles: with the string-Hamiltonian values of the alpha singles
+    int na, add;  // add: accumulate
 };
 
-// S[Ia][j] (+)= Hd c(Ia, j) + sum over alpha singles (h + s U[pq][j]) c(Ja, j). Bound by
-// L2: two coalesced reads per term.
-template <typename T>
+// S[Ia][j] (+)= Hd c(Ia, j) + sum over alpha singles ([h +] s U[pq][j]) c(Ja, j), one vector
+// per blockIdx.z; SINGLES: with their string-Hamiltonian values h. FP64 is bound by the
+// FP64 pipe, FP32 by L2 (two coalesced reads per term). CTAs run column chunk by column
+// chunk, so that those in flight share the chunk's columns of U and c (norb 16, 3,000 x
+// 3,000 strings, FP64, a vector: 0.58 ms; 1.42 with an FP64 compare per sign).
+constexpr int64_t kUdCols = 512;  // columns of a CTA
+
+__device__ __forceinline__ double flip(double x, int m) { return __hiloint2double(__double2hiint(x) ^ m, __double2loint(x)); }
+__device__ __forceinline__ float flip(float x, int m) { return __int_as_float(__float_as_int(x) ^ m); }
+
+template <typename T, bool SINGLES>
 __global__ void __launch_bounds__(256) k_udiag(UdArgs<T> A) {
-    if (A.info && !A.info[0]) return;
+    if (A.info && !A.info[2 * blockIdx.z]) return;
     __shared__ int64_t sC[256], sU[256];
-    __shared__ T sH[256], sS[256];
+    __shared__ T sH[256];
+    __shared__ int sS[256];  // sign bit of the term
     __shared__ int sOcc[64];
     const int64_t Ia = blockIdx.x, lb = A.lb;
     const int64_t t0 = A.a_soff[Ia], t1 = A.a_soff[Ia + 1];
-    const int64_t j = blockIdx.y * 256ll + threadIdx.x;
     const int tid = threadIdx.x;
-    if (tid == 0) {
-        int k = 0;
-        for (uint64_t s = A.stra[Ia]; s; s &= s - 1) {
-            const int p = __ffsll((long long)s) - 1;
-            sOcc[k++] = p * (p + 1) / 2 + p;
-        }
+    const T *__restrict__ C = A.C + blockIdx.z * A.la * lb;
+    T *__restrict__ S = A.S + blockIdx.z * A.la * lb + Ia * lb;
+    if (tid < 64) {
+        const uint64_t s = A.stra[Ia];
+        if ((s >> tid) & 1) sOcc[__popcll(s & ((1ull << tid) - 1))] = tid * (tid + 1) / 2 + tid;
     }
-    T acc = T(0), acc2 = T(0);
+    const T eIa = A.ecore + A.Ea[Ia];
     for (int64_t t = t0; t < t1 || t == t0; t += 256) {
         const int n = (int)min((int64_t)256, t1 - t);
         __syncthreads();
@@ -356,39 +390,38 @@ __global__ void __launch_bounds__(256) k_udiag(UdArgs<T> A) {
             const int2 e = A.a_sci[t + tid];
             sC[tid] = e.x * lb;
             sU[tid] = (int64_t)(e.y >> 1) * lb;
-            sS[tid] = (e.y & 1) ? T(-1) : T(1);
-            sH[tid] = A.singles ? A.a_sval[t + tid] : T(0);
+            sS[tid] = (e.y & 1) ? (int)0x80000000 : 0;
+            if (SINGLES) sH[tid] = A.a_sval[t + tid];
         }
         __syncthreads();
-        if (j >= lb) continue;
-        if (t == t0) {
-            T ed = A.ecore + A.Ea[Ia] + __ldg(A.Eb + j);
-            for (int k = 0; k < A.na; ++k) ed += __ldg(A.U + (size_t)sOcc[k] * lb + j);
-            acc = ed * __ldg(A.C + Ia * lb + j);
-        }
-        int k = 0;
-        for (; k + 3 < n; k += 4) {
-            const T u0 = __ldg(A.U + sU[k] + j), u1 = __ldg(A.U + sU[k + 1] + j);
-            const T u2 = __ldg(A.U + sU[k + 2] + j), u3 = __ldg(A.U + sU[k + 3] + j);
-            const T c0 = __ldg(A.C + sC[k] + j), c1 = __ldg(A.C + sC[k + 1] + j);
-            const T c2 = __ldg(A.C + sC[k + 2] + j), c3 = __ldg(A.C + sC[k + 3] + j);
-            if (A.singles) {
-                acc += (sH[k] + sS[k] * u0) * c0;
-                acc2 += (sH[k + 1] + sS[k + 1] * u1) * c1;
-                acc += (sH[k + 2] + sS[k + 2] * u2) * c2;
-                acc2 += (sH[k + 3] + sS[k + 3] * u3) * c3;
-            } else {  // one multiply-add per term: the sign goes to u by its sign bit
-                acc += (sS[k] < T(0) ? -u0 : u0) * c0;
-                acc2 += (sS[k + 1] < T(0) ? -u1 : u1) * c1;
-                acc += (sS[k + 2] < T(0) ? -u2 : u2) * c2;
-                acc2 += (sS[k + 3] < T(0) ? -u3 : u3) * c3;
+        for (int64_t j = blockIdx.y * kUdCols + tid; j < min(lb, (blockIdx.y + 1) * kUdCols); j += 256) {
+            T acc = T(0), acc2 = T(0);
+            if (t == t0) {
+                T ed = eIa + __ldg(A.Eb + j);
+                for (int k = 0; k < A.na; ++k) ed += __ldg(A.U + (size_t)sOcc[k] * lb + j);
+                acc = ed * __ldg(C + Ia * lb + j);
             }
+            const T *__restrict__ Uj = A.U + j, *__restrict__ Cj = C + j;
+            // one multiply-add per term: the sign goes to u by its sign bit (an FP64 compare
+            // and select would take the pipe's other half)
+            auto coef = [&](int k, T u) { return SINGLES ? sH[k] + flip(u, sS[k]) : flip(u, sS[k]); };
+            int k = 0;
+            for (; k + 3 < n; k += 4) {
+                const T u0 = __ldg(Uj + sU[k]), u1 = __ldg(Uj + sU[k + 1]), u2 = __ldg(Uj + sU[k + 2]), u3 = __ldg(Uj + sU[k + 3]);
+                const T c0 = __ldg(Cj + sC[k]), c1 = __ldg(Cj + sC[k + 1]), c2 = __ldg(Cj + sC[k + 2]), c3 = __ldg(Cj + sC[k + 3]);
+                acc += coef(k, u0) * c0;
+                acc2 += coef(k + 1, u1) * c1;
+                acc += coef(k + 2, u2) * c2;
+                acc2 += coef(k + 3, u3) * c3;
+            }
+            for (; k < n; ++k) acc += coef(k, __ldg(Uj + sU[k])) * __ldg(Cj + sC[k]);
+            S[j] = (A.add || t > t0 ? S[j] : T(0)) + (acc + acc2);
         }
-        for (; k < n; ++k) acc += (sH[k] + sS[k] * __ldg(A.U + sU[k] + j)) * __ldg(A.C + sC[k] + j);
     }
-    if (j >= lb) return;
-    T *s = A.S + Ia * lb + j;
-    *s = (A.add ? *s : T(0)) + (acc + acc2);
+}
+
+inline dim3 ud_grid(int64_t la, int64_t lb, int nv) {
+    return dim3((unsigned)la, (unsigned)((lb + kUdCols - 1) / kUdCols), (unsigned)nv);
 }
 
 // ------------------------------------------------------------------ same-spin classes
@@ -398,8 +431,7 @@ struct SsArgs {
     int64_t la, lb;
     int nchb, ncha;  // 32-column chunks of the beta / alpha phase
     const uint8_t *flb, *fla;
-    const int *info;
-    int eH;
+    const int *info, *tab;
     void *S;
     int *err;
 };
@@ -433,7 +465,8 @@ constexpr int kSsThreads = 576;  // 16 draining warps, a TMA warp, an MMA warp
 // at the end.
 template <int P>
 __global__ void __launch_bounds__(kSsThreads, 1) k_same_spin_ex(const __grid_constant__ SsArgs A) {
-    if (!A.info[0]) return;
+    const int *info = A.info + 2 * blockIdx.z;  // one vector per blockIdx.z
+    if (!info[0]) return;
     using Sh = SsShape<P>;
     typedef typename Prec<P>::T T;
     constexpr int NSA = Sh::NSA, NSC = Sh::NSC, ORD = Sh::ORD, NT = Sh::NT, NST = Sh::kStages;
@@ -482,13 +515,13 @@ __global__ void __launch_bounds__(kSsThreads, 1) k_same_spin_ex(const __grid_con
                              "r"(beta ? Sh::kBetaBytes : Sh::kAlphaBytes)
                              : "memory");
                 if (beta) {
-                    tma3(dst, &A.mCA, fb, ch * 32, (int)row0, 0);
+                    tma3(dst, &A.mCA, fb, ch * 32, (int)row0, (int)blockIdx.z * NSC);
                     tma3(dst + NSC * 128 * 64, &A.mHb, fb, ch * 32, (int)col0, 0);
                 } else {
                     const int k = (ch - A.nchb) * 32;
                     tma3(dst, &A.mHa, fb, k, (int)row0, 0);
                     for (int b = 0; b < NT / 64; ++b)
-                        tma3(dst + NSA * 128 * 64 + b * NSC * 4096, &A.mCB, fb, (int)col0 + 64 * b, k, 0);
+                        tma3(dst + NSA * 128 * 64 + b * NSC * 4096, &A.mCB, fb, (int)col0 + 64 * b, k, (int)blockIdx.z * NSC);
                 }
                 ++n;
             }
@@ -609,8 +642,8 @@ __global__ void __launch_bounds__(kSsThreads, 1) k_same_spin_ex(const __grid_con
         }
         const int64_t Ia = row0 + quarter * 32 + lane, jb = col0 + part * NC;
         if (Ia < A.la) {
-            T *S = static_cast<T *>(A.S) + Ia * A.lb;
-            const double sc = pow2(A.eH + A.info[1] - 8 * (ORD + 1));
+            T *S = static_cast<T *>(A.S) + blockIdx.z * A.la * A.lb + Ia * A.lb;
+            const double sc = pow2(A.tab[1] + info[1] - 8 * (ORD + 1));
 #pragma unroll
             for (int x = 0; x < NC; ++x)
                 if (jb + x < A.lb) {
@@ -623,7 +656,7 @@ __global__ void __launch_bounds__(kSsThreads, 1) k_same_spin_ex(const __grid_con
     __syncthreads();
     if (sAbort && tid == 0) {
         atomicExch(A.err, 1);
-        if (row0 < A.la && col0 < A.lb) static_cast<T *>(A.S)[row0 * A.lb + col0] = (T)NAN;  // fail loudly
+        if (row0 < A.la && col0 < A.lb) static_cast<T *>(A.S)[blockIdx.z * A.la * A.lb + row0 * A.lb + col0] = (T)NAN;  // fail loudly
     }
     if (warp == 17) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base));
 }
@@ -634,8 +667,7 @@ struct AbArgs {
     int64_t la, lb, lbp;
     const __nv_bfloat16 *Cs;
     void *S;
-    const int *info;
-    int eV;
+    const int *info, *tab;
     const uint4 *Vd, *Wd;  // digits of the integral columns: [pair][128], [la][128]
     const int64_t *a_soff;
     const int2 *a_sci;
@@ -658,7 +690,8 @@ struct AbArgs {
 // to a slot per beta link (the slots of a tile ordered by target column); a thread then
 // sums the slots of a target column into the row's 64-bit sums. No atomics.
 __global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab_ex(const AbArgs A) {
-    if (!A.info[0]) return;
+    const int *info = A.info + 2 * blockIdx.y;  // one vector per blockIdx.y
+    if (!info[0]) return;
     typedef double T;
     constexpr int NSA = Prec<0>::NSA, NSC = Prec<0>::NSC, ORD = Prec<0>::ORD, NW = 2;
     extern __shared__ unsigned char smem_dyn[];
@@ -825,7 +858,7 @@ __global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab_ex(const AbArgs A) {
         for (int t = g; t < ntiles && g < ng; t += ng) {
             const int st = t % nst;
             if (t >= nst && !mb_wait(bempty + 8 * st, (t / nst - 1) & 1, ab)) break;
-            gather_tile<NSC>(A.Cs, (size_t)A.la * lbp, lbp, sJa, Kp, t, sB + st * stage_sz);
+            gather_tile<NSC>(A.Cs + blockIdx.y * NSC * A.la * lbp, (size_t)A.la * lbp, lbp, sJa, Kp, t, sB + st * stage_sz);
             mb_arrive(bfull + 8 * st);
         }
     } else {
@@ -931,8 +964,8 @@ __global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab_ex(const AbArgs A) {
     }
     tc_before();
     __syncthreads();
-    T *S = static_cast<T *>(A.S) + Ia * lb;
-    const double sc = pow2(A.eV + A.info[1] - 8 * (ORD + 1));
+    T *S = static_cast<T *>(A.S) + (blockIdx.y * A.la + Ia) * lb;
+    const double sc = pow2(A.tab[0] + info[1] - 8 * (ORD + 1));
     for (int64_t j = tid; j < lb; j += kAbThreads) {
         S[j] += fma((double)sAcc[j], 4294967296.0, (double)sAcc[lb + j]) * sc;
     }
@@ -962,9 +995,9 @@ EncodeTiled encode_tiled() {
     return fn;
 }
 
-// digit planes [planes][rows][cols] (cols a multiple of 64), box [all planes][box_rows][box_cols]
-bool plane_map(CUtensorMap *m, void *base, int64_t cols, int64_t rows, int planes, int box_cols, int box_rows) {
-    const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+// digit planes [sets][planes][rows][cols] (cols a multiple of 64), box [all planes][box_rows][box_cols]
+bool plane_map(CUtensorMap *m, void *base, int64_t cols, int64_t rows, int planes, int box_cols, int box_rows, int sets = 1) {
+    const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes * sets};
     const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * rows * 2};
     const cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, (cuuint32_t)planes}, es[3] = {1, 1, 1};
     const EncodeTiled fn = encode_tiled();
@@ -975,27 +1008,27 @@ bool plane_map(CUtensorMap *m, void *base, int64_t cols, int64_t rows, int plane
 
 }  // namespace
 
-// What the exact path keeps for one prepared space: built by the first sigma that takes
-// it. Calls on several streams share the digit planes of c, so each call waits for the
-// event that the one before it recorded; `mu` keeps the launches of one call together.
+// What the exact path keeps for one prepared space and precision, in one allocation made
+// by the first sigma that takes it. Calls on several streams share the digit planes of
+// c, so each call waits for the event that the one before it recorded; `mu` keeps the
+// launches of one call together.
 struct ExactData {
     std::mutex mu;
-    cudaEvent_t busy = nullptr;
-    bool tried = false, ok = false;
     struct Type {
         bool tried = false, ready = false;
-        int eV = 0, eH = 0;
-        DevBuf<unsigned char> Vd, Wd;
-        DevBuf<__nv_bfloat16> Hb, Ha;
-        DevBuf<uint8_t> flb, fla;
+        int batch = 1;  // vectors per launch
+        cudaEvent_t busy = nullptr;
+        DevBuf<unsigned char> arena;
+        uint4 *Vd = nullptr, *Wd = nullptr;
+        __nv_bfloat16 *planes = nullptr;  // digit planes of `batch` vectors
+        double *part = nullptr;
+        int *info = nullptr, *tab = nullptr;
+        unsigned *done = nullptr;
         SsArgs ss{};
-        const void *planes = nullptr;  // the scratch that the maps point into
     } type[2];
-    DevBuf<unsigned char> planes;  // digit planes of one vector
-    DevBuf<double> part;
-    DevBuf<int> info;
     ~ExactData() {
-        if (busy) cudaEventDestroy(busy);
+        for (Type &t : type)
+            if (t.busy) cudaEventDestroy(t.busy);
     }
 };
 
@@ -1013,23 +1046,8 @@ int ab_stage_bytes(const tbsci_ctx *ctx, const Plan *P) {
     return room < one ? 0 : (int)std::min<int64_t>(room, 4 * (int64_t)one);
 }
 
-// Scale scratch and the event of a space's first call.
-tbsci_status build_common(tbsci_ctx *ctx, Plan *P, ExactData *X) {
-    X->tried = true;
-    if (P->tl_kpmax == 0) return TBSCI_OK;
-    cudaError_t e = X->part.alloc(2 * kScaleBlocks);
-    if (e == cudaSuccess) e = X->info.alloc(2);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&X->busy, cudaEventDisableTiming);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return e == cudaErrorMemoryAllocation ? TBSCI_OK : fail(ctx, TBSCI_ECUDA, std::string("scale scratch: ") + cudaGetErrorString(e));
-    }
-    X->ok = true;
-    return TBSCI_OK;
-}
-
-// Digit tables of the Hamiltonian for one precision; without room for them the space
-// stays on the SIMT kernels.
+// Digit tables of the Hamiltonian for one precision, enqueued on `st`; without room for
+// them the space stays on the SIMT kernels.
 template <int PR>
 tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData *X, cudaStream_t st) {
     typename ExactData::Type &Y = X->type[PR];
@@ -1040,142 +1058,119 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
     if ((PR == 0 && ab_stage_bytes(ctx, P) == 0) || !encode_tiled()) return TBSCI_OK;
     const int ncha = (int)((la + 31) / 32), nchb = (int)((lb + 31) / 32);
     const int64_t nba = (la + 127) / 128, nbb = (lb + Sh::NT - 1) / Sh::NT;
-    const size_t planes = (size_t)NSC * la * lbp * 2;
-    const size_t grow = planes > X->planes.n ? planes : 0;
-    // digits of the integrals: the FP64 alpha-beta kernel's (FP32 takes sigma_tc.cu's)
-    const size_t vd = PR == 0 ? (size_t)P->npair * 128 * sizeof(uint4) : 0, wd = PR == 0 ? (size_t)la * 128 * sizeof(uint4) : 0;
-    const size_t hb = (size_t)NSA * lb * lbp, ha = (size_t)NSA * la * lap;
-    const size_t bytes = vd + wd + 2 * (hb + ha) + (size_t)(nbb * nchb + nba * ncha) + grow;
-    if (charge(ctx, bytes, "digit tables") != TBSCI_OK) return TBSCI_OK;
-    cudaError_t e = cudaSuccess;
-    auto need = [&](auto &buf, size_t n) {
-        if (e == cudaSuccess) e = buf.alloc(n);
+    Y.batch = sigma_tc_batch(P);
+    // places in the allocation, 256-byte aligned
+    size_t at = 0;
+    auto place = [&](size_t n) {
+        const size_t p = at;
+        at += (n + 255) / 256 * 256;
+        return p;
     };
-    DevBuf<unsigned long long> top;
-    DevBuf<uint8_t> cnt;
-    need(top, 2);
-    need(cnt, (size_t)std::max(la * ncha, lb * nchb));
-    need(Y.Vd, vd);
-    need(Y.Wd, wd);
-    need(Y.Hb, hb);
-    need(Y.Ha, ha);
-    need(Y.flb, (size_t)nbb * nchb);
-    need(Y.fla, (size_t)nba * ncha);
-    size_t old = 0;
-    if (e == cudaSuccess && grow) {
-        old = X->planes.n;
-        if (old) e = cudaEventSynchronize(X->busy);
-        need(X->planes, planes);
-    }
-    unsigned long long ht[2] = {0, 0};
-    if (e == cudaSuccess) e = cudaMemsetAsync(top.p, 0, 16, st);
+    const size_t hb = place((size_t)NSA * lb * lbp * 2), ha = place((size_t)NSA * la * lap * 2);
+    const size_t top = place(16), done = place(4 * (size_t)Y.batch), zeroed = at;
+    const size_t vd = place(PR == 0 ? (size_t)P->npair * 128 * sizeof(uint4) : 0);  // FP32: sigma_tc.cu's planes
+    const size_t wd = place(PR == 0 ? (size_t)la * 128 * sizeof(uint4) : 0);
+    const size_t cb = place((size_t)lb * nchb), ca = place((size_t)la * ncha);
+    const size_t fb = place((size_t)nbb * nchb), fa = place((size_t)nba * ncha);
+    const size_t part = place((size_t)Y.batch * 2 * kScaleBlocks * 8), info = place(8 * (size_t)Y.batch), tab = place(12);
+    const size_t planes = place((size_t)Y.batch * NSC * la * lbp * 2);
+    if (charge(ctx, at, "digit tables") != TBSCI_OK) return TBSCI_OK;
+    cudaError_t e = Y.arena.alloc(at);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&Y.busy, cudaEventDisableTiming);
+    unsigned char *B = Y.arena.p;
+    if (e == cudaSuccess) e = cudaMemsetAsync(B, 0, zeroed, st);
+    SsArgs &S = Y.ss;
     if (e == cudaSuccess) {
-        const int64_t nv = (int64_t)P->npair * P->npair;
-        k_absmax<<<64, 256, 0, st>>>(ham->d_V.p, nv, top.p);
+        Y.Vd = reinterpret_cast<uint4 *>(B + vd);
+        Y.Wd = reinterpret_cast<uint4 *>(B + wd);
+        Y.planes = reinterpret_cast<__nv_bfloat16 *>(B + planes);
+        Y.part = reinterpret_cast<double *>(B + part);
+        Y.info = reinterpret_cast<int *>(B + info);
+        Y.tab = reinterpret_cast<int *>(B + tab);
+        Y.done = reinterpret_cast<unsigned *>(B + done);
+        unsigned long long *tp = reinterpret_cast<unsigned long long *>(B + top);
+        auto blocks = [](size_t n) { return (unsigned)std::min<size_t>(152, (n + 255) / 256); };
+        k_absmax<<<blocks((size_t)P->npair * P->npair), 256, 0, st>>>(ham->d_V.p, (int64_t)P->npair * P->npair, tp);
         for (const SpinPlan *sp : {&P->A, &P->B}) {
-            if (sp->d_sval.n) k_absmax<<<152, 256, 0, st>>>(sp->d_sval.p, (int64_t)sp->d_sval.n, top.p + 1);
-            if (sp->d_dval.n) k_absmax<<<152, 256, 0, st>>>(sp->d_dval.p, (int64_t)sp->d_dval.n, top.p + 1);
+            if (sp->d_sval.n) k_absmax<<<blocks(sp->d_sval.n), 256, 0, st>>>(sp->d_sval.p, (int64_t)sp->d_sval.n, tp + 1);
+            if (sp->d_dval.n) k_absmax<<<blocks(sp->d_dval.n), 256, 0, st>>>(sp->d_dval.p, (int64_t)sp->d_dval.n, tp + 1);
         }
-        e = cudaMemcpyAsync(ht, top.p, 16, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    }
-    double tv, th;
-    std::memcpy(&tv, &ht[0], 8);
-    std::memcpy(&th, &ht[1], 8);
-    tv *= std::max(1.0, P->A.nelec / 8.0);  // W_Ia / 8 shares the integrals' scale
-    // scales far from 1 stay on the SIMT kernels (an all-zero class needs no scale)
-    const bool fair = (tv == 0.0 || (tv > 1e-15 && tv < 1e15)) && (th == 0.0 || (th > 1e-15 && th < 1e15));
-    if (e == cudaSuccess && fair) {
-        Y.eV = tv > 0.0 ? scale_exponent(tv) : 0;
-        Y.eH = th > 0.0 ? scale_exponent(th) : 0;
+        k_table_scales<<<1, 1, 0, st>>>(tp, std::max(1.0, P->A.nelec / 8.0), Y.tab);
         if (PR == 0) {
-            k_ab_digits<<<(unsigned)(((int64_t)P->npair * 128 + 255) / 256), 256, 0, st>>>(
-                ham->d_V.p, P->npair, P->npoff, P->d_offpair.p, nullptr, P->npair, Y.eV, reinterpret_cast<uint4 *>(Y.Vd.p));
-            k_ab_digits<<<(unsigned)((la * 128 + 255) / 256), 256, 0, st>>>(
-                ham->d_V.p, P->npair, P->npoff, P->d_offpair.p, P->A.d_str, la, Y.eV, reinterpret_cast<uint4 *>(Y.Wd.p));
+            k_ab_digits<<<(unsigned)(((int64_t)P->npair * 128 + 255) / 256), 256, 0, st>>>(ham->d_V.p, P->npair, P->npoff, P->d_offpair.p,
+                                                                                          nullptr, P->npair, Y.tab, Y.Vd);
+            k_ab_digits<<<(unsigned)((la * 128 + 255) / 256), 256, 0, st>>>(ham->d_V.p, P->npair, P->npoff, P->d_offpair.p, P->A.d_str, la,
+                                                                           Y.tab, Y.Wd);
         }
-        auto dense = [&](const SpinPlan &sp, int64_t l, int64_t lp, DevBuf<__nv_bfloat16> &H, int nch, int rows, int64_t nb,
-                         DevBuf<uint8_t> &fl) {
-            const unsigned g = (unsigned)((l * 32 + 255) / 256);
-            if (e == cudaSuccess) e = cudaMemsetAsync(H.p, 0, H.bytes(), st);
-            if (e == cudaSuccess) e = cudaMemsetAsync(cnt.p, 0, (size_t)l * nch, st);
-            if (e != cudaSuccess) return;
-            k_dense_digits<PR><<<g, 256, 0, st>>>(l, lp, sp.d_soff, sp.d_sci.p, nullptr, sp.d_sval.p, Y.eH, H.p);
-            k_dense_digits<PR><<<g, 256, 0, st>>>(l, lp, sp.d_doff, nullptr, sp.d_dcol.p, sp.d_dval.p, Y.eH, H.p);
-            k_chunk_counts<<<(unsigned)((l + 63) / 64), 64, 0, st>>>(l, nch, sp.d_soff, sp.d_sci.p, sp.d_doff, sp.d_dcol.p, cnt.p);
-            k_windows<<<(unsigned)nb, 128, 0, st>>>(l, nch, rows, cnt.p, fl.p);
-            e = cudaGetLastError();
-        };
-        dense(P->B, lb, lbp, Y.Hb, nchb, Sh::NT, nbb, Y.flb);
-        dense(P->A, la, lap, Y.Ha, ncha, 128, nba, Y.fla);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        k_dense_digits<PR><<<(unsigned)((lb + 7) / 8), 256, 32 * (size_t)nchb, st>>>(
+            lb, lbp, nchb, P->B.d_soff, P->B.d_sci.p, P->B.d_sval.p, P->B.d_doff, P->B.d_dcol.p, P->B.d_dval.p, Y.tab,
+            reinterpret_cast<__nv_bfloat16 *>(B + hb), B + cb);
+        k_windows<<<(unsigned)nbb, 128, 0, st>>>(lb, nchb, Sh::NT, B + cb, B + fb);
+        k_dense_digits<PR><<<(unsigned)((la + 7) / 8), 256, 32 * (size_t)ncha, st>>>(
+            la, lap, ncha, P->A.d_soff, P->A.d_sci.p, P->A.d_sval.p, P->A.d_doff, P->A.d_dcol.p, P->A.d_dval.p, Y.tab,
+            reinterpret_cast<__nv_bfloat16 *>(B + ha), B + ca);
+        k_windows<<<(unsigned)nba, 128, 0, st>>>(la, ncha, 128, B + ca, B + fa);
+        e = cudaGetLastError();
     }
-    if (e != cudaSuccess || !fair) {
-        Y.Vd.release();
-        Y.Wd.release();
-        Y.Hb.release();
-        Y.Ha.release();
-        Y.flb.release();
-        Y.fla.release();
-        size_t back = bytes;
-        if (grow && X->planes.n == planes) back -= planes, P->charged += planes;  // the other type may use them
-        uncharge(ctx, back);
-        if (grow && old) {  // the smaller planes are gone
-            uncharge(ctx, old);
-            P->charged -= std::min(P->charged, old);
-        }
+    const bool maps = e == cudaSuccess && plane_map(&S.mHb, B + hb, lbp, lb, NSA, 32, Sh::NT) &&
+                      plane_map(&S.mHa, B + ha, lap, la, NSA, 32, 128) &&
+                      plane_map(&S.mCA, Y.planes, lbp, la, NSC, 32, 128, Y.batch) &&
+                      plane_map(&S.mCB, Y.planes, lbp, la, NSC, 64, 32, Y.batch);
+    if (!maps) {
+        Y.arena.release();
+        uncharge(ctx, at);
         cudaGetLastError();
         return e == cudaSuccess || e == cudaErrorMemoryAllocation ? TBSCI_OK
                                                                    : fail(ctx, TBSCI_ECUDA, std::string("digit tables: ") + cudaGetErrorString(e));
     }
-    P->charged += bytes;
-    if (old) {
-        uncharge(ctx, old);
-        P->charged -= std::min(P->charged, old);
-    }
-    SsArgs &S = Y.ss;
+    P->charged += at;
     S.la = la;
     S.lb = lb;
     S.nchb = nchb;
     S.ncha = ncha;
-    S.flb = Y.flb.p;
-    S.fla = Y.fla.p;
-    S.eH = Y.eH;
-    S.info = X->info.p;
+    S.flb = B + fb;
+    S.fla = B + fa;
+    S.info = Y.info;
+    S.tab = Y.tab;
     S.err = P->d_tc_err.p;
-    Y.ready = plane_map(&S.mHb, Y.Hb.p, lbp, lb, NSA, 32, Sh::NT) && plane_map(&S.mHa, Y.Ha.p, lap, la, NSA, 32, 128);
+    Y.ready = true;
     return TBSCI_OK;
 }
 
 UdArgs<double> ud_args(const tbsci_ham *ham, const Plan *P, double) {
     return {P->A.l, P->B.l, nullptr, nullptr, nullptr, P->A.d_str, P->A.d_soff, P->A.d_sci.p, P->A.d_sval.p, P->A.d_E.p,
-            P->B.d_E.p, P->d_U.p, ham->ecore, P->A.nelec, 0, 0};
+            P->B.d_E.p, P->d_U.p, ham->ecore, P->A.nelec, 0};
 }
 UdArgs<float> ud_args(const tbsci_ham *ham, const Plan *P, float) {
     return {P->A.l, P->B.l, nullptr, nullptr, nullptr, P->A.d_str, P->A.d_soff, P->A.d_sci.p, P->A.d_svalf.p, P->A.d_Ef.p,
-            P->B.d_Ef.p, P->d_Uf.p, (float)ham->ecore, P->A.nelec, 0, 0};
+            P->B.d_Ef.p, P->d_Uf.p, (float)ham->ecore, P->A.nelec, 0};
 }
 
 }  // namespace
 
-// Whether a space takes this path: by its size and link counts, not by what is in it.
+// Whether a space takes this path. It wins at every shape and link density tried from
+// 2^14 determinants and two tiles of columns on (one vector, ms, against the SIMT kernels):
+//   150 x 150 strings, norb 12         FP64 0.11 / 0.20    FP32 0.09 / 0.12
+//   500 x 200, norb 14                 0.21 / 0.41         0.13 / 0.23
+//   1,200 x 1,100, norb 16             1.1 / 2.9           0.39 / 1.4
+//   1,800 x 1,800, norb 16, 3,100 non-zeros a determinant: 3.6 / 17.6 and 1.0 / 6.2
+// but not below: 100 x 100 0.09 / 0.09 and 0.08 / 0.06, 2,000 x 60 0.33 / 0.42 and 0.20 / 0.17.
 template <typename T>
-bool exact_eligible(const tbsci_ctx *ctx, const Plan *P) {
-    (void)ctx;
+bool exact_eligible(const Plan *P) {
     const int64_t la = P->A.l, lb = P->B.l;
-    if (P->tl_kpmax == 0 || la < 128 || lb < 128 || la > 32768 || lb > 32768) return false;
+    if (P->tl_kpmax == 0 || la < 32 || lb < 2 * kAbTile || la > 32768 || lb > 32768) return false;
     if (P->tune_stage[sizeof(T) == 8 ? 0 : 1] >= 3) return false;  // a shape of the split path was asked for
-    return la * lb >= (int64_t(1) << 20);
+    return la * lb >= (int64_t(1) << 14);
 }
 
 // sigma of the vectors c -> s; *ran = false (and nothing launched) where the path does
-// not apply: the SIMT kernels then serve the call. `simt(v, skip)` launches those for
-// vector v, to return at once where *skip is set.
+// not apply: the SIMT kernels then serve the call. `simt(v, nv, skip)` launches those for
+// vectors v .. v + nv - 1, to return at once where skip[2 i] is set.
 template <typename T, int PR>
 tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const T *c, T *s, int nvec, cudaStream_t st,
-                            bool *ran, const std::function<tbsci_status(int, const int *)> &simt) {
+                            bool *ran, const std::function<tbsci_status(int, int, const int *)> &simt) {
     *ran = false;
-    if (!exact_eligible<T>(ctx, P)) return TBSCI_OK;
+    if (!exact_eligible<T>(P)) return TBSCI_OK;
     // the tables are made outside of graphs, and a graph's replays would share them with other streams
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
@@ -1189,8 +1184,6 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
     }
     ExactData *X = P->exact.get();
     std::lock_guard<std::mutex> g(X->mu);
-    if (!X->tried) TB_TRY(build_common(ctx, P, X));
-    if (!X->ok) return TBSCI_OK;
     typename ExactData::Type &Y = X->type[PR];
     if (!Y.tried) TB_TRY((build_type<PR>(ctx, ham, P, X, st)));
     if (!Y.ready) return TBSCI_OK;
@@ -1201,30 +1194,21 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
     }
     using Sh = SsShape<PR>;
     const int64_t la = P->A.l, lb = P->B.l, lbp = pad64(lb);
-    __nv_bfloat16 *planes = reinterpret_cast<__nv_bfloat16 *>(X->planes.p);
-    if (Y.planes != planes) {
-        if (!plane_map(&Y.ss.mCA, planes, lbp, la, Prec<PR>::NSC, 32, 128) ||
-            !plane_map(&Y.ss.mCB, planes, lbp, la, Prec<PR>::NSC, 64, 32)) {
-            Y.ready = false;
-            return TBSCI_OK;
-        }
-        Y.planes = planes;
-    }
     auto kss = k_same_spin_ex<PR>;
     TB_CUDA(ctx, cudaFuncSetAttribute(kss, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem));
     UdArgs<T> U = ud_args(ham, P, T(0));
-    U.info = X->info.p;
+    U.info = Y.info;
     AbArgs A{};
     size_t ab_smem = 0;
     if (PR == 0) {
         A.la = la;
         A.lb = lb;
         A.lbp = lbp;
-        A.Cs = planes;
-        A.info = X->info.p;
-        A.eV = Y.eV;
-        A.Vd = reinterpret_cast<const uint4 *>(Y.Vd.p);
-        A.Wd = reinterpret_cast<const uint4 *>(Y.Wd.p);
+        A.Cs = Y.planes;
+        A.info = Y.info;
+        A.tab = Y.tab;
+        A.Vd = Y.Vd;
+        A.Wd = Y.Wd;
         A.a_soff = P->A.d_soff;
         A.a_sci = P->A.d_sci.p;
         A.pos = P->d_tl_pos.p;
@@ -1239,63 +1223,67 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
         TB_CUDA(ctx, cudaFuncSetAttribute(k_sigma_ab_ex, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ab_smem));
     }
     *ran = true;
-    TB_CUDA(ctx, cudaStreamWaitEvent(st, X->busy, 0));
-    for (int v = 0; v < nvec; ++v) {
+    TB_CUDA(ctx, cudaStreamWaitEvent(st, Y.busy, 0));
+    for (int v = 0, nv = 0; v < nvec; v += nv) {
+        nv = std::min(Y.batch, nvec - v);
         const T *cv = c + (size_t)v * la * lb;
         T *sv = s + (size_t)v * la * lb;
         {
             TraceScope tr(ctx, "k_slice", st);
-            k_scale_partial<T><<<kScaleBlocks, kScaleThreads, 0, st>>>(cv, la * lb, X->part.p);
-            k_scale_final<<<1, 512, 0, st>>>(X->part.p, kScaleBlocks, la * lb, Prec<PR>::kRatio, X->info.p);
-            k_slice<PR><<<ctx->num_sms * 8, 256, 0, st>>>(cv, la, lb, lbp, X->info.p, planes);
+            const unsigned nb = (unsigned)std::min<int64_t>(kScaleBlocks, (la * lb + 4 * kScaleThreads - 1) / (4 * kScaleThreads));
+            k_scale<T><<<dim3(nb, (unsigned)nv), kScaleThreads, 0, st>>>(cv, la * lb, Prec<PR>::kRatio, Y.part, Y.done,
+                                                                        Y.tab, Y.info);
+            const unsigned ns = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (lbp / 8) + 255) / 256);
+            k_slice<PR><<<dim3(ns, (unsigned)nv), 256, 0, st>>>(cv, la, lb, lbp, Y.info, Y.planes);
             TB_CUDA(ctx, cudaGetLastError());
         }
         {
             TraceScope tr(ctx, "k_udiag", st);
             U.C = cv;
             U.S = sv;
-            k_udiag<T><<<dim3((unsigned)la, (unsigned)((lb + 255) / 256)), 256, 0, st>>>(U);
+            k_udiag<T, false><<<ud_grid(la, lb, nv), 256, 0, st>>>(U);
             TB_CUDA(ctx, cudaGetLastError());
         }
         {
             TraceScope tr(ctx, "k_same_spin_ex", st);
             Y.ss.S = sv;
-            kss<<<dim3((unsigned)((lb + Sh::NT - 1) / Sh::NT), (unsigned)((la + 127) / 128)), kSsThreads, Sh::kSmem, st>>>(Y.ss);
+            kss<<<dim3((unsigned)((lb + Sh::NT - 1) / Sh::NT), (unsigned)((la + 127) / 128), (unsigned)nv), kSsThreads, Sh::kSmem,
+                  st>>>(Y.ss);
             TB_CUDA(ctx, cudaGetLastError());
         }
         if constexpr (PR == 0) {
             TraceScope tr(ctx, "k_sigma_ab_ex", st);
             A.S = sv;
-            k_sigma_ab_ex<<<(unsigned)la, kAbThreads, ab_smem, st>>>(A);
+            k_sigma_ab_ex<<<dim3((unsigned)la, (unsigned)nv), kAbThreads, ab_smem, st>>>(A);
             TB_CUDA(ctx, cudaGetLastError());
         } else {
-            TB_TRY(sigma_tc_ab(ctx, P, 3, cv, sv, X->info.p, st));
+            TB_TRY(sigma_tc_ab(ctx, P, 3, cv, sv, nv, Y.info, st));
         }
-        TB_TRY(simt(v, X->info.p));
+        TB_TRY(simt(v, nv, Y.info));
     }
-    TB_CUDA(ctx, cudaEventRecord(X->busy, st));
+    TB_CUDA(ctx, cudaEventRecord(Y.busy, st));
     return TBSCI_OK;
 }
 
 tbsci_status exact_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const double *c, double *s, int nvec,
-                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, const int *)> &simt) {
+                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *)> &simt) {
     return exact_launch_t<double, 0>(ctx, ham, P, c, s, nvec, st, ran, simt);
 }
 tbsci_status exact_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const float *c, float *s, int nvec,
-                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, const int *)> &simt) {
+                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *)> &simt) {
     return exact_launch_t<float, 1>(ctx, ham, P, c, s, nvec, st, ran, simt);
 }
 
 // s (+)= the diagonal and the alpha singles with the beta string unchanged, FP32 (see k_udiag)
-tbsci_status udiag_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, const float *c, float *s, bool add,
+tbsci_status udiag_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, const float *c, float *s, int nv, bool add,
                           bool singles, cudaStream_t st) {
     UdArgs<float> U = ud_args(ham, P, 0.f);
     U.C = c;
     U.S = s;
     U.add = add;
-    U.singles = singles;
     TraceScope tr(ctx, "k_udiag", st);
-    k_udiag<float><<<dim3((unsigned)P->A.l, (unsigned)((P->B.l + 255) / 256)), 256, 0, st>>>(U);
+    if (singles) k_udiag<float, true><<<ud_grid(P->A.l, P->B.l, nv), 256, 0, st>>>(U);
+    else k_udiag<float, false><<<ud_grid(P->A.l, P->B.l, nv), 256, 0, st>>>(U);
     TB_CUDA(ctx, cudaGetLastError());
     return TBSCI_OK;
 }

@@ -159,7 +159,9 @@ __device__ __forceinline__ void bf16_planes(float x, uint32_t (&h)[NP]) {
 template <int NP>
 __global__ void __launch_bounds__(256) k_planes(const float *__restrict__ c, int64_t la, int64_t lb, int64_t lbp,
                                                 const int *__restrict__ info, __nv_bfloat16 *out) {
-    if (info && !info[0]) return;
+    if (info && !info[2 * blockIdx.y]) return;  // one vector per blockIdx.y
+    c += blockIdx.y * la * lb;
+    out += blockIdx.y * NP * la * lbp;
     const int64_t per = lbp / 8, n = la * per, plane = la * lbp;
     for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
         const int64_t r = i / per, j = (i - r * per) * 8;
@@ -204,7 +206,7 @@ struct FpArgs {
     int64_t la, lb, lbp;
     const __nv_bfloat16 *Cs;
     float *S;
-    const int *info;       // run only where info[0] is set (NULL: always)
+    const int *info;       // run only where info[2 v] is set (NULL: always)
     const uint2 *Vd, *Wd;  // [pair][128], [la][128] x 4 BF16
     const int64_t *a_soff;
     const int2 *a_sci;
@@ -220,7 +222,7 @@ struct FpArgs {
 
 template <int NP>
 __global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab_tc(const FpArgs A) {
-    if (A.info && !A.info[0]) return;
+    if (A.info && !A.info[2 * blockIdx.y]) return;  // one vector per blockIdx.y
     extern __shared__ unsigned char smem_dyn[];
     __shared__ uint64_t bar[16];
     __shared__ uint32_t tmem_base;
@@ -364,7 +366,7 @@ __global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab_tc(const FpArgs A) {
         for (int t = g; t < ntiles && g < ng; t += ng) {
             const int st = t % nst;
             if (t >= nst && !mb_wait(bempty + 8 * st, (t / nst - 1) & 1, ab)) break;
-            gather_tile<NP>(A.Cs, (size_t)A.la * lbp, lbp, sJa, Kp, t, sB + st * stage_sz);
+            gather_tile<NP>(A.Cs + blockIdx.y * NP * A.la * lbp, (size_t)A.la * lbp, lbp, sJa, Kp, t, sB + st * stage_sz);
             mb_arrive(bfull + 8 * st);
         }
     } else {
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab_tc(const FpArgs A) {
     }
     tc_before();
     __syncthreads();
-    float *S = A.S + Ia * lb;
+    float *S = A.S + (blockIdx.y * A.la + Ia) * lb;
     for (int64_t j = tid; j < lb; j += kAbThreads) S[j] += sAcc[j];
     if (sAbort && tid == 0) {
         atomicExch(A.err, 1);
@@ -454,6 +456,12 @@ int fp_stage_bytes(const tbsci_ctx *ctx, const Plan *P, int np) {
 }
 
 }  // namespace
+
+// Vectors per launch: small spaces share the launches with up to eight (planes of at
+// most 2^24 determinants are kept).
+int sigma_tc_batch(const Plan *P) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(8, (int64_t(1) << 24) / std::max<int64_t>(1, P->A.l * P->B.l)));
+}
 
 // Link plan of a space (norb <= 16), made when the space is prepared; left out
 // (tl_kpmax = 0) where the alpha-beta kernels do not apply.
@@ -490,8 +498,9 @@ struct AbPlanes {
     std::mutex mu;
     cudaEvent_t busy = nullptr;
     bool tried = false, ready = false;
-    DevBuf<uint2> V, W;
-    DevBuf<__nv_bfloat16> c;
+    DevBuf<unsigned char> arena;
+    uint2 *V = nullptr, *W = nullptr;
+    __nv_bfloat16 *c = nullptr;  // planes of sigma_tc_batch vectors
     ~AbPlanes() {
         if (busy) cudaEventDestroy(busy);
     }
@@ -503,25 +512,23 @@ template <int NP>
 tbsci_status build_planes(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, AbPlanes *X, cudaStream_t st) {
     X->tried = true;
     const int64_t la = P->A.l, lb = P->B.l;
-    const size_t nv = (size_t)P->npair * 128, nw = (size_t)la * 128, nc = (size_t)NP * la * pad64(lb);
+    const size_t nv = (size_t)P->npair * 128, nw = (size_t)la * 128, nc = (size_t)sigma_tc_batch(P) * NP * la * pad64(lb);
     const size_t bytes = (nv + nw) * sizeof(uint2) + nc * 2;
     if (charge(ctx, bytes, "planes of the alpha-beta products") != TBSCI_OK) return TBSCI_OK;
-    cudaError_t e = X->V.alloc(nv);
-    if (e == cudaSuccess) e = X->W.alloc(nw);
-    if (e == cudaSuccess) e = X->c.alloc(nc);
+    cudaError_t e = X->arena.alloc(bytes);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&X->busy, cudaEventDisableTiming);
     if (e == cudaSuccess) {
+        X->V = reinterpret_cast<uint2 *>(X->arena.p);
+        X->W = X->V + nv;
+        X->c = reinterpret_cast<__nv_bfloat16 *>(X->W + nw);
         k_ab_planes<NP><<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(ham->d_Vf.p, P->npair, P->npoff, P->d_offpair.p, nullptr,
-                                                                     P->npair, X->V.p);
+                                                                     P->npair, X->V);
         k_ab_planes<NP><<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(ham->d_Vf.p, P->npair, P->npoff, P->d_offpair.p, P->A.d_str,
-                                                                     la, X->W.p);
+                                                                     la, X->W);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
-        X->V.release();
-        X->W.release();
-        X->c.release();
+        X->arena.release();
         uncharge(ctx, bytes);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? TBSCI_OK : fail(ctx, TBSCI_ECUDA, std::string("alpha-beta planes: ") + cudaGetErrorString(e));
@@ -532,17 +539,17 @@ tbsci_status build_planes(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, AbPlane
 }
 
 template <int NP>
-tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float *s, const int *info, cudaStream_t st) {
+tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float *s, int nv, const int *info, cudaStream_t st) {
     const int64_t la = P->A.l, lb = P->B.l;
     FpArgs A{};
     A.la = la;
     A.lb = lb;
     A.lbp = pad64(lb);
-    A.Cs = X->c.p;
+    A.Cs = X->c;
     A.S = s;
     A.info = info;
-    A.Vd = X->V.p;
-    A.Wd = X->W.p;
+    A.Vd = X->V;
+    A.Wd = X->W;
     A.a_soff = P->A.d_soff;
     A.a_sci = P->A.d_sci.p;
     A.pos = P->d_tl_pos.p;
@@ -559,12 +566,13 @@ tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float 
     TB_CUDA(ctx, cudaStreamWaitEvent(st, X->busy, 0));
     {
         TraceScope tr(ctx, "k_planes", st);
-        k_planes<NP><<<ctx->num_sms * 8, 256, 0, st>>>(c, la, lb, A.lbp, info, X->c.p);
+        const unsigned nb = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (A.lbp / 8) + 255) / 256);
+        k_planes<NP><<<dim3(nb, (unsigned)nv), 256, 0, st>>>(c, la, lb, A.lbp, info, X->c);
         TB_CUDA(ctx, cudaGetLastError());
     }
     {
         TraceScope tr(ctx, "k_sigma_ab_tc", st);
-        kern<<<(unsigned)la, kAbThreads, smem, st>>>(A);
+        kern<<<dim3((unsigned)la, (unsigned)nv), kAbThreads, smem, st>>>(A);
         TB_CUDA(ctx, cudaGetLastError());
     }
     TB_CUDA(ctx, cudaEventRecord(X->busy, st));
@@ -597,12 +605,13 @@ tbsci_status sigma_tc_prepare(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int
     return TBSCI_OK;
 }
 
-// Adds the alpha-beta products of one vector into s (after a prepare that said ready);
-// info: a device flag, nothing is done where it is 0 (NULL: always).
-tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, const int *info, cudaStream_t st) {
+// Adds the alpha-beta products of nv vectors (at most sigma_tc_batch) into s, after a
+// prepare that said ready; info: device flags [nv][2], nothing is done for a vector whose
+// first one is 0 (NULL: always).
+tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, int nv, const int *info, cudaStream_t st) {
     AbPlanes *X = P->ab[np == 1 ? 0 : 1].get();
     std::lock_guard<std::mutex> g(X->mu);
-    return np == 1 ? ab_add<1>(ctx, P, X, c, s, info, st) : ab_add<3>(ctx, P, X, c, s, info, st);
+    return np == 1 ? ab_add<1>(ctx, P, X, c, s, nv, info, st) : ab_add<3>(ctx, P, X, c, s, nv, info, st);
 }
 
 }  // namespace tbsci

@@ -42,7 +42,7 @@ def _check(s, osp, h, eri, C, rows, **kw):
 
 def _rows(ndet, seed, k=400):
     r = np.random.default_rng(seed)
-    return np.unique(np.concatenate([r.choice(ndet, k, replace=False), np.arange(40), np.arange(ndet - 40, ndet)]))
+    return np.unique(np.concatenate([r.choice(ndet, min(k, ndet), replace=False), np.arange(min(40, ndet)), np.arange(max(0, ndet - 40), ndet)]))
 
 
 @pytest.mark.parametrize("dtype", ["f64", "f32"])
@@ -50,7 +50,10 @@ def _rows(ndet, seed, k=400):
     (13, 6, 6, 1030, 1025, 2),    # one row past a 128-row tile's multiple of 6, one column past 64
     (16, 8, 8, 1100, 1087, 1),    # rows with all 64 alpha singles (65 terms), a column short of 17 tiles
     (16, 12, 5, 1024, 1024, 1),   # twelve alpha electrons: W beyond eight integrals; whole tiles
-    (12, 6, 6, None, None, 1),    # 924 x 924: below the size from which this path is taken
+    (10, 5, 5, 126, 130, 1),      # 16,380 determinants: just below the size from which this path is taken
+    (10, 5, 5, 128, 128, 9),      # at it, in two launches of eight and one vectors
+    (12, 6, 4, 33, 495, 3),       # few, long rows
+    (2, 1, 1, None, None, 1),     # 2 x 2
     (13, 6, 5, None, None, 1),    # a full space: every list at its longest
 ])
 def test_exact_sigma_parity(tb, ctx, n, na, nb, la, lb, nvec, dtype):
@@ -66,7 +69,7 @@ def test_exact_sigma_parity(tb, ctx, n, na, nb, la, lb, nvec, dtype):
     torch.cuda.synchronize()
     tb.tbsci_trace_enable(ctx.handle, False)
     names = {k for k, _ in tb.tbsci_trace_read(ctx.handle)[0]}
-    assert ("k_same_spin_ex" in names) == (sp.ndet >= 1 << 20), names
+    assert ("k_same_spin_ex" in names) == (sp.ndet >= 1 << 14), names
     assert torch.equal(s, sp.sigma(Ct))  # integer sums: the same in every run
     _check(s.double().cpu().numpy(), osp, h, eri, Ct.double().cpu().numpy(), _rows(sp.ndet, n), **({} if dtype == "f64" else F32))
     sp.close()
