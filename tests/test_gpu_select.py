@@ -112,3 +112,20 @@ def test_selection_argument_errors(tb, ctx):
             call()
         assert err.value.status == tb.TBSCI_EINVAL
     sp.close()
+
+
+@pytest.mark.parametrize("edges", [[0.5], [-1.0, -0.0, 1e-300, 1.0], [1.0, 2.0, 3.0], list(10.0 ** np.linspace(-12, 0, 255)),
+                                   list(10.0 ** np.linspace(-12, 0, 256)), [1.0, np.inf]])
+@pytest.mark.parametrize("n", [1, 255, 1025, 300001])
+def test_histogram_bins_at_their_edges(tb, ctx, edges, n):
+    """Values equal to an edge, one unit below it, zeros, infinities and NaN: the bin
+    of x is the number of edges at or below |x| (none for NaN)."""
+    import torch
+    e = np.array(edges)
+    r = np.random.default_rng(n)
+    special = np.concatenate([np.abs(e), np.nextafter(np.abs(e), 0), [0.0, np.inf, np.nan, 5e-324, 1.7e308]])
+    x = np.where(r.random(n) < 0.5, r.choice(special, n), 10.0 ** r.uniform(-14, 2, n)) * r.choice([-1.0, 1.0], n)
+    got = tb.tbsci_coefficient_histogram(ctx.handle, torch.from_numpy(x).cuda(), e)
+    a = np.abs(x)
+    want = np.bincount(np.where(np.isnan(a), 0, np.searchsorted(e, a, side="right")), minlength=len(e) + 1)
+    assert np.array_equal(got, want)
