@@ -288,6 +288,7 @@ tbsci_status plan_get(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *a, con
         int64_t s1 = a->h_off1[i + 1] - a->h_off1[i];
         int64_t d2 = a->h_off2[i + 1] - a->h_off2[i];
         S1a += s1;
+        plan->a_smax = std::max<int>(plan->a_smax, (int)s1);
         D2a += d2;
         work[i] = (double)(1 + s1) * (double)(lb + S1b) + (double)d2 * (double)lb + (double)D2b;
     }

@@ -307,6 +307,121 @@ __global__ void __launch_bounds__(kThreads) k_sigma(SigArgs<T> A) {
     sigma_row<T, NV, STAGE, ACCS, kThreads, REST>(A, A.rowsa[blockIdx.x], smem_raw);
 }
 
+__device__ __forceinline__ double flip_sign(double x, int m) {
+    return __hiloint2double(__double2hiint(x) ^ m, __double2loint(x));
+}
+__device__ __forceinline__ float flip_sign(float x, int m) { return __int_as_float(__float_as_int(x) ^ m); }
+
+template <typename T>
+__host__ __device__ size_t small_smem_bytes(int npair, int64_t la, int64_t lb, int nsmax) {
+    return (size_t)(la * lb + (int64_t)(nsmax + 1) * (npair + 1) + nsmax + 512) * sizeof(T) + (size_t)nsmax * 8;
+}
+
+// Spaces whose whole vector fits in shared memory. k_sigma's CTA walks a row's alpha terms
+// one after the other, two barriers and a round trip to L2 for each; here c and the
+// coefficients of all the row's alpha singles are staged once, SL slices of 32 columns
+// (permb2 order) take a CTA, and G = 16 / SL warps per slice share the terms: alpha singles
+// and doubles by their place, the links of Ja = Ia by theirs. The warps' sums are added in
+// warp order. What is left is the FP64 pipe (norb 8 full space: 4,900 x 397 multiply-adds,
+// 3 us of 152 SMs), so a slice per CTA is taken until the grid covers the GPU twice.
+// Norb 8 full space, one vector, FP64: 22 us; 46 on k_sigma, and 16 orbitals with 60 x 60
+// strings, two vectors, 53; 405.
+template <typename T, int SL>
+__global__ void __launch_bounds__(512) k_sigma_small(SigArgs<T> A, int nsmax) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int G = 16 / SL;
+    const int npair = A.npair, np1 = npair + 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int lb = (int)A.lb, ndet = (int)(A.la * A.lb);
+    T *sC = reinterpret_cast<T *>(smem_raw);  // [ndet]
+    T *sW = sC + ndet;                        // [np1]: sum_{p in Ia} (pp|x); the last is zero (padding)
+    T *sV = sW + np1;                         // [nsmax][np1]: s_a (pq|x) of each alpha single
+    T *sH = sV + nsmax * np1;                 // [nsmax]
+    T *sRed = sH + nsmax;                     // [512]
+    int *sJ = reinterpret_cast<int *>(sRed + 512), *sP = sJ + nsmax;  // start of row Ja, pair | sign << 31
+    const int64_t Ia = A.rowsa[blockIdx.x];
+    const T *__restrict__ C = A.C + blockIdx.z * A.vstride;
+    T *__restrict__ S = A.S + blockIdx.z * A.vstride;
+    const int64_t t0 = A.a_soff[Ia];
+    const int ns = (int)(A.a_soff[Ia + 1] - t0);
+    const uint64_t str = A.stra[Ia];
+#pragma unroll 4
+    for (int x = tid; x < ndet; x += 512) sC[x] = __ldg(C + x);
+    for (int t = tid; t < ns; t += 512) {
+        const int2 e = __ldg(A.a_sci + t0 + t);
+        sJ[t] = e.x * lb;
+        sP[t] = (e.y >> 1) | (e.y << 31);
+        sH[t] = __ldg(A.a_sval + t0 + t);
+    }
+    for (int x = tid; x < np1; x += 512) {
+        T w = 0;
+        if (x < npair)
+            for (uint64_t s = str; s; s &= s - 1) {
+                const int p = __ffsll((long long)s) - 1;
+                w += __ldg(A.V + (size_t)(p * (p + 1) / 2 + p) * npair + x);
+            }
+        sW[x] = w;
+    }
+    for (int t = warp; t < ns; t += 16) {
+        const int2 e = __ldg(A.a_sci + t0 + t);
+        for (int x = lane; x < np1; x += 32)
+            sV[t * np1 + x] = x < npair ? flip_sign(__ldg(A.V + (size_t)(e.y >> 1) * npair + x), e.y << 31) : T(0);
+    }
+    __syncthreads();
+    const int64_t sl = blockIdx.y * SL + warp % SL;
+    const int g = warp / SL;
+    const bool live = sl * 32 < lb;  // warp-uniform
+    const int64_t j = sl * 32 + lane;
+    const int ib = live && j < lb ? __ldg(A.permb2 + j) : 0;
+    if (live) {
+        const T *row = sC + Ia * lb;
+        T acc = T(0), acc2 = T(0);
+        const int2 *ci = A.s2_ci + A.s2_off[sl] + lane;
+        const T *cv = A.s2_val + A.s2_off[sl] + lane;
+        const int w1 = A.s2_w[sl], w2 = A.d2_w[sl];
+        // ---- Ja = Ia
+        if (g == 0 && j < lb) {
+            T ed = A.ecore + A.Ea[Ia] + __ldg(A.Eb2 + j);
+            for (uint64_t s = str; s; s &= s - 1) {
+                const int p = __ffsll((long long)s) - 1;
+                ed += __ldg(A.U2 + (size_t)(p * (p + 1) / 2 + p) * lb + j);
+            }
+            acc = ed * row[ib];
+        }
+#pragma unroll 2
+        for (int k = g; k < w1; k += G) {
+            const int2 e = __ldg(ci + 32 * k);
+            acc2 += (__ldg(cv + 32 * k) + flip_sign(sW[e.y >> 1], e.y << 31)) * row[e.x];
+        }
+        const int32_t *dc = A.d2_col + A.d2_off[sl] + lane;
+        const T *dv = A.d2_val + A.d2_off[sl] + lane;
+#pragma unroll 4
+        for (int k = g; k < w2; k += G) acc += __ldg(dv + 32 * k) * row[__ldg(dc + 32 * k)];
+        // ---- alpha doubles
+        const int64_t u0 = A.a_doff[Ia];
+        const int nd = (int)(A.a_doff[Ia + 1] - u0);
+#pragma unroll 4
+        for (int t = g; t < nd; t += G) acc2 += __ldg(A.a_dval + u0 + t) * sC[__ldg(A.a_dcol + u0 + t) * lb + ib];
+        // ---- alpha singles: the column's own c, then its beta links
+        if (j < lb)
+            for (int t = g; t < ns; t += G)
+                acc += (sH[t] + flip_sign(__ldg(A.U2 + (size_t)(sP[t] & 0x7FFFFFFF) * lb + j), sP[t] & (int)0x80000000)) * sC[sJ[t] + ib];
+        for (int k = 0; k < w1; ++k) {
+            const int2 e = __ldg(ci + 32 * k);
+            const T *v = sV + (e.y >> 1), *c = sC + e.x;
+            const int m = e.y << 31;
+#pragma unroll 2
+            for (int t = g; t < ns; t += G) acc2 += flip_sign(v[t * np1], m) * c[sJ[t]];
+        }
+        sRed[tid] = acc + acc2;
+    }
+    __syncthreads();
+    if (live && g == 0 && j < lb) {
+        T v = sRed[tid];
+        for (int k = 1; k < G; ++k) v += sRed[tid + 32 * SL * k];
+        S[Ia * lb + ib] = v;
+    }
+}
+
 // The vectors (one per blockIdx.y) that the exact tensor-core path leaves: skip[2 v] = 0.
 // Its own kernel, so that k_sigma's arguments stay constants.
 template <typename T, bool STAGE, bool ACCS>
@@ -1115,6 +1230,35 @@ tbsci_status sigma_launch_rest(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan 
 
 namespace {
 
+// k_sigma_small where it applies (*ran): a vector that fits in shared memory, up to the
+// size from which the exact tensor-core path is the faster one (ms, FP64, one vector:
+// 126 x 129 strings 0.047 here, 0.092 there; 150 x 150 0.066, 160 x 155 there 0.109), and no shape of the
+// split path asked for
+constexpr int64_t kSmallDets = 24000;
+
+template <typename T>
+tbsci_status launch_small(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, const T *c, T *s, int nvec, cudaStream_t st,
+                          bool *ran) {
+    *ran = false;
+    const int64_t la = P->A.l, lb = P->B.l;
+    if (la == 0 || lb == 0 || la * lb >= kSmallDets || nvec > 65535) return TBSCI_OK;
+    if (P->tune_stage[sizeof(T) == 8 ? 0 : 1] >= 3) return TBSCI_OK;
+    const size_t sm = small_smem_bytes<T>(P->npair, la, lb, P->a_smax);
+    if (sm > ctx->smem_optin) return TBSCI_OK;
+    SigArgs<T> A = make_args<T>(ham, P);
+    A.C = c;
+    A.S = s;
+    const int64_t nsl = (lb + 31) / 32, work = la * nsl * nvec;
+    const int sl = work <= 2 * ctx->num_sms ? 1 : work <= 4 * ctx->num_sms ? 2 : 4;
+    auto k = sl == 1 ? k_sigma_small<T, 1> : sl == 2 ? k_sigma_small<T, 2> : k_sigma_small<T, 4>;
+    TB_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    TraceScope tr(ctx, "k_sigma", st);
+    k<<<dim3((unsigned)la, (unsigned)((nsl + sl - 1) / sl), (unsigned)nvec), 512, sm, st>>>(A, P->a_smax);
+    TB_CUDA(ctx, cudaGetLastError());
+    *ran = true;
+    return TBSCI_OK;
+}
+
 template <typename T, bool STAGE, bool ACCS>
 tbsci_status launch_left(tbsci_ctx *ctx, const SigArgs<T> &A, int nv, const int *skip, cudaStream_t st) {
     const size_t sm = smem_bytes<T>(A.npair, A.lb, 1, STAGE, ACCS);
@@ -1132,6 +1276,8 @@ tbsci_status launch_full(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan,
                          cudaStream_t st) {
     const size_t n = (size_t)plan->A.l * plan->B.l;
     bool ran = false;
+    TB_TRY(launch_small<T>(ctx, ham, plan, c, s, nvec, st, &ran));
+    if (ran) return TBSCI_OK;
     TB_TRY(exact_launch(ctx, ham, const_cast<Plan *>(plan), c, s, nvec, st, &ran, [&](int v, int nv, const int *skip) {
         SigArgs<T> A = make_args<T>(ham, plan);
         A.C = c + v * n;

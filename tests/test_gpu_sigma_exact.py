@@ -50,9 +50,12 @@ def _rows(ndet, seed, k=400):
     (13, 6, 6, 1030, 1025, 2),    # one row past a 128-row tile's multiple of 6, one column past 64
     (16, 8, 8, 1100, 1087, 1),    # rows with all 64 alpha singles (65 terms), a column short of 17 tiles
     (16, 12, 5, 1024, 1024, 1),   # twelve alpha electrons: W beyond eight integrals; whole tiles
-    (10, 5, 5, 126, 130, 1),      # 16,380 determinants: just below the size from which this path is taken
-    (10, 5, 5, 128, 128, 9),      # at it, in two launches of eight and one vectors
-    (12, 6, 4, 33, 495, 3),       # few, long rows
+    (10, 5, 5, 154, 155, 1),      # 23,870 determinants: the small-space kernel, four column slices per CTA
+    (10, 5, 5, 160, 150, 9),      # 24,000: this path, in two launches of eight and one vectors
+    (12, 6, 4, 33, 495, 3),       # small-space kernel, few long rows
+    (16, 8, 8, 390, 60, 2),       # 23,400: too much for shared memory in FP64
+    (8, 4, 4, None, None, 1),     # small-space kernel, one slice per CTA
+    (8, 4, 3, 40, 33, 4),         # a column past a slice
     (2, 1, 1, None, None, 1),     # 2 x 2
     (13, 6, 5, None, None, 1),    # a full space: every list at its longest
 ])
@@ -69,7 +72,7 @@ def test_exact_sigma_parity(tb, ctx, n, na, nb, la, lb, nvec, dtype):
     torch.cuda.synchronize()
     tb.tbsci_trace_enable(ctx.handle, False)
     names = {k for k, _ in tb.tbsci_trace_read(ctx.handle)[0]}
-    assert ("k_same_spin_ex" in names) == (sp.ndet >= 1 << 14), names
+    assert ("k_same_spin_ex" in names) == (sp.ndet >= 24000), names
     assert torch.equal(s, sp.sigma(Ct))  # integer sums: the same in every run
     _check(s.double().cpu().numpy(), osp, h, eri, Ct.double().cpu().numpy(), _rows(sp.ndet, n), **({} if dtype == "f64" else F32))
     sp.close()
