@@ -303,6 +303,26 @@ void tbsci_tables_destroy(tbsci_tables *t) {
     delete t;
 }
 
+// Pair-packed integrals V[pq][rs] = (pq|rs) in both precisions, and the checks of the input:
+// flags 1 a non-finite entry, 2 an entry that differs from a permuted one by over 1e-12
+// (norb 24: the same loops took 0.7 ms on the host).
+static __global__ void k_integrals(const double *__restrict__ eri, int n, int npair, double *V, float *Vf, int *flags) {
+    const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, n4 = (int64_t)n * n * n * n;
+    if (x >= n4) return;
+    int64_t y = x;
+    const int l = (int)(y % n), k = (int)((y /= n) % n), j = (int)((y /= n) % n), i = (int)(y / n);
+    auto E = [&](int a, int b, int c, int d) { return eri[(((int64_t)a * n + b) * n + c) * n + d]; };
+    const double v = eri[x];
+    int f = isfinite(v) ? 0 : 1;
+    if (!f && (fabs(v - E(j, i, k, l)) > 1e-12 || fabs(v - E(i, j, l, k)) > 1e-12 || fabs(v - E(k, l, i, j)) > 1e-12)) f = 2;
+    if (f) atomicOr(flags, f);
+    if (j <= i && l <= k) {
+        const size_t at = (size_t)(i * (i + 1) / 2 + j) * npair + k * (k + 1) / 2 + l;
+        V[at] = v;
+        Vf[at] = (float)v;
+    }
+}
+
 tbsci_status tbsci_hamiltonian_create(tbsci_ctx *ctx, int norb, const double *h, const double *eri, double ecore,
                                       tbsci_ham **out) {
     TB_GUARD_CTX(ctx);
@@ -316,48 +336,38 @@ tbsci_status tbsci_hamiltonian_create(tbsci_ctx *ctx, int norb, const double *h,
             if (!std::isfinite(h[i * n + j])) return fail(ctx, TBSCI_EINVAL, "h has a non-finite entry");
             if (std::fabs(h[i * n + j] - h[j * n + i]) > 1e-12) return fail(ctx, TBSCI_EINVAL, "h is not symmetric");
         }
-    auto E = [&](int i, int j, int k, int l) { return eri[(((size_t)i * n + j) * n + k) * n + l]; };
-    for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j)
-            for (int k = 0; k < n; ++k)
-                for (int l = 0; l < n; ++l) {
-                    double v = E(i, j, k, l);
-                    if (!std::isfinite(v)) return fail(ctx, TBSCI_EINVAL, "eri has a non-finite entry");
-                    if (std::fabs(v - E(j, i, k, l)) > 1e-12 || std::fabs(v - E(i, j, l, k)) > 1e-12 ||
-                        std::fabs(v - E(k, l, i, j)) > 1e-12)
-                        return fail(ctx, TBSCI_EINVAL, "eri lacks the 8-fold symmetry of real orbitals");
-                }
     tbsci_ham *H = new (std::nothrow) tbsci_ham();
     if (!H) return fail(ctx, TBSCI_ENOMEM, "host allocation failed");
     H->ctx = ctx;
     H->norb = n;
     H->npair = n * (n + 1) / 2;
     H->ecore = ecore;
-    H->h_h.assign(h, h + n2);
-    H->h_eri.assign(eri, eri + n4);
-    const int P = H->npair;
-    std::vector<double> V((size_t)P * P);
-    std::vector<float> Vf((size_t)P * P);
-    for (int p = 0; p < n; ++p)
-        for (int q = 0; q <= p; ++q)
-            for (int r = 0; r < n; ++r)
-                for (int s = 0; s <= r; ++s) {
-                    size_t idx = (size_t)pair_index(p, q) * P + pair_index(r, s);
-                    V[idx] = E(p, q, r, s);
-                    Vf[idx] = (float)V[idx];
-                }
+    const size_t P2 = (size_t)H->npair * H->npair;
     auto cleanup = [&](tbsci_status st, const char *msg) {
         delete H;
         return fail(ctx, st, msg);
     };
-    if (H->d_h.alloc(n2) != cudaSuccess || H->d_V.alloc(V.size()) != cudaSuccess ||
-        H->d_Vf.alloc(Vf.size()) != cudaSuccess || H->d_eri.alloc(n4) != cudaSuccess)
-        return cleanup(TBSCI_ENOMEM, "device allocation failed");
-    if (cudaMemcpy(H->d_h.p, h, n2 * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(H->d_V.p, V.data(), V.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(H->d_Vf.p, Vf.data(), Vf.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(H->d_eri.p, eri, n4 * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
-        return cleanup(TBSCI_ECUDA, "copy of integrals failed");
+    DevBuf<int> flags;
+    H->arena.add(H->d_h, n2);
+    H->arena.add(H->d_V, P2);
+    H->arena.add(H->d_Vf, P2);
+    H->arena.add(H->d_eri, n4);
+    H->arena.add(flags, 1);
+    if (H->arena.commit() != cudaSuccess) return cleanup(TBSCI_ENOMEM, "device allocation failed");
+    cudaStream_t st = ctx->stream;
+    int bad = 0;
+    cudaError_t e = cudaMemcpyAsync(H->d_h.p, h, n2 * sizeof(double), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(H->d_eri.p, eri, n4 * sizeof(double), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(flags.p, 0, sizeof(int), st);
+    if (e == cudaSuccess) {
+        k_integrals<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(H->d_eri.p, n, H->npair, H->d_V.p, H->d_Vf.p, flags.p);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, flags.p, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cleanup(TBSCI_ECUDA, "copy of integrals failed");
+    if (bad & 1) return cleanup(TBSCI_EINVAL, "eri has a non-finite entry");
+    if (bad & 2) return cleanup(TBSCI_EINVAL, "eri lacks the 8-fold symmetry of real orbitals");
     *out = H;
     return TBSCI_OK;
 }

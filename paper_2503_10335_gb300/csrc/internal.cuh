@@ -55,14 +55,16 @@ template <typename T>
 struct DevBuf {
     T *p = nullptr;
     size_t n = 0;
+    bool view = false;  // a piece of an Arena, which owns the memory
     DevBuf() = default;
     DevBuf(const DevBuf &) = delete;
     DevBuf &operator=(const DevBuf &) = delete;
     ~DevBuf() { release(); }
     void release() {
-        if (p) cudaFree(p);
+        if (p && !view) cudaFree(p);
         p = nullptr;
         n = 0;
+        view = false;
     }
     // n is set only once the allocation succeeded: a failed alloc leaves an
     // empty buffer (p == nullptr, n == 0), so a later size check re-allocates
@@ -78,6 +80,37 @@ struct DevBuf {
         return cudaSuccess;
     }
     size_t bytes() const { return n * sizeof(T); }
+};
+
+// One device allocation for many buffers: allocating and freeing a buffer of a few MB
+// takes 37 us each way, and a prepared space has some forty.
+struct Arena {
+    DevBuf<unsigned char> mem;
+    struct Piece {
+        void **p;
+        size_t at;
+    };
+    std::vector<Piece> pieces;
+    size_t total = 0;
+    // b gets n elements at commit(), 256-byte aligned; n = 0 leaves it empty
+    template <typename T>
+    size_t add(DevBuf<T> &b, size_t n) {
+        b.release();
+        if (n == 0) return total;
+        const size_t at = total;
+        b.n = n;
+        b.view = true;
+        pieces.push_back({(void **)&b.p, at});
+        total += (n * sizeof(T) + 255) / 256 * 256;
+        return at;
+    }
+    cudaError_t commit() {
+        const cudaError_t e = mem.alloc(total);
+        if (e == cudaSuccess)
+            for (const Piece &x : pieces) *x.p = mem.p + x.at;
+        pieces.clear();
+        return e;
+    }
 };
 
 }  // namespace tbsci
@@ -223,6 +256,7 @@ struct AbPlanes;   // sigma_tc.cu
 
 struct Plan {
     uint64_t ida = 0, idb = 0;
+    Arena arena;  // holds what is made when the space is prepared
     int norb = 0, npair = 0;
     SpinPlan A, B;
     DevBuf<double> d_U;      // [npair][l_b]: sum_{r in occ(Ib)} (pair|rr)
@@ -308,9 +342,9 @@ struct tbsci_ham {
     tbsci_ctx *ctx = nullptr;
     int norb = 0, npair = 0;
     double ecore = 0.0;
+    tbsci::Arena arena;  // holds the integrals
     tbsci::DevBuf<double> d_h, d_V, d_eri;  // h[n][n], V[npair][npair] = (pq|rs) pair-packed, eri[n^4]
     tbsci::DevBuf<float> d_Vf;
-    std::vector<double> h_h, h_eri;
     std::vector<std::unique_ptr<tbsci::Plan>> plans;
 };
 
@@ -396,6 +430,7 @@ tbsci_status udiag_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, c
                           bool singles, cudaStream_t st);
 // sigma_tc.cu: the alpha-beta classes on the tensor cores with np = 1 or 3 BF16 planes
 // per operand, FP32 accumulation, added into s
+void tile_links_size(tbsci_ctx *ctx, Plan *P);  // adds the plan's buffers to its arena
 tbsci_status tile_links_build(tbsci_ctx *ctx, Plan *P, cudaStream_t st);
 tbsci_status sigma_tc_prepare(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int np, cudaStream_t st, bool *ready);
 tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, int nv, const int *info, cudaStream_t st);

@@ -21,22 +21,28 @@ __device__ __forceinline__ double eri_at(const double *__restrict__ eri, int n, 
     return __ldg(eri + (((size_t)i * n + j) * n + k) * n + l);
 }
 
+// One warp per string, lanes over its orbitals i (a thread per string left most of the GPU
+// idle: 5,000 strings of 12 electrons took 51 us, now 15 us).
 __global__ void k_string_energy(const uint64_t *__restrict__ str, int64_t l, int n, const double *__restrict__ h,
                                 const double *__restrict__ eri, double *E, float *Ef) {
-    int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (w >= l) return;
-    uint64_t s = str[w];
+    const uint64_t s = str[w];
     double e = 0.0;
-    for (uint64_t a = s; a; a &= a - 1) {
-        int i = __ffsll((long long)a) - 1;
+    for (int i = lane; i < n; i += 32) {
+        if (!((s >> i) & 1)) continue;
         e += h[i * n + i];
         for (uint64_t b = s; b; b &= b - 1) {
-            int j = __ffsll((long long)b) - 1;
+            const int j = __ffsll((long long)b) - 1;
             e += 0.5 * (eri_at(eri, n, i, i, j, j) - eri_at(eri, n, i, j, j, i));
         }
     }
-    E[w] = e;
-    Ef[w] = (float)e;
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (lane == 0) {
+        E[w] = e;
+        Ef[w] = (float)e;
+    }
 }
 
 // one warp per source row; lanes over the row's single links
@@ -90,7 +96,8 @@ __global__ void k_coulomb_table(const uint64_t *__restrict__ strb, int64_t lb, i
     Uf[(size_t)pr * lb + ib] = (float)u;
 }
 
-// Sliced-ELL copy of CSR rows taken in the column order `perm` (see Plan).
+// Sliced-ELL copy of CSR rows taken in the column order `perm` (see Plan); entries are
+// split over blockIdx.y (a thread per lane alone left the GPU idle).
 __global__ void k_sell_singles(const int32_t *__restrict__ perm, int64_t lb, const int64_t *__restrict__ off,
                                const int2 *__restrict__ sci, const double *__restrict__ sval,
                                const int64_t *__restrict__ soff, const int32_t *__restrict__ sw, int64_t nsl,
@@ -103,7 +110,7 @@ __global__ void k_sell_singles(const int32_t *__restrict__ perm, int64_t lb, con
     const int64_t a = j < lb ? off[ib] : 0, cnt = j < lb ? off[ib + 1] - a : 0;
     const int64_t base = soff[sl] + lane;
     const int w = sw[sl];
-    for (int k = 0; k < w; ++k) {
+    for (int k = blockIdx.y; k < w; k += gridDim.y) {
         const int64_t pos = base + 32 * (int64_t)k;
         if (k < cnt) {
             out_ci[pos] = sci[a + k];
@@ -133,7 +140,7 @@ __global__ void k_sell_doubles(const int32_t *__restrict__ perm, int64_t lb, con
     const int64_t a = j < lb ? off[ib] : 0, cnt = j < lb ? off[ib + 1] - a : 0;
     const int64_t base = soff[sl] + lane;
     const int w = sw[sl];
-    for (int k = 0; k < w; ++k) {
+    for (int k = blockIdx.y; k < w; k += gridDim.y) {
         const int64_t pos = base + 32 * (int64_t)k;
         const bool real = k < cnt;
         out_col[pos] = real ? dcol[a + k] : (int32_t)ib;
@@ -182,8 +189,7 @@ void sell_shape(const std::vector<int32_t> &perm, const std::vector<int64_t> &of
     }
 }
 
-tbsci_status build_spin(tbsci_ctx *ctx, const tbsci_ham *ham, const tbsci_tables *t, SpinPlan &sp, cudaStream_t st) {
-    const int n = ham->norb;
+void size_spin(const tbsci_tables *t, SpinPlan &sp, Arena &arena) {
     sp.l = t->count;
     sp.nelec = t->nelec;
     sp.d_str = t->d_str.p;
@@ -191,33 +197,48 @@ tbsci_status build_spin(tbsci_ctx *ctx, const tbsci_ham *ham, const tbsci_tables
     sp.d_doff = t->d_off2.p;
     sp.h_soff = t->h_off1;
     sp.h_doff = t->h_off2;
-    TB_CUDA(ctx, sp.d_E.alloc(sp.l));
-    TB_CUDA(ctx, sp.d_Ef.alloc(sp.l));
-    TB_CUDA(ctx, sp.d_sci.alloc(t->nsingle));
-    TB_CUDA(ctx, sp.d_sval.alloc(t->nsingle));
-    TB_CUDA(ctx, sp.d_svalf.alloc(t->nsingle));
-    TB_CUDA(ctx, sp.d_dcol.alloc(t->ndouble));
-    TB_CUDA(ctx, sp.d_dval.alloc(t->ndouble));
-    TB_CUDA(ctx, sp.d_dvalf.alloc(t->ndouble));
+    arena.add(sp.d_E, sp.l);
+    arena.add(sp.d_Ef, sp.l);
+    arena.add(sp.d_sci, t->nsingle);
+    arena.add(sp.d_sval, t->nsingle);
+    arena.add(sp.d_svalf, t->nsingle);
+    arena.add(sp.d_dcol, t->ndouble);
+    arena.add(sp.d_dval, t->ndouble);
+    arena.add(sp.d_dvalf, t->ndouble);
+}
+
+tbsci_status build_spin(tbsci_ctx *ctx, const tbsci_ham *ham, const tbsci_tables *t, SpinPlan &sp, cudaStream_t st) {
+    const int n = ham->norb;
     const double *eri = ham->d_eri.p;
-    if (sp.l > 0) {
-        k_string_energy<<<(unsigned)((sp.l + 127) / 128), 128, 0, st>>>(sp.d_str, sp.l, n, ham->d_h.p, eri, sp.d_E.p,
-                                                                       sp.d_Ef.p);
-        TB_CUDA(ctx, cudaGetLastError());
-        if (t->nsingle > 0) {
-            k_single_values<<<(unsigned)((sp.l * 32 + 255) / 256), 256, 0, st>>>(
-                sp.d_str, sp.l, n, t->d_off1.p, t->d_ent1.p, ham->d_h.p, eri, sp.d_sci.p, sp.d_sval.p, sp.d_svalf.p);
-            TB_CUDA(ctx, cudaGetLastError());
-        }
-        if (t->ndouble > 0) {
-            k_double_values<<<(unsigned)((t->ndouble + 255) / 256), 256, 0, st>>>(t->ndouble, n, t->d_ent2.p, eri,
-                                                                                 sp.d_dcol.p, sp.d_dval.p,
-                                                                                 sp.d_dvalf.p);
-            TB_CUDA(ctx, cudaGetLastError());
-        }
-    }
-    TB_CUDA(ctx, cudaStreamSynchronize(st));
+    if (sp.l == 0) return TBSCI_OK;
+    k_string_energy<<<(unsigned)((sp.l * 32 + 127) / 128), 128, 0, st>>>(sp.d_str, sp.l, n, ham->d_h.p, eri, sp.d_E.p, sp.d_Ef.p);
+    if (t->nsingle > 0)
+        k_single_values<<<(unsigned)((sp.l * 32 + 255) / 256), 256, 0, st>>>(
+            sp.d_str, sp.l, n, t->d_off1.p, t->d_ent1.p, ham->d_h.p, eri, sp.d_sci.p, sp.d_sval.p, sp.d_svalf.p);
+    if (t->ndouble > 0)
+        k_double_values<<<(unsigned)((t->ndouble + 255) / 256), 256, 0, st>>>(t->ndouble, n, t->d_ent2.p, eri, sp.d_dcol.p,
+                                                                             sp.d_dval.p, sp.d_dvalf.p);
+    TB_CUDA(ctx, cudaGetLastError());
     return TBSCI_OK;
+}
+
+// indices 0 .. n - 1 by key, largest first, equal keys in index order
+std::vector<int32_t> order_desc(const std::vector<int64_t> &key) {
+    const int64_t top = key.empty() ? 0 : *std::max_element(key.begin(), key.end());
+    const size_t n = key.size();
+    std::vector<int32_t> out(n);
+    if (top > 4 * (int64_t)n + 65536) {
+        std::vector<std::pair<int64_t, int32_t>> a(n);
+        for (size_t i = 0; i < n; ++i) a[i] = {-key[i], (int32_t)i};
+        std::sort(a.begin(), a.end());
+        for (size_t i = 0; i < n; ++i) out[i] = a[i].second;
+        return out;
+    }
+    std::vector<int32_t> at(top + 2, 0);  // link counts are small: a counting sort
+    for (int64_t k : key) ++at[top - k + 1];
+    for (int64_t k = 0; k <= top; ++k) at[k + 1] += at[k];
+    for (size_t i = 0; i < n; ++i) out[at[top - key[i]]++] = (int32_t)i;
+    return out;
 }
 
 // device bytes a prepared space holds
@@ -255,150 +276,115 @@ tbsci_status plan_get(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *a, con
     plan->idb = b->id;
     plan->norb = ham->norb;
     plan->npair = ham->npair;
-    TB_TRY(build_spin(ctx, ham, a, plan->A, st));
-    TB_TRY(build_spin(ctx, ham, b, plan->B, st));
-    const int64_t la = a->count, lb = b->count;
-    TB_CUDA(ctx, plan->d_U.alloc((size_t)ham->npair * lb));
-    TB_CUDA(ctx, plan->d_Uf.alloc((size_t)ham->npair * lb));
-    if (lb > 0) {
-        dim3 grid((unsigned)((lb + 127) / 128), (unsigned)ham->npair);
-        k_coulomb_table<<<grid, 128, 0, st>>>(b->d_str.p, lb, ham->npair, ham->d_V.p, plan->d_U.p, plan->d_Uf.p);
-        TB_CUDA(ctx, cudaGetLastError());
-    }
-    // schedules
-    std::vector<int64_t> s1b(lb), idx_b(lb);
-    int64_t S1b = 0, D2b = 0;
+    plan->npoff = ham->norb * (ham->norb - 1) / 2;
+    const int64_t la = a->count, lb = b->count, np = ham->npair, nsl = (lb + 31) / 32;
+    // schedules: beta columns by their single-link count and by all their links, alpha rows
+    // and pairs of rows (2k, 2k + 1; even l_alpha only: the SIMT pass of the tensor-core
+    // sigma types may serve two rows per CTA) by their work, heaviest first
+    std::vector<int64_t> s1b(lb), tot_b(lb), work(la);
+    int64_t S1b = 0, D2b = 0, S1a = 0, D2a = 0;
     for (int64_t i = 0; i < lb; ++i) {
         s1b[i] = b->h_off1[i + 1] - b->h_off1[i];
+        tot_b[i] = s1b[i] + (b->h_off2[i + 1] - b->h_off2[i]);
         S1b += s1b[i];
         D2b += b->h_off2[i + 1] - b->h_off2[i];
     }
-    std::iota(idx_b.begin(), idx_b.end(), 0);
-    std::stable_sort(idx_b.begin(), idx_b.end(), [&](int64_t x, int64_t y) { return s1b[x] > s1b[y]; });
-    std::vector<int32_t> permb(idx_b.begin(), idx_b.end());
-    std::vector<int64_t> tot_b(lb);
-    for (int64_t i = 0; i < lb; ++i) tot_b[i] = s1b[i] + (b->h_off2[i + 1] - b->h_off2[i]);
-    std::iota(idx_b.begin(), idx_b.end(), 0);
-    std::stable_sort(idx_b.begin(), idx_b.end(), [&](int64_t x, int64_t y) { return tot_b[x] > tot_b[y]; });
-    std::vector<int32_t> permb2(idx_b.begin(), idx_b.end());
-    std::vector<double> work(la);
-    std::vector<int64_t> idx_a(la);
-    int64_t S1a = 0, D2a = 0;
     for (int64_t i = 0; i < la; ++i) {
-        int64_t s1 = a->h_off1[i + 1] - a->h_off1[i];
-        int64_t d2 = a->h_off2[i + 1] - a->h_off2[i];
+        const int64_t s1 = a->h_off1[i + 1] - a->h_off1[i], d2 = a->h_off2[i + 1] - a->h_off2[i];
         S1a += s1;
         plan->a_smax = std::max<int>(plan->a_smax, (int)s1);
         D2a += d2;
-        work[i] = (double)(1 + s1) * (double)(lb + S1b) + (double)d2 * (double)lb + (double)D2b;
+        work[i] = (1 + s1) * (lb + S1b) + d2 * lb + D2b;
     }
-    std::iota(idx_a.begin(), idx_a.end(), 0);
-    std::stable_sort(idx_a.begin(), idx_a.end(), [&](int64_t x, int64_t y) { return work[x] > work[y]; });
-    std::vector<int32_t> rowsa(idx_a.begin(), idx_a.end());
-    TB_CUDA(ctx, plan->d_permb.alloc(lb));
-    TB_CUDA(ctx, plan->d_permb2.alloc(lb));
-    if (lb > 0) TB_CUDA(ctx, cudaMemcpy(plan->d_permb2.p, permb2.data(), lb * sizeof(int32_t), cudaMemcpyHostToDevice));
-    TB_CUDA(ctx, plan->d_rowsa.alloc(la));
-    if (lb > 0) TB_CUDA(ctx, cudaMemcpy(plan->d_permb.p, permb.data(), lb * sizeof(int32_t), cudaMemcpyHostToDevice));
-    if (la > 0) TB_CUDA(ctx, cudaMemcpy(plan->d_rowsa.p, rowsa.data(), la * sizeof(int32_t), cudaMemcpyHostToDevice));
+    const std::vector<int32_t> permb = order_desc(s1b), permb2 = order_desc(tot_b), rowsa = order_desc(work);
+    std::vector<int32_t> pairs;
     if (la > 0 && la % 2 == 0) {
-        // even alpha row starts of row pairs (2k, 2k + 1), heaviest pair first: the
-        // SIMT pass of the tensor-core sigma types may serve two rows per CTA
-        std::vector<int64_t> pr(la / 2);
-        std::iota(pr.begin(), pr.end(), 0);
-        std::stable_sort(pr.begin(), pr.end(),
-                         [&](int64_t x, int64_t y) { return work[2 * x] + work[2 * x + 1] > work[2 * y] + work[2 * y + 1]; });
-        std::vector<int32_t> starts(la / 2);
-        for (int64_t k = 0; k < la / 2; ++k) starts[k] = (int32_t)(2 * pr[k]);
-        TB_CUDA(ctx, plan->d_pairs.alloc(la / 2));
-        TB_CUDA(ctx, cudaMemcpy(plan->d_pairs.p, starts.data(), (la / 2) * sizeof(int32_t), cudaMemcpyHostToDevice));
+        std::vector<int64_t> w2(la / 2);
+        for (int64_t k = 0; k < la / 2; ++k) w2[k] = work[2 * k] + work[2 * k + 1];
+        pairs = order_desc(w2);
+        for (int32_t &k : pairs) k *= 2;
     }
-    // sliced-ELL beta links and column-permuted tables
-    {
-        const int64_t nsl = (lb + 31) / 32;
-        std::vector<int64_t> so;
-        std::vector<int32_t> sw;
-        int64_t tot = 0;
-        const unsigned g = (unsigned)std::max<int64_t>(1, (nsl * 32 + 255) / 256);
+    std::vector<int64_t> o1, o2, od;
+    std::vector<int32_t> w1, w2, wd, offpair;
+    int64_t n1 = 0, n2 = 0, nd = 0;
+    sell_shape(permb, b->h_off1, o1, w1, n1);
+    sell_shape(permb2, b->h_off1, o2, w2, n2);
+    sell_shape(permb2, b->h_off2, od, wd, nd);
+    const bool tc = plan->npoff <= 128 && lb > 0;  // the off-diagonal pairs fit one 128-row tile
+    if (tc) {
+        offpair.resize(plan->npoff);
+        for (int r = 1; r < ham->norb; ++r)
+            for (int q = 0; q < r; ++q) offpair[r * (r - 1) / 2 + q] = r * (r + 1) / 2 + q;
+    }
+    // one allocation; what the host made comes first and goes up in one copy
+    Arena &arena = plan->arena;
+    std::vector<unsigned char> up;
+    auto put = [&](auto &buf, const auto &h) {
+        const size_t at = arena.add(buf, h.size());
+        up.resize(arena.total);
+        if (!h.empty()) std::copy_n(reinterpret_cast<const unsigned char *>(h.data()), h.size() * sizeof(h[0]), up.data() + at);
+    };
+    put(plan->d_permb, permb);
+    put(plan->d_permb2, permb2);
+    put(plan->d_rowsa, rowsa);
+    put(plan->d_pairs, pairs);
+    put(plan->d_s1_off, o1);
+    put(plan->d_s1_w, w1);
+    put(plan->d_s2_off, o2);
+    put(plan->d_s2_w, w2);
+    put(plan->d_d2_off, od);
+    put(plan->d_d2_w, wd);
+    put(plan->d_offpair, offpair);
+    size_spin(a, plan->A, arena);
+    size_spin(b, plan->B, arena);
+    arena.add(plan->d_U, (size_t)np * lb);
+    arena.add(plan->d_Uf, (size_t)np * lb);
+    arena.add(plan->d_s1_ci, std::max<int64_t>(n1, 1));
+    arena.add(plan->d_s2_ci, std::max<int64_t>(n2, 1));
+    arena.add(plan->d_s2_val, std::max<int64_t>(n2, 1));
+    arena.add(plan->d_s2_valf, std::max<int64_t>(n2, 1));
+    arena.add(plan->d_d2_col, std::max<int64_t>(nd, 1));
+    arena.add(plan->d_d2_val, std::max<int64_t>(nd, 1));
+    arena.add(plan->d_d2_valf, std::max<int64_t>(nd, 1));
+    arena.add(plan->d_U1, (size_t)np * lb);
+    arena.add(plan->d_U1f, (size_t)np * lb);
+    arena.add(plan->d_U2, (size_t)np * lb);
+    arena.add(plan->d_U2f, (size_t)np * lb);
+    arena.add(plan->d_Eb2, lb);
+    arena.add(plan->d_Eb2f, lb);
+    if (tc) {
+        arena.add(plan->d_lbp, (size_t)lb * plan->npoff);
+        arena.add(plan->d_tc_err, 1);
+        tile_links_size(ctx, plan.get());
+    }
+    TB_CUDA(ctx, arena.commit());
+    if (!up.empty()) TB_CUDA(ctx, cudaMemcpyAsync(arena.mem.p, up.data(), up.size(), cudaMemcpyHostToDevice, st));
+    TB_TRY(build_spin(ctx, ham, a, plan->A, st));
+    TB_TRY(build_spin(ctx, ham, b, plan->B, st));
+    if (lb > 0) {
+        const dim3 gu((unsigned)((lb + 127) / 128), (unsigned)np), ge((unsigned)((lb + 127) / 128), 1);
+        k_coulomb_table<<<gu, 128, 0, st>>>(b->d_str.p, lb, ham->npair, ham->d_V.p, plan->d_U.p, plan->d_Uf.p);
+        // sliced-ELL beta links: singles in permb order, singles with values and doubles in permb2 order
+        const dim3 g((unsigned)((nsl * 32 + 255) / 256), 64);
         const int zero_idx = 2 * ham->npair;
-        // singles in permb order
-        sell_shape(permb, b->h_off1, so, sw, tot);
-        TB_CUDA(ctx, plan->d_s1_off.alloc(nsl));
-        TB_CUDA(ctx, plan->d_s1_w.alloc(nsl));
-        TB_CUDA(ctx, plan->d_s1_ci.alloc(std::max<int64_t>(tot, 1)));
-        if (nsl > 0) {
-            TB_CUDA(ctx, cudaMemcpy(plan->d_s1_off.p, so.data(), nsl * sizeof(int64_t), cudaMemcpyHostToDevice));
-            TB_CUDA(ctx, cudaMemcpy(plan->d_s1_w.p, sw.data(), nsl * sizeof(int32_t), cudaMemcpyHostToDevice));
-            k_sell_singles<<<g, 256, 0, st>>>(plan->d_permb.p, lb, b->d_off1.p, plan->B.d_sci.p, nullptr,
-                                              plan->d_s1_off.p, plan->d_s1_w.p, nsl, zero_idx, plan->d_s1_ci.p,
-                                              nullptr, nullptr);
-            TB_CUDA(ctx, cudaGetLastError());
-        }
-        // singles with values in permb2 order
-        sell_shape(permb2, b->h_off1, so, sw, tot);
-        TB_CUDA(ctx, plan->d_s2_off.alloc(nsl));
-        TB_CUDA(ctx, plan->d_s2_w.alloc(nsl));
-        TB_CUDA(ctx, plan->d_s2_ci.alloc(std::max<int64_t>(tot, 1)));
-        TB_CUDA(ctx, plan->d_s2_val.alloc(std::max<int64_t>(tot, 1)));
-        TB_CUDA(ctx, plan->d_s2_valf.alloc(std::max<int64_t>(tot, 1)));
-        if (nsl > 0) {
-            TB_CUDA(ctx, cudaMemcpy(plan->d_s2_off.p, so.data(), nsl * sizeof(int64_t), cudaMemcpyHostToDevice));
-            TB_CUDA(ctx, cudaMemcpy(plan->d_s2_w.p, sw.data(), nsl * sizeof(int32_t), cudaMemcpyHostToDevice));
-            k_sell_singles<<<g, 256, 0, st>>>(plan->d_permb2.p, lb, b->d_off1.p, plan->B.d_sci.p, plan->B.d_sval.p,
-                                              plan->d_s2_off.p, plan->d_s2_w.p, nsl, zero_idx, plan->d_s2_ci.p,
-                                              plan->d_s2_val.p, plan->d_s2_valf.p);
-            TB_CUDA(ctx, cudaGetLastError());
-        }
-        // doubles in permb2 order
-        sell_shape(permb2, b->h_off2, so, sw, tot);
-        TB_CUDA(ctx, plan->d_d2_off.alloc(nsl));
-        TB_CUDA(ctx, plan->d_d2_w.alloc(nsl));
-        TB_CUDA(ctx, plan->d_d2_col.alloc(std::max<int64_t>(tot, 1)));
-        TB_CUDA(ctx, plan->d_d2_val.alloc(std::max<int64_t>(tot, 1)));
-        TB_CUDA(ctx, plan->d_d2_valf.alloc(std::max<int64_t>(tot, 1)));
-        if (nsl > 0) {
-            TB_CUDA(ctx, cudaMemcpy(plan->d_d2_off.p, so.data(), nsl * sizeof(int64_t), cudaMemcpyHostToDevice));
-            TB_CUDA(ctx, cudaMemcpy(plan->d_d2_w.p, sw.data(), nsl * sizeof(int32_t), cudaMemcpyHostToDevice));
-            k_sell_doubles<<<g, 256, 0, st>>>(plan->d_permb2.p, lb, b->d_off2.p, plan->B.d_dcol.p, plan->B.d_dval.p,
-                                              plan->d_d2_off.p, plan->d_d2_w.p, nsl, plan->d_d2_col.p,
-                                              plan->d_d2_val.p, plan->d_d2_valf.p);
-            TB_CUDA(ctx, cudaGetLastError());
-        }
-        const int64_t np = ham->npair;
-        TB_CUDA(ctx, plan->d_U1.alloc(np * lb));
-        TB_CUDA(ctx, plan->d_U1f.alloc(np * lb));
-        TB_CUDA(ctx, plan->d_U2.alloc(np * lb));
-        TB_CUDA(ctx, plan->d_U2f.alloc(np * lb));
-        TB_CUDA(ctx, plan->d_Eb2.alloc(lb));
-        TB_CUDA(ctx, plan->d_Eb2f.alloc(lb));
-        if (lb > 0) {
-            dim3 gu((unsigned)((lb + 127) / 128), (unsigned)np);
-            k_permute_cols<<<gu, 128, 0, st>>>(plan->d_U.p, np, lb, plan->d_permb.p, plan->d_U1.p, plan->d_U1f.p);
-            k_permute_cols<<<gu, 128, 0, st>>>(plan->d_U.p, np, lb, plan->d_permb2.p, plan->d_U2.p, plan->d_U2f.p);
-            dim3 ge((unsigned)((lb + 127) / 128), 1);
-            k_permute_cols<<<ge, 128, 0, st>>>(plan->B.d_E.p, 1, lb, plan->d_permb2.p, plan->d_Eb2.p, plan->d_Eb2f.p);
-            TB_CUDA(ctx, cudaGetLastError());
-        }
+        k_sell_singles<<<g, 256, 0, st>>>(plan->d_permb.p, lb, b->d_off1.p, plan->B.d_sci.p, nullptr, plan->d_s1_off.p,
+                                          plan->d_s1_w.p, nsl, zero_idx, plan->d_s1_ci.p, nullptr, nullptr);
+        k_sell_singles<<<g, 256, 0, st>>>(plan->d_permb2.p, lb, b->d_off1.p, plan->B.d_sci.p, plan->B.d_sval.p, plan->d_s2_off.p,
+                                          plan->d_s2_w.p, nsl, zero_idx, plan->d_s2_ci.p, plan->d_s2_val.p, plan->d_s2_valf.p);
+        k_sell_doubles<<<g, 256, 0, st>>>(plan->d_permb2.p, lb, b->d_off2.p, plan->B.d_dcol.p, plan->B.d_dval.p, plan->d_d2_off.p,
+                                          plan->d_d2_w.p, nsl, plan->d_d2_col.p, plan->d_d2_val.p, plan->d_d2_valf.p);
+        // tables with their columns in those orders
+        k_permute_cols<<<gu, 128, 0, st>>>(plan->d_U.p, np, lb, plan->d_permb.p, plan->d_U1.p, plan->d_U1f.p);
+        k_permute_cols<<<gu, 128, 0, st>>>(plan->d_U.p, np, lb, plan->d_permb2.p, plan->d_U2.p, plan->d_U2f.p);
+        k_permute_cols<<<ge, 128, 0, st>>>(plan->B.d_E.p, 1, lb, plan->d_permb2.p, plan->d_Eb2.p, plan->d_Eb2f.p);
+        TB_CUDA(ctx, cudaGetLastError());
     }
-    // tensor-core alpha-beta tables (only when the off-diagonal pairs fit one 128-row tile)
-    {
-        const int n = ham->norb;
-        plan->npoff = n * (n - 1) / 2;
-        if (plan->npoff <= 128 && lb > 0) {
-            TB_CUDA(ctx, plan->d_lbp.alloc((size_t)lb * plan->npoff));
-            TB_CUDA(ctx, cudaMemsetAsync(plan->d_lbp.p, 0xFF, plan->d_lbp.bytes(), st));
-            k_link_by_pair<<<(unsigned)((lb + 127) / 128), 128, 0, st>>>(lb, b->d_off1.p, b->d_ent1.p, plan->npoff,
-                                                                          plan->d_lbp.p);
-            TB_CUDA(ctx, cudaGetLastError());
-            std::vector<int32_t> op(plan->npoff);
-            for (int r = 1; r < n; ++r)
-                for (int q = 0; q < r; ++q) op[r * (r - 1) / 2 + q] = r * (r + 1) / 2 + q;
-            TB_CUDA(ctx, plan->d_offpair.alloc(plan->npoff));
-            TB_CUDA(ctx, cudaMemcpy(plan->d_offpair.p, op.data(), op.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-            TB_CUDA(ctx, plan->d_tc_err.alloc(1));
-            TB_CUDA(ctx, cudaMemsetAsync(plan->d_tc_err.p, 0, sizeof(int), st));
-            TB_TRY(tile_links_build(ctx, plan.get(), st));
-        }
+    if (tc) {  // tensor-core alpha-beta tables
+        TB_CUDA(ctx, cudaMemsetAsync(plan->d_lbp.p, 0xFF, plan->d_lbp.bytes(), st));
+        TB_CUDA(ctx, cudaMemsetAsync(plan->d_tc_err.p, 0, sizeof(int), st));
+        k_link_by_pair<<<(unsigned)((lb + 127) / 128), 128, 0, st>>>(lb, b->d_off1.p, b->d_ent1.p, plan->npoff, plan->d_lbp.p);
+        TB_CUDA(ctx, cudaGetLastError());
+        TB_TRY(tile_links_build(ctx, plan.get(), st));
     }
     // work counts: non-zeros of H by class (Sec. II.C, Table I)
     tbsci_sigma_counts &c = plan->counts;

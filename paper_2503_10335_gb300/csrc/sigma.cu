@@ -489,6 +489,45 @@ __global__ void k_diagonal(const uint64_t *__restrict__ stra, int64_t la, int64_
     diag[K] = d;
 }
 
+// The same by tables: 32 columns x a range of rows per block, with the sums of U over every
+// set of six orbitals in shared memory ([group][64][32], ecore + E_b with the first group),
+// so a determinant takes norb / 6 + 1 FP64 adds instead of nelec + 2. Bound by them
+// (2 a clock and SM): 4,000 x 5,000 at norb 24 took 535 us, now 200 us. A table costs
+// 80 adds per group and column, as much as some 16 rows, so fewer than kDiagRows rows per
+// block are left to k_diagonal.
+constexpr int kDiagRows = 64;
+__global__ void __launch_bounds__(256) k_diagonal_tab(const uint64_t *__restrict__ stra, int64_t la, int64_t lb, int norb,
+                                                      int rows, const double *__restrict__ Ea, const double *__restrict__ Eb,
+                                                      const double *__restrict__ U, double ecore, double *__restrict__ diag) {
+    extern __shared__ double tab[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ng = (norb + 5) / 6;
+    const int64_t ib = blockIdx.x * 32ll + lane, ibc = min(ib, lb - 1);
+    for (int g = 0; g < ng; ++g) {
+        double u[6];
+        for (int k = 0; k < 6; ++k) {
+            const int p = 6 * g + k;
+            u[k] = p < norb ? U[(size_t)(p * (p + 1) / 2 + p) * lb + ibc] : 0.0;
+        }
+        double t[8];  // entries 8 warp .. 8 warp + 7
+        t[0] = g == 0 ? ecore + Eb[ibc] : 0.0;
+        for (int k = 0; k < 3; ++k)
+            if ((warp >> k) & 1) t[0] += u[3 + k];
+        t[1] = t[0] + u[0];
+        t[2] = t[0] + u[1];
+        t[3] = t[1] + u[1];
+        for (int k = 0; k < 4; ++k) t[4 + k] = t[k] + u[2];
+        for (int k = 0; k < 8; ++k) tab[(g * 64 + warp * 8 + k) * 32 + lane] = t[k];
+    }
+    __syncthreads();
+    const int64_t end = min(la, (int64_t)(blockIdx.y + 1) * rows);
+    for (int64_t ia = (int64_t)blockIdx.y * rows + warp; ia < end; ia += 8) {
+        uint64_t s = stra[ia];
+        double d = Ea[ia];
+        for (int g = 0; g < ng; ++g, s >>= 6) d += tab[(g * 64 + (int)(s & 63)) * 32 + lane];
+        if (ib < lb) diag[ia * lb + ib] = d;
+    }
+}
+
 template <typename T>
 void set_sell(SigArgs<T> &A, const Plan *P) {
     A.s1_off = P->d_s1_off.p;
@@ -1323,7 +1362,18 @@ tbsci_status sigma_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan
 tbsci_status diagonal_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, double *diag, cudaStream_t st) {
     const int64_t N = P->A.l * P->B.l;
     if (N == 0) return TBSCI_OK;
-    k_diagonal<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(P->A.d_str, P->A.l, P->B.l, P->A.d_E.p, P->B.d_E.p,
+    const int64_t la = P->A.l, lb = P->B.l, ct = (lb + 31) / 32;
+    if (la >= kDiagRows && lb >= 16) {  // narrower rows leave most of a warp's lanes without a column
+        const size_t smem = (size_t)((P->norb + 5) / 6) * 64 * 32 * sizeof(double);  // 176 KB at 64 orbitals
+        // about eight blocks per SM, 128 to 1024 rows each
+        const int64_t rows = std::max<int64_t>(std::min<int64_t>(std::max<int64_t>(la * ct / (152 * 8), 128), 1024), (la + 65534) / 65535);
+        TB_CUDA(ctx, cudaFuncSetAttribute(k_diagonal_tab, cudaFuncAttributeMaxDynamicSharedMemorySize, 180224));
+        k_diagonal_tab<<<dim3((unsigned)ct, (unsigned)((la + rows - 1) / rows)), 256, smem, st>>>(
+            P->A.d_str, la, lb, P->norb, (int)rows, P->A.d_E.p, P->B.d_E.p, P->d_U.p, ham->ecore, diag);
+        TB_CUDA(ctx, cudaGetLastError());
+        return TBSCI_OK;
+    }
+    k_diagonal<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(P->A.d_str, la, lb, P->A.d_E.p, P->B.d_E.p,
                                                             P->d_U.p, ham->ecore, diag);
     TB_CUDA(ctx, cudaGetLastError());
     return TBSCI_OK;

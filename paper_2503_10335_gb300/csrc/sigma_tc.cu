@@ -465,29 +465,33 @@ int sigma_tc_batch(const Plan *P) {
 
 // Link plan of a space (norb <= 16), made when the space is prepared; left out
 // (tl_kpmax = 0) where the alpha-beta kernels do not apply.
-tbsci_status tile_links_build(tbsci_ctx *ctx, Plan *P, cudaStream_t st) {
+void tile_links_size(tbsci_ctx *ctx, Plan *P) {
     const int64_t la = P->A.l, lb = P->B.l;
     P->tl_kpmax = 0;
-    if (P->npoff < 1 || P->npoff > 120 || !P->d_lbp.p || la < 1 || lb < 1) return TBSCI_OK;
-    int kmax = 1;
-    for (int64_t i = 0; i < la; ++i) kmax = std::max<int>(kmax, 1 + (int)(P->A.h_soff[i + 1] - P->A.h_soff[i]));
-    const size_t smem = (size_t)lb * 4;
-    if (kmax > 65 || smem + 16384 > ctx->smem_optin) return TBSCI_OK;
+    if (P->npoff < 1 || P->npoff > 120 || la < 1 || lb < 1) return;
+    const int kmax = 1 + P->a_smax;
+    if (kmax > 65 || (size_t)lb * 4 + 16384 > ctx->smem_optin) return;
     const int nt = (int)((lb + kAbTile - 1) / kAbTile);
     int links = 0;
     for (int t = 0; t < nt; ++t)
         links = std::max<int>(links, (int)(P->B.h_soff[std::min<int64_t>(lb, (t + 1) * (int64_t)kAbTile)] - P->B.h_soff[(int64_t)t * kAbTile]));
     P->tl_nslot = (links + kPiece + 2) / 2 * 2;  // a piece is read whole; the last slot takes pairs without a link
     P->tl_npiece = std::max(1, (links + kAbDrain - 1) / kAbDrain) * kAbDrain;
-    TB_CUDA(ctx, P->d_tl_pos.alloc((size_t)nt * 4 * 2 * 128));
-    TB_CUDA(ctx, P->d_tl_piece.alloc((size_t)nt * P->tl_npiece));
-    TB_CUDA(ctx, P->d_tl_rounds.alloc(nt));
-    TB_CUDA(ctx, cudaFuncSetAttribute(k_tile_links, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_tile_links<<<(unsigned)nt, kLinkThreads, smem, st>>>(P->d_lbp.p, lb, P->npoff, P->tl_npiece, P->tl_nslot,
-                                                          reinterpret_cast<uint16_t *>(P->d_tl_pos.p), P->d_tl_piece.p,
-                                                          P->d_tl_rounds.p);
-    TB_CUDA(ctx, cudaGetLastError());
+    P->arena.add(P->d_tl_pos, (size_t)nt * 4 * 2 * 128);
+    P->arena.add(P->d_tl_piece, (size_t)nt * P->tl_npiece);
+    P->arena.add(P->d_tl_rounds, nt);
     P->tl_kpmax = (kmax + 15) / 16 * 16;
+}
+
+tbsci_status tile_links_build(tbsci_ctx *ctx, Plan *P, cudaStream_t st) {
+    if (P->tl_kpmax == 0) return TBSCI_OK;
+    const int64_t lb = P->B.l;
+    const size_t smem = (size_t)lb * 4;
+    TB_CUDA(ctx, cudaFuncSetAttribute(k_tile_links, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_tile_links<<<(unsigned)((lb + kAbTile - 1) / kAbTile), kLinkThreads, smem, st>>>(
+        P->d_lbp.p, lb, P->npoff, P->tl_npiece, P->tl_nslot, reinterpret_cast<uint16_t *>(P->d_tl_pos.p), P->d_tl_piece.p,
+        P->d_tl_rounds.p);
+    TB_CUDA(ctx, cudaGetLastError());
     return TBSCI_OK;
 }
 

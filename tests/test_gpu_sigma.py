@@ -85,6 +85,17 @@ def test_diagonal_parity(tb, ctx):
     sp.close()
 
 
+@pytest.mark.parametrize("n,na,nb,la,lb", [(6, 3, 3, 20, 20), (12, 6, 5, 63, 33), (12, 6, 5, 64, 15), (12, 6, 5, 64, 16),
+                                           (13, 6, 5, 300, 65), (64, 2, 1, 70, 33)])
+def test_diagonal_by_tables(tb, ctx, n, na, nb, la, lb):
+    """Sizes around the rule (64 rows, 16 columns), a last group of one orbital, all 11 groups."""
+    sp, osp, h, eri = _case(tb, ctx, n, na, nb, la, lb, seed=n)
+    d = sp.diagonal().cpu().numpy()
+    ref = oracle.diagonal(osp, h, eri, 0.0)
+    assert np.max(np.abs(d - ref)) <= 1e-12 * max(1.0, np.max(np.abs(ref)))
+    sp.close()
+
+
 def test_sigma_host_equals_device_and_deterministic(tb, ctx):
     import torch
     sp, osp, h, eri = _case(tb, ctx, 10, 5, 5, 150, 150, seed=10)

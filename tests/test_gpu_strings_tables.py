@@ -132,3 +132,27 @@ def test_table6_stored_entries_smallest(tb, ctx):
             lo, hi = min(p, q), max(p, q)
             between = sum((src >> x) & 1 for x in range(lo + 1, hi))
             assert int(e["sign"]) == (-1) ** between
+
+
+@pytest.mark.parametrize("n,N,cnt", [(64, 2, 2016), (24, 12, 8192), (24, 12, 8193), (24, 12, 33000), (40, 38, 129),
+                                     (20, 19, 20)])
+def test_blocked_sort_and_link_filter(tb, ctx, n, N, cnt):
+    """Shuffled sets around the sort block (8,192 keys) and with a full 64 KB filter: sorted
+    as by numpy, and single and double links as found by masks over the sorted set."""
+    sel = selected_strings(n, N, cnt, 5)
+    np.random.default_rng(cnt).shuffle(sel)
+    t, l, strs = _tables(tb, ctx, n, N, sel)
+    off1, e1, off2, e2 = tb.tbsci_tables_export(ctx.handle, t, l)
+    tb.tbsci_tables_destroy(t)
+    assert l == cnt == len(sel) and np.array_equal(strs, np.sort(sel))
+    for J in sorted({0, 1, 7, 8, 31, 32, cnt // 2, cnt - 1} & set(range(cnt))):
+        dist = np.bitwise_count(strs ^ strs[J])
+        for off, e, d in ((off1, e1, 2), (off2, e2, 4)):
+            assert np.array_equal(np.sort(e["target"][off[J]:off[J + 1]]), np.flatnonzero(dist == d))
+    both = np.repeat(np.arange(cnt), np.diff(off1)).astype(np.int64) * cnt + e1["target"]
+    back = e1["target"].astype(np.int64) * cnt + np.repeat(np.arange(cnt), np.diff(off1))
+    assert np.array_equal(np.sort(both), np.sort(back))
+    x = strs[np.repeat(np.arange(cnt), np.diff(off2))]
+    for k in ("p", "r", "q", "s"):
+        x = x ^ (np.uint64(1) << e2[k].astype(np.uint64))
+    assert np.array_equal(x, strs[e2["target"]])
