@@ -228,7 +228,7 @@ struct SpinPlan {
 // padding entries point at the part's first column with a zero coefficient.
 // U is the beta Coulomb table with its columns in `perm` order.
 struct PartLayout {
-    int P = 0;
+    int P = 0, elem = 0;  // column parts; element bytes the link order is for
     int64_t W = 0;
     DevBuf<int32_t> perm, iperm;  // column order and its inverse
     DevBuf<int64_t> off;          // [nslices * P]

@@ -322,12 +322,94 @@ __global__ void k_combine(T *y, const T *__restrict__ pz, const int32_t *__restr
     }
 }
 
-// Part layout of the beta single links for `nparts` column parts (built on the host).
-tbsci_status build_parts(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int nparts, PartLayout **out) {
+// Order of the links of each column of a part layout. The 32 columns of a slice read their
+// k-th links together: c at the target and the coefficient at its pair, both from shared
+// memory at scattered places (some 3.5 lanes on one bank in each). A column's links may be
+// summed in any fixed order, so lane by lane, at every k, the link is taken that adds least
+// to the fullest bank of either read; equal coefficients are one read. One warp per slice
+// and part, kSpread links of a column at a time. FP32 only, whose k_sigma_parts is bound by
+// these reads: 20,000 x 40,000 at norb 24 took 238 ms, now 198. FP64 is bound by the FP64
+// pipe and gained nothing (432 and 431 ms at 10,000 x 40,000).
+constexpr int kSpread = 64;
+__global__ void __launch_bounds__(32) k_spread_links(const int64_t *__restrict__ off, const int32_t *__restrict__ w, uint32_t *ci,
+                                                     double *val, float *valf) {
+    __shared__ double buf[kSpread * 33];  // ci, then val, then valf, of kSpread links x 32 lanes
+    __shared__ uint8_t take[kSpread * 33];
+    uint32_t *code = reinterpret_cast<uint32_t *>(buf);
+    float *bf = reinterpret_cast<float *>(buf);
+    const int lane = threadIdx.x;
+    const int64_t o = off[blockIdx.x] + lane;
+    const int wide = w[blockIdx.x];
+    for (int k0 = 0; k0 < wide; k0 += kSpread) {
+        const int n = min(kSpread, wide - k0);
+        const int64_t at = o + 32 * (int64_t)k0;
+        for (int k = 0; k < n; ++k) code[k * 33 + lane] = ci[at + 32 * k];
+        __syncwarp();
+        uint64_t left = n == 64 ? ~0ull : (1ull << n) - 1;  // of this lane's column
+        for (int k = 0; k < n; ++k) {
+            int nc = 0, nv = 0, maxc = 0, maxv = 0;  // reads on this lane's bank
+            uint32_t av = ~0u;                       // a coefficient read from it
+            for (int turn = 0; turn < 32; ++turn) {
+                const int L = (turn + k) & 31;
+                const uint64_t mine = __shfl_sync(0xffffffffu, left, L);
+                uint32_t best = ~0u;
+                for (int h = 0; h < n; h += 32) {
+                    const int j = h + lane;
+                    const uint32_t e = j < n ? code[j * 33 + L] : 0u;
+                    const uint32_t x = e & ((1u << kPartLinkBits) - 1), tg = e >> kPartLinkBits;
+                    const int bx = (int)(x & 31);
+                    const int bt = (int)(tg & 31);
+                    const int c1 = __shfl_sync(0xffffffffu, nc, bt) + 1;
+                    const int vb = __shfl_sync(0xffffffffu, nv, bx);
+                    const bool same = __shfl_sync(0xffffffffu, av, bx) == x;
+                    const int v1 = same ? 0 : vb + 1;
+                    const uint32_t cost = ((c1 > maxc) + (v1 > maxv)) * 128u + c1 + v1;
+                    if (j < n && ((mine >> j) & 1)) best = min(best, cost << 8 | (uint32_t)j);
+                }
+                best = __reduce_min_sync(0xffffffffu, best);
+                const int j = best & 255;
+                const uint32_t e = code[j * 33 + L];
+                const uint32_t x = e & ((1u << kPartLinkBits) - 1), tg = e >> kPartLinkBits;
+                const int bx = (int)(x & 31);
+                const int bt = (int)(tg & 31);
+                if (lane == bt) ++nc;
+                if (lane == bx && av != x) {
+                    ++nv;
+                    av = x;
+                }
+                maxc = max(maxc, __shfl_sync(0xffffffffu, nc, bt));
+                maxv = max(maxv, __shfl_sync(0xffffffffu, nv, bx));
+                if (lane == L) {
+                    left &= ~(1ull << j);
+                    take[k * 33 + L] = (uint8_t)j;
+                }
+            }
+        }
+        __syncwarp();
+        for (int k = 0; k < n; ++k) ci[at + 32 * k] = code[take[k * 33 + lane] * 33 + lane];
+        __syncwarp();
+        for (int k = 0; k < n; ++k) buf[k * 33 + lane] = val[at + 32 * k];
+        __syncwarp();
+        for (int k = 0; k < n; ++k) val[at + 32 * k] = buf[take[k * 33 + lane] * 33 + lane];
+        __syncwarp();
+        for (int k = 0; k < n; ++k) bf[k * 33 + lane] = valf[at + 32 * k];
+        __syncwarp();
+        for (int k = 0; k < n; ++k) valf[at + 32 * k] = bf[take[k * 33 + lane] * 33 + lane];
+        __syncwarp();
+    }
+}
+
+// Part layout of the beta single links for `nparts` column parts (built on the host) and
+// elements of `elem` bytes.
+tbsci_status build_parts(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int nparts, int elem, PartLayout **out) {
+    PartLayout *other = nullptr;  // the same parts in the other type's order
     for (auto &pl : P->parts)
         if (pl->P == nparts) {
-            *out = pl.get();
-            return TBSCI_OK;
+            if (pl->elem == elem) {
+                *out = pl.get();
+                return TBSCI_OK;
+            }
+            other = pl.get();
         }
     const int64_t lb = P->B.l, nsl = (lb + 31) / 32;
     const int64_t W = (lb + nparts - 1) / nparts;
@@ -403,9 +485,14 @@ tbsci_status build_parts(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int npar
     }
     auto pl = std::make_unique<PartLayout>();
     pl->P = nparts;
+    pl->elem = elem;
     pl->W = W;
     const size_t bytes = loff.size() * 12 + ci.size() * (sizeof(uint32_t) + 12) + (size_t)lb * 28;
-    TB_TRY(charge(ctx, bytes, "column-part link layout"));
+    if (other && charge(ctx, bytes, "column-part link layout") != TBSCI_OK) {  // no room for a second one
+        *out = other;
+        return TBSCI_OK;
+    }
+    if (!other) TB_TRY(charge(ctx, bytes, "column-part link layout"));
     cudaError_t e = pl->off.alloc(loff.size());
     if (e == cudaSuccess) e = pl->w.alloc(lw.size());
     if (e == cudaSuccess) e = pl->ci.alloc(ci.size());
@@ -428,6 +515,11 @@ tbsci_status build_parts(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int npar
     if (e == cudaSuccess) e = cudaMemcpy(pl->str.p, pstr.data(), lb * sizeof(uint64_t), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(pl->Eb.p, pE.data(), lb * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(pl->Ebf.p, pEf.data(), lb * sizeof(float), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && total > 0 && elem == 4) {  // on the default stream, after the copies
+        k_spread_links<<<(unsigned)(nsl * nparts), 32>>>(pl->off.p, pl->w.p, pl->ci.p, pl->val.p, pl->valf.p);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    }
     if (e != cudaSuccess) {
         uncharge(ctx, bytes);
         return fail(ctx, e == cudaErrorMemoryAllocation ? TBSCI_ENOMEM : TBSCI_ECUDA,
@@ -571,7 +663,7 @@ tbsci_status split_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const T
     TB_CHECK(ctx, (la + 31) / 32 <= 65535, TBSCI_EINVAL, "split sigma: too many alpha strings");
     nparts = (int)std::min<int64_t>(lb, nparts);
     PartLayout *pl = nullptr;
-    TB_TRY(build_parts(ctx, ham, P, nparts, &pl));
+    TB_TRY(build_parts(ctx, ham, P, nparts, (int)sizeof(T), &pl));
     const size_t need = 2 * (size_t)la * lb * sizeof(T);
     if (P->d_trans.n < need) {
         uncharge(ctx, P->d_trans.bytes());

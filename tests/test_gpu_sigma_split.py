@@ -125,3 +125,18 @@ def test_split_davidson_matches_dense(tb, tmp_path):
         assert info["converged"] and np.max(np.abs(e - w[:4])) < 1e-8
     sp.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("n,na,nb,acnt,bcnt", [(20, 10, 10, 40, 300), (24, 12, 12, 20, 161), (16, 8, 8, 33, 64)])
+def test_link_order_of_fp32_layout(tb, tmp_path, n, na, nb, acnt, bcnt):
+    """The FP32 layout's link order with columns of over 64 links (the aufbau string has up to
+    144) and a ragged last slice."""
+    import torch
+    ctx = _ctx_with_shape(tb, tmp_path, n, acnt, bcnt, "f32", 512, 3)
+    sp, osp, h, eri = _space(tb, ctx, n, na, nb, acnt, bcnt, seed=800 + n, ecore=0.15)
+    C = np.random.default_rng(n).standard_normal((2, sp.la, sp.lb)).astype(np.float32)
+    s = sp.sigma(torch.from_numpy(C).cuda()).double().cpu().numpy().reshape(2, -1)
+    ref, bound = oracle.sigma(osp, h, eri, 0.15, C.astype(np.float64), with_bound=True)
+    assert_sigma_close(s, ref, bound, rel=64 * 2.0 ** -24, norm_rel=1e-5)
+    sp.close()
+    ctx.close()
