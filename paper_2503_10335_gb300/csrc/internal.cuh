@@ -352,6 +352,25 @@ namespace tbsci {
 
 inline int pair_index(int p, int q) { return p >= q ? p * (p + 1) / 2 + q : q * (q + 1) / 2 + p; }
 
+// Elements of the vectors of an exact launch that its digits leave out (FP64 only), and what
+// their links need (k_sigma_left adds them)
+constexpr int kOutliers = 256;
+struct Outliers {
+    double *thr;    // [vector] an outlier's magnitude exceeds it
+    int *count;     // [vector]
+    int64_t *list;  // [vector][kOutliers], in no order
+};
+struct OutlierArgs {
+    Outliers O;
+    int64_t lb;
+    const uint64_t *stra;
+    const int64_t *a_soff, *a_doff, *b_soff, *b_doff;
+    const int2 *a_sci, *b_sci;
+    const double *a_sval, *b_sval, *a_dval, *b_dval, *V;
+    const int32_t *a_dcol, *b_dcol;
+    int npair;
+};
+
 // strings.cu
 tbsci_status strings_build(tbsci_ctx *ctx, int norb, int nelec, const uint64_t *sel, int64_t nsel,
                            tbsci_strings *out);
@@ -423,9 +442,9 @@ void dense_context_release(tbsci_ctx *ctx);
 // *ran = false where it does not apply. simt(v, nv, skip) launches the SIMT sigma of
 // vectors v .. v + nv - 1, each of which returns at once where skip[2 i] (device memory) is set.
 tbsci_status exact_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const double *c, double *s, int nvec,
-                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *)> &simt);
+                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *, const OutlierArgs &)> &simt);
 tbsci_status exact_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const float *c, float *s, int nvec,
-                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *)> &simt);
+                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *, const OutlierArgs &)> &simt);
 tbsci_status udiag_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, const float *c, float *s, int nv, bool add,
                           bool singles, cudaStream_t st);
 // sigma_tc.cu: the alpha-beta classes on the tensor cores with np = 1 or 3 BF16 planes

@@ -422,12 +422,72 @@ __global__ void __launch_bounds__(512) k_sigma_small(SigArgs<T> A, int nsmax) {
     }
 }
 
-// The vectors (one per blockIdx.y) that the exact tensor-core path leaves: skip[2 v] = 0.
+// The outliers' share of what the digit kernels sum for row Ia, in FP64: their same-spin
+// links and their alpha-beta links (k_udiag has their diagonal and the rest of the alpha
+// singles). Outlier by outlier in the order of their places, so every element is summed in
+// a fixed order without atomics. C and S: the vector; sJ: kOutliers + 1 places.
+__device__ void outliers_row(const OutlierArgs &A, int v, const double *C, double *S, int64_t Ia, int64_t *sJ) {
+    const int n = min(A.O.count[v], kOutliers), tid = threadIdx.x, th = blockDim.x;
+    const int64_t *list = A.O.list + (size_t)v * kOutliers, lb = A.lb;
+    for (int x = tid; x < n; x += th) {
+        const int64_t mine = list[x];
+        int rank = 0;
+        for (int k = 0; k < n; ++k) rank += list[k] < mine;
+        sJ[rank] = mine;
+    }
+    __syncthreads();
+    S += Ia * lb;
+    const uint64_t sI = A.stra[Ia];
+    for (int o = 0; o < n; ++o) {
+        const int64_t J = sJ[o], Ja = J / lb, Jb = J - Ja * lb;
+        const double x = C[J];
+        const uint64_t sj = A.stra[Ja];
+        const int d = __popcll(sI ^ sj);  // 0, 2 or 4 where Ia and Ja are linked
+        if (d > 4) continue;
+        if (d == 0) {
+            for (int64_t t = A.b_soff[Jb] + tid; t < A.b_soff[Jb + 1]; t += th) {
+                const int2 e = A.b_sci[t];
+                double w = 0.0;
+                for (uint64_t m = sj; m; m &= m - 1) {
+                    const int p = __ffsll((long long)m) - 1;
+                    w += A.V[(size_t)(p * (p + 1) / 2 + p) * A.npair + (e.y >> 1)];
+                }
+                S[e.x] += x * (A.b_sval[t] + ((e.y & 1) ? -w : w));
+            }
+            for (int64_t t = A.b_doff[Jb] + tid; t < A.b_doff[Jb + 1]; t += th) S[A.b_dcol[t]] += x * A.b_dval[t];
+        } else if (d == 2) {
+            for (int64_t t = A.a_soff[Ja] + tid; t < A.a_soff[Ja + 1]; t += th)
+                if (A.a_sci[t].x == Ia) sJ[kOutliers] = t;
+            __syncthreads();
+            const int64_t ta = sJ[kOutliers];
+            const int2 ea = A.a_sci[ta];
+            if (tid == 0) S[Jb] += x * A.a_sval[ta];
+            for (int64_t t = A.b_soff[Jb] + tid; t < A.b_soff[Jb + 1]; t += th) {
+                const int2 e = A.b_sci[t];
+                const double h = A.V[(size_t)(ea.y >> 1) * A.npair + (e.y >> 1)];
+                S[e.x] += x * (((ea.y ^ e.y) & 1) ? -h : h);
+            }
+        } else {
+            for (int64_t t = A.a_doff[Ja] + tid; t < A.a_doff[Ja + 1]; t += th)
+                if (A.a_dcol[t] == Ia) S[Jb] += x * A.a_dval[t];
+        }
+        __syncthreads();
+    }
+}
+
+// The vectors (one per blockIdx.y) that the exact tensor-core path leaves: skip[2 v] = 0;
+// of the others, the links of their outliers (a launch of their own cost 4 us a call).
 // Its own kernel, so that k_sigma's arguments stay constants.
 template <typename T, bool STAGE, bool ACCS>
-__global__ void __launch_bounds__(256) k_sigma_left(SigArgs<T> A, const int *__restrict__ skip) {
+__global__ void __launch_bounds__(256) k_sigma_left(SigArgs<T> A, const int *__restrict__ skip, const OutlierArgs out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (skip[2 * blockIdx.y]) return;
+    if (skip[2 * blockIdx.y]) {
+        if constexpr (sizeof(T) == 8)
+            if (out.O.count[blockIdx.y])
+                outliers_row(out, blockIdx.y, A.C + blockIdx.y * A.vstride, A.S + blockIdx.y * A.vstride, A.rowsa[blockIdx.x],
+                             reinterpret_cast<int64_t *>(smem_raw));
+        return;
+    }
     A.C += blockIdx.y * A.vstride;
     A.S += blockIdx.y * A.vstride;
     sigma_row<T, 1, STAGE, ACCS, 256>(A, A.rowsa[blockIdx.x], smem_raw);
@@ -1299,12 +1359,12 @@ tbsci_status launch_small(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, c
 }
 
 template <typename T, bool STAGE, bool ACCS>
-tbsci_status launch_left(tbsci_ctx *ctx, const SigArgs<T> &A, int nv, const int *skip, cudaStream_t st) {
-    const size_t sm = smem_bytes<T>(A.npair, A.lb, 1, STAGE, ACCS);
+tbsci_status launch_left(tbsci_ctx *ctx, const SigArgs<T> &A, int nv, const int *skip, const OutlierArgs &out, cudaStream_t st) {
+    const size_t sm = std::max(smem_bytes<T>(A.npair, A.lb, 1, STAGE, ACCS), (kOutliers + 1) * sizeof(int64_t));
     auto k = k_sigma_left<T, STAGE, ACCS>;
     TB_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     TraceScope tr(ctx, "k_sigma_left", st);
-    k<<<dim3((unsigned)A.la, (unsigned)nv), 256, sm, st>>>(A, skip);
+    k<<<dim3((unsigned)A.la, (unsigned)nv), 256, sm, st>>>(A, skip, out);
     TB_CUDA(ctx, cudaGetLastError());
     return TBSCI_OK;
 }
@@ -1317,14 +1377,14 @@ tbsci_status launch_full(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan,
     bool ran = false;
     TB_TRY(launch_small<T>(ctx, ham, plan, c, s, nvec, st, &ran));
     if (ran) return TBSCI_OK;
-    TB_TRY(exact_launch(ctx, ham, const_cast<Plan *>(plan), c, s, nvec, st, &ran, [&](int v, int nv, const int *skip) {
+    TB_TRY(exact_launch(ctx, ham, const_cast<Plan *>(plan), c, s, nvec, st, &ran, [&](int v, int nv, const int *skip, const OutlierArgs &out) {
         SigArgs<T> A = make_args<T>(ham, plan);
         A.C = c + v * n;
         A.S = s + v * n;
         switch (stage_variant<T>(ctx, A.npair, A.lb, 1, 0)) {
-            case 0: return launch_left<T, true, true>(ctx, A, nv, skip, st);
-            case 1: return launch_left<T, false, true>(ctx, A, nv, skip, st);
-            default: return launch_left<T, false, false>(ctx, A, nv, skip, st);
+            case 0: return launch_left<T, true, true>(ctx, A, nv, skip, out, st);
+            case 1: return launch_left<T, false, true>(ctx, A, nv, skip, out, st);
+            default: return launch_left<T, false, false>(ctx, A, nv, skip, out, st);
         }
     }));
     return ran ? TBSCI_OK : launch_typed<T>(ctx, ham, plan, c, s, nvec, st);

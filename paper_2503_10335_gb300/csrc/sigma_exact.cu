@@ -126,12 +126,23 @@ __host__ __device__ inline int scale_exponent(double top) {
 constexpr int kScaleThreads = 256;
 constexpr int kScaleBlocks = 304;
 
+// Elements that tower over the rest of a vector (trial vectors of an eigensolver start as
+// single determinants and stay close to them) are kept out of the digits: at most
+// n / 256^2 of a vector's n elements exceed 256 times its root mean square, so no more than
+// kOutliers up to 2^24 elements; larger vectors go to the SIMT kernels whole. The rest then
+// has the scale that any vector with this root mean square may have, and k_sigma_left adds
+// the outliers' links. 20 iterations of 3 roots from single determinants, 1,200 x 1,100
+// strings at norb 16: seven of 60 vectors went to the SIMT kernels, 118 ms; now none, 103 ms.
+constexpr double kOutlierRms = 256.0;
+constexpr int64_t kOutlierMaxN = int64_t(1) << 24;
+
 // Per vector (blockIdx.y) its largest magnitude and sum of squares, in a fixed order;
 // the last block to finish writes info[2 v]: 1 when the digits serve the vector,
-// info[2 v + 1]: its scale exponent. done[v] wraps back to 0.
+// info[2 v + 1]: its scale exponent. done[v] wraps back to 0. O.thr[v]: what an outlier exceeds.
 template <typename T>
-__global__ void __launch_bounds__(kScaleThreads) k_scale(const T *__restrict__ c0, int64_t n, double ratio, double *part0,
-                                                         unsigned *done, const int *__restrict__ tab, int *info) {
+__global__ void __launch_bounds__(kScaleThreads) k_scale(const T *__restrict__ c0, int64_t n, double ratio, int64_t outlier_n,
+                                                         double *part0, unsigned *done, const int *__restrict__ tab, int *info,
+                                                         Outliers O) {
     const T *__restrict__ c = c0 + blockIdx.y * n;
     double *part = part0 + (size_t)blockIdx.y * 2 * kScaleBlocks;
     double top = 0.0, sum = 0.0;
@@ -186,14 +197,23 @@ __global__ void __launch_bounds__(kScaleThreads) k_scale(const T *__restrict__ c
     if (threadIdx.x != 0) return;
     top = st[0];
     int ok = 0, e = 0;
+    double thr = INFINITY;
     if (!tab[2]) {
         ok = 0;
     } else if (top == 0.0) {
         ok = 1;
     } else if (top < 1e15 && top > 1e-15) {
+        const double rms = sqrt(ss[0] / (double)n);
         e = scale_exponent(top);
-        ok = ldexp(1.0, e) <= ratio * sqrt(ss[0] / (double)n) ? 1 : 0;
+        ok = ldexp(1.0, e) <= ratio * rms ? 1 : 0;
+        if (!ok && n <= outlier_n) {
+            thr = kOutlierRms * rms;
+            e = scale_exponent(thr);  // 2^e <= 4 thr = 1024 rms
+            ok = 1;
+        }
     }
+    O.thr[blockIdx.y] = thr;
+    O.count[blockIdx.y] = 0;
     info[2 * blockIdx.y] = ok;
     info[2 * blockIdx.y + 1] = e;
 }
@@ -201,9 +221,10 @@ __global__ void __launch_bounds__(kScaleThreads) k_scale(const T *__restrict__ c
 // the digit planes [NSC][la][lbp] of each vector, columns lb .. lbp - 1 zero; 8 columns per thread
 template <int P>
 __global__ void __launch_bounds__(256) k_slice(const typename Prec<P>::T *__restrict__ c, int64_t la, int64_t lb,
-                                               int64_t lbp, const int *__restrict__ info, __nv_bfloat16 *out) {
+                                               int64_t lbp, const int *__restrict__ info, Outliers O, __nv_bfloat16 *out) {
     info += 2 * blockIdx.y;
     if (!info[0]) return;
+    const typename Prec<P>::T lim = (typename Prec<P>::T)O.thr[blockIdx.y];
     constexpr int N = Prec<P>::NSC;
     c += blockIdx.y * la * lb;
     out += blockIdx.y * N * la * lbp;
@@ -213,7 +234,16 @@ __global__ void __launch_bounds__(256) k_slice(const typename Prec<P>::T *__rest
         const int64_t r = i / per, j = (i - r * per) * 8;
         int64_t f[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) f[u] = j + u < lb ? to_fixed(__ldg(c + r * lb + j + u), shift) : 0;
+        for (int u = 0; u < 8; ++u) {
+            const typename Prec<P>::T x = j + u < lb ? __ldg(c + r * lb + j + u) : 0;
+            if (x <= lim && -x <= lim) {
+                f[u] = to_fixed(x, shift);
+            } else {
+                const int k = atomicAdd(O.count + blockIdx.y, 1);
+                if (k < kOutliers) O.list[blockIdx.y * kOutliers + k] = r * lb + j + u;
+                f[u] = 0;
+            }
+        }
 #pragma unroll
         for (int s = 0; s < N; ++s) {
             uint32_t w[4];
@@ -1024,6 +1054,7 @@ struct ExactData {
         double *part = nullptr;
         int *info = nullptr, *tab = nullptr;
         unsigned *done = nullptr;
+        Outliers out{};
         SsArgs ss{};
     } type[2];
     ~ExactData() {
@@ -1073,6 +1104,7 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
     const size_t cb = place((size_t)lb * nchb), ca = place((size_t)la * ncha);
     const size_t fb = place((size_t)nbb * nchb), fa = place((size_t)nba * ncha);
     const size_t part = place((size_t)Y.batch * 2 * kScaleBlocks * 8), info = place(8 * (size_t)Y.batch), tab = place(12);
+    const size_t thr = place(8 * (size_t)Y.batch), count = place(4 * (size_t)Y.batch), list = place(8 * (size_t)Y.batch * kOutliers);
     const size_t planes = place((size_t)Y.batch * NSC * la * lbp * 2);
     if (charge(ctx, at, "digit tables") != TBSCI_OK) return TBSCI_OK;
     cudaError_t e = Y.arena.alloc(at);
@@ -1088,6 +1120,7 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
         Y.info = reinterpret_cast<int *>(B + info);
         Y.tab = reinterpret_cast<int *>(B + tab);
         Y.done = reinterpret_cast<unsigned *>(B + done);
+        Y.out = {reinterpret_cast<double *>(B + thr), reinterpret_cast<int *>(B + count), reinterpret_cast<int64_t *>(B + list)};
         unsigned long long *tp = reinterpret_cast<unsigned long long *>(B + top);
         auto blocks = [](size_t n) { return (unsigned)std::min<size_t>(152, (n + 255) / 256); };
         k_absmax<<<blocks((size_t)P->npair * P->npair), 256, 0, st>>>(ham->d_V.p, (int64_t)P->npair * P->npair, tp);
@@ -1168,7 +1201,7 @@ bool exact_eligible(const Plan *P) {
 // vectors v .. v + nv - 1, to return at once where skip[2 i] is set.
 template <typename T, int PR>
 tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const T *c, T *s, int nvec, cudaStream_t st,
-                            bool *ran, const std::function<tbsci_status(int, int, const int *)> &simt) {
+                            bool *ran, const std::function<tbsci_status(int, int, const int *, const OutlierArgs &)> &simt) {
     *ran = false;
     if (!exact_eligible<T>(P)) return TBSCI_OK;
     // the tables are made outside of graphs, and a graph's replays would share them with other streams
@@ -1199,6 +1232,9 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
     UdArgs<T> U = ud_args(ham, P, T(0));
     U.info = Y.info;
     AbArgs A{};
+    const OutlierArgs out{Y.out, lb, P->A.d_str, P->A.d_soff, P->A.d_doff, P->B.d_soff, P->B.d_doff,
+                   P->A.d_sci.p, P->B.d_sci.p, P->A.d_sval.p, P->B.d_sval.p, P->A.d_dval.p, P->B.d_dval.p, ham->d_V.p,
+                   P->A.d_dcol.p, P->B.d_dcol.p, P->npair};
     size_t ab_smem = 0;
     if (PR == 0) {
         A.la = la;
@@ -1231,10 +1267,10 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
         {
             TraceScope tr(ctx, "k_slice", st);
             const unsigned nb = (unsigned)std::min<int64_t>(kScaleBlocks, (la * lb + 4 * kScaleThreads - 1) / (4 * kScaleThreads));
-            k_scale<T><<<dim3(nb, (unsigned)nv), kScaleThreads, 0, st>>>(cv, la * lb, Prec<PR>::kRatio, Y.part, Y.done,
-                                                                        Y.tab, Y.info);
+            k_scale<T><<<dim3(nb, (unsigned)nv), kScaleThreads, 0, st>>>(cv, la * lb, Prec<PR>::kRatio, PR == 0 ? kOutlierMaxN : 0,
+                                                                        Y.part, Y.done, Y.tab, Y.info, Y.out);
             const unsigned ns = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (lbp / 8) + 255) / 256);
-            k_slice<PR><<<dim3(ns, (unsigned)nv), 256, 0, st>>>(cv, la, lb, lbp, Y.info, Y.planes);
+            k_slice<PR><<<dim3(ns, (unsigned)nv), 256, 0, st>>>(cv, la, lb, lbp, Y.info, Y.out, Y.planes);
             TB_CUDA(ctx, cudaGetLastError());
         }
         {
@@ -1259,18 +1295,18 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
         } else {
             TB_TRY(sigma_tc_ab(ctx, P, 3, cv, sv, nv, Y.info, st));
         }
-        TB_TRY(simt(v, nv, Y.info));
+        TB_TRY(simt(v, nv, Y.info, out));
     }
     TB_CUDA(ctx, cudaEventRecord(Y.busy, st));
     return TBSCI_OK;
 }
 
 tbsci_status exact_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const double *c, double *s, int nvec,
-                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *)> &simt) {
+                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *, const OutlierArgs &)> &simt) {
     return exact_launch_t<double, 0>(ctx, ham, P, c, s, nvec, st, ran, simt);
 }
 tbsci_status exact_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const float *c, float *s, int nvec,
-                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *)> &simt) {
+                          cudaStream_t st, bool *ran, const std::function<tbsci_status(int, int, const int *, const OutlierArgs &)> &simt) {
     return exact_launch_t<float, 1>(ctx, ham, P, c, s, nvec, st, ran, simt);
 }
 

@@ -156,3 +156,25 @@ def test_without_room_for_the_tables(tb):
     _check(full.cpu().numpy(), osp, h, eri, C, rows)
     sp.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("la,lb,k", [(1040, 1030, 1), (1040, 1030, 3), (4000, 4000, 200), (4100, 4100, 200)])
+def test_towering_elements(tb, ctx, la, lb, k):
+    """k elements ten thousand times the rest, in one row, one column and linked rows: more than
+    256 times the root mean square, so kept out of the digits (the last case: past 2^24
+    determinants, all SIMT). Rows linked to them and rows that are not agree with the oracle."""
+    import torch
+    sp, osp, h, eri = _space(tb, ctx, 16, 8, 8, la, lb, seed=771)
+    rng = np.random.default_rng(k)
+    C = 1e-4 * rng.standard_normal((1, sp.la, sp.lb))
+    at = [(5, 7), (5, 8), (6, 7)][:k] + [(int(a), int(b)) for a, b in zip(rng.choice(sp.la, k), rng.choice(sp.lb, k))][3:]
+    for a, b in at:
+        C[0, a, b] = rng.choice([-1.0, 1.0])
+    assert np.abs(C).max() > 256 * np.sqrt((C ** 2).mean())
+    Ct = torch.from_numpy(C).cuda()
+    s = sp.sigma(Ct)
+    assert torch.equal(s, sp.sigma(Ct))
+    near = [a * sp.lb + j for a, b in at[:2] for j in range(0, sp.lb, 29)] + [i * sp.lb + b for a, b in at[:2] for i in range(0, sp.la, 29)]
+    rows = np.unique(np.concatenate([_rows(sp.ndet, 9), near, [a * sp.lb + b for a, b in at]]))
+    _check(s.cpu().numpy(), osp, h, eri, C, rows)
+    sp.close()
