@@ -137,6 +137,16 @@ def _kernel_work(name, c, nvec, dtype):
         noff = c["norb"] * (c["norb"] - 1) // 2
         return (2.0 * noff * c["n1a"] * lb * nvec, "tensor",
                 "2 flops per (alpha single, off-diagonal pair kl, beta column) of the dense contraction per vector")
+    if name == "k_sigma_ab_ex":
+        noff = c["norb"] * (c["norb"] - 1) // 2
+        return (35 * 2.0 * noff * c["n1a"] * lb * nvec, "tensor",
+                "2 flops per digit product (35), alpha single, off-diagonal pair kl and beta column per vector")
+    if name == "k_same_spin_ex":
+        return ((35 if dtype == "f64" else 10) * 2.0 * la * lb * (la + lb) * nvec, "tensor",
+                "2 flops per digit product (35 in FP64, 10 in FP32) of the dense c Hb^T + Ha c per vector, chunks without a "
+                "link counted though skipped")
+    if name == "k_udiag":
+        return 2.0 * (nd + c["n1a"] * lb) * nvec, "fp", "2 flops per determinant and alpha single's column per vector"
     if name == "k_transpose":
         return None, "bytes", "read + write of one vector"
     if name == "k_combine":

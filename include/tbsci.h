@@ -124,7 +124,8 @@ const char *tbsci_status_string(tbsci_status st);
  * row kernel, the split path's row kernel, double-class products, transposes
  * and combine, the tensor-core kernel and its SIMT pass, the dense same-spin
  * products of rest mode 5 (one entry for the cuBLAS calls of a vector, plus
- * the split and unpad passes), the pruned kernel).
+ * the split and unpad passes), the small-space kernel (as k_sigma), the passes of
+ * the exact tensor-core path, the pruned kernels).
  * While tracing is on, every such launch made through this context is
  * bracketed by two CUDA events recorded on its own stream (launches made while
  * that stream is being captured into a graph are not traced). The trace keeps
@@ -457,8 +458,9 @@ tbsci_status tbsci_coefficient_histogram(tbsci_ctx *ctx, const double *x, int64_
  * a request that arrives while others run joins as soon as a slot and memory
  * are free, its sigma work goes into the same batched launches and its vector
  * work overlaps on its own stream. Each solve is the Davidson of tbsci_davidson,
- * so a result does not depend on what else was running (batched sigma launches
- * compute every job exactly as a launch of its own would). */
+ * so a result does not depend on what else was running (in a batched sigma launch
+ * no job sees another; it agrees with tbsci_sigma, which may take another kernel,
+ * to rounding). */
 typedef struct tbsci_server tbsci_server;
 
 typedef struct tbsci_server_opts {

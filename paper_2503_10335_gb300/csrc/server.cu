@@ -12,8 +12,8 @@
 //      host logic of whichever solves have finished a phase runs while the
 //      device keeps working on the others (each solve has its own stream);
 //   3. gathers the sigma work that solves are waiting for and issues the small
-//      jobs as one batched launch per precision (every job computed exactly as a
-//      launch of its own would: CTAs never mix jobs), ordered after each solve's
+//      jobs as one batched launch per precision (a job's result does not depend on
+//      the others: CTAs never mix jobs), ordered after each solve's
 //      stream and before the solve continues; jobs above 2^20 determinant-vectors
 //      get launches of their own on their solve's stream, so the small batch runs
 //      beside them instead of waiting for them;

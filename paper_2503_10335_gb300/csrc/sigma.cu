@@ -22,6 +22,10 @@
 // is staged in shared memory for the in-row beta gathers, the accumulator row
 // lives in shared memory, threads own beta columns in an order sorted by
 // single-link count so a warp's lanes have nearly equal trip counts.
+//
+// Before this kernel (k_sigma) come two others where they apply (launch_full):
+// k_sigma_small for vectors that fit in shared memory, and the exact products on the
+// tensor cores of sigma_exact.cu, whose remaining vectors k_sigma_left serves.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -506,7 +510,7 @@ __global__ void __launch_bounds__(kThreads) k_sigma_rest_pair(SigArgs<float> A) 
 // the next row of the concatenated job list from a device counter until the
 // list is exhausted. Row b is row b - cta_off[j] of job j, the last j with
 // cta_off[j] <= b; jobs are ordered heaviest rows first, each job's rows in its
-// own work order. Jobs are independent, so results equal per-job launches.
+// own work order. Jobs are independent, so results equal those of k_sigma on one job.
 template <typename T, int kThreads>
 __global__ void __launch_bounds__(kThreads) k_sigma_batch(const SigArgs<T> *__restrict__ jobs,
                                                           const int64_t *__restrict__ cta_off, int njobs,
