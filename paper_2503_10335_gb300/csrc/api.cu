@@ -562,7 +562,7 @@ tbsci_status tbsci_diagonal(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *
     TB_TRY(plan_get(ctx, ham, a, b, &p));
     if (p->A.l * p->B.l == 0) return TBSCI_OK;
     if (!diag) return fail(ctx, TBSCI_EINVAL, "null diag pointer");
-    return diagonal_launch(ctx, ham, p, diag, (cudaStream_t)stream);
+    return diagonal_launch(ctx, ham, p, diag, (cudaStream_t)stream, true);
 }
 
 tbsci_status tbsci_sigma_counts_get(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *a, const tbsci_tables *b,

@@ -587,7 +587,7 @@ struct DavEngine {
         rnorm.assign(nroots, INFINITY);
         e32.assign(nroots, 0.0);
         if (pr) TB_TRY(pruned_diagonal_launch(ctx, ham, plan, pr, diag.p, st));
-        else TB_TRY(diagonal_launch(ctx, ham, plan, diag.p, st));
+        else TB_TRY(diagonal_launch(ctx, ham, plan, diag.p, st, false));
         // guess: unit vectors at the nroots lowest (H_KK, K), each mixed with the next
         // four lowest determinants so that every symmetry sector is present
         const int extra = (int)std::min<int64_t>(4, N - nroots);

@@ -455,7 +455,7 @@ tbsci_status sigma_tc_prepare(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int
 tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, int nv, const int *info, cudaStream_t st);
 int sigma_tc_batch(const Plan *P);
 tbsci_status diagonal_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan, double *diag,
-                             cudaStream_t st);
+                             cudaStream_t st, bool tables);
 
 // davidson.cu: resumable Davidson engine (one solve) and its drivers
 struct DavEngine;

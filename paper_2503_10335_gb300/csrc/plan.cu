@@ -21,28 +21,25 @@ __device__ __forceinline__ double eri_at(const double *__restrict__ eri, int n, 
     return __ldg(eri + (((size_t)i * n + j) * n + k) * n + l);
 }
 
-// One warp per string, lanes over its orbitals i (a thread per string left most of the GPU
-// idle: 5,000 strings of 12 electrons took 51 us, now 15 us).
+// One thread per string: the order of this sum decides which of two determinants with
+// mathematically equal diagonals (spin-flipped pairs) a Davidson guess starts from, so it
+// stays as it is (a warp per string took 15 us instead of 51 for 5,000 strings).
 __global__ void k_string_energy(const uint64_t *__restrict__ str, int64_t l, int n, const double *__restrict__ h,
                                 const double *__restrict__ eri, double *E, float *Ef) {
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (w >= l) return;
-    const uint64_t s = str[w];
+    uint64_t s = str[w];
     double e = 0.0;
-    for (int i = lane; i < n; i += 32) {
-        if (!((s >> i) & 1)) continue;
+    for (uint64_t a = s; a; a &= a - 1) {
+        int i = __ffsll((long long)a) - 1;
         e += h[i * n + i];
         for (uint64_t b = s; b; b &= b - 1) {
-            const int j = __ffsll((long long)b) - 1;
+            int j = __ffsll((long long)b) - 1;
             e += 0.5 * (eri_at(eri, n, i, i, j, j) - eri_at(eri, n, i, j, j, i));
         }
     }
-    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-    if (lane == 0) {
-        E[w] = e;
-        Ef[w] = (float)e;
-    }
+    E[w] = e;
+    Ef[w] = (float)e;
 }
 
 // one warp per source row; lanes over the row's single links
@@ -211,7 +208,7 @@ tbsci_status build_spin(tbsci_ctx *ctx, const tbsci_ham *ham, const tbsci_tables
     const int n = ham->norb;
     const double *eri = ham->d_eri.p;
     if (sp.l == 0) return TBSCI_OK;
-    k_string_energy<<<(unsigned)((sp.l * 32 + 127) / 128), 128, 0, st>>>(sp.d_str, sp.l, n, ham->d_h.p, eri, sp.d_E.p, sp.d_Ef.p);
+    k_string_energy<<<(unsigned)((sp.l + 127) / 128), 128, 0, st>>>(sp.d_str, sp.l, n, ham->d_h.p, eri, sp.d_E.p, sp.d_Ef.p);
     if (t->nsingle > 0)
         k_single_values<<<(unsigned)((sp.l * 32 + 255) / 256), 256, 0, st>>>(
             sp.d_str, sp.l, n, t->d_off1.p, t->d_ent1.p, ham->d_h.p, eri, sp.d_sci.p, sp.d_sval.p, sp.d_svalf.p);

@@ -1423,11 +1423,13 @@ tbsci_status sigma_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan
     return fail(ctx, TBSCI_EINVAL, "unknown dtype");
 }
 
-tbsci_status diagonal_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, double *diag, cudaStream_t st) {
+// tables: any order of the sum will do (else k_diagonal's, on which the choice among
+// determinants with mathematically equal diagonals depends: the Davidson guess)
+tbsci_status diagonal_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, double *diag, cudaStream_t st, bool tables) {
     const int64_t N = P->A.l * P->B.l;
     if (N == 0) return TBSCI_OK;
     const int64_t la = P->A.l, lb = P->B.l, ct = (lb + 31) / 32;
-    if (la >= kDiagRows && lb >= 16) {  // narrower rows leave most of a warp's lanes without a column
+    if (tables && la >= kDiagRows && lb >= 16) {  // narrower rows leave most of a warp's lanes without a column
         const size_t smem = (size_t)((P->norb + 5) / 6) * 64 * 32 * sizeof(double);  // 176 KB at 64 orbitals
         // about eight blocks per SM, 128 to 1024 rows each
         const int64_t rows = std::max<int64_t>(std::min<int64_t>(std::max<int64_t>(la * ct / (152 * 8), 128), 1024), (la + 65534) / 65535);
