@@ -327,8 +327,10 @@ __host__ __device__ size_t small_smem_bytes(int npair, int64_t la, int64_t lb, i
 // (permb2 order) take a CTA, and G = 16 / SL warps per slice share the terms: alpha singles
 // and doubles by their place, the links of Ja = Ia by theirs. The warps' sums are added in
 // warp order. What is left is the FP64 pipe (norb 8 full space: 4,900 x 397 multiply-adds,
-// 3 us of 152 SMs), so a slice per CTA is taken until the grid covers the GPU twice.
-// Norb 8 full space, one vector, FP64: 22 us; 46 on k_sigma, and 16 orbitals with 60 x 60
+// 3 us of 152 SMs), so a slice per CTA is taken until the grid of one vector covers the GPU
+// twice. SL decides in which order a column is summed, so it depends on the space alone:
+// a vector's sigma is the same whichever vectors share its launch.
+// Norb 8 full space, one vector, FP64: 15 us; 45 on k_sigma, and 16 orbitals with 60 x 60
 // strings, two vectors, 53; 405.
 template <typename T, int SL>
 __global__ void __launch_bounds__(512) k_sigma_small(SigArgs<T> A, int nsmax) {
@@ -1351,7 +1353,7 @@ tbsci_status launch_small(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, c
     SigArgs<T> A = make_args<T>(ham, P);
     A.C = c;
     A.S = s;
-    const int64_t nsl = (lb + 31) / 32, work = la * nsl * nvec;
+    const int64_t nsl = (lb + 31) / 32, work = la * nsl;
     const int sl = work <= 2 * ctx->num_sms ? 1 : work <= 4 * ctx->num_sms ? 2 : 4;
     auto k = sl == 1 ? k_sigma_small<T, 1> : sl == 2 ? k_sigma_small<T, 2> : k_sigma_small<T, 4>;
     TB_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));

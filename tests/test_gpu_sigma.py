@@ -127,6 +127,25 @@ def test_sigma_host_pipelined_groups(tb, ctx):
     sp.close()
 
 
+@pytest.mark.parametrize("n,na,nb,acnt,bcnt,dtype", [(8, 4, 4, None, None, "f64"), (8, 4, 4, None, None, "f32"),
+                                                      (8, 4, 3, 52, 33, "f64"), (12, 6, 6, 90, 97, "f64"),
+                                                      (12, 6, 6, 102, 97, "f32"), (10, 5, 5, 150, 150, "f64")])
+def test_vector_is_the_same_in_any_company(tb, ctx, n, na, nb, acnt, bcnt, dtype):
+    """A space whose vector fits in shared memory, at 1, 2, 4 column slices per CTA: a vector's
+    sigma has the same bits alone, among five, and (FP64) through the host call's groups."""
+    import torch
+    sp, _, _, _ = _case(tb, ctx, n, na, nb, acnt, bcnt, seed=87)
+    C = np.random.default_rng(88).standard_normal((5, sp.la, sp.lb))
+    Ct = torch.from_numpy(C).cuda().to(torch.float64 if dtype == "f64" else torch.float32)
+    together = sp.sigma(Ct)
+    for k in (1, 2, 3):
+        for v in range(0, 6 - k):
+            assert torch.equal(sp.sigma(Ct[v:v + k].contiguous()), together[v:v + k]), (v, k)
+    if dtype == "f64":
+        assert np.array_equal(sp.sigma_host(C), together.cpu().numpy())
+    sp.close()
+
+
 def test_fci8_sigma(tb, ctx):
     import torch
     wl = WORKLOADS["fci8"]
