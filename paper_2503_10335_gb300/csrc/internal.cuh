@@ -287,6 +287,7 @@ struct Plan {
     DevBuf<uint4> d_tl_pos;
     DevBuf<int2> d_tl_piece;
     DevBuf<int> d_tl_rounds;
+    DevBuf<uint2> d_ab_v, d_ab_w;  // BF16 planes of the integrals and of W_Ia
     int tl_nslot = 0, tl_npiece = 0, tl_kpmax = 0;
     std::shared_ptr<AbPlanes> ab[2];  // one BF16 plane per operand, three
     // autotuned launch shape per sigma type (index = tbsci_dtype F64 / F32): threads per CTA, vectors per CTA
@@ -450,9 +451,10 @@ tbsci_status udiag_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, c
 // sigma_tc.cu: the alpha-beta classes on the tensor cores with np = 1 or 3 BF16 planes
 // per operand, FP32 accumulation, added into s
 void tile_links_size(tbsci_ctx *ctx, Plan *P);  // adds the plan's buffers to its arena
-tbsci_status tile_links_build(tbsci_ctx *ctx, Plan *P, cudaStream_t st);
-tbsci_status sigma_tc_prepare(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int np, cudaStream_t st, bool *ready);
-tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, int nv, const int *info, cudaStream_t st);
+tbsci_status tile_links_build(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, cudaStream_t st);
+bool sigma_tc_serves(const tbsci_ctx *ctx, const Plan *P, int np);
+tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, int nv,
+                         const int *info, cudaStream_t st);
 int sigma_tc_batch(const Plan *P);
 tbsci_status diagonal_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan, double *diag,
                              cudaStream_t st, bool tables);

@@ -250,7 +250,7 @@ size_t plan_device_bytes(const Plan &P) {
          P.d_s2_valf.bytes() + P.d_d2_valf.bytes() + P.d_d2_col.bytes();
     b += P.d_U1.bytes() + P.d_U2.bytes() + P.d_Eb2.bytes() + P.d_U1f.bytes() + P.d_U2f.bytes() + P.d_Eb2f.bytes();
     b += P.d_rowsa.bytes() + P.d_pairs.bytes() + P.d_lbp.bytes() + P.d_offpair.bytes() + P.d_tc_err.bytes();
-    b += P.d_tl_pos.bytes() + P.d_tl_piece.bytes() + P.d_tl_rounds.bytes();
+    b += P.d_tl_pos.bytes() + P.d_tl_piece.bytes() + P.d_tl_rounds.bytes() + P.d_ab_v.bytes() + P.d_ab_w.bytes();
     return b;
 }
 
@@ -381,7 +381,7 @@ tbsci_status plan_get(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *a, con
         TB_CUDA(ctx, cudaMemsetAsync(plan->d_tc_err.p, 0, sizeof(int), st));
         k_link_by_pair<<<(unsigned)((lb + 127) / 128), 128, 0, st>>>(lb, b->d_off1.p, b->d_ent1.p, plan->npoff, plan->d_lbp.p);
         TB_CUDA(ctx, cudaGetLastError());
-        TB_TRY(tile_links_build(ctx, plan.get(), st));
+        TB_TRY(tile_links_build(ctx, ham, plan.get(), st));
     }
     // work counts: non-zeros of H by class (Sec. II.C, Table I)
     tbsci_sigma_counts &c = plan->counts;

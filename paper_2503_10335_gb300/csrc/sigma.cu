@@ -1408,9 +1408,7 @@ tbsci_status sigma_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan
         const float *cf = static_cast<const float *>(c);
         float *sf = static_cast<float *>(s);
         const int np = dt == TBSCI_F32_TC_BF16 ? 1 : 3;
-        bool ready = false;
-        TB_TRY(sigma_tc_prepare(ctx, ham, const_cast<Plan *>(plan), np, st, &ready));
-        if (!ready)  // no tensor-core tile for this norb, or no room for its planes: FP32 on the SIMT path
+        if (!sigma_tc_serves(ctx, plan, np))  // no tensor-core tile for this norb, or rows too long: FP32 on the SIMT path
             return launch_typed<float>(ctx, ham, plan, cf, sf, nvec, st);
         TB_TRY(sigma_launch_rest(ctx, ham, plan, cf, sf, nvec, st, -1, 0, nullptr, 0, np == 1));
         const size_t n = (size_t)plan->A.l * plan->B.l;

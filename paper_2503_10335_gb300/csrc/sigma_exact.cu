@@ -1086,7 +1086,7 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
     using Sh = SsShape<PR>;
     const int64_t la = P->A.l, lb = P->B.l, lap = pad64(la), lbp = pad64(lb);
     constexpr int NSA = Prec<PR>::NSA, NSC = Prec<PR>::NSC;
-    if ((PR == 0 && ab_stage_bytes(ctx, P) == 0) || !encode_tiled()) return TBSCI_OK;
+    if ((PR == 0 ? ab_stage_bytes(ctx, P) == 0 : !sigma_tc_serves(ctx, P, 3)) || !encode_tiled()) return TBSCI_OK;
     const int ncha = (int)((la + 31) / 32), nchb = (int)((lb + 31) / 32);
     const int64_t nba = (la + 127) / 128, nbb = (lb + Sh::NT - 1) / Sh::NT;
     Y.batch = sigma_tc_batch(P);
@@ -1220,11 +1220,6 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
     typename ExactData::Type &Y = X->type[PR];
     if (!Y.tried) TB_TRY((build_type<PR>(ctx, ham, P, X, st)));
     if (!Y.ready) return TBSCI_OK;
-    if (PR == 1) {
-        bool ready = false;
-        TB_TRY(sigma_tc_prepare(ctx, ham, P, 3, st, &ready));
-        if (!ready) return TBSCI_OK;
-    }
     using Sh = SsShape<PR>;
     const int64_t la = P->A.l, lb = P->B.l, lbp = pad64(lb);
     auto kss = k_same_spin_ex<PR>;

@@ -20,11 +20,15 @@
 //
 // What bounds it: not the products (512 to 960 tensor-core cycles per 64 columns) but
 // the way of G into the sigma row. So it keeps the products' operands out of the
-// warps' hands (A lies in TMEM for the whole row; c arrives as BF16 planes cut once
-// per vector, a 128-byte segment per coupled row) and gives the accumulators a plan of
-// the links made once per space: every link of a 64-column tile has a slot, the slots
-// of a target column are consecutive, and a thread sums up to four of them. No atomics:
-// results are run-to-run identical.
+// draining warps' hands (A lies in TMEM for the whole row; three warps stage the coupled
+// c rows, a tile each) and gives the accumulators a plan of the links made once per space:
+// every link of a 64-column tile has a slot, the slots of a target column are consecutive,
+// and a thread sums up to four of them. No atomics: results are run-to-run identical.
+// c arrives as BF16 planes cut once per vector into memory of the space (a 128-byte
+// segment per coupled row). In a graph, whose replays would share that memory with other
+// streams, and where there is no room for it, the staging warps cut c themselves, to the
+// same bits: 100 ms instead of 67 on the full norb-16 space with three planes, 54 instead
+// of 42 with one.
 // Norb 16, full space (165.6M determinants), one vector: 35.7 ms with three planes, 30.4
 // ms with one; 85 and 53 ms with operands staged element by element and sums by
 // shared-memory atomics.
@@ -175,8 +179,48 @@ __global__ void __launch_bounds__(256) k_planes(const float *__restrict__ c, int
     }
 }
 
-// planes of the integral columns, [pair][128 off-diagonal pairs] x 4 BF16, or of W_Ia, [la][128] x 4
-template <int NP>
+// Cuts the columns 64 t .. 64 t + 63 of the rows sJa[0 .. Kp - 1] of c into planes in stage
+// `dst0` by one warp, two columns per lane: MN-major operand planes of Kp rows of 128 bytes,
+// 128-byte swizzle. PAIR: rows of c start on 8 bytes (even length), else scalar loads. Eight
+// rows of loads are in flight (a warp has three tile times for its tile).
+template <int NP, bool PAIR>
+__device__ __forceinline__ void stage_tile(const float *__restrict__ C, int64_t lb, const int *sJa, int Kp, int t, uint32_t dst0) {
+    constexpr int kRows = 8;  // Kp is a multiple of 16
+    const int lane = threadIdx.x & 31;
+    const int64_t j = (int64_t)t * kAbTile + 2 * lane;
+    const bool in0 = j < lb, in1 = j + 1 < lb;
+    const float *src0 = C + j;
+    for (int k0 = 0; k0 < Kp; k0 += kRows) {
+        float x[kRows], y[kRows];
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) {
+            const float *src = src0 + (size_t)sJa[k0 + u] * lb;
+            if (PAIR) {
+                const float2 v = in0 ? __ldg(reinterpret_cast<const float2 *>(src)) : make_float2(0.f, 0.f);
+                x[u] = v.x;
+                y[u] = v.y;
+            } else {
+                x[u] = in0 ? __ldg(src) : 0.f;
+                y[u] = in1 ? __ldg(src + 1) : 0.f;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) {
+            const int k = k0 + u;
+            uint32_t hx[NP], hy[NP];
+            bf16_planes<NP>(x[u], hx);
+            bf16_planes<NP>(y[u], hy);
+            const uint32_t dst = dst0 + k * 128 + (((lane >> 2) ^ (k & 7)) << 4) + ((lane & 3) << 2);
+#pragma unroll
+            for (int s = 0; s < NP; ++s)
+                asm volatile("st.shared.b32 [%0], %1;" ::"r"(dst + s * Kp * 128), "r"(hx[s] | (hy[s] << 16)) : "memory");
+        }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+// planes of the integral columns, [pair][128 off-diagonal pairs] x 4 BF16 (the last zero), or of
+// W_Ia, [la][128] x 4; one plane is the first of three
 __global__ void k_ab_planes(const float *__restrict__ V, int npair, int npoff, const int32_t *__restrict__ offpair,
                             const uint64_t *__restrict__ str, int64_t rows, uint2 *out) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -195,16 +239,17 @@ __global__ void k_ab_planes(const float *__restrict__ V, int npair, int npoff, c
             x = V[(size_t)row * npair + col];
         }
     }
-    uint32_t h[NP];
-    bf16_planes<NP>(x, h);
-    out[i] = make_uint2(h[0] | (NP > 1 ? h[NP > 1 ? 1 : 0] << 16 : 0u), NP > 2 ? h[NP > 2 ? 2 : 0] : 0u);
+    uint32_t h[3];
+    bf16_planes<3>(x, h);
+    out[i] = make_uint2(h[0] | (h[1] << 16), h[2]);
 }
 
 // ------------------------------------------------------------------ the kernel
 
 struct FpArgs {
     int64_t la, lb, lbp;
-    const __nv_bfloat16 *Cs;
+    const float *C;
+    const __nv_bfloat16 *Cs;  // planes of c (PLANES)
     float *S;
     const int *info;       // run only where info[2 v] is set (NULL: always)
     const uint2 *Vd, *Wd;  // [pair][128], [la][128] x 4 BF16
@@ -215,12 +260,13 @@ struct FpArgs {
                            // positive links << 16 | negative links << 20 | further pieces << 24}
     const int *rounds;     // [tile] pieces / kAbDrain, rounded up
     int npiece, nslot;
-    int stage_bytes;       // shared memory for the gathered c rows
+    int stage_bytes;       // shared memory for the staged c rows
+    int pair;              // rows of c start on 8 bytes
     const int32_t *rowsa;
     int *err;
 };
 
-template <int NP>
+template <int NP, bool PLANES>
 __global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab_tc(const FpArgs A) {
     if (A.info && !A.info[2 * blockIdx.y]) return;  // one vector per blockIdx.y
     extern __shared__ unsigned char smem_dyn[];
@@ -229,7 +275,7 @@ __global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab_tc(const FpArgs A) {
     __shared__ int sAbort;
     __shared__ int sJa[kAbMaxK], sPq[kAbMaxK];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t lb = A.lb, lbp = A.lbp, Ia = A.rowsa[blockIdx.x], t0 = A.a_soff[Ia];
+    const int64_t lb = A.lb, Ia = A.rowsa[blockIdx.x], t0 = A.a_soff[Ia];
     const int K = 1 + (int)(A.a_soff[Ia + 1] - t0), Kp = (K + 15) / 16 * 16;
     const uint32_t stage_sz = (uint32_t)NP * Kp * kAbTile * 2;
     const int nst = min(4, A.stage_bytes / (int)stage_sz);
@@ -360,13 +406,17 @@ __global__ void __launch_bounds__(kAbThreads, 1) k_sigma_ab_tc(const FpArgs A) {
             for (int it = 0; it < 4096; ++it) __nanosleep(100);
         __syncwarp();
     } else if (warp >= 16) {
-        // a warp gathers a whole tile; three tiles are on their way (not more than there are
+        // a warp stages a whole tile; three tiles are on their way (not more than there are
         // stages: a wait must not run a phase ahead of its barrier)
         const int ng = min(3, nst), g = warp - 16;
         for (int t = g; t < ntiles && g < ng; t += ng) {
             const int st = t % nst;
             if (t >= nst && !mb_wait(bempty + 8 * st, (t / nst - 1) & 1, ab)) break;
-            gather_tile<NP>(A.Cs + blockIdx.y * NP * A.la * lbp, (size_t)A.la * lbp, lbp, sJa, Kp, t, sB + st * stage_sz);
+            const float *C = A.C + blockIdx.y * A.la * lb;
+            if (PLANES)
+                gather_tile<NP>(A.Cs + blockIdx.y * NP * A.la * A.lbp, (size_t)A.la * A.lbp, A.lbp, sJa, Kp, t, sB + st * stage_sz);
+            else if (A.pair) stage_tile<NP, true>(C, lb, sJa, Kp, t, sB + st * stage_sz);
+            else stage_tile<NP, false>(C, lb, sJa, Kp, t, sB + st * stage_sz);
             mb_arrive(bfull + 8 * st);
         }
     } else {
@@ -457,13 +507,13 @@ int fp_stage_bytes(const tbsci_ctx *ctx, const Plan *P, int np) {
 
 }  // namespace
 
-// Vectors per launch: small spaces share the launches with up to eight (planes of at
-// most 2^24 determinants are kept).
+// Vectors per launch: small spaces share the launches with up to eight (up to 2^24
+// determinants together).
 int sigma_tc_batch(const Plan *P) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(8, (int64_t(1) << 24) / std::max<int64_t>(1, P->A.l * P->B.l)));
 }
 
-// Link plan of a space (norb <= 16), made when the space is prepared; left out
+// Link plan of a space (norb <= 16) and planes of its integrals, made when the space is prepared; left out
 // (tl_kpmax = 0) where the alpha-beta kernels do not apply.
 void tile_links_size(tbsci_ctx *ctx, Plan *P) {
     const int64_t la = P->A.l, lb = P->B.l;
@@ -480,31 +530,35 @@ void tile_links_size(tbsci_ctx *ctx, Plan *P) {
     P->arena.add(P->d_tl_pos, (size_t)nt * 4 * 2 * 128);
     P->arena.add(P->d_tl_piece, (size_t)nt * P->tl_npiece);
     P->arena.add(P->d_tl_rounds, nt);
+    P->arena.add(P->d_ab_v, (size_t)P->npair * 128);
+    P->arena.add(P->d_ab_w, (size_t)la * 128);
     P->tl_kpmax = (kmax + 15) / 16 * 16;
 }
 
-tbsci_status tile_links_build(tbsci_ctx *ctx, Plan *P, cudaStream_t st) {
+tbsci_status tile_links_build(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, cudaStream_t st) {
     if (P->tl_kpmax == 0) return TBSCI_OK;
-    const int64_t lb = P->B.l;
+    const int64_t la = P->A.l, lb = P->B.l;
     const size_t smem = (size_t)lb * 4;
     TB_CUDA(ctx, cudaFuncSetAttribute(k_tile_links, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_tile_links<<<(unsigned)((lb + kAbTile - 1) / kAbTile), kLinkThreads, smem, st>>>(
         P->d_lbp.p, lb, P->npoff, P->tl_npiece, P->tl_nslot, reinterpret_cast<uint16_t *>(P->d_tl_pos.p), P->d_tl_piece.p,
         P->d_tl_rounds.p);
+    k_ab_planes<<<(unsigned)((P->npair * 128 + 255) / 256), 256, 0, st>>>(ham->d_Vf.p, P->npair, P->npoff, P->d_offpair.p, nullptr,
+                                                                         P->npair, P->d_ab_v.p);
+    k_ab_planes<<<(unsigned)((la * 128 + 255) / 256), 256, 0, st>>>(ham->d_Vf.p, P->npair, P->npoff, P->d_offpair.p, P->A.d_str, la,
+                                                                   P->d_ab_w.p);
     TB_CUDA(ctx, cudaGetLastError());
     return TBSCI_OK;
 }
 
-// What the kernel keeps for one space and number of planes, made by the first sigma that
-// needs it. Calls on several streams share the planes of c: each waits for the event
-// that the one before it recorded, and `mu` keeps the launches of one call together.
+// The planes of c of one space and number of planes, made by the first sigma that has
+// room for them. Calls on several streams share them: each waits for the event that the
+// one before it recorded, and `mu` keeps the launches of one call together.
 struct AbPlanes {
     std::mutex mu;
     cudaEvent_t busy = nullptr;
-    bool tried = false, ready = false;
-    DevBuf<unsigned char> arena;
-    uint2 *V = nullptr, *W = nullptr;
-    __nv_bfloat16 *c = nullptr;  // planes of sigma_tc_batch vectors
+    bool tried = false;
+    DevBuf<__nv_bfloat16> c;  // planes of sigma_tc_batch vectors
     ~AbPlanes() {
         if (busy) cudaEventDestroy(busy);
     }
@@ -512,48 +566,35 @@ struct AbPlanes {
 
 namespace {
 
-template <int NP>
-tbsci_status build_planes(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, AbPlanes *X, cudaStream_t st) {
+tbsci_status build_planes(tbsci_ctx *ctx, Plan *P, int np, AbPlanes *X) {
     X->tried = true;
-    const int64_t la = P->A.l, lb = P->B.l;
-    const size_t nv = (size_t)P->npair * 128, nw = (size_t)la * 128, nc = (size_t)sigma_tc_batch(P) * NP * la * pad64(lb);
-    const size_t bytes = (nv + nw) * sizeof(uint2) + nc * 2;
+    const size_t n = (size_t)sigma_tc_batch(P) * np * P->A.l * pad64(P->B.l), bytes = n * sizeof(__nv_bfloat16);
     if (charge(ctx, bytes, "planes of the alpha-beta products") != TBSCI_OK) return TBSCI_OK;
-    cudaError_t e = X->arena.alloc(bytes);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&X->busy, cudaEventDisableTiming);
-    if (e == cudaSuccess) {
-        X->V = reinterpret_cast<uint2 *>(X->arena.p);
-        X->W = X->V + nv;
-        X->c = reinterpret_cast<__nv_bfloat16 *>(X->W + nw);
-        k_ab_planes<NP><<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(ham->d_Vf.p, P->npair, P->npoff, P->d_offpair.p, nullptr,
-                                                                     P->npair, X->V);
-        k_ab_planes<NP><<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(ham->d_Vf.p, P->npair, P->npoff, P->d_offpair.p, P->A.d_str,
-                                                                     la, X->W);
-        e = cudaGetLastError();
-    }
+    cudaError_t e = cudaEventCreateWithFlags(&X->busy, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = X->c.alloc(n);
     if (e != cudaSuccess) {
-        X->arena.release();
         uncharge(ctx, bytes);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? TBSCI_OK : fail(ctx, TBSCI_ECUDA, std::string("alpha-beta planes: ") + cudaGetErrorString(e));
     }
     P->charged += bytes;
-    X->ready = true;
     return TBSCI_OK;
 }
 
 template <int NP>
-tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float *s, int nv, const int *info, cudaStream_t st) {
+tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float *s, int nv, const int *info,
+                    cudaStream_t st) {
     const int64_t la = P->A.l, lb = P->B.l;
     FpArgs A{};
     A.la = la;
     A.lb = lb;
     A.lbp = pad64(lb);
-    A.Cs = X->c;
+    A.C = c;
+    A.Cs = X ? X->c.p : nullptr;
     A.S = s;
     A.info = info;
-    A.Vd = X->V;
-    A.Wd = X->W;
+    A.Vd = P->d_ab_v.p;
+    A.Wd = P->d_ab_w.p;
     A.a_soff = P->A.d_soff;
     A.a_sci = P->A.d_sci.p;
     A.pos = P->d_tl_pos.p;
@@ -562,16 +603,17 @@ tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float 
     A.npiece = P->tl_npiece;
     A.nslot = P->tl_nslot;
     A.stage_bytes = fp_stage_bytes(ctx, P, NP);
+    A.pair = lb % 2 == 0 && (uintptr_t)c % 8 == 0;
     A.rowsa = P->d_rowsa.p;
     A.err = P->d_tc_err.p;
     const size_t smem = 1024 + (size_t)A.stage_bytes + 4 * ((size_t)lb + 2 * (size_t)A.nslot);
-    auto kern = k_sigma_ab_tc<NP>;
+    auto kern = X ? k_sigma_ab_tc<NP, true> : k_sigma_ab_tc<NP, false>;
     TB_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    TB_CUDA(ctx, cudaStreamWaitEvent(st, X->busy, 0));
-    {
+    if (X) {
+        TB_CUDA(ctx, cudaStreamWaitEvent(st, X->busy, 0));
         TraceScope tr(ctx, "k_planes", st);
         const unsigned nb = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (A.lbp / 8) + 255) / 256);
-        k_planes<NP><<<dim3(nb, (unsigned)nv), 256, 0, st>>>(c, la, lb, A.lbp, info, X->c);
+        k_planes<NP><<<dim3(nb, (unsigned)nv), 256, 0, st>>>(c, la, lb, A.lbp, info, X->c.p);
         TB_CUDA(ctx, cudaGetLastError());
     }
     {
@@ -579,42 +621,33 @@ tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float 
         kern<<<dim3((unsigned)la, (unsigned)nv), kAbThreads, smem, st>>>(A);
         TB_CUDA(ctx, cudaGetLastError());
     }
-    TB_CUDA(ctx, cudaEventRecord(X->busy, st));
+    if (X) TB_CUDA(ctx, cudaEventRecord(X->busy, st));
     return TBSCI_OK;
 }
 
 }  // namespace
 
-// Makes the kernel's tables for `np` planes (1 or 3); *ready = false where the space, the
-// budget or a stream being captured (the tables are made outside of graphs, and a
-// graph's replays would share the planes of c with other streams) leaves it to the
-// SIMT kernels.
-tbsci_status sigma_tc_prepare(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int np, cudaStream_t st, bool *ready) {
-    *ready = false;
-    if (P->tl_kpmax == 0 || fp_stage_bytes(ctx, P, np) == 0) return TBSCI_OK;
+// Whether the kernel serves a space with `np` planes (1 or 3)
+bool sigma_tc_serves(const tbsci_ctx *ctx, const Plan *P, int np) { return P->tl_kpmax > 0 && fp_stage_bytes(ctx, P, np) > 0; }
+
+// Adds the alpha-beta products of nv vectors (at most sigma_tc_batch) into s; info: device
+// flags [nv][2], nothing is done for a vector whose first one is 0 (NULL: always).
+tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, int nv,
+                         const int *info, cudaStream_t st) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
-        return TBSCI_OK;
+        return np == 1 ? ab_add<1>(ctx, P, nullptr, c, s, nv, info, st) : ab_add<3>(ctx, P, nullptr, c, s, nv, info, st);
     }
-    std::shared_ptr<AbPlanes> &X = P->ab[np == 1 ? 0 : 1];
+    std::shared_ptr<AbPlanes> &own = P->ab[np == 1 ? 0 : 1];
     {
         static std::mutex make;
         std::lock_guard<std::mutex> g(make);
-        if (!X) X = std::make_shared<AbPlanes>();
+        if (!own) own = std::make_shared<AbPlanes>();
     }
-    std::lock_guard<std::mutex> g(X->mu);
-    if (!X->tried) TB_TRY(np == 1 ? build_planes<1>(ctx, ham, P, X.get(), st) : build_planes<3>(ctx, ham, P, X.get(), st));
-    *ready = X->ready;
-    return TBSCI_OK;
-}
-
-// Adds the alpha-beta products of nv vectors (at most sigma_tc_batch) into s, after a
-// prepare that said ready; info: device flags [nv][2], nothing is done for a vector whose
-// first one is 0 (NULL: always).
-tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, int nv, const int *info, cudaStream_t st) {
-    AbPlanes *X = P->ab[np == 1 ? 0 : 1].get();
-    std::lock_guard<std::mutex> g(X->mu);
+    std::lock_guard<std::mutex> g(own->mu);
+    if (!own->tried) TB_TRY(build_planes(ctx, P, np, own.get()));
+    AbPlanes *X = own->c.p ? own.get() : nullptr;
     return np == 1 ? ab_add<1>(ctx, P, X, c, s, nv, info, st) : ab_add<3>(ctx, P, X, c, s, nv, info, st);
 }
 

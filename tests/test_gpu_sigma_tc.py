@@ -59,6 +59,47 @@ def test_tc_sigma_parity(tb, ctx, mode, n, na, nb, acnt, bcnt, nvec):
     sp.close()
 
 
+@pytest.mark.parametrize("mode", ["tf32", "bf16"])
+@pytest.mark.parametrize("n,na,nb,la,lb", [(12, 6, 6, 200, 129), (12, 6, 6, 200, 130), (16, 8, 8, 150, 64), (13, 6, 5, 90, 1)])
+def test_tc_sigma_under_capture_and_without_room(tb, ctx, mode, n, na, nb, la, lb):
+    """A captured call runs the tensor-core kernel too: the bits of the eager call, on odd and
+    even rows and on vectors that start on 4 bytes only. So does a context whose budget is
+    spent by the prepared space, and it takes nothing more."""
+    import torch
+    h, eri, _ = synth_hamiltonian(n, seed=310 + n)
+    asel, bsel = selected_strings(n, na, la, 41), selected_strings(n, nb, lb, 42)
+    dt = tb.TBSCI_F32_TC_TF32 if mode == "tf32" else tb.TBSCI_F32_TC_BF16
+    c = torch.from_numpy(random_vectors(3, la, lb, seed=43)).float().cuda()
+    sp = tb.Space(ctx, n, na, nb, h, eri, 0.2, alpha=asel, beta=bsel)
+    out = torch.empty_like(c)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):  # the first call on this space
+        sp.sigma(c, out, dtype=dt)
+    g.replay()
+    want = sp.sigma(c, dtype=dt)
+    assert torch.equal(out, want)
+    tb.tbsci_trace_enable(ctx.handle, True)
+    buf = torch.empty(c.numel() + 1, device="cuda")
+    shifted = buf[1:].view(c.shape)
+    shifted.copy_(c)
+    assert torch.equal(sp.sigma(shifted, dtype=dt), want)
+    torch.cuda.synchronize()
+    tb.tbsci_trace_enable(ctx.handle, False)
+    assert "k_sigma_ab_tc" in {k for k, _ in tb.tbsci_trace_read(ctx.handle)[0]}
+    sp.close()
+    probe = tb.Context(0)
+    sp = tb.Space(probe, n, na, nb, h, eri, 0.2, alpha=asel, beta=bsel)
+    need = tb.tbsci_hbm_used(probe.handle)
+    sp.close()
+    probe.close()
+    full = tb.Context(0, hbm_budget=need)
+    sp = tb.Space(full, n, na, nb, h, eri, 0.2, alpha=asel, beta=bsel)
+    assert torch.equal(sp.sigma(c, dtype=dt), want)
+    assert tb.tbsci_hbm_used(full.handle) == need
+    sp.close()
+    full.close()
+
+
 def test_tc_sigma_sel16_sampled(tb, ctx):
     """norb=16, 3,000 x 3,000 (9.0M determinants), split TF32, 3 vectors."""
     import torch
