@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_bf16.h>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -454,7 +455,9 @@ void tile_links_size(tbsci_ctx *ctx, Plan *P);  // adds the plan's buffers to it
 tbsci_status tile_links_build(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, cudaStream_t st);
 bool sigma_tc_serves(const tbsci_ctx *ctx, const Plan *P, int np);
 tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, int nv,
-                         const int *info, cudaStream_t st);
+                         const int *info, cudaStream_t st, const __nv_bfloat16 *planes);
+tbsci_status sigma_tc_planes(tbsci_ctx *ctx, const Plan *P, const float *c, int nv, const int *info, __nv_bfloat16 *out,
+                             cudaStream_t st);
 int sigma_tc_batch(const Plan *P);
 tbsci_status diagonal_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan, double *diag,
                              cudaStream_t st, bool tables);

@@ -1416,7 +1416,7 @@ tbsci_status sigma_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan
         for (int v = 0; v < nvec; v += batch) {
             const int nv = std::min(batch, nvec - v);
             TB_TRY(udiag_launch(ctx, ham, plan, cf + v * n, sf + v * n, nv, true, true, st));
-            TB_TRY(sigma_tc_ab(ctx, const_cast<Plan *>(plan), np, cf + v * n, sf + v * n, nv, nullptr, st));
+            TB_TRY(sigma_tc_ab(ctx, const_cast<Plan *>(plan), np, cf + v * n, sf + v * n, nv, nullptr, st, nullptr));
         }
         return TBSCI_OK;
     }

@@ -9,9 +9,17 @@
 // (below 2^-64 of the vector's scale, 2^-56 of the Hamiltonian's) and the products of
 // weight below 256^-9 are lost: less than the rounding of the FP64 sums that they
 // replace (norb 16, 3,000 x 3,000 strings: 6.1e-16 of the norm from 64-bit values, the
-// SIMT kernel 1.5e-15). FP32 sigma takes 4 + 4 digits and weights to 256^-5 for the
-// same-spin classes (1.3e-7 in all, the SIMT kernel 6.2e-7).
+// SIMT kernel 1.5e-15).
 // Integer sums are associative: results do not depend on the order of the work.
+//
+// FP32 sigma takes the same kernels of the same-spin classes with three BF16 planes per
+// value in the place of digits (all 24 bits of an FP32 value, each with its own exponent)
+// and the six products x_i y_j with i + j <= 2, summed in FP32: what an element loses is
+// relative to the terms of its own sum, as in the SIMT kernel, however far the elements of
+// a vector or the integrals lie apart. (FP32 digits, of 32 bits below one scale for the whole
+// vector, were up to 1e-3 of (|H||c|)_I off on vectors that decay by a decade per excitation.)
+// norb 16, 3,000 x 3,000 strings, three vectors: 5.3 ms, 1.4e-7 of the norm from 64-bit values;
+// the SIMT kernel 13.6 ms, 6.2e-7.
 //
 // Parts of a sigma (Sec. II.B, Eq. 7; the classes [a,b] of Sec. II.C):
 //   k_udiag         the diagonal and the opposite-spin term of the alpha singles
@@ -44,7 +52,8 @@ namespace tbsci {
 
 namespace {
 
-// digits of a matrix element / of c, and accumulated weights 256^-2 .. 256^-(ORD + 1)
+// digits (FP32: planes) of a matrix element / of c, and accumulated weights 256^-2 ..
+// 256^-(ORD + 1) (FP32: sums i + j)
 template <int P>
 struct Prec;
 template <>
@@ -55,9 +64,9 @@ struct Prec<0> {  // FP64
 };
 template <>
 struct Prec<1> {  // FP32
-    static constexpr int NSA = 4, NSC = 4, ORD = 4;
+    static constexpr int NSA = 3, NSC = 3, ORD = 3;
     typedef float T;
-    static constexpr double kRatio = 256.0;
+    static constexpr double kRatio = INFINITY;  // planes have their own exponents
 };
 
 // Two accumulators of integers x0, x1 as the integer 256 x0 + x1, plus kPairBias (mod
@@ -95,22 +104,10 @@ __device__ __forceinline__ int64_t to_fixed(double x, int shift_base) {
     else v = sh < -54 ? 0 : (m + ((int64_t)1 << (-sh - 1))) >> -sh;
     return (int64_t)b < 0 ? -v : v;
 }
-__device__ __forceinline__ int64_t to_fixed(float x, int shift_base) {
-    const uint32_t b = __float_as_uint(x);
-    const int ex = (int)((b >> 23) & 0xFF);
-    if (ex == 0) return 0;
-    const int64_t m = (int64_t)((b & 0x7FFFFFu) | 0x800000u);
-    const int sh = ex - 150 + shift_base;
-    int64_t v;
-    if (sh >= 0) v = m << min(sh, 62);
-    else v = sh < -25 ? 0 : (m + ((int64_t)1 << (-sh - 1))) >> -sh;
-    return (int32_t)b < 0 ? -v : v;
-}
-
 // digit s (0 = leading) of an N-digit fixed-point value, as BF16 bits
 template <int N>
 __device__ __forceinline__ uint32_t digit_bf16(int64_t fixed, int s) {
-    constexpr uint64_t kBias = N == 8 ? 0x0080808080808080ull : N == 7 ? 0x0000808080808080ull : 0x0000000000808080ull;
+    constexpr uint64_t kBias = N == 8 ? 0x0080808080808080ull : 0x0000808080808080ull;
     const uint64_t u = (uint64_t)fixed + kBias;
     const int d = s == 0 ? (int)((int64_t)u >> (8 * (N - 1))) : (int)((u >> (8 * (N - 1 - s))) & 0xFF) - 128;
     return __float_as_uint((float)d) >> 16;
@@ -219,13 +216,12 @@ __global__ void __launch_bounds__(kScaleThreads) k_scale(const T *__restrict__ c
 }
 
 // the digit planes [NSC][la][lbp] of each vector, columns lb .. lbp - 1 zero; 8 columns per thread
-template <int P>
-__global__ void __launch_bounds__(256) k_slice(const typename Prec<P>::T *__restrict__ c, int64_t la, int64_t lb,
-                                               int64_t lbp, const int *__restrict__ info, Outliers O, __nv_bfloat16 *out) {
+__global__ void __launch_bounds__(256) k_slice(const double *__restrict__ c, int64_t la, int64_t lb, int64_t lbp,
+                                               const int *__restrict__ info, Outliers O, __nv_bfloat16 *out) {
     info += 2 * blockIdx.y;
     if (!info[0]) return;
-    const typename Prec<P>::T lim = (typename Prec<P>::T)O.thr[blockIdx.y];
-    constexpr int N = Prec<P>::NSC;
+    const double lim = O.thr[blockIdx.y];
+    constexpr int N = Prec<0>::NSC;
     c += blockIdx.y * la * lb;
     out += blockIdx.y * N * la * lbp;
     const int shift = 8 * N - info[1];
@@ -235,7 +231,7 @@ __global__ void __launch_bounds__(256) k_slice(const typename Prec<P>::T *__rest
         int64_t f[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-            const typename Prec<P>::T x = j + u < lb ? __ldg(c + r * lb + j + u) : 0;
+            const double x = j + u < lb ? __ldg(c + r * lb + j + u) : 0;
             if (x <= lim && -x <= lim) {
                 f[u] = to_fixed(x, shift);
             } else {
@@ -280,8 +276,8 @@ __global__ void k_table_scales(const unsigned long long *__restrict__ top, doubl
     tab[1] = tab[2] && h > 0.0 ? scale_exponent(h) : 0;
 }
 
-// the links of one CSR row per warp into dense digit planes [NSA][l][ld] (zeroed before),
-// and their number per 32-column chunk
+// the links of one CSR row per warp into dense digit (FP32: BF16) planes [NSA][l][ld] (zeroed
+// before), and their number per 32-column chunk
 template <int P>
 __global__ void __launch_bounds__(256) k_dense_digits(int64_t l, int64_t ld, int nch, const int64_t *__restrict__ soff,
                                                       const int2 *__restrict__ sci, const double *__restrict__ sval,
@@ -299,9 +295,16 @@ __global__ void __launch_bounds__(256) k_dense_digits(int64_t l, int64_t ld, int
     __syncwarp();
     const int shift = 8 * N - tab[1];
     auto put = [&](int col, double x) {
-        const int64_t f = to_fixed(x, shift);
+        uint32_t h[N];
+        if constexpr (P == 0) {
+            const int64_t f = to_fixed(x, shift);
 #pragma unroll
-        for (int s = 0; s < N; ++s) out[s * plane + r * ld + col] = __ushort_as_bfloat16((unsigned short)digit_bf16<N>(f, s));
+            for (int s = 0; s < N; ++s) h[s] = digit_bf16<N>(f, s);
+        } else {
+            bf16_planes<N>((float)x, h);
+        }
+#pragma unroll
+        for (int s = 0; s < N; ++s) out[s * plane + r * ld + col] = __ushort_as_bfloat16((unsigned short)h[s]);
         atomicAdd(c + (col >> 5), 1u);
     };
     for (int64_t t = soff[r] + lane; t < soff[r + 1]; t += 32) put(sci[t].x, sval[t]);
@@ -311,8 +314,9 @@ __global__ void __launch_bounds__(256) k_dense_digits(int64_t l, int64_t ld, int
 }
 
 // The accumulators stay exact while a row has met at most kWindow links: 7 products
-// of digits below 2^7 each per link and weight, 7 * 144 * 2^14 < 2^24 (and 4 * 144 *
-// 2^22 + 144 * 2^16 < 2^31 where two weights share a 32-bit word).
+// of digits below 2^7 each per link and weight, 7 * 144 * 2^14 < 2^24. FP32 sums keep the
+// same windows: they are added up in registers, rounded to nearest, where the tensor core's
+// accumulator truncates.
 constexpr int kWindow = 144;
 
 // flush[b][ch] = 1: drain the accumulators before chunk ch (rows of block b); 2: no link, skip it
@@ -477,8 +481,8 @@ __device__ __forceinline__ void tma3(uint32_t dst, const CUtensorMap *m, uint32_
 template <int P>
 struct SsShape {
     static constexpr int NSA = Prec<P>::NSA, NSC = Prec<P>::NSC, ORD = Prec<P>::ORD;
-    static constexpr int NT = 512 / ORD;  // every weight's accumulator of a tile is resident: ORD x NT = 512 TMEM columns
-    static constexpr int kStages = P == 0 ? 2 : 3;
+    static constexpr int NT = P == 0 ? 64 : 128;  // every weight's accumulator of a tile is resident: ORD x NT <= 512 TMEM columns
+    static constexpr int kStages = P == 0 ? 2 : 4;
     static constexpr uint32_t kBetaBytes = NSC * 128 * 64 + NSA * NT * 64;
     static constexpr uint32_t kAlphaBytes = NSA * 128 * 64 + NSC * 32 * NT * 2;
     static constexpr uint32_t kStageBytes = ((kBetaBytes > kAlphaBytes ? kBetaBytes : kAlphaBytes) + 1023) / 1024 * 1024;
@@ -629,12 +633,13 @@ __global__ void __launch_bounds__(kSsThreads, 1) k_same_spin_ex(const __grid_con
     } else {
         constexpr int NC = NT / 4;  // columns of a draining warp
         const int quarter = warp & 3, part = warp >> 2;
-        int64_t hi[NC], lo[P == 0 ? NC : 1];
+        int64_t hi[P == 0 ? NC : 1], lo[P == 0 ? NC : 1];
+        float sum[P == 0 ? 1 : NC];
 #pragma unroll
-        for (int x = 0; x < NC; ++x) hi[x] = 0;
-        if (P == 0)
-#pragma unroll
-            for (int x = 0; x < NC; ++x) lo[P == 0 ? x : 0] = 0;
+        for (int x = 0; x < NC; ++x) {
+            if (P == 0) hi[P == 0 ? x : 0] = lo[P == 0 ? x : 0] = 0;
+            else sum[P == 0 ? 0 : x] = 0.f;
+        }
         // the same walk as the MMA warp's, to know the number of drains and which is empty
         int drains = 0, phase = 0;
         bool any = false;
@@ -653,15 +658,21 @@ __global__ void __launch_bounds__(kSsThreads, 1) k_same_spin_ex(const __grid_con
             if (ok && any) {
 #pragma unroll
                 for (int x0 = 0; x0 < NC; x0 += 16) {
+                    float t[16];  // FP32: the window's sums, smallest products first
 #pragma unroll
-                    for (int o = 0; o < ORD; ++o) {
+                    for (int o = ORD - 1; o >= 0; --o) {
                         uint32_t r[16];
                         tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + o * NT + part * NC + x0, r);
 #pragma unroll
                         for (int x = 0; x < 16; ++x) {
-                            const int64_t v = (int64_t)__float2int_rn(__uint_as_float(r[x])) << (8 * (3 - (o & 3)));
-                            if (o < 4) hi[x0 + x] += v;
-                            else lo[P == 0 ? x0 + x : 0] += v;
+                            if constexpr (P == 0) {
+                                const int64_t v = (int64_t)__float2int_rn(__uint_as_float(r[x])) << (8 * (3 - (o & 3)));
+                                if (o < 4) hi[x0 + x] += v;
+                                else lo[x0 + x] += v;
+                            } else {
+                                t[x] = o == ORD - 1 ? __uint_as_float(r[x]) : t[x] + __uint_as_float(r[x]);
+                                if (o == 0) sum[x0 + x] += t[x];
+                            }
                         }
                     }
                 }
@@ -673,12 +684,12 @@ __global__ void __launch_bounds__(kSsThreads, 1) k_same_spin_ex(const __grid_con
         const int64_t Ia = row0 + quarter * 32 + lane, jb = col0 + part * NC;
         if (Ia < A.la) {
             T *S = static_cast<T *>(A.S) + blockIdx.z * A.la * A.lb + Ia * A.lb;
-            const double sc = pow2(A.tab[1] + info[1] - 8 * (ORD + 1));
+            const double sc = P == 0 ? pow2(A.tab[1] + info[1] - 8 * (ORD + 1)) : 1.0;
 #pragma unroll
             for (int x = 0; x < NC; ++x)
                 if (jb + x < A.lb) {
-                    const double v = P == 0 ? fma((double)hi[x], 4294967296.0, (double)lo[P == 0 ? x : 0]) : (double)hi[x];
-                    S[jb + x] += (T)(v * sc);
+                    if constexpr (P == 0) S[jb + x] += fma((double)hi[x], 4294967296.0, (double)lo[x]) * sc;
+                    else S[jb + x] += sum[x];
                 }
         }
     }
@@ -1099,7 +1110,7 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
     };
     const size_t hb = place((size_t)NSA * lb * lbp * 2), ha = place((size_t)NSA * la * lap * 2);
     const size_t top = place(16), done = place(4 * (size_t)Y.batch), zeroed = at;
-    const size_t vd = place(PR == 0 ? (size_t)P->npair * 128 * sizeof(uint4) : 0);  // FP32: sigma_tc.cu's planes
+    const size_t vd = place(PR == 0 ? (size_t)P->npair * 128 * sizeof(uint4) : 0);
     const size_t wd = place(PR == 0 ? (size_t)la * 128 * sizeof(uint4) : 0);
     const size_t cb = place((size_t)lb * nchb), ca = place((size_t)la * ncha);
     const size_t fb = place((size_t)nbb * nchb), fa = place((size_t)nba * ncha);
@@ -1264,10 +1275,13 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
             const unsigned nb = (unsigned)std::min<int64_t>(kScaleBlocks, (la * lb + 4 * kScaleThreads - 1) / (4 * kScaleThreads));
             k_scale<T><<<dim3(nb, (unsigned)nv), kScaleThreads, 0, st>>>(cv, la * lb, Prec<PR>::kRatio, PR == 0 ? kOutlierMaxN : 0,
                                                                         Y.part, Y.done, Y.tab, Y.info, Y.out);
-            const unsigned ns = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (lbp / 8) + 255) / 256);
-            k_slice<PR><<<dim3(ns, (unsigned)nv), 256, 0, st>>>(cv, la, lb, lbp, Y.info, Y.out, Y.planes);
+            if constexpr (PR == 0) {
+                const unsigned ns = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (lbp / 8) + 255) / 256);
+                k_slice<<<dim3(ns, (unsigned)nv), 256, 0, st>>>(cv, la, lb, lbp, Y.info, Y.out, Y.planes);
+            }
             TB_CUDA(ctx, cudaGetLastError());
         }
+        if constexpr (PR == 1) TB_TRY(sigma_tc_planes(ctx, P, cv, nv, Y.info, Y.planes, st));
         {
             TraceScope tr(ctx, "k_udiag", st);
             U.C = cv;
@@ -1288,7 +1302,7 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
             k_sigma_ab_ex<<<dim3((unsigned)la, (unsigned)nv), kAbThreads, ab_smem, st>>>(A);
             TB_CUDA(ctx, cudaGetLastError());
         } else {
-            TB_TRY(sigma_tc_ab(ctx, P, 3, cv, sv, nv, Y.info, st));
+            TB_TRY(sigma_tc_ab(ctx, P, 3, cv, sv, nv, Y.info, st, Y.planes));
         }
         TB_TRY(simt(v, nv, Y.info, out));
     }

@@ -145,20 +145,6 @@ __global__ void __launch_bounds__(kLinkThreads) k_tile_links(const int32_t *__re
 
 // ------------------------------------------------------------------ planes
 
-// x = sum of NP BF16 values, each the rounded rest of the ones before
-template <int NP>
-__device__ __forceinline__ void bf16_planes(float x, uint32_t (&h)[NP]) {
-#pragma unroll
-    for (int s = 0; s < NP; ++s) {
-        const __nv_bfloat16 b = __float2bfloat16_rn(x);
-        h[s] = __bfloat16_as_ushort(b);
-        if (s + 1 < NP) {
-            const float r = x - __bfloat162float(b);
-            x = isfinite(r) ? r : 0.f;  // infinities and NaN lie in the first plane
-        }
-    }
-}
-
 // planes [NP][la][lbp] of a vector, columns lb .. lbp - 1 zero; 8 columns per thread
 template <int NP>
 __global__ void __launch_bounds__(256) k_planes(const float *__restrict__ c, int64_t la, int64_t lb, int64_t lbp,
@@ -582,15 +568,15 @@ tbsci_status build_planes(tbsci_ctx *ctx, Plan *P, int np, AbPlanes *X) {
 }
 
 template <int NP>
-tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float *s, int nv, const int *info,
-                    cudaStream_t st) {
+tbsci_status ab_launch(tbsci_ctx *ctx, const Plan *P, const __nv_bfloat16 *planes, const float *c, float *s,
+                       int nv, const int *info, cudaStream_t st) {
     const int64_t la = P->A.l, lb = P->B.l;
     FpArgs A{};
     A.la = la;
     A.lb = lb;
     A.lbp = pad64(lb);
     A.C = c;
-    A.Cs = X ? X->c.p : nullptr;
+    A.Cs = planes;
     A.S = s;
     A.info = info;
     A.Vd = P->d_ab_v.p;
@@ -607,22 +593,29 @@ tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float 
     A.rowsa = P->d_rowsa.p;
     A.err = P->d_tc_err.p;
     const size_t smem = 1024 + (size_t)A.stage_bytes + 4 * ((size_t)lb + 2 * (size_t)A.nslot);
-    auto kern = X ? k_sigma_ab_tc<NP, true> : k_sigma_ab_tc<NP, false>;
+    auto kern = planes ? k_sigma_ab_tc<NP, true> : k_sigma_ab_tc<NP, false>;
     TB_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (X) {
-        TB_CUDA(ctx, cudaStreamWaitEvent(st, X->busy, 0));
-        TraceScope tr(ctx, "k_planes", st);
-        const unsigned nb = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (A.lbp / 8) + 255) / 256);
-        k_planes<NP><<<dim3(nb, (unsigned)nv), 256, 0, st>>>(c, la, lb, A.lbp, info, X->c.p);
-        TB_CUDA(ctx, cudaGetLastError());
-    }
-    {
-        TraceScope tr(ctx, "k_sigma_ab_tc", st);
-        kern<<<dim3((unsigned)la, (unsigned)nv), kAbThreads, smem, st>>>(A);
-        TB_CUDA(ctx, cudaGetLastError());
-    }
-    if (X) TB_CUDA(ctx, cudaEventRecord(X->busy, st));
+    TraceScope tr(ctx, "k_sigma_ab_tc", st);
+    kern<<<dim3((unsigned)la, (unsigned)nv), kAbThreads, smem, st>>>(A);
+    TB_CUDA(ctx, cudaGetLastError());
     return TBSCI_OK;
+}
+
+template <int NP>
+tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float *s, int nv, const int *info,
+                    cudaStream_t st) {
+    if (!X) return ab_launch<NP>(ctx, P, nullptr, c, s, nv, info, st);
+    const int64_t la = P->A.l, lb = P->B.l, lbp = pad64(lb);
+    TB_CUDA(ctx, cudaStreamWaitEvent(st, X->busy, 0));
+    {
+        TraceScope tr(ctx, "k_planes", st);
+        const unsigned nb = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (lbp / 8) + 255) / 256);
+        k_planes<NP><<<dim3(nb, (unsigned)nv), 256, 0, st>>>(c, la, lb, lbp, info, X->c.p);
+        TB_CUDA(ctx, cudaGetLastError());
+    }
+    const tbsci_status r = ab_launch<NP>(ctx, P, X->c.p, c, s, nv, info, st);
+    TB_CUDA(ctx, cudaEventRecord(X->busy, st));  // also behind a failed launch: the planes are in use
+    return r;
 }
 
 }  // namespace
@@ -630,10 +623,23 @@ tbsci_status ab_add(tbsci_ctx *ctx, Plan *P, AbPlanes *X, const float *c, float 
 // Whether the kernel serves a space with `np` planes (1 or 3)
 bool sigma_tc_serves(const tbsci_ctx *ctx, const Plan *P, int np) { return P->tl_kpmax > 0 && fp_stage_bytes(ctx, P, np) > 0; }
 
+// The three planes [nv][3][la][pad64(lb)] of nv vectors, for the vectors whose info is set
+tbsci_status sigma_tc_planes(tbsci_ctx *ctx, const Plan *P, const float *c, int nv, const int *info, __nv_bfloat16 *out,
+                             cudaStream_t st) {
+    const int64_t la = P->A.l, lb = P->B.l, lbp = pad64(lb);
+    TraceScope tr(ctx, "k_planes", st);
+    const unsigned nb = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (lbp / 8) + 255) / 256);
+    k_planes<3><<<dim3(nb, (unsigned)nv), 256, 0, st>>>(c, la, lb, lbp, info, out);
+    TB_CUDA(ctx, cudaGetLastError());
+    return TBSCI_OK;
+}
+
 // Adds the alpha-beta products of nv vectors (at most sigma_tc_batch) into s; info: device
-// flags [nv][2], nothing is done for a vector whose first one is 0 (NULL: always).
+// flags [nv][2], nothing is done for a vector whose first one is 0 (NULL: always); planes:
+// those of c if the caller has them (np = 3).
 tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float *s, int nv,
-                         const int *info, cudaStream_t st) {
+                         const int *info, cudaStream_t st, const __nv_bfloat16 *planes) {
+    if (planes) return ab_launch<3>(ctx, P, planes, c, s, nv, info, st);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
         cudaGetLastError();

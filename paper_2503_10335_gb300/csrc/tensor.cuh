@@ -1,9 +1,24 @@
 // tcgen05, TMEM and mbarrier helpers shared by the tensor-core kernels.
 #pragma once
 
+#include <cuda_bf16.h>
 #include <stdint.h>
 
 namespace tbsci {
+
+// x = sum of NP BF16 values, each the rounded rest of the ones before
+template <int NP>
+__device__ __forceinline__ void bf16_planes(float x, uint32_t (&h)[NP]) {
+#pragma unroll
+    for (int s = 0; s < NP; ++s) {
+        const __nv_bfloat16 b = __float2bfloat16_rn(x);
+        h[s] = __bfloat16_as_ushort(b);
+        if (s + 1 < NP) {
+            const float r = x - __bfloat162float(b);
+            x = isfinite(r) ? r : 0.f;  // infinities and NaN lie in the first plane
+        }
+    }
+}
 
 __device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 

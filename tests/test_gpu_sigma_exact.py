@@ -45,6 +45,74 @@ def _rows(ndet, seed, k=400):
     return np.unique(np.concatenate([r.choice(ndet, min(k, ndet), replace=False), np.arange(min(40, ndet)), np.arange(max(0, ndet - 40), ndet)]))
 
 
+def _graded(sp, decades, rng):
+    """Normal deviates that fall by `decades` per excitation, in both spins; and the sampled rows: any, and the most excited."""
+    a, b = sp.strings()
+    level = (np.bitwise_count(a >> np.uint64(sp.nalpha)).astype(int)[:, None] + np.bitwise_count(b >> np.uint64(sp.nbeta)).astype(int))
+    C = rng.standard_normal((1, sp.la, sp.lb)) * 10.0 ** (-decades * level)
+    top = np.argsort(level.reshape(-1), kind="stable")[-500:]
+    return C / np.linalg.norm(C), np.unique(np.concatenate([_rows(sp.ndet, 11, 1500), top]))
+
+
+@pytest.mark.parametrize("dtype", ["f32"])
+@pytest.mark.parametrize("n,na,nb,la,lb,decades", [
+    (11, 5, 5, None, None, 0.8),
+    (11, 5, 5, None, None, 1.0),
+    (11, 5, 5, None, None, 1.5),
+    (16, 8, 8, 700, 650, 1.0),
+    (16, 8, 8, 700, 650, 1.5),
+])
+def test_small_elements_keep_their_accuracy(tb, ctx, n, na, nb, la, lb, decades, dtype):
+    """Vectors that decay by orders of magnitude per excitation, as CI vectors do: every element
+    is as close, relative to the terms of its own sum, as anywhere else."""
+    import torch
+    sp, osp, h, eri = _space(tb, ctx, n, na, nb, la, lb, seed=760 + n)
+    C, rows = _graded(sp, decades, np.random.default_rng(n))
+    Ct = torch.from_numpy(C).to(torch.float64 if dtype == "f64" else torch.float32).cuda()
+    s = sp.sigma(Ct)
+    assert torch.equal(s, sp.sigma(Ct))
+    _check(s.double().cpu().numpy(), osp, h, eri, Ct.double().cpu().numpy(), rows, **({} if dtype == "f64" else F32))
+    sp.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32"])
+@pytest.mark.parametrize("decades", [0.0, 0.5])
+def test_small_integrals_keep_their_accuracy(tb, ctx, decades, dtype):
+    """Integrals that spread over five decades from orbital to orbital: elements whose links are
+    all small are as close as the others."""
+    import torch
+    n = 11
+    h, eri, _ = synth_hamiltonian(n, seed=768)
+    g = 10.0 ** (-np.linspace(0, 1.25, n))
+    h = h * g[:, None] * g[None, :]
+    eri = eri * np.einsum("i,j,k,l->ijkl", g, g, g, g)
+    sp = tb.Space(ctx, n, 5, 5, h, eri, 0.25)
+    osp = oracle.make_space(n, 5, 5)
+    C, rows = _graded(sp, decades, np.random.default_rng(12))
+    Ct = torch.from_numpy(C).to(torch.float64 if dtype == "f64" else torch.float32).cuda()
+    _check(sp.sigma(Ct).double().cpu().numpy(), osp, h, eri, Ct.double().cpu().numpy(), rows, **({} if dtype == "f64" else F32))
+    sp.close()
+
+
+def test_f32_takes_peaked_vectors(tb, ctx):
+    """The trial vectors of a mixed solve: one element thousands of times the root mean square.
+    They stay on the tensor cores (the bits are not those of a captured call, which is SIMT)."""
+    import torch
+    sp, osp, h, eri = _space(tb, ctx, 13, 6, 6, 1040, 1030, seed=733)
+    C = 1e-4 * np.random.default_rng(8).standard_normal((1, sp.la, sp.lb))
+    C[0, 0, 0] = 0.9
+    assert np.abs(C).max() > 256 * np.sqrt((C ** 2).mean())
+    Ct = torch.from_numpy(C).float().cuda()
+    s, out = sp.sigma(Ct), torch.empty_like(Ct)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        sp.sigma(Ct, out)
+    g.replay()
+    assert not torch.equal(s, out)
+    _check(s.double().cpu().numpy(), osp, h, eri, Ct.double().cpu().numpy(), _rows(sp.ndet, 13), **F32)
+    sp.close()
+
+
 @pytest.mark.parametrize("dtype", ["f64", "f32"])
 @pytest.mark.parametrize("n,na,nb,la,lb,nvec", [
     (13, 6, 6, 1030, 1025, 2),    # one row past a 128-row tile's multiple of 6, one column past 64
