@@ -362,8 +362,16 @@ struct Outliers {
     int *count;     // [vector]
     int64_t *list;  // [vector][kOutliers], in no order
 };
+// Elements of sigma for which the digits are too coarse (FP64 only): k_sigma_repair sums these
+struct Coarse {
+    float *need;      // [vector] an element's terms add up to this, or it is listed
+    unsigned *count;  // [vector]
+    int32_t *list;    // [vector][limit]: element, in no order
+    unsigned limit;   // past it the vector goes to the SIMT kernels whole (its info[0] becomes 0)
+};
 struct OutlierArgs {
     Outliers O;
+    Coarse R;
     int64_t lb;
     const uint64_t *stra;
     const int64_t *a_soff, *a_doff, *b_soff, *b_doff;

@@ -481,9 +481,74 @@ __device__ void outliers_row(const OutlierArgs &A, int v, const double *C, doubl
     }
 }
 
+// The elements of sigma listed by the exact path (Coarse), a warp each: every term of the row
+// of H, lanes over the beta links and over the alpha links, added up in a fixed order. Behind
+// k_sigma_left, whose outliers they include. At most 64 single links per string.
+// Bound by the gathers of V and c: 244,000 elements of three vectors of 1,200 x 1,100 strings
+// in 0.85 ms.
+__global__ void __launch_bounds__(256) k_sigma_repair(SigArgs<double> A, const int *__restrict__ info, const Coarse R) {
+    const int v = blockIdx.y, lane = threadIdx.x & 31;
+    if (!info[2 * v]) return;
+    const unsigned n = R.count[v];
+    const int64_t lb = A.lb;
+    const double *__restrict__ C = A.C + v * A.vstride;
+    double *__restrict__ S = A.S + v * A.vstride;
+    for (unsigned x = blockIdx.x * 8 + (threadIdx.x >> 5); x < n; x += gridDim.x * 8) {
+        const int64_t I = R.list[(size_t)v * R.limit + x], Ia = I / lb, Ib = I - Ia * lb;
+        const uint64_t str = A.stra[Ia];
+        const int64_t a0 = A.a_soff[Ia], b0 = A.b_soff[Ib];
+        const int ns = (int)(A.a_soff[Ia + 1] - a0), nb = (int)(A.b_soff[Ib + 1] - b0);
+        double acc = 0.0;
+        if (lane == 0) {
+            double ed = A.ecore + A.Ea[Ia] + A.Eb[Ib];
+            for (uint64_t s = str; s; s &= s - 1) {
+                const int p = __ffsll((long long)s) - 1;
+                ed += A.U[(size_t)(p * (p + 1) / 2 + p) * lb + Ib];
+            }
+            acc = ed * C[I];
+        }
+        // alpha links with the beta string unchanged
+        for (int t = lane; t < ns; t += 32) {
+            const int2 e = __ldg(A.a_sci + a0 + t);
+            const double h = __ldg(A.a_sval + a0 + t) + flip_sign(__ldg(A.U + (size_t)(e.y >> 1) * lb + Ib), e.y << 31);
+            acc += h * __ldg(C + e.x * lb + Ib);
+        }
+        for (int64_t t = A.a_doff[Ia] + lane; t < A.a_doff[Ia + 1]; t += 32)
+            acc += __ldg(A.a_dval + t) * __ldg(C + __ldg(A.a_dcol + t) * lb + Ib);
+        // beta links with the alpha string unchanged
+        int2 eb[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            eb[q] = lane + 32 * q < nb ? __ldg(A.b_sci + b0 + lane + 32 * q) : make_int2(-1, 0);
+            if (eb[q].x < 0) continue;
+            double w = 0.0;
+            for (uint64_t s = str; s; s &= s - 1) {
+                const int p = __ffsll((long long)s) - 1;
+                w += __ldg(A.V + (size_t)(p * (p + 1) / 2 + p) * A.npair + (eb[q].y >> 1));
+            }
+            acc += (__ldg(A.b_sval + b0 + lane + 32 * q) + flip_sign(w, eb[q].y << 31)) * __ldg(C + Ia * lb + eb[q].x);
+        }
+        for (int64_t t = A.b_doff[Ib] + lane; t < A.b_doff[Ib + 1]; t += 32)
+            acc += __ldg(A.b_dval + t) * __ldg(C + Ia * lb + __ldg(A.b_dcol + t));
+        // both
+#pragma unroll 4
+        for (int t = 0; t < ns; ++t) {
+            const int2 e = __ldg(A.a_sci + a0 + t);
+            const double *V = A.V + (size_t)(e.y >> 1) * A.npair, *c = C + e.x * lb;
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (eb[q].x >= 0) acc += flip_sign(__ldg(V + (eb[q].y >> 1)), (e.y ^ eb[q].y) << 31) * __ldg(c + eb[q].x);
+        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) S[I] = acc;
+    }
+}
+
 // The vectors (one per blockIdx.y) that the exact tensor-core path leaves: skip[2 v] = 0;
 // of the others, the links of their outliers (a launch of their own cost 4 us a call).
-// Its own kernel, so that k_sigma's arguments stay constants.
+// Its own kernel, so that k_sigma's arguments stay constants. One vector per CTA, since each
+// may be left or not: a vector of 1,200 x 1,100 strings at norb 16 takes 2.81 ms (2.92 with 512
+// threads), 2.63 with three of them in k_sigma.
 template <typename T, bool STAGE, bool ACCS>
 __global__ void __launch_bounds__(256) k_sigma_left(SigArgs<T> A, const int *__restrict__ skip, const OutlierArgs out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1388,10 +1453,17 @@ tbsci_status launch_full(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan,
         A.C = c + v * n;
         A.S = s + v * n;
         switch (stage_variant<T>(ctx, A.npair, A.lb, 1, 0)) {
-            case 0: return launch_left<T, true, true>(ctx, A, nv, skip, out, st);
-            case 1: return launch_left<T, false, true>(ctx, A, nv, skip, out, st);
-            default: return launch_left<T, false, false>(ctx, A, nv, skip, out, st);
+            case 0: TB_TRY((launch_left<T, true, true>(ctx, A, nv, skip, out, st))); break;
+            case 1: TB_TRY((launch_left<T, false, true>(ctx, A, nv, skip, out, st))); break;
+            default: TB_TRY((launch_left<T, false, false>(ctx, A, nv, skip, out, st)));
         }
+        if constexpr (sizeof(T) == 8) {
+            TraceScope tr(ctx, "k_sigma_repair", st);
+            const unsigned nb = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (out.R.limit + 7) / 8);
+            k_sigma_repair<<<dim3(std::max(1u, nb), (unsigned)nv), 256, 0, st>>>(A, skip, out.R);
+            TB_CUDA(ctx, cudaGetLastError());
+        }
+        return TBSCI_OK;
     }));
     return ran ? TBSCI_OK : launch_typed<T>(ctx, ham, plan, c, s, nvec, st);
 }

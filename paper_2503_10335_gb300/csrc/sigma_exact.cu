@@ -31,11 +31,13 @@
 //                   (rs|pq), F: the coupled c rows), then G summed into the columns
 //                   its beta links point to
 // Small spaces take several vectors per launch.
-// A vector is scaled by one power of two. Digits are relative to that scale, so a
-// vector whose largest entry is far above its root mean square would lose digits of
-// the others: k_scale_final refuses such vectors (and NaN, infinities, extreme
-// magnitudes) by a flag in device memory, and the SIMT kernels, launched behind with
-// the same flag, compute those instead. The flag costs no synchronisation.
+// FP64 digits are relative to one power of two per vector, so an element of sigma whose
+// terms are all far below the vector's largest would be summed from few bits. Its terms are
+// therefore looked at on the way (k_udiag, see kCoarse): elements for which the digits are too
+// coarse are listed and summed again, term by term, by k_sigma_repair; a vector with many of
+// them goes to the SIMT kernels, launched behind, as do NaN, infinities and extreme
+// magnitudes, by a flag in device memory. Nothing of this costs a synchronisation. Elements of
+// c that tower over the rest are kept out of the digits (see kOutlierRms).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -133,13 +135,32 @@ constexpr int kScaleBlocks = 304;
 constexpr double kOutlierRms = 256.0;
 constexpr int64_t kOutlierMaxN = int64_t(1) << 24;
 
+// How far digits carry. With c below 2^(e - 1), the string Hamiltonians below 2^(h - 1) and n
+// links, an element of sigma is off by the products dropped, 2^-66 of 2^(e + h) a link or
+// 7e-19 of it (root mean square) at 3,000 links, and by the digits cut off H, 2^-58 of it for
+// the largest c: 8e-18 of 2^(e + h) where six standard deviations meet the worst H. (The W
+// row's digits are doubled thrice, so the integrals count with one more power of two.) The
+// terms of an element, (|H||c|)_I, are at least those of its diagonal and of its alpha singles
+// with the beta string unchanged, which k_udiag has at hand; where these reach 2^-14 of
+// 2^(e + h), the element is within 1.3e-13 of (|H||c|)_I, and 3e-15 where they are not all at
+// the limit. Two decades of string weights in each spin: up to 3 elements in a thousand are
+// below it.
+constexpr double kCoarse = 1.0 / 16384;
+// A listed element costs 1.7 times its share of the SIMT kernel (1,200 x 1,100 strings at
+// norb 16: 3.5 ns against 2.1), and the digits save two thirds of that kernel: past a quarter
+// of the elements the vector goes there. Of the 60 vectors of a 20-iteration Davidson run on
+// these strings, 12 do (the first four iterations, on which most elements are still zero or
+// nearly so); the run takes 127 ms, 103 without this look at the elements, when some were off
+// by up to 5e-9 of their terms, and 204 on the SIMT kernel.
+constexpr int64_t kCoarseShare = 4;
+
 // Per vector (blockIdx.y) its largest magnitude and sum of squares, in a fixed order;
 // the last block to finish writes info[2 v]: 1 when the digits serve the vector,
 // info[2 v + 1]: its scale exponent. done[v] wraps back to 0. O.thr[v]: what an outlier exceeds.
 template <typename T>
 __global__ void __launch_bounds__(kScaleThreads) k_scale(const T *__restrict__ c0, int64_t n, double ratio, int64_t outlier_n,
                                                          double *part0, unsigned *done, const int *__restrict__ tab, int *info,
-                                                         Outliers O) {
+                                                         Outliers O, Coarse R) {
     const T *__restrict__ c = c0 + blockIdx.y * n;
     double *part = part0 + (size_t)blockIdx.y * 2 * kScaleBlocks;
     double top = 0.0, sum = 0.0;
@@ -211,6 +232,8 @@ __global__ void __launch_bounds__(kScaleThreads) k_scale(const T *__restrict__ c
     }
     O.thr[blockIdx.y] = thr;
     O.count[blockIdx.y] = 0;
+    R.need[blockIdx.y] = top == 0.0 ? 0.f : (float)ldexp(kCoarse, e + max(tab[1], tab[0] + 1));
+    R.count[blockIdx.y] = 0;
     info[2 * blockIdx.y] = ok;
     info[2 * blockIdx.y + 1] = e;
 }
@@ -256,6 +279,22 @@ __global__ void k_absmax(const double *__restrict__ v, int64_t n, unsigned long 
     unsigned long long m = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(v[i]) & 0x7FFFFFFFFFFFFFFFull;
+        m = b > m ? b : m;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xffffffffu, m, o);
+        m = y > m ? y : m;
+    }
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(top, m);
+}
+
+// the same over the off-diagonal columns of the integrals, the only ones cut into digits
+__global__ void k_absmax_off(const double *__restrict__ V, int npair, int npoff, const int32_t *__restrict__ offpair,
+                             unsigned long long *top) {
+    unsigned long long m = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < npair * npoff; i += gridDim.x * blockDim.x) {
+        const unsigned long long b =
+            (unsigned long long)__double_as_longlong(V[(size_t)(i / npoff) * npair + offpair[i % npoff]]) & 0x7FFFFFFFFFFFFFFFull;
         m = b > m ? b : m;
     }
     for (int o = 16; o > 0; o >>= 1) {
@@ -388,6 +427,9 @@ struct UdArgs {
     const T *a_sval, *Ea, *Eb, *U;
     T ecore;
     int na, add;  // add: accumulate
+    const float *a_svalf;  // CHECK
+    int *flag;             // = info
+    Coarse R;
 };
 
 // S[Ia][j] (+)= Hd c(Ia, j) + sum over alpha singles ([h +] s U[pq][j]) c(Ja, j), one vector
@@ -399,17 +441,32 @@ constexpr int64_t kUdCols = 512;  // columns of a CTA
 
 __device__ __forceinline__ double flip(double x, int m) { return __hiloint2double(__double2hiint(x) ^ m, __double2loint(x)); }
 __device__ __forceinline__ float flip(float x, int m) { return __int_as_float(__float_as_int(x) ^ m); }
+// |x| rounded towards zero, on the integer units (a conversion instruction would take the
+// FP64 pipe); 0 below the smallest normal float, the largest float above it
+__device__ __forceinline__ float low_abs(double x) {
+    const uint32_t h = min((uint32_t)__double2hiint(x) & 0x7FFFFFFFu, 0x47EFFFFFu);
+    const uint32_t f = __funnelshift_l((uint32_t)__double2loint(x), h - 0x38000000u, 3);
+    return h < 0x38100000u ? 0.f : __uint_as_float(f);
+}
 
-template <typename T, bool SINGLES>
+// CHECK (FP64): the magnitudes of the terms are added up in FP32 beside them, with the
+// alpha singles' own values; what cancels between those and U is taken off by its rounding.
+// Elements that stay below R.need are listed (see kCoarse). At most 64 alpha singles.
+template <typename T, bool SINGLES, bool CHECK>
 __global__ void __launch_bounds__(256) k_udiag(UdArgs<T> A) {
-    if (A.info && !A.info[2 * blockIdx.z]) return;
     __shared__ int64_t sC[256], sU[256];
     __shared__ T sH[256];
+    __shared__ float sF[CHECK ? 64 : 1];
     __shared__ int sS[256];  // sign bit of the term
     __shared__ int sOcc[64];
+    __shared__ int sOn;
     const int64_t Ia = blockIdx.x, lb = A.lb;
     const int64_t t0 = A.a_soff[Ia], t1 = A.a_soff[Ia + 1];
     const int tid = threadIdx.x;
+    // read once for the whole CTA: with CHECK another CTA may clear it at any time
+    if (tid == 0) sOn = A.info ? *reinterpret_cast<const volatile int *>(A.info + 2 * blockIdx.z) : 1;
+    __syncthreads();
+    if (!sOn) return;
     const T *__restrict__ C = A.C + blockIdx.z * A.la * lb;
     T *__restrict__ S = A.S + blockIdx.z * A.la * lb + Ia * lb;
     if (tid < 64) {
@@ -426,14 +483,24 @@ __global__ void __launch_bounds__(256) k_udiag(UdArgs<T> A) {
             sU[tid] = (int64_t)(e.y >> 1) * lb;
             sS[tid] = (e.y & 1) ? (int)0x80000000 : 0;
             if (SINGLES) sH[tid] = A.a_sval[t + tid];
+            if (CHECK) sF[tid] = flip(A.a_svalf[t + tid], sS[tid]);  // with the sign of the term taken out
         }
         __syncthreads();
         for (int64_t j = blockIdx.y * kUdCols + tid; j < min(lb, (blockIdx.y + 1) * kUdCols); j += 256) {
             T acc = T(0), acc2 = T(0);
+            float mag = 0.f;
+            auto look = [&](int k, T u, T c) {
+                if constexpr (CHECK) {
+                    const float h = sF[k], v = copysignf(low_abs(u), __int_as_float(__double2hiint(u)));
+                    mag = fmaf(fmaxf(fmaf(fabsf(h) + fabsf(v), -1e-6f, fabsf(h + v)), 0.f), low_abs(c), mag);
+                }
+            };
             if (t == t0) {
                 T ed = eIa + __ldg(A.Eb + j);
                 for (int k = 0; k < A.na; ++k) ed += __ldg(A.U + (size_t)sOcc[k] * lb + j);
-                acc = ed * __ldg(C + Ia * lb + j);
+                const T c = __ldg(C + Ia * lb + j);
+                acc = ed * c;
+                if constexpr (CHECK) mag = low_abs(ed) * low_abs(c);
             }
             const T *__restrict__ Uj = A.U + j, *__restrict__ Cj = C + j;
             // one multiply-add per term: the sign goes to u by its sign bit (an FP64 compare
@@ -447,9 +514,34 @@ __global__ void __launch_bounds__(256) k_udiag(UdArgs<T> A) {
                 acc2 += coef(k + 1, u1) * c1;
                 acc += coef(k + 2, u2) * c2;
                 acc2 += coef(k + 3, u3) * c3;
+                look(k, u0, c0);
+                look(k + 1, u1, c1);
+                look(k + 2, u2, c2);
+                look(k + 3, u3, c3);
             }
-            for (; k < n; ++k) acc += coef(k, __ldg(Uj + sU[k])) * __ldg(Cj + sC[k]);
+            for (; k < n; ++k) {
+                const T u = __ldg(Uj + sU[k]), c = __ldg(Cj + sC[k]);
+                acc += coef(k, u) * c;
+                look(k, u, c);
+            }
             S[j] = (A.add || t > t0 ? S[j] : T(0)) + (acc + acc2);
+            if constexpr (CHECK) {
+                const int lane = tid & 31;
+                const int64_t left = min(lb, (blockIdx.y + 1) * kUdCols) - (j - lane);  // lanes with a column
+                const unsigned on = left >= 32 ? 0xFFFFFFFFu : (1u << left) - 1u;
+                const unsigned low = __ballot_sync(on, mag < A.R.need[blockIdx.z]);
+                if (low) {
+                    const unsigned cnt = __popc(low), lead = __ffs(low) - 1;
+                    unsigned at = 0;
+                    if (lane == lead) {
+                        at = atomicAdd(A.R.count + blockIdx.z, cnt);
+                        if (at + cnt > A.R.limit) A.flag[2 * blockIdx.z] = 0;
+                    }
+                    at = __shfl_sync(on, at, lead) + __popc(low & ((1u << lane) - 1u));
+                    if (((low >> lane) & 1) && at < A.R.limit)
+                        A.R.list[(size_t)blockIdx.z * A.R.limit + at] = (int32_t)(Ia * lb + j);
+                }
+            }
         }
     }
 }
@@ -1066,6 +1158,7 @@ struct ExactData {
         int *info = nullptr, *tab = nullptr;
         unsigned *done = nullptr;
         Outliers out{};
+    Coarse low{};
         SsArgs ss{};
     } type[2];
     ~ExactData() {
@@ -1116,6 +1209,9 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
     const size_t fb = place((size_t)nbb * nchb), fa = place((size_t)nba * ncha);
     const size_t part = place((size_t)Y.batch * 2 * kScaleBlocks * 8), info = place(8 * (size_t)Y.batch), tab = place(12);
     const size_t thr = place(8 * (size_t)Y.batch), count = place(4 * (size_t)Y.batch), list = place(8 * (size_t)Y.batch * kOutliers);
+    const size_t need = place(4 * (size_t)Y.batch), lows = place(4 * (size_t)Y.batch);
+    Y.low.limit = PR == 0 ? (unsigned)(la * lb / kCoarseShare) : 0;
+    const size_t lowl = place(4 * (size_t)Y.batch * Y.low.limit);
     const size_t planes = place((size_t)Y.batch * NSC * la * lbp * 2);
     if (charge(ctx, at, "digit tables") != TBSCI_OK) return TBSCI_OK;
     cudaError_t e = Y.arena.alloc(at);
@@ -1132,9 +1228,12 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
         Y.tab = reinterpret_cast<int *>(B + tab);
         Y.done = reinterpret_cast<unsigned *>(B + done);
         Y.out = {reinterpret_cast<double *>(B + thr), reinterpret_cast<int *>(B + count), reinterpret_cast<int64_t *>(B + list)};
+        Y.low.need = reinterpret_cast<float *>(B + need);
+        Y.low.count = reinterpret_cast<unsigned *>(B + lows);
+        Y.low.list = reinterpret_cast<int32_t *>(B + lowl);
         unsigned long long *tp = reinterpret_cast<unsigned long long *>(B + top);
         auto blocks = [](size_t n) { return (unsigned)std::min<size_t>(152, (n + 255) / 256); };
-        k_absmax<<<blocks((size_t)P->npair * P->npair), 256, 0, st>>>(ham->d_V.p, (int64_t)P->npair * P->npair, tp);
+        k_absmax_off<<<blocks((size_t)P->npair * P->npoff), 256, 0, st>>>(ham->d_V.p, P->npair, P->npoff, P->d_offpair.p, tp);
         for (const SpinPlan *sp : {&P->A, &P->B}) {
             if (sp->d_sval.n) k_absmax<<<blocks(sp->d_sval.n), 256, 0, st>>>(sp->d_sval.p, (int64_t)sp->d_sval.n, tp + 1);
             if (sp->d_dval.n) k_absmax<<<blocks(sp->d_dval.n), 256, 0, st>>>(sp->d_dval.p, (int64_t)sp->d_dval.n, tp + 1);
@@ -1183,11 +1282,11 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
 
 UdArgs<double> ud_args(const tbsci_ham *ham, const Plan *P, double) {
     return {P->A.l, P->B.l, nullptr, nullptr, nullptr, P->A.d_str, P->A.d_soff, P->A.d_sci.p, P->A.d_sval.p, P->A.d_E.p,
-            P->B.d_E.p, P->d_U.p, ham->ecore, P->A.nelec, 0};
+            P->B.d_E.p, P->d_U.p, ham->ecore, P->A.nelec, 0, P->A.d_svalf.p, nullptr, {}};
 }
 UdArgs<float> ud_args(const tbsci_ham *ham, const Plan *P, float) {
     return {P->A.l, P->B.l, nullptr, nullptr, nullptr, P->A.d_str, P->A.d_soff, P->A.d_sci.p, P->A.d_svalf.p, P->A.d_Ef.p,
-            P->B.d_Ef.p, P->d_Uf.p, (float)ham->ecore, P->A.nelec, 0};
+            P->B.d_Ef.p, P->d_Uf.p, (float)ham->ecore, P->A.nelec, 0, nullptr, nullptr, {}};
 }
 
 }  // namespace
@@ -1236,9 +1335,10 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
     auto kss = k_same_spin_ex<PR>;
     TB_CUDA(ctx, cudaFuncSetAttribute(kss, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem));
     UdArgs<T> U = ud_args(ham, P, T(0));
-    U.info = Y.info;
+    U.info = U.flag = Y.info;
+    U.R = Y.low;
     AbArgs A{};
-    const OutlierArgs out{Y.out, lb, P->A.d_str, P->A.d_soff, P->A.d_doff, P->B.d_soff, P->B.d_doff,
+    const OutlierArgs out{Y.out, Y.low, lb, P->A.d_str, P->A.d_soff, P->A.d_doff, P->B.d_soff, P->B.d_doff,
                    P->A.d_sci.p, P->B.d_sci.p, P->A.d_sval.p, P->B.d_sval.p, P->A.d_dval.p, P->B.d_dval.p, ham->d_V.p,
                    P->A.d_dcol.p, P->B.d_dcol.p, P->npair};
     size_t ab_smem = 0;
@@ -1271,23 +1371,26 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
         const T *cv = c + (size_t)v * la * lb;
         T *sv = s + (size_t)v * la * lb;
         {
-            TraceScope tr(ctx, "k_slice", st);
+            TraceScope tr(ctx, "k_scale", st);
             const unsigned nb = (unsigned)std::min<int64_t>(kScaleBlocks, (la * lb + 4 * kScaleThreads - 1) / (4 * kScaleThreads));
             k_scale<T><<<dim3(nb, (unsigned)nv), kScaleThreads, 0, st>>>(cv, la * lb, Prec<PR>::kRatio, PR == 0 ? kOutlierMaxN : 0,
-                                                                        Y.part, Y.done, Y.tab, Y.info, Y.out);
-            if constexpr (PR == 0) {
-                const unsigned ns = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (lbp / 8) + 255) / 256);
-                k_slice<<<dim3(ns, (unsigned)nv), 256, 0, st>>>(cv, la, lb, lbp, Y.info, Y.out, Y.planes);
-            }
+                                                                        Y.part, Y.done, Y.tab, Y.info, Y.out, Y.low);
             TB_CUDA(ctx, cudaGetLastError());
         }
-        if constexpr (PR == 1) TB_TRY(sigma_tc_planes(ctx, P, cv, nv, Y.info, Y.planes, st));
         {
             TraceScope tr(ctx, "k_udiag", st);
             U.C = cv;
             U.S = sv;
-            k_udiag<T, false><<<ud_grid(la, lb, nv), 256, 0, st>>>(U);
+            k_udiag<T, false, PR == 0><<<ud_grid(la, lb, nv), 256, 0, st>>>(U);
             TB_CUDA(ctx, cudaGetLastError());
+        }
+        if constexpr (PR == 0) {
+            TraceScope tr(ctx, "k_slice", st);
+            const unsigned ns = (unsigned)std::min<int64_t>(8ll * ctx->num_sms, (la * (lbp / 8) + 255) / 256);
+            k_slice<<<dim3(ns, (unsigned)nv), 256, 0, st>>>(cv, la, lb, lbp, Y.info, Y.out, Y.planes);
+            TB_CUDA(ctx, cudaGetLastError());
+        } else {
+            TB_TRY(sigma_tc_planes(ctx, P, cv, nv, Y.info, Y.planes, st));
         }
         {
             TraceScope tr(ctx, "k_same_spin_ex", st);
@@ -1327,8 +1430,8 @@ tbsci_status udiag_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, c
     U.S = s;
     U.add = add;
     TraceScope tr(ctx, "k_udiag", st);
-    if (singles) k_udiag<float, true><<<ud_grid(P->A.l, P->B.l, nv), 256, 0, st>>>(U);
-    else k_udiag<float, false><<<ud_grid(P->A.l, P->B.l, nv), 256, 0, st>>>(U);
+    if (singles) k_udiag<float, true, false><<<ud_grid(P->A.l, P->B.l, nv), 256, 0, st>>>(U);
+    else k_udiag<float, false, false><<<ud_grid(P->A.l, P->B.l, nv), 256, 0, st>>>(U);
     TB_CUDA(ctx, cudaGetLastError());
     return TBSCI_OK;
 }

@@ -54,13 +54,14 @@ def _graded(sp, decades, rng):
     return C / np.linalg.norm(C), np.unique(np.concatenate([_rows(sp.ndet, 11, 1500), top]))
 
 
-@pytest.mark.parametrize("dtype", ["f32"])
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
 @pytest.mark.parametrize("n,na,nb,la,lb,decades", [
     (11, 5, 5, None, None, 0.8),
     (11, 5, 5, None, None, 1.0),
     (11, 5, 5, None, None, 1.5),
     (16, 8, 8, 700, 650, 1.0),
     (16, 8, 8, 700, 650, 1.5),
+    (16, 8, 8, 1500, 1400, 1.5),  # more CTAs than run at once
 ])
 def test_small_elements_keep_their_accuracy(tb, ctx, n, na, nb, la, lb, decades, dtype):
     """Vectors that decay by orders of magnitude per excitation, as CI vectors do: every element
@@ -75,7 +76,7 @@ def test_small_elements_keep_their_accuracy(tb, ctx, n, na, nb, la, lb, decades,
     sp.close()
 
 
-@pytest.mark.parametrize("dtype", ["f32"])
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
 @pytest.mark.parametrize("decades", [0.0, 0.5])
 def test_small_integrals_keep_their_accuracy(tb, ctx, decades, dtype):
     """Integrals that spread over five decades from orbital to orbital: elements whose links are
