@@ -19,6 +19,10 @@ tbsci_status charge(tbsci_ctx *ctx, size_t bytes, const char *what) {
     if (!ctx || bytes == 0) return TBSCI_OK;
     size_t cur = ctx->hbm_used.load();
     for (;;) {
+        if (ctx->hbm_budget && cur + bytes > ctx->hbm_budget && spare_reclaim(ctx)) {
+            cur = ctx->hbm_used.load();
+            continue;
+        }
         if (ctx->hbm_budget && cur + bytes > ctx->hbm_budget)
             return fail(ctx, TBSCI_ENOMEM,
                         std::string(what) + ": " + std::to_string(bytes) + " device bytes would exceed the context's "
@@ -29,6 +33,60 @@ tbsci_status charge(tbsci_ctx *ctx, size_t bytes, const char *what) {
 
 void uncharge(tbsci_ctx *ctx, size_t bytes) {
     if (ctx && bytes) ctx->hbm_used.fetch_sub(std::min(bytes, ctx->hbm_used.load()));
+}
+
+bool spare_charge(tbsci_ctx *ctx, size_t bytes) {
+    size_t held = ctx->spare_used.load();
+    do {
+        const size_t room = ctx->spare_room.load();
+        if (held > room || bytes > room - held) return false;
+    } while (!ctx->spare_used.compare_exchange_weak(held, held + bytes));
+    size_t cur = ctx->hbm_used.load();
+    do {
+        if (ctx->hbm_budget && cur + bytes > ctx->hbm_budget) {
+            ctx->spare_used.fetch_sub(bytes);
+            return false;
+        }
+    } while (!ctx->hbm_used.compare_exchange_weak(cur, cur + bytes));
+    return true;
+}
+
+void spare_uncharge(tbsci_ctx *ctx, size_t bytes) {
+    ctx->spare_used.fetch_sub(bytes);
+    uncharge(ctx, bytes);
+}
+
+namespace {
+std::mutex spare_mu;
+std::vector<Spare *> spares;
+}  // namespace
+
+void Spare::enlist() {
+    std::lock_guard<std::mutex> g(spare_mu);
+    spares.push_back(this);
+}
+
+void Spare::retire() {
+    std::lock_guard<std::mutex> g(spare_mu);
+    for (size_t i = 0; i < spares.size(); ++i)
+        if (spares[i] == this) {
+            spares[i] = spares.back();
+            spares.pop_back();
+            return;
+        }
+}
+
+bool spare_reclaim(tbsci_ctx *ctx) {
+    int dev = -1;
+    if (!ctx && cudaGetDevice(&dev) != cudaSuccess) return false;
+    bool freed = false;
+    std::lock_guard<std::mutex> g(spare_mu);
+    for (Spare *s : spares) {
+        if (ctx ? s->ctx != ctx : s->ctx->device != dev) continue;
+        std::unique_lock<std::mutex> lk(s->mu, std::try_to_lock);
+        if (lk.owns_lock()) freed |= s->give_back();
+    }
+    return freed;
 }
 
 constexpr size_t kTraceCap = 1 << 16;  // launches held before the oldest unread ones are dropped

@@ -2,7 +2,6 @@
 #pragma once
 
 #include <cuda_bf16.h>
-#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -29,6 +28,32 @@ tbsci_status fail(tbsci_ctx *ctx, tbsci_status st, const std::string &msg);
 // uncharge() gives them back when the object is freed.
 tbsci_status charge(tbsci_ctx *ctx, size_t bytes, const char *what);
 void uncharge(tbsci_ctx *ctx, size_t bytes);
+
+// Spare memory: device memory that only makes calls faster (digit tables, planes of c, link
+// lists of classes, a second part layout). It counts against the budget like any other, but
+// whoever needs room for something required takes it back: charge() before it refuses, and a
+// device allocation that fails. Its holder works without it and may make it again.
+// spare_charge: false, nothing counted and no error recorded, where there is no room.
+bool spare_charge(tbsci_ctx *ctx, size_t bytes);
+void spare_uncharge(tbsci_ctx *ctx, size_t bytes);
+struct Spare {
+    tbsci_ctx *const ctx;
+    std::mutex mu;  // held while launches that use the memory are enqueued
+    explicit Spare(tbsci_ctx *c) : ctx(c) {}
+    Spare(const Spare &) = delete;
+    Spare &operator=(const Spare &) = delete;
+    virtual ~Spare() = default;
+    // waits for the last use, frees, takes the bytes off the count (mu is held);
+    // false where it holds nothing
+    virtual bool give_back() = 0;
+
+  protected:
+    void enlist();  // at the end of the holder's constructor
+    void retire();  // at the start of its destructor
+};
+// Takes back what is not being enqueued at the moment: of one context, or (NULL) of all on
+// the current device. True where something was freed. Not to be called with a Spare's mu held.
+bool spare_reclaim(tbsci_ctx *ctx);
 
 // A failed device allocation returns ENOMEM (the context stays usable); any
 // other CUDA error returns ECUDA.
@@ -68,11 +93,16 @@ struct DevBuf {
         view = false;
     }
     // n is set only once the allocation succeeded: a failed alloc leaves an
-    // empty buffer (p == nullptr, n == 0), so a later size check re-allocates
-    cudaError_t alloc(size_t count) {
+    // empty buffer (p == nullptr, n == 0), so a later size check re-allocates.
+    // spare: for spare memory (above), which takes none back from others
+    cudaError_t alloc(size_t count, bool spare = false) {
         release();
         if (count == 0) return cudaSuccess;
         cudaError_t e = cudaMalloc((void **)&p, count * sizeof(T));
+        if (e == cudaErrorMemoryAllocation && !spare && spare_reclaim(nullptr)) {
+            cudaGetLastError();
+            e = cudaMalloc((void **)&p, count * sizeof(T));
+        }
         if (e != cudaSuccess) {
             p = nullptr;
             return e;
@@ -127,6 +157,7 @@ struct tbsci_ctx {
     // bytes they hold now, Davidson mode when no options are given, tune-cache file
     size_t hbm_budget = 0;
     std::atomic<size_t> hbm_used{0};
+    std::atomic<size_t> spare_used{0}, spare_room{SIZE_MAX};  // spare bytes held, and at most to be held
     int default_mixed = 0;
     std::string tune_path;
     cudaStream_t stream = nullptr;
@@ -323,6 +354,7 @@ struct tbsci_pruned {
     tbsci::DevBuf<int32_t> d_rows;  // alpha rows ordered by work (descending)
     std::vector<int64_t> h_off;
     size_t charged = 0;
+    std::unique_ptr<tbsci::Spare> classes;  // holds what follows
     // Classes of alpha rows with equal I_w (none when ncls == 0): the links of every
     // class's columns into every class's columns, as positions in the compressed rows,
     // in sliced-ELL slices of 32 consecutive members (see pruned.cu).
@@ -447,6 +479,8 @@ tbsci_status rest_products_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P,
 // cuBLAS handle is released by dense_context_release.
 tbsci_status rest_dense_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const float *c, float *s, int nvec,
                                bool bf16, cudaStream_t st);
+// device bytes that rest_dense_launch would still take for this plan
+size_t rest_dense_bytes(const Plan *P, bool bf16);
 void dense_context_release(tbsci_ctx *ctx);
 // sigma_exact.cu: FP64 / FP32 sigma summed exactly on the tensor cores (norb <= 16);
 // *ran = false where it does not apply. simt(v, nv, skip) launches the SIMT sigma of

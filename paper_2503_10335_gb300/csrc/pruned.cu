@@ -555,6 +555,8 @@ tbsci_status launch_pruned(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, 
     if (pr->nd == 0 || A.la == 0) return TBSCI_OK;
     // rows in classes: the warps of a CTA take 32 members each, so a row of a few
     // hundred members runs on 4 warps and many CTAs share an SM
+    std::unique_lock<std::mutex> lk;
+    if (pr->classes) lk = std::unique_lock<std::mutex>(pr->classes->mu);
     const int cls_threads = pr->cmax > 1024 ? 512 : pr->cmax > 256 ? 256 : 128;
     if (pr->ncls > 0 && nvec <= 65535 && cls_smem_bytes<T>(A.npair, pr->cmax, cls_threads) <= ctx->smem_optin) {
         ClsArgs K{pr->ncls, pr->cmax, pr->d_cls.p, pr->d_ccnt.p, pr->d_pos.p, pr->d_ov.p, pr->d_sbase.p, pr->d_dbase.p,
@@ -570,6 +572,7 @@ tbsci_status launch_pruned(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, 
         TB_CUDA(ctx, cudaGetLastError());
         return TBSCI_OK;
     }
+    if (lk.owns_lock()) lk.unlock();
     const size_t head = pr_head_bytes<T>(A.npair), full = head + (size_t)A.lb * sizeof(T);
     const bool expand = full <= ctx->smem_optin;
     for (int v = 0; v < nvec; ++v) {
@@ -587,6 +590,43 @@ tbsci_status launch_pruned(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, 
     }
     return TBSCI_OK;
 }
+
+// The lists of a pruned space's classes as spare memory; without them the space runs on the
+// general kernel.
+struct ClassLists : Spare {
+    tbsci_pruned *const pr;
+    size_t charged = 0;
+    ClassLists(tbsci_ctx *c, tbsci_pruned *p) : Spare(c), pr(p) {}
+    void publish() { enlist(); }  // once the lists are there
+    ~ClassLists() override {
+        retire();
+        spare_uncharge(ctx, charged);
+    }
+    void release() {
+        pr->ncls = 0;
+        pr->d_cls.release();
+        pr->d_cbeg.release();
+        pr->d_ccnt.release();
+        pr->d_pos.release();
+        pr->d_ov.release();
+        pr->d_sbase.release();
+        pr->d_dbase.release();
+        pr->d_s_off.release();
+        pr->d_d_off.release();
+        pr->d_s_w.release();
+        pr->d_d_w.release();
+        pr->d_s_ci.release();
+        pr->d_s_li.release();
+        pr->d_d_ent.release();
+    }
+    bool give_back() override {
+        if (pr->ncls == 0 || cudaDeviceSynchronize() != cudaSuccess) return false;
+        release();
+        spare_uncharge(ctx, charged);
+        charged = 0;
+        return true;
+    }
+};
 
 // Groups the alpha rows by equal I_w and lists the links between the classes on the
 // device. Not more than kMaxClasses classes (their pair tables grow with the square),
@@ -627,10 +667,11 @@ tbsci_status build_classes(tbsci_ctx *ctx, const tbsci_tables *a, const tbsci_ta
     const size_t left = ctx->hbm_budget ? ctx->hbm_budget - std::min(ctx->hbm_budget, ctx->hbm_used.load()) : SIZE_MAX;
     if (fixed > left / 8) return TBSCI_OK;
     cudaStream_t st = ctx->stream;
+    auto lists = std::make_unique<ClassLists>(ctx, pr);
     DevBuf<int64_t> s_cnt, d_cnt;
     cudaError_t e = cudaSuccess;
     auto need = [&](auto &buf, size_t n) {
-        if (e == cudaSuccess) e = buf.alloc(n);
+        if (e == cudaSuccess) e = buf.alloc(n, true);
     };
     auto put = [&](auto &buf, const auto &h) {
         need(buf, h.size());
@@ -670,7 +711,7 @@ tbsci_status build_classes(tbsci_ctx *ctx, const tbsci_tables *a, const tbsci_ta
         if (e == cudaSuccess) e = cudaMemcpy(&tot[1], pr->d_d_off.p + nds, 8, cudaMemcpyDeviceToHost);
     }
     const size_t bytes = fixed + 8 * (size_t)(tot[0] + tot[1]);
-    const bool fits = e == cudaSuccess && ret == TBSCI_OK && bytes <= left / 8 && charge(ctx, bytes, "pruned space classes") == TBSCI_OK;
+    const bool fits = e == cudaSuccess && ret == TBSCI_OK && bytes <= left / 8 && spare_charge(ctx, bytes);
     if (fits) {
         need(pr->d_s_ci, std::max<int64_t>(tot[0], 1));
         need(pr->d_s_li, std::max<int64_t>(tot[0], 1));
@@ -686,26 +727,14 @@ tbsci_status build_classes(tbsci_ctx *ctx, const tbsci_tables *a, const tbsci_ta
         if (e == cudaSuccess) {
             pr->ncls = ncls;
             pr->cmax = cmax;
-            pr->charged += bytes;
+            lists->charged = bytes;
+            lists->publish();
+            pr->classes = std::move(lists);
             return TBSCI_OK;
         }
-        uncharge(ctx, bytes);
+        spare_uncharge(ctx, bytes);
     }
-    // without the tables the space runs on the general kernel
-    pr->d_cls.release();
-    pr->d_cbeg.release();
-    pr->d_ccnt.release();
-    pr->d_pos.release();
-    pr->d_ov.release();
-    pr->d_sbase.release();
-    pr->d_dbase.release();
-    pr->d_s_off.release();
-    pr->d_d_off.release();
-    pr->d_s_w.release();
-    pr->d_d_w.release();
-    pr->d_s_ci.release();
-    pr->d_s_li.release();
-    pr->d_d_ent.release();
+    lists->release();
     cudaGetLastError();  // a failed allocation is not the caller's error
     return e == cudaSuccess || e == cudaErrorMemoryAllocation ? TBSCI_OK
                                                                : fail(ctx, TBSCI_ECUDA, std::string("pruned space classes: ") + cudaGetErrorString(e));
@@ -838,6 +867,7 @@ tbsci_status tbsci_pruned_count(const tbsci_pruned *pr, int64_t *ndet) {
 void tbsci_pruned_destroy(tbsci_pruned *pr) {
     if (!pr) return;
     if (pr->ctx) cudaSetDevice(pr->ctx->device);
+    pr->classes.reset();  // nothing is taken back from here on
     uncharge(pr->ctx, pr->charged);
     delete pr;
 }

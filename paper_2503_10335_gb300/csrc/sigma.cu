@@ -1076,6 +1076,8 @@ tbsci_status autotune_rest(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *plan, con
     // timed on one. Mode 5 is skipped when its dense matrices do not fit the
     // context's budget or the device (the failed set-up leaves the plan as it was).
     for (int mode = 4; mode <= 5 && ret == TBSCI_OK; ++mode) {
+        // a trial does not drive out what other calls keep: no room beside that, no trial
+        if (mode == 5 && ctx->hbm_budget && ctx->hbm_used.load() + rest_dense_bytes(plan, bf16) > ctx->hbm_budget) continue;
         float ms = 0.f;
         tbsci_status r5 = timed([&] { return sigma_launch_rest(ctx, ham, plan, c, s, nvec, st, mode, 256, nullptr, 0,
                                                                bf16); }, 1, &ms);

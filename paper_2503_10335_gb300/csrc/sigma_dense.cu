@@ -145,6 +145,13 @@ tbsci_status ensure_dense(tbsci_ctx *ctx, Plan *P, bool bf16, cudaStream_t st) {
 
 }  // namespace
 
+size_t rest_dense_bytes(const Plan *P, bool bf16) {
+    const size_t lap = (size_t)padded(P->A.l), lbp = (size_t)padded(P->B.l);
+    const DenseSameSpin &D = P->dense;
+    const size_t held = bf16 ? D.a_bf.n : D.a_hi.n, scratch = lap * lbp * (bf16 ? 6 : 12);
+    return (held ? 0 : (bf16 ? 2 : 8) * (lap * lap + lbp * lbp)) + (scratch > D.scratch.n ? scratch - D.scratch.n : 0);
+}
+
 tbsci_status rest_dense_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const float *c, float *s, int nvec,
                                bool bf16, cudaStream_t st) {
     (void)ham;

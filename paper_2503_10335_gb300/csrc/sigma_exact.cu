@@ -1141,16 +1141,16 @@ bool plane_map(CUtensorMap *m, void *base, int64_t cols, int64_t rows, int plane
 
 }  // namespace
 
-// What the exact path keeps for one prepared space and precision, in one allocation made
-// by the first sigma that takes it. Calls on several streams share the digit planes of
-// c, so each call waits for the event that the one before it recorded; `mu` keeps the
+// What the exact path keeps for one prepared space and precision, in one allocation of spare
+// memory made by the first sigma that takes it. Calls on several streams share the digit planes
+// of c, so each call waits for the event that the one before it recorded; `mu` keeps the
 // launches of one call together.
-struct ExactData {
-    std::mutex mu;
+struct ExactData : Spare {
     struct Type {
         bool tried = false, ready = false;
         int batch = 1;  // vectors per launch
         cudaEvent_t busy = nullptr;
+        size_t charged = 0;
         DevBuf<unsigned char> arena;
         uint4 *Vd = nullptr, *Wd = nullptr;
         __nv_bfloat16 *planes = nullptr;  // digit planes of `batch` vectors
@@ -1158,12 +1158,28 @@ struct ExactData {
         int *info = nullptr, *tab = nullptr;
         unsigned *done = nullptr;
         Outliers out{};
-    Coarse low{};
+        Coarse low{};
         SsArgs ss{};
     } type[2];
-    ~ExactData() {
-        for (Type &t : type)
+    explicit ExactData(tbsci_ctx *x) : Spare(x) { enlist(); }
+    ~ExactData() override {
+        retire();
+        for (Type &t : type) {
+            spare_uncharge(ctx, t.charged);
             if (t.busy) cudaEventDestroy(t.busy);
+        }
+    }
+    bool give_back() override {
+        bool freed = false;
+        for (Type &t : type) {
+            if (!t.arena.p || cudaEventSynchronize(t.busy) != cudaSuccess) continue;
+            t.arena.release();
+            spare_uncharge(ctx, t.charged);
+            t.charged = 0;
+            t.tried = t.ready = false;
+            freed = true;
+        }
+        return freed;
     }
 };
 
@@ -1186,11 +1202,13 @@ int ab_stage_bytes(const tbsci_ctx *ctx, const Plan *P) {
 template <int PR>
 tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData *X, cudaStream_t st) {
     typename ExactData::Type &Y = X->type[PR];
-    Y.tried = true;
     using Sh = SsShape<PR>;
     const int64_t la = P->A.l, lb = P->B.l, lap = pad64(la), lbp = pad64(lb);
     constexpr int NSA = Prec<PR>::NSA, NSC = Prec<PR>::NSC;
-    if ((PR == 0 ? ab_stage_bytes(ctx, P) == 0 : !sigma_tc_serves(ctx, P, 3)) || !encode_tiled()) return TBSCI_OK;
+    if ((PR == 0 ? ab_stage_bytes(ctx, P) == 0 : !sigma_tc_serves(ctx, P, 3)) || !encode_tiled()) {
+        Y.tried = true;
+        return TBSCI_OK;
+    }
     const int ncha = (int)((la + 31) / 32), nchb = (int)((lb + 31) / 32);
     const int64_t nba = (la + 127) / 128, nbb = (lb + Sh::NT - 1) / Sh::NT;
     Y.batch = sigma_tc_batch(P);
@@ -1213,9 +1231,11 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
     Y.low.limit = PR == 0 ? (unsigned)(la * lb / kCoarseShare) : 0;
     const size_t lowl = place(4 * (size_t)Y.batch * Y.low.limit);
     const size_t planes = place((size_t)Y.batch * NSC * la * lbp * 2);
-    if (charge(ctx, at, "digit tables") != TBSCI_OK) return TBSCI_OK;
-    cudaError_t e = Y.arena.alloc(at);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&Y.busy, cudaEventDisableTiming);
+    if (!spare_charge(ctx, at)) return TBSCI_OK;  // asked for again by the next call
+    Y.tried = true;
+    Y.charged = at;
+    cudaError_t e = Y.busy ? cudaSuccess : cudaEventCreateWithFlags(&Y.busy, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = Y.arena.alloc(at, true);
     unsigned char *B = Y.arena.p;
     if (e == cudaSuccess) e = cudaMemsetAsync(B, 0, zeroed, st);
     SsArgs &S = Y.ss;
@@ -1261,12 +1281,12 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
                       plane_map(&S.mCB, Y.planes, lbp, la, NSC, 64, 32, Y.batch);
     if (!maps) {
         Y.arena.release();
-        uncharge(ctx, at);
+        Y.charged = 0;
+        spare_uncharge(ctx, at);
         cudaGetLastError();
         return e == cudaSuccess || e == cudaErrorMemoryAllocation ? TBSCI_OK
                                                                    : fail(ctx, TBSCI_ECUDA, std::string("digit tables: ") + cudaGetErrorString(e));
     }
-    P->charged += at;
     S.la = la;
     S.lb = lb;
     S.nchb = nchb;
@@ -1276,6 +1296,7 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
     S.info = Y.info;
     S.tab = Y.tab;
     S.err = P->d_tc_err.p;
+    TB_CUDA(ctx, cudaEventRecord(Y.busy, st));  // other streams wait for the tables
     Y.ready = true;
     return TBSCI_OK;
 }
@@ -1323,7 +1344,7 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
     {
         static std::mutex make;
         std::lock_guard<std::mutex> g(make);
-        if (!P->exact) P->exact = std::make_shared<ExactData>();
+        if (!P->exact) P->exact = std::make_shared<ExactData>(ctx);
     }
     ExactData *X = P->exact.get();
     std::lock_guard<std::mutex> g(X->mu);
@@ -1366,6 +1387,12 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
     }
     *ran = true;
     TB_CUDA(ctx, cudaStreamWaitEvent(st, Y.busy, 0));
+    // whatever became of the launches, the next user of the tables waits for those made
+    struct Record {
+        cudaEvent_t e;
+        cudaStream_t st;
+        ~Record() { cudaEventRecord(e, st); }
+    } record{Y.busy, st};
     for (int v = 0, nv = 0; v < nvec; v += nv) {
         nv = std::min(Y.batch, nvec - v);
         const T *cv = c + (size_t)v * la * lb;
@@ -1409,7 +1436,6 @@ tbsci_status exact_launch_t(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const
         }
         TB_TRY(simt(v, nv, Y.info, out));
     }
-    TB_CUDA(ctx, cudaEventRecord(Y.busy, st));
     return TBSCI_OK;
 }
 

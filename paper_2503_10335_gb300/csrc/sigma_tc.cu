@@ -537,33 +537,41 @@ tbsci_status tile_links_build(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, cud
     return TBSCI_OK;
 }
 
-// The planes of c of one space and number of planes, made by the first sigma that has
-// room for them. Calls on several streams share them: each waits for the event that the
-// one before it recorded, and `mu` keeps the launches of one call together.
-struct AbPlanes {
-    std::mutex mu;
+// The planes of c of one space and number of planes (spare memory), made by the first sigma
+// that has room for them. Calls on several streams share them: each waits for the event that
+// the one before it recorded, and `mu` keeps the launches of one call together.
+struct AbPlanes : Spare {
     cudaEvent_t busy = nullptr;
     bool tried = false;
     DevBuf<__nv_bfloat16> c;  // planes of sigma_tc_batch vectors
-    ~AbPlanes() {
+    explicit AbPlanes(tbsci_ctx *x) : Spare(x) { enlist(); }
+    ~AbPlanes() override {
+        retire();
+        spare_uncharge(ctx, c.bytes());
         if (busy) cudaEventDestroy(busy);
+    }
+    bool give_back() override {
+        if (!c.p || cudaEventSynchronize(busy) != cudaSuccess) return false;
+        spare_uncharge(ctx, c.bytes());
+        c.release();
+        tried = false;
+        return true;
     }
 };
 
 namespace {
 
-tbsci_status build_planes(tbsci_ctx *ctx, Plan *P, int np, AbPlanes *X) {
-    X->tried = true;
+tbsci_status build_planes(tbsci_ctx *ctx, const Plan *P, int np, AbPlanes *X) {
     const size_t n = (size_t)sigma_tc_batch(P) * np * P->A.l * pad64(P->B.l), bytes = n * sizeof(__nv_bfloat16);
-    if (charge(ctx, bytes, "planes of the alpha-beta products") != TBSCI_OK) return TBSCI_OK;
-    cudaError_t e = cudaEventCreateWithFlags(&X->busy, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = X->c.alloc(n);
+    if (!spare_charge(ctx, bytes)) return TBSCI_OK;  // asked for again by the next call
+    X->tried = true;
+    cudaError_t e = X->busy ? cudaSuccess : cudaEventCreateWithFlags(&X->busy, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = X->c.alloc(n, true);
     if (e != cudaSuccess) {
-        uncharge(ctx, bytes);
+        spare_uncharge(ctx, bytes);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? TBSCI_OK : fail(ctx, TBSCI_ECUDA, std::string("alpha-beta planes: ") + cudaGetErrorString(e));
     }
-    P->charged += bytes;
     return TBSCI_OK;
 }
 
@@ -649,7 +657,7 @@ tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float 
     {
         static std::mutex make;
         std::lock_guard<std::mutex> g(make);
-        if (!own) own = std::make_shared<AbPlanes>();
+        if (!own) own = std::make_shared<AbPlanes>(ctx);
     }
     std::lock_guard<std::mutex> g(own->mu);
     if (!own->tried) TB_TRY(build_planes(ctx, P, np, own.get()));

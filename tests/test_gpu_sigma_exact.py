@@ -247,3 +247,58 @@ def test_towering_elements(tb, ctx, la, lb, k):
     rows = np.unique(np.concatenate([_rows(sp.ndet, 9), near, [a * sp.lb + b for a, b in at]]))
     _check(s.cpu().numpy(), osp, h, eri, C, rows)
     sp.close()
+
+
+@pytest.mark.parametrize("kind", ["f64", "f32", "tf32", "pruned"])
+def test_tables_make_room(tb, kind):
+    """What a sigma keeps to be faster (digit tables, planes, class lists) gives way to what a
+    later call cannot do without: under a budget that holds the space and the vectors of that
+    call alone, the call runs, and the sigma after it agrees with the one before."""
+    import torch
+
+    def make(budget):
+        ctx = tb.Context(0, hbm_budget=budget)
+        sp, _, h, eri = _space(tb, ctx, 13, 6, 6, 640, 630, seed=781)
+        pr = None
+        if kind == "pruned":
+            a, b = sp.strings()
+            keep = (np.bitwise_count(a >> np.uint64(6)).astype(int)[:, None] + np.bitwise_count(b >> np.uint64(6))) <= 6
+            pr = sp.prune(np.concatenate([[0], np.cumsum(keep.sum(1))]).astype(np.int64), np.nonzero(keep)[1].astype(np.int32))
+        return ctx, sp, pr
+    ctx, sp, pr = make(0)
+    need = tb.tbsci_hbm_used(ctx.handle)
+    nvec = 24  # the host call's buffers: 155 MB, more than any of the tables
+    H = np.random.default_rng(9).standard_normal((nvec, sp.la, sp.lb))
+    want = sp.sigma_host(H)
+    sp.close()
+    ctx.close()
+    extra = 1 << 16
+    while pr:  # the space alone: under the smallest budget that it fits, there is no room for its lists
+        try:
+            ctx, sp, small = make(need // 2 + extra)
+        except tb.B.TbsciError:
+            extra += extra // 4
+            continue
+        need = tb.tbsci_hbm_used(ctx.handle)
+        small.close()
+        sp.close()
+        ctx.close()
+        break
+    ctx, sp, pr = make(need + 2 * H.nbytes)
+    before = tb.tbsci_hbm_used(ctx.handle)
+    assert (before > need) == (kind == "pruned")
+    dt = {"f64": (torch.float64, None), "pruned": (torch.float64, None), "f32": (torch.float32, None),
+          "tf32": (torch.float32, tb.TBSCI_F32_TC_TF32)}[kind]
+    c = torch.randn((1, pr.ndet) if pr else (1, sp.la, sp.lb), dtype=dt[0], device="cuda")
+    sigma = (lambda: pr.sigma(c)) if pr else (lambda: sp.sigma(c, dtype=dt[1]))
+    first = sigma()
+    assert tb.tbsci_hbm_used(ctx.handle) > need
+    got = sp.sigma_host(H)
+    assert np.abs(got - want).max() <= 1e-11 * np.abs(want).max()
+    again = sigma()
+    assert torch.linalg.vector_norm(again - first) <= (1e-13 if dt[0] == torch.float64 else 2e-6) * torch.linalg.vector_norm(first)
+    if pr:
+        pr.close()
+    sp.close()
+    assert tb.tbsci_hbm_used(ctx.handle) <= 2 * H.nbytes  # the host call's buffers, which the context keeps
+    ctx.close()
