@@ -36,24 +36,11 @@ void uncharge(tbsci_ctx *ctx, size_t bytes) {
 }
 
 bool spare_charge(tbsci_ctx *ctx, size_t bytes) {
-    size_t held = ctx->spare_used.load();
-    do {
-        const size_t room = ctx->spare_room.load();
-        if (held > room || bytes > room - held) return false;
-    } while (!ctx->spare_used.compare_exchange_weak(held, held + bytes));
     size_t cur = ctx->hbm_used.load();
     do {
-        if (ctx->hbm_budget && cur + bytes > ctx->hbm_budget) {
-            ctx->spare_used.fetch_sub(bytes);
-            return false;
-        }
+        if (ctx->hbm_budget && cur + bytes > ctx->hbm_budget) return false;
     } while (!ctx->hbm_used.compare_exchange_weak(cur, cur + bytes));
     return true;
-}
-
-void spare_uncharge(tbsci_ctx *ctx, size_t bytes) {
-    ctx->spare_used.fetch_sub(bytes);
-    uncharge(ctx, bytes);
 }
 
 namespace {

@@ -35,7 +35,6 @@ void uncharge(tbsci_ctx *ctx, size_t bytes);
 // device allocation that fails. Its holder works without it and may make it again.
 // spare_charge: false, nothing counted and no error recorded, where there is no room.
 bool spare_charge(tbsci_ctx *ctx, size_t bytes);
-void spare_uncharge(tbsci_ctx *ctx, size_t bytes);
 struct Spare {
     tbsci_ctx *const ctx;
     std::mutex mu;  // held while launches that use the memory are enqueued
@@ -157,7 +156,6 @@ struct tbsci_ctx {
     // bytes they hold now, Davidson mode when no options are given, tune-cache file
     size_t hbm_budget = 0;
     std::atomic<size_t> hbm_used{0};
-    std::atomic<size_t> spare_used{0}, spare_room{SIZE_MAX};  // spare bytes held, and at most to be held
     int default_mixed = 0;
     std::string tune_path;
     cudaStream_t stream = nullptr;
@@ -339,6 +337,7 @@ struct Plan {
     std::shared_ptr<ExactData> exact;  // tables of the exact tensor-core path, made on first use
     tbsci_sigma_counts counts{};
     size_t charged = 0;  // device bytes counted against the context's budget
+    bool no_spare = false;  // its sigma takes no spare memory (set before the first one)
 };
 
 }  // namespace tbsci
@@ -500,7 +499,9 @@ tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float 
                          const int *info, cudaStream_t st, const __nv_bfloat16 *planes);
 tbsci_status sigma_tc_planes(tbsci_ctx *ctx, const Plan *P, const float *c, int nv, const int *info, __nv_bfloat16 *out,
                              cudaStream_t st);
-int sigma_tc_batch(const Plan *P);
+int sigma_tc_batch(int64_t ndet);
+size_t sigma_tc_device_bytes(int norb, int64_t la, int64_t lb, int np);
+size_t exact_device_bytes(int norb, int64_t la, int64_t lb, int type);
 tbsci_status diagonal_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan, double *diag,
                              cudaStream_t st, bool tables);
 

@@ -600,7 +600,7 @@ struct ClassLists : Spare {
     void publish() { enlist(); }  // once the lists are there
     ~ClassLists() override {
         retire();
-        spare_uncharge(ctx, charged);
+        uncharge(ctx, charged);
     }
     void release() {
         pr->ncls = 0;
@@ -622,7 +622,7 @@ struct ClassLists : Spare {
     bool give_back() override {
         if (pr->ncls == 0 || cudaDeviceSynchronize() != cudaSuccess) return false;
         release();
-        spare_uncharge(ctx, charged);
+        uncharge(ctx, charged);
         charged = 0;
         return true;
     }
@@ -732,7 +732,7 @@ tbsci_status build_classes(tbsci_ctx *ctx, const tbsci_tables *a, const tbsci_ta
             pr->classes = std::move(lists);
             return TBSCI_OK;
         }
-        spare_uncharge(ctx, bytes);
+        uncharge(ctx, bytes);
     }
     lists->release();
     cudaGetLastError();  // a failed allocation is not the caller's error

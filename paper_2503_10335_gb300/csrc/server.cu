@@ -48,6 +48,7 @@ struct Req {
     bool full_a = false, full_b = false;
     double t_submit = 0, t_admit = -1, t_first = -1;
     size_t bytes = 0;
+    bool no_spare = false;  // the budget has no room for the tables that its sigma would keep
     int64_t la = 0, lb = 0;
     tbsci_strings *sa = nullptr, *sb = nullptr;
     tbsci_tables *ta = nullptr, *tb = nullptr;
@@ -160,6 +161,7 @@ struct tbsci_server {
         TB_TRY(tbsci_build_excitation_tables(c, q.sb, 0, &q.tb));
         TB_TRY(tbsci_hamiltonian_create(c, q.r.norb, q.h.data(), q.eri.data(), q.r.ecore, &q.ham));
         TB_TRY(tbsci::plan_get(c, q.ham, q.ta, q.tb, &q.plan));
+        q.plan->no_spare = q.no_spare;
         // small solves get the highest stream priority: the block scheduler then
         // prefers their CTAs over the queued CTAs of large solves
         const bool small = (double)q.la * (double)q.lb * q.r.nroots <= (double)big_job_det;
@@ -410,6 +412,18 @@ tbsci_status tbsci_submit(tbsci_server *srv, const tbsci_request *req, uint64_t 
     o.mixed = r.mixed;
     q->bytes = spin_bytes(r.norb, r.nalpha, q->la) + spin_bytes(r.norb, r.nbeta, q->lb) +
                tbsci::engine_device_bytes(q->la * q->lb, r.nroots, &o) + (size_t)r.norb * r.norb * 64 * (q->lb + 64);
+    // What its sigma keeps to be faster counts too, and where the budget has no room for it
+    // the solve does without: by the request alone, so that a result does not depend on
+    // what else runs. Solves whose sigma always goes into the batched launches keep nothing
+    // (the tensor-core types have planes of c there too).
+    size_t spare = 0;
+    if (srv->opts.fuse_sigma < 0 || (double)q->la * (double)q->lb * r.nroots > (double)srv->big_job_det) {
+        spare += tbsci::exact_device_bytes(r.norb, q->la, q->lb, 0);
+        if (r.mixed == 1) spare += tbsci::exact_device_bytes(r.norb, q->la, q->lb, 1);
+    }
+    if (r.mixed >= 2) spare += tbsci::sigma_tc_device_bytes(r.norb, q->la, q->lb, r.mixed == 3 ? 1 : 3);
+    if (q->bytes + spare <= srv->opts.hbm_budget) q->bytes += spare;
+    else q->no_spare = true;
     std::lock_guard<std::mutex> lk(srv->mu);
     if (srv->stop) return TBSCI_EBUSY;
     if ((int)srv->queue.size() >= srv->opts.max_queue) return TBSCI_EAGAIN;

@@ -1486,7 +1486,7 @@ tbsci_status sigma_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *plan
             return launch_typed<float>(ctx, ham, plan, cf, sf, nvec, st);
         TB_TRY(sigma_launch_rest(ctx, ham, plan, cf, sf, nvec, st, -1, 0, nullptr, 0, np == 1));
         const size_t n = (size_t)plan->A.l * plan->B.l;
-        const int batch = sigma_tc_batch(plan);
+        const int batch = sigma_tc_batch((int64_t)n);
         for (int v = 0; v < nvec; v += batch) {
             const int nv = std::min(batch, nvec - v);
             TB_TRY(udiag_launch(ctx, ham, plan, cf + v * n, sf + v * n, nv, true, true, st));

@@ -1165,7 +1165,7 @@ struct ExactData : Spare {
     ~ExactData() override {
         retire();
         for (Type &t : type) {
-            spare_uncharge(ctx, t.charged);
+            uncharge(ctx, t.charged);
             if (t.busy) cudaEventDestroy(t.busy);
         }
     }
@@ -1174,7 +1174,7 @@ struct ExactData : Spare {
         for (Type &t : type) {
             if (!t.arena.p || cudaEventSynchronize(t.busy) != cudaSuccess) continue;
             t.arena.release();
-            spare_uncharge(ctx, t.charged);
+            uncharge(ctx, t.charged);
             t.charged = 0;
             t.tried = t.ready = false;
             freed = true;
@@ -1197,6 +1197,47 @@ int ab_stage_bytes(const tbsci_ctx *ctx, const Plan *P) {
     return room < one ? 0 : (int)std::min<int64_t>(room, 4 * (int64_t)one);
 }
 
+// Places in the allocation of one precision, 256-byte aligned, and its size
+struct Places {
+    size_t hb, ha, top, done, zeroed, vd, wd, cb, ca, fb, fa, part, info, tab, thr, count, list, need, lows, lowl, planes, bytes;
+};
+template <int PR>
+Places places_of(int64_t la, int64_t lb, int npair) {
+    constexpr int NSA = Prec<PR>::NSA, NSC = Prec<PR>::NSC, NT = SsShape<PR>::NT;
+    const size_t batch = (size_t)sigma_tc_batch(la * lb), lap = (size_t)pad64(la), lbp = (size_t)pad64(lb);
+    const size_t ncha = (size_t)(la + 31) / 32, nchb = (size_t)(lb + 31) / 32;
+    Places p;
+    size_t at = 0;
+    auto place = [&](size_t n) {
+        const size_t q = at;
+        at += (n + 255) / 256 * 256;
+        return q;
+    };
+    p.hb = place(NSA * lb * lbp * 2);
+    p.ha = place(NSA * la * lap * 2);
+    p.top = place(16);
+    p.done = place(4 * batch);
+    p.zeroed = at;
+    p.vd = place(PR == 0 ? (size_t)npair * 128 * sizeof(uint4) : 0);
+    p.wd = place(PR == 0 ? (size_t)la * 128 * sizeof(uint4) : 0);
+    p.cb = place(lb * nchb);
+    p.ca = place(la * ncha);
+    p.fb = place((size_t)(lb + NT - 1) / NT * nchb);
+    p.fa = place((size_t)(la + 127) / 128 * ncha);
+    p.part = place(batch * 2 * kScaleBlocks * 8);
+    p.info = place(8 * batch);
+    p.tab = place(12);
+    p.thr = place(8 * batch);
+    p.count = place(4 * batch);
+    p.list = place(8 * batch * kOutliers);
+    p.need = place(4 * batch);
+    p.lows = place(4 * batch);
+    p.lowl = place(PR == 0 ? 4 * batch * (size_t)(la * lb / kCoarseShare) : 0);
+    p.planes = place(batch * NSC * la * lbp * 2);
+    p.bytes = at;
+    return p;
+}
+
 // Digit tables of the Hamiltonian for one precision, enqueued on `st`; without room for
 // them the space stays on the SIMT kernels.
 template <int PR>
@@ -1211,26 +1252,10 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
     }
     const int ncha = (int)((la + 31) / 32), nchb = (int)((lb + 31) / 32);
     const int64_t nba = (la + 127) / 128, nbb = (lb + Sh::NT - 1) / Sh::NT;
-    Y.batch = sigma_tc_batch(P);
-    // places in the allocation, 256-byte aligned
-    size_t at = 0;
-    auto place = [&](size_t n) {
-        const size_t p = at;
-        at += (n + 255) / 256 * 256;
-        return p;
-    };
-    const size_t hb = place((size_t)NSA * lb * lbp * 2), ha = place((size_t)NSA * la * lap * 2);
-    const size_t top = place(16), done = place(4 * (size_t)Y.batch), zeroed = at;
-    const size_t vd = place(PR == 0 ? (size_t)P->npair * 128 * sizeof(uint4) : 0);
-    const size_t wd = place(PR == 0 ? (size_t)la * 128 * sizeof(uint4) : 0);
-    const size_t cb = place((size_t)lb * nchb), ca = place((size_t)la * ncha);
-    const size_t fb = place((size_t)nbb * nchb), fa = place((size_t)nba * ncha);
-    const size_t part = place((size_t)Y.batch * 2 * kScaleBlocks * 8), info = place(8 * (size_t)Y.batch), tab = place(12);
-    const size_t thr = place(8 * (size_t)Y.batch), count = place(4 * (size_t)Y.batch), list = place(8 * (size_t)Y.batch * kOutliers);
-    const size_t need = place(4 * (size_t)Y.batch), lows = place(4 * (size_t)Y.batch);
+    Y.batch = sigma_tc_batch(la * lb);
     Y.low.limit = PR == 0 ? (unsigned)(la * lb / kCoarseShare) : 0;
-    const size_t lowl = place(4 * (size_t)Y.batch * Y.low.limit);
-    const size_t planes = place((size_t)Y.batch * NSC * la * lbp * 2);
+    const auto [hb, ha, top, done, zeroed, vd, wd, cb, ca, fb, fa, part, info, tab, thr, count, list, need, lows, lowl, planes, at] =
+        places_of<PR>(la, lb, P->npair);
     if (!spare_charge(ctx, at)) return TBSCI_OK;  // asked for again by the next call
     Y.tried = true;
     Y.charged = at;
@@ -1282,7 +1307,7 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
     if (!maps) {
         Y.arena.release();
         Y.charged = 0;
-        spare_uncharge(ctx, at);
+        uncharge(ctx, at);
         cudaGetLastError();
         return e == cudaSuccess || e == cudaErrorMemoryAllocation ? TBSCI_OK
                                                                    : fail(ctx, TBSCI_ECUDA, std::string("digit tables: ") + cudaGetErrorString(e));
@@ -1322,9 +1347,17 @@ UdArgs<float> ud_args(const tbsci_ham *ham, const Plan *P, float) {
 template <typename T>
 bool exact_eligible(const Plan *P) {
     const int64_t la = P->A.l, lb = P->B.l;
-    if (P->tl_kpmax == 0 || la < 32 || lb < 2 * kAbTile || la > 32768 || lb > 32768) return false;
+    if (P->no_spare || P->tl_kpmax == 0 || la < 32 || lb < 2 * kAbTile || la > 32768 || lb > 32768) return false;
     if (P->tune_stage[sizeof(T) == 8 ? 0 : 1] >= 3) return false;  // a shape of the split path was asked for
     return la * lb >= (int64_t(1) << 14);
+}
+
+// Spare bytes that sigma of a type (0 FP64, 1 FP32) takes on a space of these sizes; an upper
+// bound, without a look at its links
+size_t exact_device_bytes(int norb, int64_t la, int64_t lb, int type) {
+    if (norb < 2 || norb > 16 || la < 32 || lb < 2 * kAbTile || la > 32768 || lb > 32768 || la * lb < (int64_t(1) << 14)) return 0;
+    const int npair = norb * (norb + 1) / 2;
+    return type == 0 ? places_of<0>(la, lb, npair).bytes : places_of<1>(la, lb, npair).bytes;
 }
 
 // sigma of the vectors c -> s; *ran = false (and nothing launched) where the path does

@@ -495,8 +495,13 @@ int fp_stage_bytes(const tbsci_ctx *ctx, const Plan *P, int np) {
 
 // Vectors per launch: small spaces share the launches with up to eight (up to 2^24
 // determinants together).
-int sigma_tc_batch(const Plan *P) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>(8, (int64_t(1) << 24) / std::max<int64_t>(1, P->A.l * P->B.l)));
+int sigma_tc_batch(int64_t ndet) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(8, (int64_t(1) << 24) / std::max<int64_t>(1, ndet)));
+}
+
+// Spare bytes that a tensor-core type takes on a space of these sizes: planes of c
+size_t sigma_tc_device_bytes(int norb, int64_t la, int64_t lb, int np) {
+    return norb < 2 || norb > 16 ? 0 : (size_t)sigma_tc_batch(la * lb) * np * la * pad64(lb) * sizeof(__nv_bfloat16);
 }
 
 // Link plan of a space (norb <= 16) and planes of its integrals, made when the space is prepared; left out
@@ -547,12 +552,12 @@ struct AbPlanes : Spare {
     explicit AbPlanes(tbsci_ctx *x) : Spare(x) { enlist(); }
     ~AbPlanes() override {
         retire();
-        spare_uncharge(ctx, c.bytes());
+        uncharge(ctx, c.bytes());
         if (busy) cudaEventDestroy(busy);
     }
     bool give_back() override {
         if (!c.p || cudaEventSynchronize(busy) != cudaSuccess) return false;
-        spare_uncharge(ctx, c.bytes());
+        uncharge(ctx, c.bytes());
         c.release();
         tried = false;
         return true;
@@ -562,13 +567,13 @@ struct AbPlanes : Spare {
 namespace {
 
 tbsci_status build_planes(tbsci_ctx *ctx, const Plan *P, int np, AbPlanes *X) {
-    const size_t n = (size_t)sigma_tc_batch(P) * np * P->A.l * pad64(P->B.l), bytes = n * sizeof(__nv_bfloat16);
+    const size_t n = (size_t)sigma_tc_batch(P->A.l * P->B.l) * np * P->A.l * pad64(P->B.l), bytes = n * sizeof(__nv_bfloat16);
     if (!spare_charge(ctx, bytes)) return TBSCI_OK;  // asked for again by the next call
     X->tried = true;
     cudaError_t e = X->busy ? cudaSuccess : cudaEventCreateWithFlags(&X->busy, cudaEventDisableTiming);
     if (e == cudaSuccess) e = X->c.alloc(n, true);
     if (e != cudaSuccess) {
-        spare_uncharge(ctx, bytes);
+        uncharge(ctx, bytes);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? TBSCI_OK : fail(ctx, TBSCI_ECUDA, std::string("alpha-beta planes: ") + cudaGetErrorString(e));
     }
@@ -649,8 +654,9 @@ tbsci_status sigma_tc_ab(tbsci_ctx *ctx, Plan *P, int np, const float *c, float 
                          const int *info, cudaStream_t st, const __nv_bfloat16 *planes) {
     if (planes) return ab_launch<3>(ctx, P, planes, c, s, nv, info, st);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
+    const cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e != cudaSuccess) cudaGetLastError();
+    if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone || P->no_spare) {
         return np == 1 ? ab_add<1>(ctx, P, nullptr, c, s, nv, info, st) : ab_add<3>(ctx, P, nullptr, c, s, nv, info, st);
     }
     std::shared_ptr<AbPlanes> &own = P->ab[np == 1 ? 0 : 1];

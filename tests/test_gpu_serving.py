@@ -195,3 +195,30 @@ def test_tensor_core_mixed_requests_in_the_mix(tb):
         assert np.max(np.abs(np.array(d["energies"]) - w)) < 1e-8, (r["mixed"], d["energies"], w)
         if r["mixed"]:
             assert d["nsigma_f32"] > 0
+
+
+def test_budget_decides_on_tables(tb):
+    """The tables that a large solve's sigma keeps to be faster count at admission. Under a
+    budget that its vectors fill, the solve does without: other kernels, other last bits, the
+    same energies; and a request that fitted before is not refused."""
+    h, eri, _ = synth_hamiltonian(12, seed=5013)
+    req = dict(norb=12, nalpha=6, nbeta=6, h=h, eri=eri, ecore=0.0, alpha=None, beta=None, nroots=2, mixed=False)
+
+    def solve(budget):
+        srv = tb.Server(0, hbm_budget=budget)
+        try:
+            return _solve_all(srv, [req])[0]
+        finally:
+            srv.close()
+    lo, hi = 1 << 20, 4 << 30  # refused, accepted
+    while hi - lo > 1 << 20:
+        mid = (lo + hi) // 2
+        if solve(mid)["status"] == tb.TBSCI_ENOMEM:
+            lo = mid
+        else:
+            hi = mid
+    tight, roomy, again = solve(hi), solve(0), solve(hi)
+    assert tight["status"] == 0 and roomy["status"] == 0
+    bits = lambda d: (list(d["energies"][:2]), list(d["residual"][:2]))  # noqa: E731
+    assert bits(tight) == bits(again) and bits(tight) != bits(roomy)
+    assert np.max(np.abs(np.array(tight["energies"][:2]) - np.array(roomy["energies"][:2]))) < 1e-8
