@@ -258,7 +258,7 @@ struct SpinPlan {
 // padding entries point at the part's first column with a zero coefficient.
 // U is the beta Coulomb table with its columns in `perm` order.
 struct PartLayout {
-    int P = 0, elem = 0;  // column parts; element bytes the link order is for
+    int P = 0;  // column parts
     int64_t W = 0;
     DevBuf<int32_t> perm, iperm;  // column order and its inverse
     DevBuf<int64_t> off;          // [nslices * P]
@@ -267,6 +267,9 @@ struct PartLayout {
     DevBuf<uint32_t> ci;
     DevBuf<double> val;           // same-spin string-Hamiltonian value
     DevBuf<float> valf;
+    // the links in another order for FP32 (spare memory, see k_spread_links); valf goes with it
+    DevBuf<uint32_t> ci4;
+    bool ci4_failed = false;      // the device had no room for it
     DevBuf<uint64_t> str;         // beta string of each column, in perm order
     DevBuf<double> Eb;            // its one-electron energy, same order
     DevBuf<float> Ebf;
@@ -327,6 +330,7 @@ struct Plan {
     // split path for rows longer than shared memory: part layouts by part count,
     // and the transposed c / sigma scratch of the beta-double class
     std::vector<std::unique_ptr<PartLayout>> parts;
+    std::unique_ptr<Spare> link_order;  // of the layouts' ci4
     DevBuf<unsigned char> d_trans;
     // same-spin beta links (singles, then doubles, per source string) with FP32
     // values: the beta classes of the tensor-core types' product pass
@@ -478,6 +482,8 @@ tbsci_status rest_products_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P,
 // cuBLAS handle is released by dense_context_release.
 tbsci_status rest_dense_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const float *c, float *s, int nvec,
                                bool bf16, cudaStream_t st);
+// sigma_split.cu
+std::unique_ptr<Spare> make_link_order(tbsci_ctx *ctx, Plan *P);
 // device bytes that rest_dense_launch would still take for this plan
 size_t rest_dense_bytes(const Plan *P, bool bf16);
 void dense_context_release(tbsci_ctx *ctx);

@@ -273,6 +273,7 @@ tbsci_status plan_get(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *a, con
     plan->idb = b->id;
     plan->norb = ham->norb;
     plan->npair = ham->npair;
+    plan->link_order = make_link_order(ctx, plan.get());
     plan->npoff = ham->norb * (ham->norb - 1) / 2;
     const int64_t la = a->count, lb = b->count, np = ham->npair, nsl = (lb + 31) / 32;
     // schedules: beta columns by their single-link count and by all their links, alpha rows

@@ -332,11 +332,10 @@ __global__ void k_combine(T *y, const T *__restrict__ pz, const int32_t *__restr
 // pipe and gained nothing (432 and 431 ms at 10,000 x 40,000).
 constexpr int kSpread = 64;
 __global__ void __launch_bounds__(32) k_spread_links(const int64_t *__restrict__ off, const int32_t *__restrict__ w, uint32_t *ci,
-                                                     double *val, float *valf) {
-    __shared__ double buf[kSpread * 33];  // ci, then val, then valf, of kSpread links x 32 lanes
+                                                     float *valf) {
+    __shared__ float bf[kSpread * 33];  // ci, then valf, of kSpread links x 32 lanes
     __shared__ uint8_t take[kSpread * 33];
-    uint32_t *code = reinterpret_cast<uint32_t *>(buf);
-    float *bf = reinterpret_cast<float *>(buf);
+    uint32_t *code = reinterpret_cast<uint32_t *>(bf);
     const int lane = threadIdx.x;
     const int64_t o = off[blockIdx.x] + lane;
     const int wide = w[blockIdx.x];
@@ -388,10 +387,6 @@ __global__ void __launch_bounds__(32) k_spread_links(const int64_t *__restrict__
         __syncwarp();
         for (int k = 0; k < n; ++k) ci[at + 32 * k] = code[take[k * 33 + lane] * 33 + lane];
         __syncwarp();
-        for (int k = 0; k < n; ++k) buf[k * 33 + lane] = val[at + 32 * k];
-        __syncwarp();
-        for (int k = 0; k < n; ++k) val[at + 32 * k] = buf[take[k * 33 + lane] * 33 + lane];
-        __syncwarp();
         for (int k = 0; k < n; ++k) bf[k * 33 + lane] = valf[at + 32 * k];
         __syncwarp();
         for (int k = 0; k < n; ++k) valf[at + 32 * k] = bf[take[k * 33 + lane] * 33 + lane];
@@ -399,17 +394,59 @@ __global__ void __launch_bounds__(32) k_spread_links(const int64_t *__restrict__
     }
 }
 
-// Part layout of the beta single links for `nparts` column parts (built on the host) and
-// elements of `elem` bytes.
-tbsci_status build_parts(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int nparts, int elem, PartLayout **out) {
-    PartLayout *other = nullptr;  // the same parts in the other type's order
+__global__ void k_round_values(const double *__restrict__ val, int64_t n, float *valf) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) valf[i] = (float)val[i];
+}
+
+// The FP32 link orders of a plan's layouts
+struct LinkOrder : Spare {
+    Plan *const P;
+    LinkOrder(tbsci_ctx *c, Plan *p) : Spare(c), P(p) { enlist(); }
+    ~LinkOrder() override {
+        retire();
+        for (auto &pl : P->parts) uncharge(ctx, pl->ci4.bytes());
+    }
+    // makes the order of a layout where there is room (mu is held); on the default stream,
+    // behind the copies of the layout
+    tbsci_status make(PartLayout *pl, int64_t nslices) {
+        const size_t bytes = pl->ci.bytes();
+        if (pl->ci4.p || pl->ci4_failed || bytes == 0 || P->no_spare || !spare_charge(ctx, bytes)) return TBSCI_OK;
+        cudaError_t e = pl->ci4.alloc(pl->ci.n, true);
+        if (e == cudaSuccess) {
+            e = cudaMemcpy(pl->ci4.p, pl->ci.p, bytes, cudaMemcpyDeviceToDevice);
+            if (e == cudaSuccess) {
+                k_spread_links<<<(unsigned)(nslices * pl->P), 32>>>(pl->off.p, pl->w.p, pl->ci4.p, pl->valf.p);
+                e = cudaGetLastError();
+            }
+            if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+            if (e == cudaSuccess) return TBSCI_OK;
+            pl->ci4.release();
+        }
+        pl->ci4_failed = true;
+        uncharge(ctx, bytes);
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? TBSCI_OK : fail(ctx, TBSCI_ECUDA, std::string("link order: ") + cudaGetErrorString(e));
+    }
+    bool give_back() override {
+        bool freed = false;
+        for (auto &pl : P->parts) {
+            if (!pl->ci4.p || cudaDeviceSynchronize() != cudaSuccess) continue;
+            k_round_values<<<608, 256>>>(pl->val.p, (int64_t)pl->valf.n, pl->valf.p);  // back in ci's order
+            if (cudaStreamSynchronize(nullptr) != cudaSuccess) continue;
+            uncharge(ctx, pl->ci4.bytes());
+            pl->ci4.release();
+            freed = true;
+        }
+        return freed;
+    }
+};
+
+// Part layout of the beta single links for `nparts` column parts (built on the host).
+tbsci_status build_parts(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int nparts, PartLayout **out) {
     for (auto &pl : P->parts)
         if (pl->P == nparts) {
-            if (pl->elem == elem) {
-                *out = pl.get();
-                return TBSCI_OK;
-            }
-            other = pl.get();
+            *out = pl.get();
+            return TBSCI_OK;
         }
     const int64_t lb = P->B.l, nsl = (lb + 31) / 32;
     const int64_t W = (lb + nparts - 1) / nparts;
@@ -485,14 +522,9 @@ tbsci_status build_parts(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int npar
     }
     auto pl = std::make_unique<PartLayout>();
     pl->P = nparts;
-    pl->elem = elem;
     pl->W = W;
     const size_t bytes = loff.size() * 12 + ci.size() * (sizeof(uint32_t) + 12) + (size_t)lb * 28;
-    if (other && charge(ctx, bytes, "column-part link layout") != TBSCI_OK) {  // no room for a second one
-        *out = other;
-        return TBSCI_OK;
-    }
-    if (!other) TB_TRY(charge(ctx, bytes, "column-part link layout"));
+    TB_TRY(charge(ctx, bytes, "column-part link layout"));
     cudaError_t e = pl->off.alloc(loff.size());
     if (e == cudaSuccess) e = pl->w.alloc(lw.size());
     if (e == cudaSuccess) e = pl->ci.alloc(ci.size());
@@ -515,11 +547,6 @@ tbsci_status build_parts(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int npar
     if (e == cudaSuccess) e = cudaMemcpy(pl->str.p, pstr.data(), lb * sizeof(uint64_t), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(pl->Eb.p, pE.data(), lb * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(pl->Ebf.p, pEf.data(), lb * sizeof(float), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && total > 0 && elem == 4) {  // on the default stream, after the copies
-        k_spread_links<<<(unsigned)(nsl * nparts), 32>>>(pl->off.p, pl->w.p, pl->ci.p, pl->val.p, pl->valf.p);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
-    }
     if (e != cudaSuccess) {
         uncharge(ctx, bytes);
         return fail(ctx, e == cudaErrorMemoryAllocation ? TBSCI_ENOMEM : TBSCI_ECUDA,
@@ -527,6 +554,7 @@ tbsci_status build_parts(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, int npar
     }
     P->charged += bytes;
     *out = pl.get();
+    std::lock_guard<std::mutex> g(P->link_order->mu);  // which walks over the layouts
     P->parts.push_back(std::move(pl));
     return TBSCI_OK;
 }
@@ -639,6 +667,8 @@ int split_min_parts(const tbsci_ctx *ctx, int npair, int norb, int64_t lb, size_
     return (int)std::max<int64_t>(1, (lb + wmax - 1) / wmax);
 }
 
+std::unique_ptr<Spare> make_link_order(tbsci_ctx *ctx, Plan *P) { return std::make_unique<LinkOrder>(ctx, P); }
+
 // mode 0: the whole sigma; 1: K1 alone on the listed alpha rows (a tuning
 // sample; its output is scratch); 2: K2, K3 and the combine alone (the part of
 // the time that does not depend on the K1 shape; sigma is not meaningful)
@@ -663,7 +693,7 @@ tbsci_status split_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const T
     TB_CHECK(ctx, (la + 31) / 32 <= 65535, TBSCI_EINVAL, "split sigma: too many alpha strings");
     nparts = (int)std::min<int64_t>(lb, nparts);
     PartLayout *pl = nullptr;
-    TB_TRY(build_parts(ctx, ham, P, nparts, (int)sizeof(T), &pl));
+    TB_TRY(build_parts(ctx, ham, P, nparts, &pl));
     const size_t need = 2 * (size_t)la * lb * sizeof(T);
     if (P->d_trans.n < need) {
         uncharge(ctx, P->d_trans.bytes());
@@ -678,7 +708,13 @@ tbsci_status split_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const T
         }
         P->charged += need;
     }
+    std::unique_lock<std::mutex> lk;
+    if (sizeof(T) == 4) {  // its own link order, held while the launches are enqueued
+        lk = std::unique_lock<std::mutex>(P->link_order->mu);
+        TB_TRY(static_cast<LinkOrder *>(P->link_order.get())->make(pl, (lb + 31) / 32));
+    }
     SplitArgs<T> A = split_args<T>(ham, P, pl);
+    if (sizeof(T) == 4 && pl->ci4.p) A.pci = pl->ci4.p;
     A.NC = nc;
     if (rows) {
         A.rowsa = rows;

@@ -140,3 +140,42 @@ def test_link_order_of_fp32_layout(tb, tmp_path, n, na, nb, acnt, bcnt):
     assert_sigma_close(s, ref, bound, rel=64 * 2.0 ** -24, norm_rel=1e-5)
     sp.close()
     ctx.close()
+
+
+def test_link_order_gives_way(tb, tmp_path):
+    """One layout serves both types; the FP32 order of its links is kept only where there is
+    room. A host call that needs the room gets it, the FP32 sigma after it agrees with the one
+    before, and the FP64 sigma has the same bits whether an FP32 one ran or not."""
+    import torch
+    n, la, lb = 14, 90, 3432
+    h, eri, _ = synth_hamiltonian(n, seed=97)
+    asel = selected_strings(n, 7, la, 98)
+    path = tmp_path / "tune.txt"
+    path.write_text("tbsci-tune 1\n%d %d %d 512 1 3 512 1 3 0 0\n" % (n, la, lb))
+    c = torch.randn((1, la, lb), dtype=torch.float64, device="cuda")
+    H = np.random.default_rng(1).standard_normal((2, la, lb))
+
+    def make(budget):
+        ctx = tb.Context(0, hbm_budget=budget)
+        tb.tbsci_tune_cache_load(ctx.handle, str(path))
+        return ctx, tb.Space(ctx, n, 7, 7, h, eri, 0.0, alpha=asel)
+    ctx, sp = make(0)
+    want = sp.sigma(c)
+    torch.cuda.synchronize()
+    want_host = sp.sigma_host(H)
+    need = tb.tbsci_hbm_used(ctx.handle)  # space, layout, scratch, host buffers
+    sp.close()
+    ctx.close()
+    ctx, sp = make(need)
+    assert torch.equal(sp.sigma(c), want)
+    without = tb.tbsci_hbm_used(ctx.handle)
+    f32 = sp.sigma(c.float())
+    torch.cuda.synchronize()
+    assert tb.tbsci_hbm_used(ctx.handle) > without
+    assert np.array_equal(sp.sigma_host(H), want_host)
+    assert tb.tbsci_hbm_used(ctx.handle) == need
+    again = sp.sigma(c.float())
+    assert torch.linalg.vector_norm(again - f32) <= 2e-6 * torch.linalg.vector_norm(f32)
+    assert torch.equal(sp.sigma(c), want)
+    sp.close()
+    ctx.close()
