@@ -332,6 +332,12 @@ struct Plan {
     std::vector<std::unique_ptr<PartLayout>> parts;
     std::unique_ptr<Spare> link_order;  // of the layouts' ci4
     DevBuf<unsigned char> d_trans;
+    // d_trans and dense.scratch are shared by all streams: see ScratchUse
+    std::mutex scratch_mu;
+    cudaEvent_t scratch_busy = nullptr;
+    ~Plan() {
+        if (scratch_busy) cudaEventDestroy(scratch_busy);
+    }
     // same-spin beta links (singles, then doubles, per source string) with FP32
     // values: the beta classes of the tensor-core types' product pass
     DevBuf<int64_t> d_bss_off;
@@ -482,6 +488,34 @@ tbsci_status rest_products_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P,
 // cuBLAS handle is released by dense_context_release.
 tbsci_status rest_dense_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const float *c, float *s, int nvec,
                                bool bf16, cudaStream_t st);
+// While it lives, the launches of one call that use a plan's scratch are enqueued on `st`: they
+// wait for the last call's, on whichever stream that was, and the next call's wait for them.
+// On a stream being captured nothing is ordered: a graph that uses the scratch must not run
+// beside other calls on its space.
+class ScratchUse {
+  public:
+    ScratchUse(Plan *P, cudaStream_t st) : P_(P), st_(st), lock_(P->scratch_mu) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+        else free_ = cap == cudaStreamCaptureStatusNone;
+        if (!free_) return;
+        if (!P->scratch_busy) err_ = cudaEventCreateWithFlags(&P->scratch_busy, cudaEventDisableTiming);
+        if (err_ == cudaSuccess) err_ = cudaStreamWaitEvent(st, P->scratch_busy, 0);
+    }
+    ~ScratchUse() {
+        if (free_ && P_->scratch_busy) cudaEventRecord(P_->scratch_busy, st_);
+    }
+    ScratchUse(const ScratchUse &) = delete;
+    ScratchUse &operator=(const ScratchUse &) = delete;
+    cudaError_t error() const { return err_; }
+
+  private:
+    Plan *P_;
+    cudaStream_t st_;
+    std::lock_guard<std::mutex> lock_;
+    bool free_ = false;
+    cudaError_t err_ = cudaSuccess;
+};
 // sigma_split.cu
 std::unique_ptr<Spare> make_link_order(tbsci_ctx *ctx, Plan *P);
 // device bytes that rest_dense_launch would still take for this plan

@@ -164,6 +164,8 @@ tbsci_status rest_dense_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, co
     // padded product, all lap x lbp
     const size_t np = (size_t)lap * lbp;
     const size_t need = np * (bf16 ? 2 + 4 : 3 * 4);
+    const ScratchUse use(P, st);
+    TB_CUDA(ctx, use.error());
     DevBuf<unsigned char> &scr = P->dense.scratch;
     if (scr.n < need) {
         uncharge(ctx, scr.bytes());

@@ -695,6 +695,8 @@ tbsci_status split_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, const T
     PartLayout *pl = nullptr;
     TB_TRY(build_parts(ctx, ham, P, nparts, &pl));
     const size_t need = 2 * (size_t)la * lb * sizeof(T);
+    const ScratchUse use(P, st);
+    TB_CUDA(ctx, use.error());
     if (P->d_trans.n < need) {
         uncharge(ctx, P->d_trans.bytes());
         P->charged -= std::min(P->charged, P->d_trans.bytes());
@@ -817,6 +819,8 @@ tbsci_status rest_products_launch(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P,
         P->charged += bytes;
     }
     const size_t need = 2 * (size_t)la * lb * sizeof(float);
+    const ScratchUse use(P, st);
+    TB_CUDA(ctx, use.error());
     if (P->d_trans.n < need) {
         uncharge(ctx, P->d_trans.bytes());
         P->charged -= std::min(P->charged, P->d_trans.bytes());

@@ -179,3 +179,36 @@ def test_link_order_gives_way(tb, tmp_path):
     assert torch.equal(sp.sigma(c), want)
     sp.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype,rest", [("f64", 0), ("f32", 0), ("tf32", 4), ("tf32", 5), ("bf16", 5)])
+def test_scratch_on_two_streams(tb, tmp_path, dtype, rest):
+    """Calls on two streams, and the host call on the context's own, share the transposed
+    vectors of the split path and the padded ones of the dense products: each result is what
+    it is alone."""
+    import torch
+    n, la, lb = 14, 300, 3432
+    h, eri, _ = synth_hamiltonian(n, seed=95)
+    path = tmp_path / "tune.txt"
+    path.write_text("tbsci-tune 1\n%d %d %d 512 1 3 512 1 3 %d %d\n" % (n, la, lb, rest, 256 if rest else 0))
+    ctx = tb.Context(0)
+    tb.tbsci_tune_cache_load(ctx.handle, str(path))
+    sp = tb.Space(ctx, n, 7, 7, h, eri, 0.0, alpha=selected_strings(n, 7, la, 96))
+    kind = {"f64": None, "f32": None, "tf32": tb.TBSCI_F32_TC_TF32, "bf16": tb.TBSCI_F32_TC_BF16}[dtype]
+    C = torch.randn((6, la, lb), dtype=torch.float64 if dtype == "f64" else torch.float32, device="cuda")
+    parts = [C[v:v + 1].contiguous() for v in range(6)]
+    want = [sp.sigma(p, dtype=kind) for p in parts]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    outs = [torch.empty_like(p) for p in parts]
+    torch.cuda.synchronize()
+    for v in range(6):
+        sp.sigma(parts[v], outs[v], stream=streams[v % 2], dtype=kind)
+    host = sp.sigma_host(C[:2].double().cpu().numpy()) if dtype == "f64" else None
+    torch.cuda.synchronize()
+    for v in range(6):
+        assert torch.equal(outs[v], want[v]), v
+    if host is not None:
+        assert np.array_equal(host, torch.cat(want[:2]).cpu().numpy())
+    sp.close()
+    ctx.close()
