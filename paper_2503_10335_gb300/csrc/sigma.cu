@@ -1506,7 +1506,7 @@ tbsci_status diagonal_launch(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P
     if (tables && la >= kDiagRows && lb >= 16) {  // narrower rows leave most of a warp's lanes without a column
         const size_t smem = (size_t)((P->norb + 5) / 6) * 64 * 32 * sizeof(double);  // 176 KB at 64 orbitals
         // about eight blocks per SM, 128 to 1024 rows each
-        const int64_t rows = std::max<int64_t>(std::min<int64_t>(std::max<int64_t>(la * ct / (152 * 8), 128), 1024), (la + 65534) / 65535);
+        const int64_t rows = std::max<int64_t>(std::min<int64_t>(std::max<int64_t>(la * ct / (8 * ctx->num_sms), 128), 1024), (la + 65534) / 65535);
         TB_CUDA(ctx, cudaFuncSetAttribute(k_diagonal_tab, cudaFuncAttributeMaxDynamicSharedMemorySize, 180224));
         k_diagonal_tab<<<dim3((unsigned)ct, (unsigned)((la + rows - 1) / rows)), 256, smem, st>>>(
             P->A.d_str, la, lb, P->norb, (int)rows, P->A.d_E.p, P->B.d_E.p, P->d_U.p, ham->ecore, diag);

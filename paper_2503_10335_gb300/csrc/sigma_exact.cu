@@ -123,7 +123,7 @@ __host__ __device__ inline int scale_exponent(double top) {
 }
 
 constexpr int kScaleThreads = 256;
-constexpr int kScaleBlocks = 304;
+constexpr int kScaleBlocks = 304;  // at most, two per SM
 
 // Elements that tower over the rest of a vector (trial vectors of an eigensolver start as
 // single determinants and stay close to them) are kept out of the digits: at most
@@ -1277,7 +1277,7 @@ tbsci_status build_type(tbsci_ctx *ctx, const tbsci_ham *ham, Plan *P, ExactData
         Y.low.count = reinterpret_cast<unsigned *>(B + lows);
         Y.low.list = reinterpret_cast<int32_t *>(B + lowl);
         unsigned long long *tp = reinterpret_cast<unsigned long long *>(B + top);
-        auto blocks = [](size_t n) { return (unsigned)std::min<size_t>(152, (n + 255) / 256); };
+        auto blocks = [&](size_t n) { return (unsigned)std::min<size_t>(ctx->num_sms, (n + 255) / 256); };
         k_absmax_off<<<blocks((size_t)P->npair * P->npoff), 256, 0, st>>>(ham->d_V.p, P->npair, P->npoff, P->d_offpair.p, tp);
         for (const SpinPlan *sp : {&P->A, &P->B}) {
             if (sp->d_sval.n) k_absmax<<<blocks(sp->d_sval.n), 256, 0, st>>>(sp->d_sval.p, (int64_t)sp->d_sval.n, tp + 1);

@@ -431,7 +431,7 @@ struct LinkOrder : Spare {
         bool freed = false;
         for (auto &pl : P->parts) {
             if (!pl->ci4.p || cudaDeviceSynchronize() != cudaSuccess) continue;
-            k_round_values<<<608, 256>>>(pl->val.p, (int64_t)pl->valf.n, pl->valf.p);  // back in ci's order
+            k_round_values<<<4 * ctx->num_sms, 256>>>(pl->val.p, (int64_t)pl->valf.n, pl->valf.p);  // back in ci's order
             if (cudaStreamSynchronize(nullptr) != cudaSuccess) continue;
             uncharge(ctx, pl->ci4.bytes());
             pl->ci4.release();
