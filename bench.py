@@ -73,8 +73,8 @@ NCU_TRAFFIC = {
         "source": "sigma.cu", "sha1": "2e38dd72db29d3137f5f54aee410b1a51db79613",
         "shapes": {(512, 3, 2): 21.10e9}},
     ("sel24", "f64", "k_sigma_parts"): {
-        "source": "sigma_split.cu", "sha1": "bbca57e694e9aafe0b9476961be6286e724c7b3a",
-        "shapes": {(1024, 3): 380.95e9}},
+        "source": "sigma_split.cu", "sha1": "24d825daa0ee7a43ee998bdce498ef0a174db926",
+        "shapes": {(1024, 3): 377.00e9}},
 }
 
 
@@ -142,9 +142,9 @@ def _kernel_work(name, c, nvec, dtype):
         return (35 * 2.0 * noff * c["n1a"] * lb * nvec, "tensor",
                 "2 flops per digit product (35), alpha single, off-diagonal pair kl and beta column per vector")
     if name == "k_same_spin_ex":
-        return ((35 if dtype == "f64" else 10) * 2.0 * la * lb * (la + lb) * nvec, "tensor",
-                "2 flops per digit product (35 in FP64, 10 in FP32) of the dense c Hb^T + Ha c per vector, chunks without a "
-                "link counted though skipped")
+        return ((35 if dtype == "f64" else 6) * 2.0 * la * lb * (la + lb) * nvec, "tensor",
+                "2 flops per product of digits (35 in FP64) or BF16 planes (6 in FP32) of the dense c Hb^T + Ha c per vector, "
+                "chunks without a link counted though skipped")
     if name == "k_udiag":
         return 2.0 * (nd + c["n1a"] * lb) * nvec, "fp", "2 flops per determinant and alpha single's column per vector"
     if name == "k_transpose":

@@ -45,13 +45,18 @@ typedef enum tbsci_status {
     TBSCI_EBUSY = 7     /* object in use */
 } tbsci_status;
 
-/* Arithmetic of a sigma evaluation. F64 and F32: c, sigma and all arithmetic
- * in that type (SIMT). F32_TC_TF32 / F32_TC_BF16: c and sigma FP32; the
- * alpha-beta classes, alpha singles and the diagonal run on the tensor cores
- * with FP32 accumulation, their products from split TF32 (3 products per term,
- * FP32-level accuracy) or from single BF16 values (about 3 significant digits);
- * the other classes on the FP32 SIMT path. Tensor-core modes need norb <= 16
- * and otherwise fall back to F32. */
+/* Arithmetic of a sigma evaluation. F64 and F32: c and sigma in that type; every
+ * element of sigma agrees with the sum of its terms H_IJ c_J to 1e-12 (F64) or
+ * 64 2^-24 (F32) of the sum of their magnitudes, whichever kernels run: SIMT
+ * sums in that type, or, for norb <= 16 from 2^14 determinants on, products on
+ * the tensor cores (F64: exact sums of fixed-point digits, with the elements
+ * that these are too coarse for summed in F64; F32: three BF16 values per
+ * operand, FP32 accumulation). F32_TC_TF32 / F32_TC_BF16: c and sigma FP32; the
+ * alpha-beta classes run on the tensor cores with FP32 accumulation, from three
+ * BF16 values per operand (FP32-level accuracy) or a single one (about 3
+ * significant digits); the diagonal and the alpha singles in FP32, the other
+ * classes on the FP32 SIMT path or as dense products (tuned_rest below).
+ * Tensor-core modes need norb <= 16 and otherwise fall back to F32. */
 typedef enum tbsci_dtype {
     TBSCI_F64 = 0,
     TBSCI_F32 = 1,
@@ -98,7 +103,12 @@ typedef struct tbsci_options {
                                link tables, prepared spaces, Davidson vectors and the
                                buffers of tbsci_sigma_host; a call whose objects would
                                exceed it frees what it made and returns ENOMEM.
-                               0 = no limit */
+                               What calls keep only to be faster (tables and planes
+                               of the tensor-core kernels, link lists of a pruned
+                               space's classes, the FP32 link order of the split
+                               path) counts too, is made only where there is room,
+                               and is given back when a call needs the room (or the
+                               device has none left). 0 = no limit */
     int default_mixed;      /* mixed mode of tbsci_davidson when its opts is NULL
                                (0..3, as tbsci_davidson_opts.mixed) */
     const char *tune_cache; /* NULL, or a tune-cache file (tbsci_tune_cache_save format):
@@ -198,15 +208,24 @@ void tbsci_hamiltonian_destroy(tbsci_ham *ham);
 /* Prepares (and caches inside `ham`) the per-space data sigma needs: string
  * Hamiltonian values of every link, per-string energies, the beta Coulomb
  * table and the work schedules. Called implicitly by tbsci_sigma; exposed to
- * keep set-up out of timed regions. `a` and `b` must have double links and
- * the same norb as `ham`. Errors: EINVAL, ENOMEM, ECUDA. */
+ * keep set-up out of timed regions. What depends on the type is made by the
+ * first sigma of that type: the digit tables (F64) and planes (F32, TF32, BF16)
+ * of the tensor-core kernels, some 14 (l_a^2 + l_b^2) and 17 n bytes (F64) or
+ * 6 (l_a^2 + l_b^2) and 6 n (F32; the others 6 n or 2 n) for the n determinants
+ * of up to eight vectors, and the split path's links. `a` and `b` must have
+ * double links and the same norb as `ham`. Errors: EINVAL, ENOMEM, ECUDA. */
 tbsci_status tbsci_prepare(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *a, const tbsci_tables *b);
 
 /* sigma = H.c over the space a x b (Sec. II.B, Eq. 7, on one device; the six
  * Slater-Condon classes of Sec. II.C, Eq. 8 and Algorithm 1). c and sigma are
  * DEVICE arrays [nvec][l_a][l_b] of `dtype`, must not overlap; sigma is
  * overwritten. Work is enqueued on `stream`; the call returns without waiting.
- * Errors: EINVAL (null pointers, nvec < 1, norb mismatch, tables without
+ * A vector's sigma does not depend on the vectors beside it. On a stream being
+ * captured into a graph, F64 and F32 take the SIMT kernels and the tensor-core
+ * types the same ones as elsewhere (the alpha-beta kernel cuts c into planes
+ * itself, the same bits); a graph that uses the split path or the dense products
+ * shares their scratch with other calls on the space and must not run beside
+ * them. Errors: EINVAL (null pointers, nvec < 1, norb mismatch, tables without
  * double links), ENOMEM, ECUDA. */
 tbsci_status tbsci_sigma(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *a, const tbsci_tables *b,
                          const void *c, void *sigma, int nvec, tbsci_dtype dtype, tbsci_stream stream);
@@ -218,8 +237,12 @@ tbsci_status tbsci_sigma(tbsci_ctx *ctx, tbsci_ham *ham, const tbsci_tables *a, 
  * it) and leaves sigma = H c computed. When one sigma takes 100 ms or more, the
  * shapes are timed on a strided sample of 64 alpha rows per SM (staging and CTA
  * size at one vector per CTA, then the vectors per CTA), else every shape on the
- * whole space. Each column is summed in the same order in every shape, so
- * tuning never changes results. For F32_TC_TF32 / F32_TC_BF16 the tensor-core
+ * whole space. Each column is summed in the same order in every shape of the
+ * fused kernel, so that tuning changes no result of it; the split path (shapes 3
+ * to 6) agrees to rounding. Spaces that other kernels serve (a vector that fits
+ * in shared memory, the tensor-core path) use the shape for captured calls and
+ * where their tables find no room; a shape of the split path, which only a
+ * cache file gives them, takes them off those kernels. For F32_TC_TF32 / F32_TC_BF16 the tensor-core
  * kernel has one shape; the SIMT pass for the classes it leaves out is tuned
  * (shared-memory mode x CTA size) and the whole sigma is then run once.
  * *best_ms: the chosen shape's time on the whole space (may be NULL).

@@ -24,8 +24,9 @@
 // single-link count so a warp's lanes have nearly equal trip counts.
 //
 // Before this kernel (k_sigma) come two others where they apply (launch_full):
-// k_sigma_small for vectors that fit in shared memory, and the exact products on the
-// tensor cores of sigma_exact.cu, whose remaining vectors k_sigma_left serves.
+// k_sigma_small for vectors that fit in shared memory, and the products on the tensor
+// cores of sigma_exact.cu, whose remaining vectors and elements k_sigma_left and
+// k_sigma_repair serve.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -1404,7 +1405,7 @@ namespace {
 
 // k_sigma_small where it applies (*ran): a vector that fits in shared memory, up to the
 // size from which the exact tensor-core path is the faster one (ms, FP64, one vector:
-// 126 x 129 strings 0.047 here, 0.092 there; 150 x 150 0.066, 160 x 155 there 0.109), and no shape of the
+// 126 x 129 strings 0.054 here, 0.092 there; 150 x 150 0.060, 160 x 155 there 0.112), and no shape of the
 // split path asked for
 constexpr int64_t kSmallDets = 24000;
 

@@ -1,4 +1,4 @@
-// sigma = H.c for norb <= 16 on the tensor cores, summed exactly in integers.
+// sigma = H.c for norb <= 16 on the tensor cores: FP64 summed exactly in integers, FP32 from BF16 planes.
 //
 // This GPU's FP64 pipe runs 2 multiply-adds per SM and clock, its BF16 tensor cores
 // 4,096. So the values are cut into 8-bit digits -- an FP64 c into 8, an FP64 matrix
@@ -1339,10 +1339,10 @@ UdArgs<float> ud_args(const tbsci_ham *ham, const Plan *P, float) {
 
 // Whether a space takes this path. It wins at every shape and link density tried from
 // 2^14 determinants and two tiles of columns on (one vector, ms, against the SIMT kernels):
-//   150 x 150 strings, norb 12         FP64 0.11 / 0.20    FP32 0.09 / 0.12
-//   500 x 200, norb 14                 0.21 / 0.41         0.13 / 0.23
-//   1,200 x 1,100, norb 16             1.1 / 2.9           0.39 / 1.4
-//   1,800 x 1,800, norb 16, 3,100 non-zeros a determinant: 3.6 / 17.6 and 1.0 / 6.2
+//   160 x 155 strings, norb 12         FP64 0.11 / 0.21    FP32 0.07 / 0.12
+//   500 x 200, norb 14                 0.18 / 0.42         0.10 / 0.24
+//   1,200 x 1,100, norb 16             1.1 / 2.9           0.31 / 1.4
+//   1,800 x 1,800, norb 16             2.4 / 5.6           0.68 / 2.4
 // but not below: 100 x 100 0.09 / 0.09 and 0.08 / 0.06, 2,000 x 60 0.33 / 0.42 and 0.20 / 0.17.
 template <typename T>
 bool exact_eligible(const Plan *P) {
