@@ -103,6 +103,7 @@ struct DevBuf {
             e = cudaMalloc((void **)&p, count * sizeof(T));
         }
         if (e != cudaSuccess) {
+            cudaGetLastError();  // the caller has it: not to be found behind a later launch
             p = nullptr;
             return e;
         }

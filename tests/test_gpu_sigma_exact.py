@@ -270,6 +270,8 @@ def test_tables_make_room(tb, kind):
     nvec = 24  # the host call's buffers: 155 MB, more than any of the tables
     H = np.random.default_rng(9).standard_normal((nvec, sp.la, sp.lb))
     want = sp.sigma_host(H)
+    if pr:
+        pr.close()
     sp.close()
     ctx.close()
     extra = 1 << 16
@@ -301,4 +303,30 @@ def test_tables_make_room(tb, kind):
         pr.close()
     sp.close()
     assert tb.tbsci_hbm_used(ctx.handle) <= 2 * H.nbytes  # the host call's buffers, which the context keeps
+    ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_failed_allocation_leaves_nothing_behind(tb, dtype):
+    """A host call with more vectors than the device holds returns ENOMEM, after the tables were
+    taken back for it in vain. The next sigma makes them again (the same kernels, the same
+    bits), and so does the first one of a space prepared then."""
+    import torch
+    ctx = tb.Context(0)
+    C = np.random.default_rng(15).standard_normal((1, 640, 630))
+    c = torch.from_numpy(C).to(torch.float64 if dtype == "f64" else torch.float32).cuda()
+    sp, _, _, _ = _space(tb, ctx, 13, 6, 6, 640, 630, seed=793)
+    want = sp.sigma(c)
+    torch.cuda.synchronize()
+    with_tables = tb.tbsci_hbm_used(ctx.handle)
+    huge = (1 << 41) // (16 * sp.ndet)  # 2 TB of vectors: refused before any is read
+    out = np.empty(1)
+    for _ in range(2):
+        assert tb.B.load().tbsci_sigma_host(ctx.handle, sp.ham, sp.ta, sp.tb, tb.B._ptr(C), tb.B._ptr(out), huge) == tb.TBSCI_ENOMEM
+        assert torch.equal(sp.sigma(c), want)
+        assert tb.tbsci_hbm_used(ctx.handle) == with_tables
+        torch.cuda.synchronize()
+        sp.close()
+        sp, _, _, _ = _space(tb, ctx, 13, 6, 6, 640, 630, seed=793)  # not evaluated before the second turn's call
+    sp.close()
     ctx.close()
