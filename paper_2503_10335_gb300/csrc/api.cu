@@ -63,6 +63,11 @@ void Spare::retire() {
         }
 }
 
+void spare_forget(tbsci_ctx *ctx) {
+    std::lock_guard<std::mutex> g(spare_mu);
+    spares.erase(std::remove_if(spares.begin(), spares.end(), [&](const Spare *s) { return s->ctx == ctx; }), spares.end());
+}
+
 bool spare_reclaim(tbsci_ctx *ctx) {
     int dev = -1;
     if (!ctx && cudaGetDevice(&dev) != cudaSuccess) return false;
@@ -203,6 +208,7 @@ tbsci_status tbsci_hbm_used(const tbsci_ctx *ctx, size_t *bytes) {
 void tbsci_destroy(tbsci_ctx *ctx) {
     if (!ctx) return;
     cudaSetDevice(ctx->device);
+    spare_forget(ctx);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     if (ctx->copy_out) cudaStreamSynchronize(ctx->copy_out);
     if (!ctx->tune_path.empty()) tbsci_tune_cache_save(ctx, ctx->tune_path.c_str());

@@ -53,6 +53,8 @@ struct Spare {
 // Takes back what is not being enqueued at the moment: of one context, or (NULL) of all on
 // the current device. True where something was freed. Not to be called with a Spare's mu held.
 bool spare_reclaim(tbsci_ctx *ctx);
+// A context ends: what is left of its spare memory is not to be taken back through it
+void spare_forget(tbsci_ctx *ctx);
 
 // A failed device allocation returns ENOMEM (the context stays usable); any
 // other CUDA error returns ECUDA.

@@ -330,3 +330,27 @@ def test_failed_allocation_leaves_nothing_behind(tb, dtype):
         sp, _, _, _ = _space(tb, ctx, 13, 6, 6, 640, 630, seed=793)  # not evaluated before the second turn's call
     sp.close()
     ctx.close()
+
+
+def test_tables_of_an_ended_context(tb):
+    """A space that outlives its context keeps its tables out of what another context's failed
+    allocation takes back."""
+    import torch
+    gone = tb.Context(0)
+    sp, _, _, _ = _space(tb, gone, 13, 6, 6, 640, 630, seed=791)
+    sp.sigma(torch.randn((1, sp.la, sp.lb), dtype=torch.float64, device="cuda"))
+    torch.cuda.synchronize()
+    sp._handles = []  # its handles are not used again
+    gone.close()
+    ctx = tb.Context(0)
+    sp, osp, h, eri = _space(tb, ctx, 13, 6, 6, 640, 630, seed=792)
+    C = np.random.default_rng(14).standard_normal((1, sp.la, sp.lb))
+    c = torch.from_numpy(C).cuda()
+    want = sp.sigma(c)
+    torch.cuda.synchronize()
+    out = np.empty(1)
+    huge = (1 << 41) // (16 * sp.ndet)  # 2 TB of vectors, refused before any is read
+    assert tb.B.load().tbsci_sigma_host(ctx.handle, sp.ham, sp.ta, sp.tb, tb.B._ptr(C), tb.B._ptr(out), huge) == tb.TBSCI_ENOMEM
+    assert torch.equal(sp.sigma(c), want)  # the tables are made again
+    sp.close()
+    ctx.close()
