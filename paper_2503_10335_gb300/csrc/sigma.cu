@@ -485,8 +485,9 @@ __device__ void outliers_row(const OutlierArgs &A, int v, const double *C, doubl
 // The elements of sigma listed by the exact path (Coarse), a warp each: every term of the row
 // of H, lanes over the beta links and over the alpha links, added up in a fixed order. Behind
 // k_sigma_left, whose outliers they include. At most 64 single links per string.
-// Bound by the gathers of V and c: 244,000 elements of three vectors of 1,200 x 1,100 strings
-// in 0.85 ms.
+// Bound by the FP64 pipe, whose instructions run with the lanes that have a beta link (shuffled
+// alpha links with eight terms in flight gained nothing): 244,000 elements of three vectors of
+// 1,200 x 1,100 strings in 0.85 ms. A few elements take their latency, some 6 us.
 __global__ void __launch_bounds__(256) k_sigma_repair(SigArgs<double> A, const int *__restrict__ info, const Coarse R) {
     const int v = blockIdx.y, lane = threadIdx.x & 31;
     if (!info[2 * v]) return;
