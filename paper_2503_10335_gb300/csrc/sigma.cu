@@ -551,8 +551,8 @@ __global__ void __launch_bounds__(256) k_sigma_repair(SigArgs<double> A, const i
 // Its own kernel, so that k_sigma's arguments stay constants. One vector per CTA, since each
 // may be left or not: a vector of 1,200 x 1,100 strings at norb 16 takes 2.81 ms (2.92 with 512
 // threads), 2.63 with three of them in k_sigma.
-template <typename T, bool STAGE, bool ACCS>
-__global__ void __launch_bounds__(256) k_sigma_left(SigArgs<T> A, const int *__restrict__ skip, const OutlierArgs out) {
+template <typename T, bool STAGE, bool ACCS, int TH>
+__global__ void __launch_bounds__(TH) k_sigma_left(SigArgs<T> A, const int *__restrict__ skip, const OutlierArgs out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (skip[2 * blockIdx.y]) {
         if constexpr (sizeof(T) == 8)
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(256) k_sigma_left(SigArgs<T> A, const int *__r
     }
     A.C += blockIdx.y * A.vstride;
     A.S += blockIdx.y * A.vstride;
-    sigma_row<T, 1, STAGE, ACCS, 256>(A, A.rowsa[blockIdx.x], smem_raw);
+    sigma_row<T, 1, STAGE, ACCS, TH>(A, A.rowsa[blockIdx.x], smem_raw);
 }
 
 // SIMT pass of the tensor-core sigma types over row pairs: A.rowsa holds even
@@ -1433,13 +1433,19 @@ tbsci_status launch_small(tbsci_ctx *ctx, const tbsci_ham *ham, const Plan *P, c
     return TBSCI_OK;
 }
 
+// 256 threads; in FP64 512 from 2,000 columns on, where shared memory leaves an SM few CTAs
+// (1,500 rows, ms: 1,500 columns 4.29 / 4.32, 2,000 5.63 / 5.53, 3,500 11.5 / 11.0; 6,000 x 4,000,
+// three vectors: 255 / 240, and 240 in k_sigma)
 template <typename T, bool STAGE, bool ACCS>
 tbsci_status launch_left(tbsci_ctx *ctx, const SigArgs<T> &A, int nv, const int *skip, const OutlierArgs &out, cudaStream_t st) {
     const size_t sm = std::max(smem_bytes<T>(A.npair, A.lb, 1, STAGE, ACCS), (kOutliers + 1) * sizeof(int64_t));
-    auto k = k_sigma_left<T, STAGE, ACCS>;
+    auto k = k_sigma_left<T, STAGE, ACCS, 256>;
+    int th = 256;
+    if constexpr (sizeof(T) == 8)
+        if (A.lb >= 2000) k = k_sigma_left<T, STAGE, ACCS, 512>, th = 512;
     TB_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     TraceScope tr(ctx, "k_sigma_left", st);
-    k<<<dim3((unsigned)A.la, (unsigned)nv), 256, sm, st>>>(A, skip, out);
+    k<<<dim3((unsigned)A.la, (unsigned)nv), th, sm, st>>>(A, skip, out);
     TB_CUDA(ctx, cudaGetLastError());
     return TBSCI_OK;
 }
