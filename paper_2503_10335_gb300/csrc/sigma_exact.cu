@@ -150,7 +150,7 @@ constexpr double kCoarse = 1.0 / 16384;
 // norb 16: 3.5 ns against 2.1), and the digits save two thirds of that kernel: past a quarter
 // of the elements the vector goes there. Of the 60 vectors of a 20-iteration Davidson run on
 // these strings, 12 do (the first four iterations, on which most elements are still zero or
-// nearly so); the run takes 127 ms, 103 without this look at the elements, when some were off
+// nearly so); the run takes 130 ms, 103 without this look at the elements, when some were off
 // by up to 5e-9 of their terms, and 204 on the SIMT kernel.
 constexpr int64_t kCoarseShare = 4;
 
